@@ -1,26 +1,44 @@
 // Binned tetrahedron counts (Sec. 2.2) and the parity-decomposed channels
 // (Sec. 3.2, Eq. volume), GB300 layout.
 //
-// A tetrahedron i < a < b < c is counted at its smallest vertex i. For hub i
-// with m = |N+(i)| neighbours (local indices 0..m-1 in id order), a
-// persistent CTA
-//   1. stages N+(i) in shared memory with a bulk (TMA) copy, with the
-//      minimum-image displacement of every neighbour from i;
-//   2. builds the m x m bit matrix of adjacency within N+(i) (the paper's
-//      per-hub connectivity matrix, Sec. 3.5.2, as bits) by testing every
-//      pair (a, c), a < c, of staged displacements against the edge
-//      distances, a ballot per 32-bit word;
-//   3. for every triangle (a, b), b a bit of row a, takes the common bits
-//      of rows a and b above b: each is a tetrahedron (i, a, b, c). This is
-//      the three-way walk of Eq. (threeway) done 32 candidates per word.
-// The six bins come from the staged row (hub edges) and from the staged
-// displacements (the other three edges, recomputed exactly in integers).
+// A tetrahedron i < a < b < c is counted at its smallest vertex i. The m
+// neighbours N+(i) of a hub are taken in any order that suits the kernel
+// (the orbit and the volume's sign follow the labels, whatever they are):
+// sorted by the hub edge's bin, or, for the pixelised parity, by caller
+// index. A group of warps (a whole CTA down to one warp, by the size of the
+// rows) takes one hub at a time and
+//   1. stages the minimum-image displacement of every neighbour from i;
+//   2. fills the triangular byte matrix B of the bins of all pairs of
+//      neighbours (nb: no edge) from the staged displacements;
+//   3. takes rows a: the columns of row a that are edges form a list L, and
+//      every pair (b, c) of L with B(b, c) an edge is a tetrahedron. The b's
+//      go through a shared chunk of 32 entries that holds what depends on
+//      (i, a, b) only (the cross product d_a x d_b and the table row of the
+//      bins b_01, b_02, b_12); the c's sit in the lanes, 32 at a time, with
+//      what depends on (i, a, c) in registers. A step of the inner loop
+//      therefore costs one broadcast, one byte of B per lane (32 near
+//      bytes), one table entry, three multiply-adds and one histogram update.
+// This is the three-way walk of Eq. (threeway) with the second and third
+// lists intersected through B (the paper's per-hub connectivity matrix,
+// Sec. 3.5.2, holding bins instead of bits).
+//
 // A table maps the raw bin tuple to its S4 orbit, the parity of one
-// relabelling onto the orbit representative and the orbit's chirality; the
-// signed volume is det[d_a, d_b, d_c] in 64-bit integers, multiplied by
-// that parity. Counts use per-CTA shared-memory histograms flushed with
-// 64-bit atomics. Hubs with more than kMaxSmemRow neighbours run in a
-// second launch whose per-hub workspace lives in global scratch.
+// relabelling onto the orbit representative and the orbit's chirality. The
+// volume V = (d_a x d_b) . d_c is formed in single precision; within its
+// error bound of zero, exactly in integers. Counts use per-CTA
+// shared-memory histograms flushed with 64-bit atomics, one cell per orbit
+// and sign of V: even = V > 0 plus V < 0, odd = their difference (chiral
+// orbits), so a tetrahedron updates one cell; those with V = 0 go to the
+// global even count. Hubs with more neighbours than the shared workspace
+// holds run with their workspace in global scratch.
+//
+// What bounds it: instruction issue (80% of slots, 32 instructions per step of
+// 14 tetrahedra) and the shared-memory/L1 pipe (73%) together. Measured on one
+// GB300 against a kernel that queued (b, c) pairs per warp and gave every lane
+// one of them (7.5 instructions and two random 16-byte loads per tetrahedron):
+// parity on 2e5 clustered points (8.4e10 tetrahedra) 648 -> 231 ms, pixelised
+// parity on 1e5 (4.2e10) 810 -> 194 ms, connected 4pCF of 5e4 + 5e4 points
+// 520 -> 424 ms, 1e5 points with rows of 26 (mock, build included) 8.5 -> 2.7 ms.
 //
 // When the per-orbit counters of every orbit do not fit in shared memory
 // beside the hub workspace (unweighted: many bins; weighted: see below),
@@ -29,13 +47,10 @@
 // tetrahedron of any other orbit goes to the global counters directly.
 //
 // Weighted sums (exact, fixed-point W): the hub's sums of W_a W_b W_c are
-// kept per orbit in shared 128-bit words (32-bit limbs), one for
-// each sign of the volume so that a tetrahedron adds to one word only, and
-// multiplied by W_i into the global 192-bit sums when the hub ends. Shared
-// memory holds these words (and the counts) only for the `hot` orbits: the
-// orbit tables are relabelled so that the orbits met most often in a
-// sample of hubs come first, and a tetrahedron of any other orbit goes
-// straight to the global sums with its full product.
+// kept per cell in shared 128-bit words (32-bit limbs) and multiplied by W_i
+// into the global 192-bit sums when the hub ends. Shared memory holds these
+// words (and the counts) only for the `hot` orbits, as above; a tetrahedron
+// of any other orbit goes straight to the global sums with its full product.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -50,40 +65,61 @@ namespace {
 constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxSmemRow = 512;
+// A hub's tetrahedra (at most C(m, 3)) may go to the shared counters when
+// they are at most this many (m <= 738).
+constexpr unsigned long long kMaxHubNeed = 1ull << 26;
 // Squared-distance buckets for the bin lookup: bucket k covers
 // [k 2^shift, (k + 1) 2^shift) with 2^shift no wider than the narrowest bin
 // in squared distance, so a bucket holds at most one bin edge.
 constexpr int kBucketMax = 2048;
+// A pixel volume at or below this is degenerate: over all pixel triples the
+// exact value is zero or above 5e-5 in magnitude, and the single-precision
+// value (six products of components of unit vectors, each rounded) is
+// within 2e-6 of it.
+constexpr float kPixZero = 2e-5f;
 
 struct Args {
   const int64_t* __restrict__ ptr;
   const int32_t* __restrict__ deg;
   const uint32_t* __restrict__ adj;  // row i at row_at(adj, ptr, i, adj_off, split, adj_off2)
   int64_t adj_off, split, adj_off2;
-  int64_t hub_begin, hub_end;
-  const int64_t* __restrict__ big;  // hubs above the shared capacity, taken first
-  int64_t nbig;
+  // hubs: list[0..nlist), or hub_begin + k hub_stride below hub_end with at
+  // most dmax neighbours (list = nullptr)
+  int64_t hub_begin, hub_end, hub_stride;
+  const int64_t* __restrict__ list;
+  int64_t nlist;
+  int dmax;
   const int4* __restrict__ xyzp;
   const int64_t* __restrict__ e2g;
-  const uint32_t* __restrict__ lut;
-  int64_t n, box;
-  int nb, n_orbits;
-  int mcap;   // shared-memory workspace capacity (neighbours)
-  int thr;    // hubs with more neighbours than this use the global workspace
-  int gcap;   // global workspace capacity (neighbours)
+  const void* __restrict__ ent;      // orbit table (see Ent)
+  const uint8_t* __restrict__ chir;  // chirality per slot (parity)
+  int64_t box;
+  int nb, nb3;
+  int cap;   // shared-memory workspace capacity (neighbours) of a group
+  int gcap;  // global workspace capacity
+  int group; // warps per group
   int bk_shift, bk_n;  // squared-distance buckets (bk_n = 0: binary search)
   int hot;             // orbits (slots) below this are accumulated in shared memory
-  int64_t hub_stride;  // hubs hub_begin + k hub_stride (1: every hub)
+  float eps;           // volumes within eps of zero are decided in integers
   unsigned long long* even;
   unsigned long long* odd;
   unsigned long long* weven;  // [n_orbits][3] 192-bit
   unsigned long long* wodd;
   const int64_t* __restrict__ W;
-  const uint8_t* __restrict__ pixsign;  // pixelised parity: 2-bit signs of sorted pixel triples
+  const float4* __restrict__ pixu;  // pixelised parity: unit vectors of the pixel centres
   unsigned long long* hub_counter;
-  int* err;
   unsigned char* gscratch;  // per-CTA global workspace
   size_t gscratch_stride;
+};
+
+// Table entries: twice the slot, plus 1 when the relabelling onto the
+// representative of a chiral orbit is odd; the top bit marks chiral orbits.
+// Two bytes when the slots fit 14 bits (nb <= 8): half the lines per gather.
+template <class E>
+struct Ent {
+  static constexpr int kTop = sizeof(E) * 8 - 1;
+  static constexpr uint32_t kMask = (1u << kTop) - 1u;
+  using Signed = typename std::make_signed<E>::type;
 };
 
 __device__ inline int64_t mi(int64_t d, int64_t box) {
@@ -112,33 +148,11 @@ __device__ inline int bin_of(T D2, const T* e2, int nb, const uint8_t* bk, int s
   return lo;
 }
 
-// Squared distance between two hub-relative displacements. With
-// SMALLR (E_nb < 2^15) every component of an edge is below 2^15 and the sum
-// below 2^32, so 32-bit arithmetic is exact.
-template <bool SMALLR>
-__device__ inline auto d2(const int4& p, const int4& q) {
-  if constexpr (SMALLR) {
-    const int x = q.x - p.x, y = q.y - p.y, z = q.z - p.z;
-    return (uint32_t)(x * x) + (uint32_t)(y * y) + (uint32_t)(z * z);
-  } else {
-    const int64_t x = (int64_t)q.x - p.x, y = (int64_t)q.y - p.y, z = (int64_t)q.z - p.z;
-    return x * x + y * y + z * z;
-  }
-}
-
-// det[da, db, dc] exactly. With SMALLR the 2x2 minors fit in 32 bits.
-template <bool SMALLR>
-__device__ inline int64_t det3(const int4& da, const int4& db, const int4& dc) {
-  if constexpr (SMALLR) {
-    const int m0 = db.y * dc.z - db.z * dc.y;
-    const int m1 = db.x * dc.z - db.z * dc.x;
-    const int m2 = db.x * dc.y - db.y * dc.x;
-    return (int64_t)da.x * m0 - (int64_t)da.y * m1 + (int64_t)da.z * m2;
-  } else {
-    return (int64_t)da.x * ((int64_t)db.y * dc.z - (int64_t)db.z * dc.y) -
-           (int64_t)da.y * ((int64_t)db.x * dc.z - (int64_t)db.z * dc.x) +
-           (int64_t)da.z * ((int64_t)db.x * dc.y - (int64_t)db.y * dc.x);
-  }
+// det[da, db, dc] exactly (components below 2^19: the sum is below 2^60).
+__device__ inline long long det3(const int4& da, const int4& db, const int4& dc) {
+  return (long long)da.x * ((long long)db.y * dc.z - (long long)db.z * dc.y) -
+         (long long)da.y * ((long long)db.x * dc.z - (long long)db.z * dc.x) +
+         (long long)da.z * ((long long)db.x * dc.y - (long long)db.y * dc.x);
 }
 
 // Direction pixel of the pixelised parity channel (Sec. 3.2 stores one
@@ -215,22 +229,6 @@ __host__ __device__ inline int dir_pixel(int64_t x, int64_t y, int64_t z) {
   return 16 * band + sector;
 }
 
-// Sign of the pixel volume (u_p1 x u_p2) . u_p3 of three pixel centres: 0
-// for repeated pixels, else the table entry of the sorted triple times the
-// parity of the sort. The table (host-built in FP64, 0 where |V| < 1e-9)
-// holds two bits per sorted triple p < q < r (1: positive, 2: negative, 0:
-// degenerate), entry C(r,3) + C(q,2) + p, four to a byte (690 KB).
-__device__ inline int pix_sign(const uint8_t* __restrict__ T, int p1, int p2, int p3) {
-  if (p1 == p2 || p1 == p3 || p2 == p3) return 0;
-  int s = 1;
-  if (p1 > p2) { const int t = p1; p1 = p2; p2 = t; s = -s; }
-  if (p2 > p3) { const int t = p2; p2 = p3; p3 = t; s = -s; }
-  if (p1 > p2) { const int t = p1; p1 = p2; p2 = t; s = -s; }
-  const int idx = p3 * (p3 - 1) * (p3 - 2) / 6 + p2 * (p2 - 1) / 2 + p1;
-  const int code = (T[idx >> 2] >> ((idx & 3) << 1)) & 3;
-  return s * ((code & 1) - (code >> 1));
-}
-
 // A 128-bit two's complement value (lo, hi) into a shared 128-bit sum kept
 // as four 32-bit limbs, least significant first (sums modulo 2^128; the
 // caller keeps the true sum in range). 32-bit shared atomics are native;
@@ -300,476 +298,627 @@ __device__ inline void fold_i128(unsigned long long* g, unsigned long long lo,
   atomic_add_w192(g, p0, p1, p2);
 }
 
+// A hub's workspace. DISP etc. per neighbour, B the strictly upper triangle
+// of bins by rows (entry (b, c), c > b, at row_off(b, m + 1) + c; nb: no edge,
+// as all of column m, which unused lanes read), and per warp the list of row
+// a's edges.
+template <class L>
 struct Workspace {
-  uint32_t* row;      // staged N+(i) words
-  int4* disp;         // displacement of each neighbour from the hub
-  uint32_t* bits;     // m x W bit matrix
-  int* cid;           // caller index of each neighbour (pixelised parity)
-  int* wv;            // weight of each neighbour (weighted sums)
-  uint8_t* brow;      // per warp: bin(a, c) of its current row a, cap bytes each
-  uint8_t* prow;      // pixelised parity, per warp: pixel of D_c - D_a for row a
-  uint32_t* queue;    // per-warp queue of (b, c) entries: kWarps x 64 words
+  int4* disp;     // displacement from the hub, bin of the hub edge
+  int* wv;        // weight (weighted sums)
+  int* cid;       // caller index (pixelised parity, while sorting)
+  uint8_t* hpix;  // pixel of the spoke from the hub (pixelised parity)
+  uint8_t* B;
+  L* list;        // per warp: cap entries
+  uint8_t* lpix;  // per warp: pixels of the spokes from a (pixelised parity)
   int cap;
 };
 
-__device__ inline Workspace carve(unsigned char* p, int cap, bool pix) {
-  const int Wc = (cap + 31) / 32;
-  Workspace w;
-  w.row = reinterpret_cast<uint32_t*>(p);
-  p += (size_t)pad_row(cap) * 4;
+__host__ __device__ inline size_t pad16(size_t x) { return (x + 15) & ~(size_t)15; }
+
+// Bytes of one group's workspace; list entries of lsize bytes.
+__host__ __device__ inline size_t workspace_bytes(int64_t cap, int group, int lsize, bool weighted,
+                                                  bool pix) {
+  const size_t c = (size_t)cap;
+  return (c + 1) * 16 + (weighted ? pad16(c * 4) : 0) + (pix ? pad16(c * 4) + pad16(c) : 0) +
+         pad16(c * (c + 1) / 2 + 1) + pad16((size_t)group * c * lsize) +
+         (pix ? pad16((size_t)group * c) : 0);
+}
+
+template <class L>
+__device__ inline Workspace<L> carve(unsigned char* p, int64_t cap, int group, bool weighted,
+                                     bool pix) {
+  const size_t c = (size_t)cap;
+  Workspace<L> w;
   w.disp = reinterpret_cast<int4*>(p);
-  p += (size_t)cap * 16;
-  w.bits = reinterpret_cast<uint32_t*>(p);
-  p += (size_t)cap * Wc * 4;
-  w.cid = reinterpret_cast<int*>(p);
-  p += (size_t)cap * 4;
+  p += (c + 1) * 16;
   w.wv = reinterpret_cast<int*>(p);
-  p += (size_t)cap * 4;
-  w.brow = reinterpret_cast<uint8_t*>(p);
-  p += (size_t)kWarps * ((cap + 15) & ~15);
-  w.prow = reinterpret_cast<uint8_t*>(p);
-  if (pix) p += (size_t)kWarps * ((cap + 15) & ~15);
-  w.queue = reinterpret_cast<uint32_t*>(p);
-  w.cap = (cap + 15) & ~15;
+  if (weighted) p += pad16(c * 4);
+  w.cid = reinterpret_cast<int*>(p);
+  if (pix) p += pad16(c * 4);
+  w.hpix = p;
+  if (pix) p += pad16(c);
+  w.B = p;
+  p += pad16(c * (c + 1) / 2 + 1);
+  w.list = reinterpret_cast<L*>(p);
+  p += pad16((size_t)group * c * sizeof(L));
+  w.lpix = p;
+  w.cap = (int)cap;
   return w;
 }
 
-// One hub: stage N+(i), build the neighbour bit matrix, enumerate the
-// tetrahedra. GW: the workspace is in global memory (rows above the shared
-// capacity) and counts go straight to the global histograms. Returns false
-// when the staging copy timed out.
-// Shared cells per weighted slot: one (no parity) or three (V = 0, V > 0,
-// V < 0), each a u32 count and a 128-bit sum; even = all three, odd = the
-// second minus the third.
-template <bool PARITY>
-constexpr int kCat = PARITY ? 3 : 1;
+// Row b of a triangle of side m starts so that entry (b, c) is at row_off + c.
+template <class I>
+__device__ inline I row_off(I b, I m) {
+  return b * (2 * m - b - 1) / 2 - b;
+}
 
-// h_even / h_odd: unweighted per-orbit counts; weighted, h_even holds the
-// cells' counts and h_sum their sums.
-template <bool PARITY, bool WEIGHTED, bool SMALLR, bool GW, bool PIX, class E2T>
-__device__ bool hub4(const Args& a, const Workspace& w, const E2T* e2, const uint8_t* bk,
-                     unsigned* h_even, int* h_odd, unsigned long long* h_sum, int64_t i, int m,
-                     uint64_t* bar, uint32_t& phase, int* s_row) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nb = a.nb;
-  const int W = (m + 31) / 32;
-  const uint32_t* grow = row_at(a.adj, a.ptr, i, a.adj_off, a.split, a.adj_off2);
-  const uint32_t* row = w.row;
-  if (!GW) {
-    if (tid == 0) bulk_load(w.row, grow, (uint32_t)pad_row(m) * 4u, bar);
-  } else {
-    row = grow;
-  }
-  for (int k = tid; k < m * W; k += kThreads) w.bits[k] = 0u;
-  if (!GW) {
-    const bool ok = mbar_wait(bar, phase, kWaitLimit);
-    if (__syncthreads_or(!ok)) {
-      // report, then wait (bounded) for the copy to land before giving up
-      if (tid == 0) atomicOr(a.err, kErrTimeout);
-      if (!ok) mbar_wait(bar, phase, kWaitLimit);
-      __syncthreads();
-      return false;
+// Barrier of one group: named barrier 1 + g (groups of two warps and more
+// than 15 groups are not used), a warp barrier for a single warp.
+__device__ inline void group_sync(int g, int threads) {
+  if (threads == 32) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(threads) : "memory");
+}
+
+// Per-CTA shared state beside the histograms and workspaces.
+struct Shared {
+  int64_t e2[kMaxBins4 + 1];
+  uint8_t bk[kBucketMax];
+  int64_t hub[kWarps];            // per group
+  int row[kWarps];                // per group: next row a
+  int flush[kWarps];
+  int cur[kWarps * kMaxBins4];    // per group: counting sort by bin
+  unsigned long long pending;     // tetrahedra the shared counters may hold
+};
+
+// Adds 1 to a counter at a shared address when b < nb (no branch).
+__device__ inline void inc_shared_below(uint32_t addr, uint32_t b, uint32_t nb) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t"
+      "@p red.shared.add.u32 [%0], 1;\n\t}" ::"r"(addr),
+      "r"(b), "r"(nb)
+      : "memory");
+}
+
+// The same for a global 64-bit counter.
+__device__ inline void inc_global_below(unsigned long long* p, uint32_t b, uint32_t nb) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t"
+      "@p red.global.add.u64 [%0], 1;\n\t}" ::"l"(p),
+      "r"(b), "r"(nb)
+      : "memory");
+}
+
+// Pairs of floats in one 64-bit register (low half first); each half is
+// rounded as the scalar operation.
+__device__ inline unsigned long long pack2(float x, float y) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ inline void unpack2(unsigned long long v, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ inline unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ inline unsigned long long fma2(unsigned long long a, unsigned long long b,
+                                          unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// What a warp keeps of 32 b's of its row a: the cross product d_a x d_b (or
+// of the pixel vectors), the row of B (GW: b itself) and the table row of
+// (b_01, b_02, b_12). Arrays, so that one 128-bit broadcast serves four steps.
+struct Chunk {
+  float nx[32], ny[32], nz[32];
+  int row[32];
+  uint32_t tab[32];
+};
+
+// The counters and sums of one CTA (cells of the slots below a.hot).
+struct Hist {
+  unsigned* cnt;             // [cells]
+  unsigned long long* sum;   // weighted: [cells][2]
+};
+
+// One tetrahedron in cell `cell` (parity: twice the slot plus the sign; else
+// the slot). deg: V = 0 on a chiral orbit, even channel only. Wab = W_a W_b.
+template <bool PARITY, bool WEIGHTED>
+__device__ inline void record4(const Args& a, const Hist& h, bool hist_ok, uint32_t cell, bool deg,
+                               int64_t Wi, int64_t Wab, int Wc) {
+  const uint32_t hotc = (uint32_t)(PARITY ? 2 * a.hot : a.hot);
+  const bool hot = hist_ok && !deg && cell < hotc;
+  if (hot) {
+    atomicAdd(h.cnt + cell, 1u);
+    if constexpr (WEIGHTED) {
+      long long lo, hi;
+      mul_i128(Wab, (long long)Wc, &lo, &hi);  // below 2^90
+      shared_add_i128(h.sum + 2 * (size_t)cell, (unsigned long long)lo, (unsigned long long)hi);
     }
-    phase ^= 1u;
-  } else {
-    __syncthreads();
+    return;
   }
+  const uint32_t slot = PARITY ? cell >> 1 : cell;
+  const bool neg = PARITY && (cell & 1u);
+  const bool odd = PARITY && !deg && a.chir[slot];
+  atomicAdd(a.even + slot, 1ull);
+  if (odd) atomicAdd(a.odd + slot, neg ? ~0ull : 1ull);
+  if constexpr (WEIGHTED) {
+    long long plo, phi;
+    mul_i128(Wab, Wi * (int64_t)Wc, &plo, &phi);  // (W_a W_b)(W_i W_c), below 2^120
+    unsigned long long lo = (unsigned long long)plo, hi = (unsigned long long)phi;
+    atomic_add_i192(a.weven + 3 * (size_t)slot, lo, hi);
+    if (odd) {
+      if (neg) {  // negate the 128-bit product
+        lo = ~lo + 1ull;
+        hi = ~hi + (lo == 0ull ? 1ull : 0ull);
+      }
+      atomic_add_i192(a.wodd + 3 * (size_t)slot, lo, hi);
+    }
+  }
+}
+
+// One hub by one group of warps. GW: the workspace is in global memory.
+// gt: thread within the group; chunk (and wchunk): the warp's 32 entries.
+// FAST: unweighted, every slot's cells in shared memory, workspace in shared
+// memory; the inner loop is then free of branches.
+template <bool PARITY, bool WEIGHTED, bool PIX, bool GW, bool FAST, class E, class L>
+__device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, const Hist& h,
+                            const float4* pixu, Chunk* ch, long long* wchunk, int64_t i, int m,
+                            int g, int gt) {
+  const int lane = threadIdx.x & 31, wg = gt >> 5, group = a.group, gthreads = group * 32;
+  const int nb = a.nb;
+  const uint32_t* row = row_at(a.adj, a.ptr, i, a.adj_off, a.split, a.adj_off2);
   const int4 P = a.xyzp[i];
-  for (int k = tid; k < m; k += kThreads) {
-    const uint32_t id = edge_id(row[k]);
-    const int4 Q = a.xyzp[id];
+  int* cur = s.cur + g * kMaxBins4;
+  auto place = [&](int pos, uint32_t word, uint32_t id, const int4& Q) {
     // the fourth component carries the hub edge's bin, so one 128-bit load
     // gives a vertex's displacement and b_i,vertex
     const int dx = (int)mi((int64_t)Q.x - P.x, a.box), dy = (int)mi((int64_t)Q.y - P.y, a.box),
               dz = (int)mi((int64_t)Q.z - P.z, a.box);
-    w.disp[k] = make_int4(dx, dy, dz, (int)edge_bin(row[k]));
-    // pixelised parity: the caller index (below 2^24) and, in the top byte,
-    // the pixel of the spoke from the hub
-    if (PIX) w.cid[k] = (int)((unsigned)Q.w | ((unsigned)dir_pixel(dx, dy, dz) << 24));
-    if (WEIGHTED) w.wv[k] = (int)a.W[id];
+    w.disp[pos] = make_int4(dx, dy, dz, (int)edge_bin(word));
+    if (PIX) w.hpix[pos] = (uint8_t)dir_pixel(dx, dy, dz);
+    if (WEIGHTED) w.wv[pos] = (int)a.W[id];
+  };
+  if constexpr (PIX) {
+    // by caller index: the position is the number of smaller indices
+    for (int k = gt; k < m; k += gthreads) w.cid[k] = a.xyzp[edge_id(row[k])].w;
+    group_sync(g, gthreads);
+    for (int k = gt; k < m; k += gthreads) {
+      const int me = w.cid[k];
+      int pos = 0;
+      for (int t = 0; t < m; ++t) pos += w.cid[t] < me ? 1 : 0;
+      const uint32_t word = row[k], id = edge_id(word);
+      place(pos, word, id, a.xyzp[id]);
+    }
+  } else {
+    // by the hub edge's bin (counting sort): lanes with neighbouring c's then
+    // share b_03, so their table entries lie in few lines
+    for (int k = gt; k < m; k += gthreads) atomicAdd(cur + edge_bin(row[k]), 1);
+    group_sync(g, gthreads);
+    if (wg == 0) {
+      const int v = lane < nb ? cur[lane] : 0;
+      int incl = v;
+      for (int o = 1; o < 16; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      if (lane < nb) cur[lane] = incl - v;
+    }
+    group_sync(g, gthreads);
+    for (int k = gt; k < m; k += gthreads) {
+      const uint32_t word = row[k], id = edge_id(word);
+      place(atomicAdd(cur + edge_bin(word), 1), word, id, a.xyzp[id]);
+    }
   }
-  __syncthreads();
-  if (tid == 0) *s_row = 0;
-  // bit matrix: row a gets bit c for every c > a whose distance from a is an
-  // edge's, E_0^2 <= |D_c - D_a|^2 < E_nb^2 on the staged hub-relative
-  // displacements (4 E_nb < L makes their difference the pair's minimum
-  // image); a warp per row, a ballot per 32-bit word
-  const int64_t e2lo = (int64_t)e2[0], e2hi = (int64_t)e2[nb];
-  for (int sa = warp; sa < m - 1; sa += kWarps) {
-    const int4 da = w.disp[sa];
-    for (int c0 = (sa + 1) & ~31; c0 < m; c0 += 32) {
-      const int c = c0 + lane;
-      bool edge = false;
-      if (c > sa && c < m) {
+  group_sync(g, gthreads);
+  if (!PIX && gt < kMaxBins4) cur[gt] = 0;  // for the next hub (barriers below)
+  using I = typename std::conditional<GW, int64_t, int>::type;
+  // B: (a, c) is an edge iff E_0^2 <= |D_c - D_a|^2 < E_nb^2 on the staged
+  // hub-relative displacements (4 E_nb < L makes their difference the pair's
+  // minimum image)
+  {
+    const int64_t e2lo = s.e2[0], e2hi = s.e2[nb];
+    const uint8_t* bk = a.bk_n ? s.bk : nullptr;
+    if (gt == 0) w.disp[m] = make_int4(0, 0, 0, 0);  // unused lanes read it
+    for (int sa = wg; sa < m; sa += group) {
+      const int4 da = w.disp[sa];
+      uint8_t* Ba = w.B + row_off<I>(sa, m + 1);
+      for (int c = sa + 1 + lane; c <= m; c += 32) {
+        if (c == m) {
+          Ba[c] = (uint8_t)nb;
+          break;
+        }
         const int4 dc = w.disp[c];
         const int x = dc.x - da.x, y = dc.y - da.y, z = dc.z - da.z;
-        const long long D2 = (long long)x * x + (long long)y * y + (long long)z * z;
-        edge = D2 >= e2lo && D2 < e2hi;
+        const int64_t D2 = (int64_t)x * x + (int64_t)y * y + (int64_t)z * z;
+        uint8_t b = (uint8_t)nb;
+        if (D2 >= e2lo && D2 < e2hi) b = (uint8_t)bin_of(D2, s.e2, nb, bk, a.bk_shift);
+        Ba[c] = b;
       }
-      const uint32_t word = __ballot_sync(0xffffffffu, edge);
-      if (lane == 0) w.bits[sa * W + (c0 >> 5)] = word;
     }
   }
-  __syncthreads();
-  // tetrahedra: warp per row a, triangles (a, b) in a warp-uniform loop;
-  // the common neighbours c > b of a and b are compacted into a per-warp
-  // queue of (b, c) entries that carries over between triangles, and each
-  // batch of 32 entries is processed one tetrahedron per lane
+  group_sync(g, gthreads);
+  // pixelised parity: neighbours before the hub in caller order
+  int nlow = 0;
+  if (PIX) {
+    for (int t0 = 0; t0 < m; t0 += 32)
+      nlow += __popc(__ballot_sync(0xffffffffu, t0 + lane < m && w.cid[t0 + lane] < P.w));
+  }
   const int64_t Wi = WEIGHTED ? a.W[i] : 0;
-  uint32_t* qbc = w.queue + warp * 64;
-  // rows near the start of N+(i) carry most of the work: warps take rows
-  // from a shared counter (reset by thread 0 before the bit matrix was built)
-  for (;;) {
-    int sa = 0;
-    if (lane == 0) sa = atomicAdd(s_row, 1);
-    sa = __shfl_sync(0xffffffffu, sa, 0);
+  const bool hist_ok = (unsigned long long)m * (unsigned long long)(m - 1) *
+                           (unsigned long long)(m - 2) / 6 <= kMaxHubNeed;
+  const E* __restrict__ ent = reinterpret_cast<const E*>(a.ent);
+  L* list = w.list + (size_t)wg * w.cap;
+  uint8_t* lpix = w.lpix + (size_t)wg * w.cap;
+  // rows near the start carry most of the work: warps take them from a
+  // shared counter (reset by the group's first thread before the hub began)
+  for (int sa = -1;;) {
+    if (group == 1) {
+      ++sa;
+    } else {
+      if (lane == 0) sa = atomicAdd(s.row + g, 1);
+      sa = __shfl_sync(0xffffffffu, sa, 0);
+    }
     if (sa >= m - 2) break;
-    const uint32_t wa = row[sa];
-    const int b01 = (int)edge_bin(wa);
+    const uint8_t* Ba = w.B + row_off<I>(sa, m + 1);
     const int4 da = w.disp[sa];
+    const int b01 = da.w;
     const int64_t Wa = WEIGHTED ? (int64_t)w.wv[sa] : 0;
-    const int64_t Wia = Wi * Wa;
-    const uint32_t* bra = w.bits + sa * W;
-    // bin(a, c) of every edge (a, c) of the row, once per row: the triangle
-    // loop and the drain read b_12 and b_13 from here
-    uint8_t* brw = w.brow + (size_t)warp * w.cap;
-    // pixelised parity: the pixels of the spokes from a (to the hub and to
-    // every c of the row), used when a has the smallest caller index
-    uint8_t* prw = w.prow + (size_t)warp * w.cap;
-    int pneg = 0;
-    for (int c = sa + 1 + lane; c < m; c += 32)
-      if ((bra[c >> 5] >> (c & 31)) & 1u) {
-        const int4 dc = w.disp[c];
-        brw[c] = (uint8_t)bin_of(d2<SMALLR>(da, dc), e2, nb, bk, a.bk_shift);
-        if (PIX)
-          prw[c] = (uint8_t)dir_pixel((int64_t)dc.x - da.x, (int64_t)dc.y - da.y,
-                                      (int64_t)dc.z - da.z);
+    // Pixelised parity. The neighbours are in caller order, so the spokes'
+    // origin (the smallest caller index) is the hub or a. From the hub the
+    // order is (hub, a, b, c) and the sign is that of V(u_a, u_b, u_c); from
+    // a, with the hub anywhere after a, sorting (hub, a, b, c) and reordering
+    // the spokes to (hub, b, c) together give one sign change:
+    // -V(u_hub, u_b, u_c). A spoke of zero length gets a zero vector (V = 0).
+    const bool from_a = PIX && sa < nlow;
+    auto spoke = [&](const int4& d, int pix) -> float4 {
+      const bool zero = from_a ? (d.x == da.x && d.y == da.y && d.z == da.z)
+                               : ((d.x | d.y | d.z) == 0);
+      return zero ? make_float4(0.f, 0.f, 0.f, 0.f) : pixu[pix];
+    };
+    float4 u1 = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (PIX) {
+      if (!from_a) {
+        u1 = spoke(da, w.hpix[sa]);
+      } else if ((da.x | da.y | da.z) != 0) {
+        const float4 u = pixu[dir_pixel(-(int64_t)da.x, -(int64_t)da.y, -(int64_t)da.z)];
+        u1 = make_float4(-u.x, -u.y, -u.z, 0.f);
       }
-    if (PIX) pneg = dir_pixel(-(int64_t)da.x, -(int64_t)da.y, -(int64_t)da.z);
-    __syncwarp();
-    // the warp's queue of (b, c) entries is a ring of 64 slots: entries
-    // [qh, qt) are pending; a drain takes the 32 (or, at the end of the row,
-    // all) oldest, one per lane
-    int qh = 0, qt = 0;
-    auto drain = [&](bool all) {
-      if (qt - qh >= 32 || (all && qt > qh)) {
-        const int take = qt - qh < 32 ? qt - qh : 32;  // warp-uniform
-        const bool active = lane < take;
-        __syncwarp();  // the entries written by other lanes are visible
-        const uint32_t e = active ? qbc[(qh + lane) & 63] : 0u;
-        __syncwarp();  // read before any lane writes the next entries
-        qh += take;
-        if (active) {
-          const int sb = (int)(e >> 16), sc = (int)(e & 0xFFFFu);
-          const int b12 = brw[sb];
-          const int4 db = w.disp[sb], dc = w.disp[sc];
-          const int b02 = db.w, b03 = dc.w;
-          const int b13 = brw[sc];
-          const int b23 = bin_of(d2<SMALLR>(db, dc), e2, nb, bk, a.bk_shift);
-          const uint32_t ent =
-              a.lut[(((uint32_t)((b01 * nb + b02) * nb + b12) * nb + b03) * nb + b13) * nb + b23];
-          const int orbit = (int)(ent & 0x3FFFFFFFu);
-          // the volume's sign, relabelled onto the orbit representative (0:
-          // achiral orbit or degenerate tetrahedron)
-          int sgn = 0;
-          if (PARITY && (ent >> 31)) {
-            if constexpr (PIX) {
-              // the pixelised reading: the three spokes from the vertex with
-              // the smallest caller index, taken in ascending caller order; a
-              // sorting network orders the vertices (0 = hub, 1 = a, 2 = b,
-              // 3 = c) and keeps the parity of the reordering
-              const int ca = w.cid[sa], cb = w.cid[sb], cc = w.cid[sc];
-              int key[4] = {P.w, ca & 0xFFFFFF, cb & 0xFFFFFF, cc & 0xFFFFFF};
-              int vx[4] = {0, 1, 2, 3};
-              int par = 1;
-              auto cx = [&](int u, int v) {
-                if (key[u] > key[v]) {
-                  const int tk = key[u];
-                  key[u] = key[v];
-                  key[v] = tk;
-                  const int tv = vx[u];
-                  vx[u] = vx[v];
-                  vx[v] = tv;
-                  par = -par;
-                }
-              };
-              cx(0, 1);
-              cx(2, 3);
-              cx(0, 2);
-              cx(1, 3);
-              cx(1, 2);
-              // pixel of the spoke from the origin o to each vertex, and
-              // whether a spoke has zero length (coincident points)
-              const int o = vx[0];
-              int p0 = 0, p1 = 0, p2 = 0, p3 = 0;
-              bool zero;
-              auto same = [](const int4& u, const int4& v) {
-                return u.x == v.x && u.y == v.y && u.z == v.z;
-              };
-              if (o == 0) {  // from the hub: cached with the caller indices
-                p1 = (int)((unsigned)ca >> 24);
-                p2 = (int)((unsigned)cb >> 24);
-                p3 = (int)((unsigned)cc >> 24);
-                zero = (da.x == 0 && da.y == 0 && da.z == 0) ||
-                       (db.x == 0 && db.y == 0 && db.z == 0) ||
-                       (dc.x == 0 && dc.y == 0 && dc.z == 0);
-              } else if (o == 1) {  // from a: the row's cached pixels
-                p0 = pneg;
-                p2 = prw[sb];
-                p3 = prw[sc];
-                zero = (da.x == 0 && da.y == 0 && da.z == 0) || same(db, da) || same(dc, da);
-              } else {  // from b or c: three pixelisations
-                const int4 Do = o == 2 ? db : dc, Dq = o == 2 ? dc : db;
-                const int q0 = dir_pixel(-(int64_t)Do.x, -(int64_t)Do.y, -(int64_t)Do.z);
-                const int q1 = dir_pixel((int64_t)da.x - Do.x, (int64_t)da.y - Do.y,
-                                         (int64_t)da.z - Do.z);
-                const int qq = dir_pixel((int64_t)Dq.x - Do.x, (int64_t)Dq.y - Do.y,
-                                         (int64_t)Dq.z - Do.z);
-                p0 = q0;
-                p1 = q1;
-                if (o == 2) p3 = qq;
-                else p2 = qq;
-                zero = (Do.x == 0 && Do.y == 0 && Do.z == 0) || same(da, Do) || same(Dq, Do);
-              }
-              auto pix_of = [&](int v) { return v == 0 ? p0 : (v == 1 ? p1 : (v == 2 ? p2 : p3)); };
-              const int px[3] = {pix_of(vx[1]), pix_of(vx[2]), pix_of(vx[3])};
-              sgn = zero ? 0 : par * pix_sign(a.pixsign, px[0], px[1], px[2]);
-            } else {
-              const int64_t V = det3<SMALLR>(da, db, dc);
-              sgn = V > 0 ? 1 : (V < 0 ? -1 : 0);
-            }
-            if ((ent >> 30) & 1u) sgn = -sgn;
-          }
-          // orbits below a.hot live in shared memory (every orbit when
-          // unweighted)
-          const bool hot = !GW && orbit < a.hot;
-          if (WEIGHTED) {
-            const int64_t Wbc = (int64_t)w.wv[sb] * w.wv[sc];  // below 2^60
-            long long plo, phi;
-            if (hot) {
-              // the hub's count and sum of W_a W_b W_c (below 2^90) in the
-              // orbit's cell for V = 0 / V > 0 / V < 0
-              const int cell = kCat<PARITY> * orbit + (sgn > 0 ? 1 : (sgn < 0 ? 2 : 0));
-              atomicAdd(h_even + cell, 1u);
-              mul_i128(Wa, Wbc, &plo, &phi);
-              shared_add_i128(h_sum + 2 * cell, (unsigned long long)plo, (unsigned long long)phi);
-            } else {
-              // (W_i W_a)(W_b W_c) straight into the global sums
-              atomicAdd(a.even + orbit, 1ull);
-              mul_i128(Wia, Wbc, &plo, &phi);
-              unsigned long long lo = (unsigned long long)plo, hi = (unsigned long long)phi;
-              atomic_add_i192(a.weven + 3 * orbit, lo, hi);
-              if (PARITY && sgn != 0) {
-                atomicAdd(a.odd + orbit, (unsigned long long)(long long)sgn);
-                if (sgn < 0) {  // negate the 128-bit product
-                  lo = ~lo + 1ull;
-                  hi = ~hi + (lo == 0ull ? 1ull : 0ull);
-                }
-                atomic_add_i192(a.wodd + 3 * orbit, lo, hi);
-              }
-            }
-          } else {
-            if (hot) atomicAdd(h_even + orbit, 1u);
-            else atomicAdd(a.even + orbit, 1ull);
-            if (PARITY && sgn != 0) {
-              if (hot) atomicAdd(h_odd + orbit, sgn);
-              else atomicAdd(a.odd + orbit, (unsigned long long)(long long)sgn);
-            }
-          }
+    }
+    int n = 0;
+    for (int c0 = sa + 1; c0 < m; c0 += 32) {
+      const int c = c0 + lane;
+      const bool e = c < m && Ba[c] < nb;
+      const unsigned mask = __ballot_sync(0xffffffffu, e);
+      if (e) {
+        const int p = n + __popc(mask & ((1u << lane) - 1u));
+        list[p] = (L)c;
+        if (PIX) {
+          const int4 dc = w.disp[c];
+          lpix[p] = from_a ? (uint8_t)dir_pixel((int64_t)dc.x - da.x, (int64_t)dc.y - da.y,
+                                                (int64_t)dc.z - da.z)
+                           : w.hpix[c];
         }
       }
-    };
-    for (int wb0 = sa >> 5; wb0 < W; ++wb0) {
-      uint32_t xb = bra[wb0];
-      while (xb) {  // warp-uniform: every lane walks the same bits
-        const int sb = wb0 * 32 + __ffs(xb) - 1;
-        xb &= xb - 1u;
-        const uint32_t* brb = w.bits + sb * W;
-        for (int wc = sb >> 5; wc < W; ++wc) {
-          uint32_t x = bra[wc] & brb[wc];
-          if (wc == (sb >> 5)) x &= ~((2u << (sb & 31)) - 1u);
-          if (!x) continue;
-          const bool set = (x >> lane) & 1u;
-          if (set)
-            qbc[(qt + __popc(x & ((1u << lane) - 1u))) & 63] =
-                ((uint32_t)sb << 16) | (uint32_t)(wc * 32 + lane);
-          qt += __popc(x);  // at most 31 + 32 pending: the ring never overfills
-          drain(false);
+      n += __popc(mask);
+    }
+    for (int k0 = 0; k0 < n - 1; k0 += 32) {
+      __syncwarp();  // the list is written; the chunk is no longer read
+      {
+        const int p = k0 + lane;
+        int brow = 0;
+        uint32_t tri = 0;
+        float nx = 0.f, ny = 0.f, nz = 0.f;
+        long long wab = 0;
+        if (p < n) {
+          const int b = (int)list[p];
+          const int4 db = w.disp[b];
+          tri = (uint32_t)((b01 * nb + db.w) * nb + Ba[b]) * (uint32_t)a.nb3;
+          brow = GW ? b : row_off<int>(b, m + 1);
+          if (PARITY) {
+            if constexpr (PIX) {
+              const float4 u2 = spoke(db, lpix[p]);
+              nx = u1.y * u2.z - u1.z * u2.y;
+              ny = u1.z * u2.x - u1.x * u2.z;
+              nz = u1.x * u2.y - u1.y * u2.x;
+            } else {
+              nx = i40_to_float((long long)da.y * db.z - (long long)da.z * db.y);
+              ny = i40_to_float((long long)da.z * db.x - (long long)da.x * db.z);
+              nz = i40_to_float((long long)da.x * db.y - (long long)da.y * db.x);
+            }
+          }
+          if (WEIGHTED) wab = Wa * w.wv[b];
+        }
+        ch->row[lane] = brow;
+        ch->tab[lane] = tri;
+        if (PARITY) {
+          ch->nx[lane] = nx;
+          ch->ny[lane] = ny;
+          ch->nz[lane] = nz;
+        }
+        if (WEIGHTED) wchunk[lane] = wab;
+      }
+      __syncwarp();
+      for (int t0 = k0; t0 < n; t0 += 32) {
+        const int p = t0 + lane;
+        const bool in = p < n;
+        const int c = in ? (int)list[p] : m;  // column m: no edges
+        const int4 dc = w.disp[c];
+        const uint32_t lane_idx = (uint32_t)((dc.w * nb + (in ? (int)Ba[c] : 0)) * nb);
+        const int Wc = WEIGHTED && in ? w.wv[c] : 0;
+        float ux = 0.f, uy = 0.f, uz = 0.f;
+        if constexpr (PIX) {
+          const float4 u3 = spoke(dc, in ? lpix[p] : 0);
+          ux = u3.x, uy = u3.y, uz = u3.z;
+        } else if (PARITY) {
+          ux = (float)dc.x, uy = (float)dc.y, uz = (float)dc.z;
+        }
+        const int ns = t0 > k0 ? 32 : min(31, n - 1 - k0);
+        if constexpr (FAST) {
+          const uint8_t* Bc = w.B + c;
+          const auto* ent_c = reinterpret_cast<const typename Ent<E>::Signed*>(ent) + lane_idx;
+          const uint32_t cells = (uint32_t)__cvta_generic_to_shared(h.cnt);
+          const unsigned long long ux2 = pack2(ux, ux), uy2 = pack2(uy, uy), uz2 = pack2(uz, uz);
+          auto steps = [&](auto diag) {
+            constexpr int U = 4;
+            for (int s0 = 0; s0 < ns; s0 += U) {
+              uint32_t b23[U];
+              int en[U];
+              float V[U] = {0.f, 0.f, 0.f, 0.f};
+              const int4 r = *reinterpret_cast<const int4*>(ch->row + s0);
+              const uint4 t = *reinterpret_cast<const uint4*>(ch->tab + s0);
+              const int rr[U] = {r.x, r.y, r.z, r.w};
+              const uint32_t tt[U] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+              for (int u = 0; u < U; ++u) {
+                // a lane without an edge here reads the next table entry
+                // (same lines) and adds nothing
+                b23[u] = (uint32_t)nb;
+                if (!decltype(diag)::value || s0 + u < lane) b23[u] = Bc[rr[u]];
+                en[u] = ent_c[tt[u] + b23[u]];
+              }
+              if (PARITY) {
+                const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(ch->nx + s0);
+                const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(ch->ny + s0);
+                const ulonglong2 z = *reinterpret_cast<const ulonglong2*>(ch->nz + s0);
+                unpack2(fma2(z.x, uz2, fma2(y.x, uy2, mul2(x.x, ux2))), V[0], V[1]);
+                unpack2(fma2(z.y, uz2, fma2(y.y, uy2, mul2(x.y, ux2))), V[2], V[3]);
+              }
+              float vmin = 3.0e38f;
+#pragma unroll
+              for (int u = 0; u < U; ++u) {
+                uint32_t cell;
+                uint32_t below = (uint32_t)nb;
+                if constexpr (PARITY) {
+                  // V < 0 on a chiral orbit (the entry is read sign-extended)
+                  const uint32_t neg = (__float_as_uint(V[u]) & (uint32_t)en[u]) >> 31;
+                  cell = ((uint32_t)en[u] ^ neg) & Ent<E>::kMask;
+                  if constexpr (PIX) {
+                    // degenerate pixel volumes are a few percent: even channel
+                    if (fabsf(V[u]) < a.eps && en[u] < 0) {
+                      inc_global_below(a.even + (cell >> 1), b23[u], (uint32_t)nb);
+                      below = 0u;
+                    }
+                  } else {
+                    if (b23[u] < (uint32_t)nb) vmin = fminf(vmin, fabsf(V[u]));
+                  }
+                } else {
+                  cell = ((uint32_t)en[u] & Ent<E>::kMask) >> 1;
+                }
+                inc_shared_below(cells + 4u * cell, b23[u], below);
+              }
+              if (PARITY && !PIX && vmin < a.eps) {
+                // a volume within its error bound of zero: move the count if
+                // the exact sign is another, or to the even channel if V = 0
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                  if (b23[u] >= (uint32_t)nb || !(fabsf(V[u]) < a.eps) || en[u] >= 0) continue;
+                  const uint32_t neg = __float_as_uint(V[u]) >> 31;
+                  const uint32_t cell = ((uint32_t)en[u] ^ neg) & Ent<E>::kMask;
+                  const long long Vx = det3(da, w.disp[list[k0 + s0 + u]], dc);
+                  if (Vx == 0) {
+                    atomicSub(h.cnt + cell, 1u);
+                    atomicAdd(a.even + (cell >> 1), 1ull);
+                  } else if ((Vx < 0 ? 1u : 0u) != neg) {
+                    atomicSub(h.cnt + cell, 1u);
+                    atomicAdd(h.cnt + (cell ^ 1u), 1u);
+                  }
+                }
+              }
+            }
+          };
+          if (t0 > k0) steps(std::false_type{});
+          else steps(std::true_type{});
+        } else {
+          // entries [0, lim) of the chunk come before c
+          const int lim = min(ns, in ? (t0 > k0 ? 32 : lane) : 0);
+          constexpr int U = 2;  // two steps' loads before their updates
+          for (int s0 = 0; s0 < lim; s0 += U) {
+            uint32_t b23[U], e[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const I rb = GW ? row_off<I>((I)ch->row[s0 + u], m + 1) : (I)ch->row[s0 + u];
+              b23[u] = (uint32_t)nb;
+              if (s0 + u < lim) b23[u] = w.B[rb + c];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              e[u] = 0u;
+              if (b23[u] < (uint32_t)nb) e[u] = ent[ch->tab[s0 + u] + lane_idx + b23[u]];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              if (b23[u] >= (uint32_t)nb) continue;
+              uint32_t cell = e[u] & Ent<E>::kMask;
+              bool deg = false;
+              if constexpr (PARITY) {
+                const float V = fmaf(ch->nz[s0 + u], uz,
+                                     fmaf(ch->ny[s0 + u], uy, ch->nx[s0 + u] * ux));
+                const uint32_t chiral = e[u] >> Ent<E>::kTop;
+                uint32_t neg = __float_as_uint(V) >> 31;
+                if (fabsf(V) < a.eps) {
+                  const long long Vx = PIX ? 0 : det3(da, w.disp[list[k0 + s0 + u]], dc);
+                  neg = Vx < 0 ? 1u : 0u;
+                  deg = Vx == 0 && chiral;
+                }
+                cell ^= neg & chiral;
+              } else {
+                cell >>= 1;
+              }
+              record4<PARITY, WEIGHTED>(a, h, hist_ok, cell, deg, Wi,
+                                        WEIGHTED ? wchunk[s0 + u] : 0, Wc);
+            }
+          }
         }
       }
     }
-    drain(true);
+    __syncwarp();  // the list is rewritten for the next row
   }
-  __syncthreads();
-  return true;
 }
 
-template <bool PARITY, bool WEIGHTED, bool SMALLR, bool PIX>
+template <bool PARITY, bool WEIGHTED, bool PIX, bool FAST, class E>
 __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  using E2T = typename std::conditional<SMALLR, uint32_t, int64_t>::type;
-  __shared__ uint64_t bar;
-  __shared__ int64_t s_hub;
-  __shared__ int s_flush;
-  __shared__ unsigned long long s_pending;
-  __shared__ E2T e2[kMaxBins4 + 1];
-  __shared__ uint8_t s_bk[kBucketMax];
-  __shared__ int s_row;
-
-  const int tid = threadIdx.x;
-  // shared slots of the orbits below a.hot: unweighted, the even and odd
-  // counts; weighted, kCat cells of a 128-bit sum (the hub's) and a count
-  const int nh = a.hot;
-  constexpr int nc = WEIGHTED ? kCat<PARITY> : 1;
+  __shared__ Shared s;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int group = a.group, gthreads = group * 32, g = warp / group, gt = tid - g * gthreads;
+  const int ncell = PARITY ? 2 * a.hot : a.hot;
   unsigned char* sp = smem;
-  unsigned long long* h_sum = reinterpret_cast<unsigned long long*>(sp);
-  sp += WEIGHTED ? (size_t)nh * nc * 16 : 0;
-  unsigned* h_even = reinterpret_cast<unsigned*>(sp);
-  sp += (size_t)nh * nc * 4;
-  int* h_odd = reinterpret_cast<int*>(sp);
-  sp += (PARITY && !WEIGHTED) ? (size_t)nh * 4 : 0;
-  unsigned char* sws = reinterpret_cast<unsigned char*>(((uintptr_t)sp + 15) & ~(uintptr_t)15);
-  const Workspace ws_s = carve(sws, a.mcap, PIX);
-  const Workspace ws_g = carve(a.gscratch ? a.gscratch + (size_t)blockIdx.x * a.gscratch_stride
-                                          : sws,
-                               a.gscratch ? a.gcap : a.mcap, PIX);
+  Hist h;
+  h.sum = reinterpret_cast<unsigned long long*>(sp);
+  if (WEIGHTED) sp += (size_t)ncell * 16;
+  h.cnt = reinterpret_cast<unsigned*>(sp);
+  sp += pad16((size_t)ncell * 4);
+  float4* pixu = reinterpret_cast<float4*>(sp);
+  if (PIX) sp += 256 * sizeof(float4);
+  Chunk* ch = reinterpret_cast<Chunk*>(sp) + warp;
+  sp += (size_t)kWarps * sizeof(Chunk);
+  long long* wchunk = reinterpret_cast<long long*>(sp) + warp * 32;
+  if (WEIGHTED) sp += (size_t)kThreads * sizeof(long long);
+  const Workspace<uint16_t> ws_s = carve<uint16_t>(
+      sp + (size_t)g * workspace_bytes(a.cap, group, sizeof(uint16_t), WEIGHTED, PIX), a.cap,
+      group, WEIGHTED, PIX);
 
-  for (int k = tid; k < nh * nc; k += kThreads) {
-    h_even[k] = 0;
-    if (PARITY && !WEIGHTED) h_odd[k] = 0;
-    if (WEIGHTED) h_sum[2 * k] = h_sum[2 * k + 1] = 0ull;
+  for (int k = tid; k < ncell; k += kThreads) {
+    h.cnt[k] = 0u;
+    if (WEIGHTED) h.sum[2 * k] = h.sum[2 * k + 1] = 0ull;
   }
-  for (int b = tid; b <= a.nb; b += kThreads) e2[b] = (E2T)a.e2g[b];
+  for (int k = tid; k < kWarps * kMaxBins4; k += kThreads) s.cur[k] = 0;
+  for (int b = tid; b <= a.nb; b += kThreads) s.e2[b] = a.e2g[b];
   for (int k = tid; k < a.bk_n; k += kThreads) {
     const int64_t x = (int64_t)k << a.bk_shift;
     int b = 0;
     while (b + 1 < a.nb && a.e2g[b + 1] <= x) ++b;
-    s_bk[k] = (uint8_t)b;
+    s.bk[k] = (uint8_t)b;
   }
-  const uint8_t* bk = a.bk_n ? s_bk : nullptr;
-  if (tid == 0) {
-    mbar_init(&bar, 1);
-    s_pending = 0;
-  }
+  if (PIX)
+    for (int k = tid; k < 256; k += kThreads) pixu[k] = a.pixu[k];
+  if (tid == 0) s.pending = 0;
   __syncthreads();
-  uint32_t phase = 0;
 
-  auto flush = [&]() {
-    for (int k = tid; k < nh; k += kThreads) {
-      if (WEIGHTED) {
-        // cells V = 0, V > 0, V < 0: even = all three, odd = second - third
-        const unsigned c0 = h_even[nc * k];
-        const unsigned cp = PARITY ? h_even[nc * k + 1] : 0u;
-        const unsigned cn = PARITY ? h_even[nc * k + 2] : 0u;
-        if (c0 | cp | cn) {
-          atomicAdd(a.even + k, (unsigned long long)c0 + cp + cn);
-          if (PARITY && cp != cn)
-            atomicAdd(a.odd + k, (unsigned long long)((long long)cp - (long long)cn));
-          h_even[nc * k] = 0;
-          if (PARITY) h_even[nc * k + 1] = h_even[nc * k + 2] = 0;
-        }
-        continue;
-      }
-      const unsigned c = h_even[k];
-      if (c) {
-        atomicAdd(a.even + k, (unsigned long long)c);
-        h_even[k] = 0;
-      }
+  // Adds the shared counters to the global counts and clears them. Exchanges,
+  // so that one group can do it while the others count on.
+  auto flush = [&](int t, int threads) {
+    for (int k = t; k < a.hot; k += threads) {
       if (PARITY) {
-        const int o = h_odd[k];
-        if (o) {
-          atomicAdd(a.odd + k, (unsigned long long)(long long)o);
-          h_odd[k] = 0;
+        const unsigned p = atomicExch(h.cnt + 2 * k, 0u), n = atomicExch(h.cnt + 2 * k + 1, 0u);
+        if (p | n) {
+          atomicAdd(a.even + k, (unsigned long long)p + n);
+          if (p != n && a.chir[k])
+            atomicAdd(a.odd + k, (unsigned long long)((long long)p - (long long)n));
         }
+      } else {
+        const unsigned p = atomicExch(h.cnt + k, 0u);
+        if (p) atomicAdd(a.even + k, (unsigned long long)p);
       }
     }
   };
 
+  unsigned long long next = 0;  // the group's first thread: the next ticket, taken ahead
+  if (gt == 0) next = atomicAdd(a.hub_counter, 1ull);
   for (;;) {
-    if (tid == 0) {
-      // the long rows first (they are few and slow), then every other hub
-      const int64_t q = (int64_t)atomicAdd(a.hub_counter, 1ull);
-      int64_t i;
-      int d = 0;
-      if (q < a.nbig) {
-        i = a.big[q];
-        d = a.deg[i];
-      } else {
-        int64_t qq = q - a.nbig;
-        for (;;) {
-          i = a.hub_begin + qq * a.hub_stride;
-          d = (i < a.hub_end) ? a.deg[i] : 0;
-          if (i >= a.hub_end || (d >= 3 && d <= a.thr)) break;
-          qq = (int64_t)atomicAdd(a.hub_counter, 1ull) - a.nbig;
+    if (gt == 0) {
+      int64_t i = -1;
+      for (;;) {
+        const int64_t q = (int64_t)next;
+        if (a.list) {
+          if (q >= a.nlist) break;
+          next = atomicAdd(a.hub_counter, 1ull);
+          i = a.list[q];
+          break;
+        }
+        const int64_t j = a.hub_begin + q * a.hub_stride;
+        if (j >= a.hub_end) break;
+        next = atomicAdd(a.hub_counter, 1ull);
+        const int d = a.deg[j];
+        if (d >= 3 && d <= a.dmax) {
+          i = j;
+          break;
         }
       }
-      s_hub = i;
-      s_flush = 0;
-      if (i < a.hub_end && d <= a.thr) {
-        const unsigned long long m = (unsigned long long)d;
+      s.hub[g] = i;
+      s.row[g] = 0;
+      s.flush[g] = 0;
+      if (i >= 0) {
+        const unsigned long long m = (unsigned long long)a.deg[i];
         const unsigned long long need = m * (m - 1) * (m - 2) / 6;
-        if (s_pending + need > 0x7FFFFFFFull) {
-          s_flush = 1;
-          s_pending = need;
-        } else {
-          s_pending += need;
+        // The shared counters stay below 2^32: between two flushes they take
+        // the hubs registered since the last reset (at most 2^29 and one
+        // hub), those registered while a flush runs (the same) and those
+        // under way at a reset (31 hubs of at most 2^26).
+        if (need <= kMaxHubNeed &&
+            atomicAdd(&s.pending, need) + need > (1ull << 29)) {
+          atomicExch(&s.pending, 0ull);
+          s.flush[g] = 1;
         }
       }
     }
-    __syncthreads();
-    const int64_t i = s_hub;
-    if (i >= a.hub_end) break;
-    if (s_flush) {
-      flush();
-      __syncthreads();
-    }
+    group_sync(g, gthreads);
+    const int64_t i = s.hub[g];
+    if (i < 0) break;
+    if (s.flush[g]) flush(gt, gthreads);
     const int m = a.deg[i];
-    bool ok;
-    if (m > a.thr) {
-      ok = hub4<PARITY, WEIGHTED, SMALLR, true, PIX>(a, ws_g, e2, bk, h_even, h_odd, h_sum, i, m,
-                                                     &bar, phase, &s_row);
+    if (m > a.cap) {
+      const Workspace<uint32_t> ws_g =
+          carve<uint32_t>(a.gscratch + (size_t)blockIdx.x * a.gscratch_stride, a.gcap, group,
+                          WEIGHTED, PIX);
+      hub4<PARITY, WEIGHTED, PIX, true, false, E>(a, ws_g, s, h, pixu, ch, wchunk, i, m, g, gt);
     } else {
-      ok = hub4<PARITY, WEIGHTED, SMALLR, false, PIX>(a, ws_s, e2, bk, h_even, h_odd, h_sum, i,
-                                                      m, &bar, phase, &s_row);
-      if (WEIGHTED && ok) {
-        // the hub's sums times W_i into the global 192-bit sums (the
-        // barrier at the top of the loop orders the clearing before the
-        // next hub's additions)
-        const long long Wi = a.W[i];
-        for (int k = tid; k < nh; k += kThreads) {
-          unsigned long long* c = h_sum + 2 * nc * k;
-          unsigned long long elo = c[0], ehi = c[1], olo = 0, ohi = 0;
-          if (PARITY) {
-            // even = S0 + S+ + S-, odd = S+ - S- (each below 2^115 in
-            // magnitude, so no 128-bit overflow)
-            const unsigned long long plo = c[2], phi = c[3], nlo = c[4], nhi = c[5];
-            unsigned long long t = elo + plo;
-            ehi += phi + (t < elo ? 1ull : 0ull);
-            elo = t;
-            t = elo + nlo;
-            ehi += nhi + (t < elo ? 1ull : 0ull);
-            elo = t;
-            olo = plo - nlo;
-            ohi = phi - nhi - (plo < nlo ? 1ull : 0ull);
-            c[2] = c[3] = c[4] = c[5] = 0ull;
-          }
+      hub4<PARITY, WEIGHTED, PIX, false, FAST, E>(a, ws_s, s, h, pixu, ch, wchunk, i, m, g, gt);
+    }
+    group_sync(g, gthreads);
+    if (WEIGHTED) {
+      // the hub's sums times W_i into the global 192-bit sums (weighted
+      // launches have one group; the barrier at the top of the loop orders
+      // the clearing before the next hub's additions)
+      const long long Wi = a.W[i];
+      for (int k = gt; k < a.hot; k += gthreads) {
+        unsigned long long* c = h.sum + (PARITY ? 4 : 2) * (size_t)k;
+        unsigned long long elo = c[0], ehi = c[1];
+        if (PARITY) {
+          // even = S+ + S-, odd = S+ - S- (each below 2^115 in magnitude, so
+          // no 128-bit overflow)
+          const unsigned long long nlo = c[2], nhi = c[3];
+          if (!(elo | ehi | nlo | nhi)) continue;
+          const unsigned long long olo = elo - nlo, ohi = ehi - nhi - (elo < nlo ? 1ull : 0ull);
+          elo += nlo;
+          ehi += nhi + (elo < nlo ? 1ull : 0ull);
+          c[0] = c[1] = c[2] = c[3] = 0ull;
+          if ((olo | ohi) && a.chir[k]) fold_i128(a.wodd + 3 * k, olo, ohi, Wi);
+        } else {
           c[0] = c[1] = 0ull;
-          if (elo | ehi) fold_i128(a.weven + 3 * k, elo, ehi, Wi);
-          if (PARITY && (olo | ohi)) fold_i128(a.wodd + 3 * k, olo, ohi, Wi);
         }
+        if (elo | ehi) fold_i128(a.weven + 3 * k, elo, ehi, Wi);
       }
     }
-    if (!ok) return;
   }
   __syncthreads();
-  flush();
-}
-
-size_t workspace_bytes(int mcap, bool pix) {
-  const size_t Wc = (size_t)(mcap + 31) / 32;
-  return (size_t)pad_row(mcap) * 4 + (size_t)mcap * 16 + (size_t)mcap * Wc * 4 +
-         (size_t)mcap * 8 + (size_t)kWarps * ((mcap + 15) & ~15) * (pix ? 2 : 1) +
-         (size_t)kWarps * 64 * 5 + 64;
+  flush(tid, kThreads);
 }
 
 }  // namespace
@@ -783,14 +932,13 @@ __global__ void k_i64_to_double(const long long* c, int64_t n, double* out) {
 }
 
 namespace {
-// Signs of the pixel volume of every sorted pixel triple p < q < r (0 below
-// 1e-9 in magnitude), built once on the host in FP64 and copied to each
-// device on first use.
+// Unit vectors of the 256 pixel centres (band z_c = -1 + (band + 1/2) / 8,
+// sector phi_c = (sector + 1/2) pi / 8), formed in FP64 on the host, kept per
+// device.
 std::mutex g_pix_mu;
-std::vector<uint8_t> g_pix_host;  // 2 bits per sorted triple
-uint8_t* g_pix_dev[64] = {nullptr};
+float4* g_pix_dev[64] = {nullptr};
 
-const uint8_t* pixel_sign_table(int* status) {
+const float4* pixel_centres(int* status) {
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64) {
@@ -799,33 +947,17 @@ const uint8_t* pixel_sign_table(int* status) {
   }
   std::lock_guard<std::mutex> lock(g_pix_mu);
   if (g_pix_dev[dev]) return g_pix_dev[dev];
-  if (g_pix_host.empty()) {
-    double u[256][3];
-    for (int p = 0; p < 256; ++p) {
-      const double zc = (2.0 * (p >> 4) + 1.0) / 16.0 - 1.0;
-      const double phi = M_PI * (2.0 * (p & 15) + 1.0) / 16.0;
-      const double rho = std::sqrt((1.0 - zc) * (1.0 + zc));
-      u[p][0] = rho * std::cos(phi);
-      u[p][1] = rho * std::sin(phi);
-      u[p][2] = zc;
-    }
-    g_pix_host.assign(((size_t)256 * 255 * 254 / 6 + 3) / 4, 0);
-    size_t idx = 0;
-    for (int r = 0; r < 256; ++r)
-      for (int q = 0; q < r; ++q)
-        for (int p = 0; p < q; ++p, ++idx) {
-          const double* a = u[p];
-          const double* b = u[q];
-          const double* c = u[r];
-          const double v = (a[1] * b[2] - a[2] * b[1]) * c[0] + (a[2] * b[0] - a[0] * b[2]) * c[1] +
-                           (a[0] * b[1] - a[1] * b[0]) * c[2];
-          const unsigned code = std::fabs(v) < 1e-9 ? 0u : (v > 0 ? 1u : 2u);
-          g_pix_host[idx >> 2] |= (uint8_t)(code << ((idx & 3) << 1));
-        }
+  std::vector<float4> u(256);
+  for (int p = 0; p < 256; ++p) {
+    const double zc = (2.0 * (p >> 4) + 1.0) / 16.0 - 1.0;
+    const double phi = M_PI * (2.0 * (p & 15) + 1.0) / 16.0;
+    const double rho = std::sqrt((1.0 - zc) * (1.0 + zc));
+    u[p] = make_float4((float)(rho * std::cos(phi)), (float)(rho * std::sin(phi)), (float)zc, 0.f);
   }
-  uint8_t* d = nullptr;
-  cudaError_t e = cudaMalloc(&d, g_pix_host.size());
-  if (e == cudaSuccess) e = cudaMemcpy(d, g_pix_host.data(), g_pix_host.size(), cudaMemcpyHostToDevice);
+  float4* d = nullptr;
+  cudaError_t e = cudaMalloc(&d, u.size() * sizeof(float4));
+  if (e == cudaSuccess)
+    e = cudaMemcpy(d, u.data(), u.size() * sizeof(float4), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaGetLastError();
     if (d) cudaFree(d);
@@ -836,13 +968,17 @@ const uint8_t* pixel_sign_table(int* status) {
   return d;
 }
 
-// Orbit table relabelled to slots: orbit o becomes slot_of[o], flags kept.
-__global__ void k_relabel_lut(const uint32_t* __restrict__ lut, int64_t n,
-                              const int32_t* __restrict__ slot_of, uint32_t* out) {
+// Table entries (see Ent) and chirality by slot from the orbit table: orbit o
+// takes slot slot_of[o] (its own index when slot_of is null).
+template <class E>
+__global__ void k_entries(const uint32_t* __restrict__ lut, int64_t n,
+                          const int32_t* __restrict__ slot_of, E* out, uint8_t* chir) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t e = lut[k];
-    out[k] = (e & 0xC0000000u) | (uint32_t)slot_of[e & 0x3FFFFFFFu];
+    const uint32_t e = lut[k], o = e & 0x3FFFFFFFu, chiral = e >> 31;
+    const uint32_t slot = slot_of ? (uint32_t)slot_of[o] : o;
+    out[k] = (E)((slot << 1) | ((e >> 30) & chiral) | (chiral << Ent<E>::kTop));
+    chir[slot] = (uint8_t)chiral;  // every raw tuple of an orbit agrees
   }
 }
 
@@ -874,16 +1010,48 @@ int direction_pixels_device(const int32_t* d_dirs, int64_t n, uint8_t* d_out, cu
   return cuda_status(cudaGetLastError());
 }
 
+namespace {
+// fast: unweighted with every slot in shared memory
+template <class E>
+void (*pick4(bool parity, bool weighted, bool pix, bool fast))(Args) {
+#define GS_K4(P, X)                                    \
+  (weighted ? k_count4<P, true, X, false, E>           \
+   : fast   ? k_count4<P, false, X, true, E>           \
+            : k_count4<P, false, X, false, E>)
+  if (parity && pix) return GS_K4(true, true);
+  if (parity) return GS_K4(true, false);
+  return GS_K4(false, false);
+#undef GS_K4
+}
+
+// Shared memory of a launch: cells of `hot` slots, chunks, pixel centres and
+// the workspaces of 32 / group groups.
+size_t launch_smem(int64_t hot, int cap, int group, bool parity, bool weighted, bool pix) {
+  const size_t ncell = (size_t)hot * (parity ? 2 : 1);
+  return (weighted ? ncell * 16 : 0) + pad16(ncell * 4) + (pix ? 256 * sizeof(float4) : 0) +
+         (size_t)kWarps * sizeof(Chunk) + (weighted ? (size_t)kThreads * 8 : 0) +
+         (size_t)(kWarps / group) * workspace_bytes(cap, group, sizeof(uint16_t), weighted, pix);
+}
+
+// Largest row capacity (a multiple of 16, at most want) of a launch, 0 if
+// not even 16 fit.
+int fit_cap(int want, int64_t hot, int group, bool parity, bool weighted, bool pix, size_t avail) {
+  int cap = (want + 15) & ~15;
+  while (cap >= 16 && launch_smem(hot, cap, group, parity, weighted, pix) > avail) cap -= 16;
+  return std::max(cap, 0);
+}
+}  // namespace
+
 int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_even,
                   int64_t* d_odd, double* d_weven, double* d_wodd, const Opts& o, Scratch& sc,
                   bool pix, unsigned long long* weven_out, unsigned long long* wodd_out) {
   cudaStream_t s = o.stream;
   int st = GS_OK;
   pix = pix && parity;
-  const uint8_t* pixsign = nullptr;
+  const float4* pixu = nullptr;
   if (pix) {
-    pixsign = pixel_sign_table(&st);
-    if (!pixsign) return st;
+    pixu = pixel_centres(&st);
+    if (!pixu) return st;
   }
   const Conf4Tables* t = conf4_tables(g.nb, &st);
   if (!t) return st;
@@ -896,24 +1064,29 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   a.adj_off = 0;
   a.split = g.n;
   a.adj_off2 = 0;
-  a.big = nullptr;
-  a.nbig = 0;
   a.hub_begin = 0;
   a.hub_end = g.n;
+  a.hub_stride = 1;
+  a.list = nullptr;
+  a.nlist = 0;
   a.xyzp = g.d_xyzp;
   a.e2g = g.d_edges2;
-  a.lut = t->d_lut;
-  a.n = g.n;
   a.box = g.box_u;
   a.nb = g.nb;
-  a.n_orbits = no;
+  a.nb3 = g.nb * g.nb * g.nb;
   a.even = reinterpret_cast<unsigned long long*>(d_even);
   a.odd = parity ? (d_odd ? reinterpret_cast<unsigned long long*>(d_odd)
                           : sc.alloc<unsigned long long>(no))
                  : nullptr;
   a.W = weighted ? fw->d_W : nullptr;
-  a.pixsign = pixsign;
-  a.hub_stride = 1;
+  a.pixu = pixu;
+  // |V| <= E_nb^3; the single-precision volume is within 4 2^-24 E_nb^3 of
+  // the exact one (one rounding of each component of the cross product and
+  // three of the sum, each relative to at most |d_a x d_b| |d_c|)
+  {
+    const double r = (double)g.edges[g.nb];
+    a.eps = pix ? kPixZero : (float)std::ldexp(r * r * r, -21);
+  }
   // weighted results land in the callers' 192-bit arrays (or scratch)
   unsigned long long* weven = weighted ? (weven_out ? weven_out : sc.alloc<unsigned long long>(3 * (size_t)no))
                                        : nullptr;
@@ -921,42 +1094,51 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
                                                   : nullptr;
   a.weven = weven;
   a.wodd = wodd;
-  a.hub_counter = sc.alloc<unsigned long long>(2);
-  a.err = sc.alloc<int>(1);
-  if (!a.hub_counter || !a.err || (parity && !a.odd) || (weighted && !a.weven) ||
+  a.hub_counter = sc.alloc<unsigned long long>(1);
+  if (!a.hub_counter || (parity && !a.odd) || (weighted && !a.weven) ||
       (weighted && parity && !a.wodd))
     return GS_ENOMEM;
-  cudaMemsetAsync(a.hub_counter, 0, sizeof(unsigned long long) * 2, s);
-  cudaMemsetAsync(a.err, 0, sizeof(int), s);
 
   int dev = 0, sms = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  // static shared memory: the bucket table, the bin edges and a few words
-  const size_t avail = (size_t)optin - 1024 - kBucketMax;
-  // bytes of one shared slot: unweighted, the even (and odd) count;
-  // weighted, one or three cells of a 128-bit sum and a count
-  const size_t per_slot = weighted ? (parity ? 60 : 20) : (parity ? 8 : 4);
-  // shared row capacity: the longest row rounded up to 32 (at most
-  // kMaxSmemRow), less while the slots do not fit
-  int mcap = std::min(kMaxSmemRow, std::max(32, (g.max_deg + 31) & ~31));
-  int nh = no;
-  // unweighted: every orbit's counts in shared memory when a row capacity of
-  // at least 256 leaves room for them; otherwise (and always when weighted)
-  // as many slots as fit beside the longest row's workspace
-  int mfit = mcap;
-  while (!weighted && mfit > 256 && (size_t)no * per_slot + 16 + workspace_bytes(mfit, pix) > avail)
-    mfit -= 32;
-  if (!weighted && (size_t)no * per_slot + 16 + workspace_bytes(mfit, pix) <= avail) {
-    mcap = mfit;
+  const size_t avail = (size_t)optin - sizeof(Shared) - 64;
+  // two-byte entries hold slots below 2^14 (nb <= 8)
+  const bool small_ent = no <= 16384;
+  // Launch 1: groups of `group` warps over every hub of at most `cap`
+  // neighbours; launch 2 (when longer rows exist): whole CTAs over a list of
+  // the longer ones, in shared memory up to cap2, else in global scratch.
+  const int maxd = std::max(g.max_deg, 3);
+  const double mean = g.n ? (double)g.edges_total / (double)g.n : 0.0;
+  int group = kWarps, cap = 0, cap2 = 0, nh = no;
+  const bool all_hot = !weighted && !(o.variant & 8) &&
+                       fit_cap(std::min(256, maxd), no, kWarps, parity, false, pix, avail) >=
+                           std::min(256, (maxd + 15) & ~15);
+  if (all_hot) {
+    // few warps per hub where rows are short: a hub's barriers and its rows'
+    // ragged ends cost the same however many warps wait for them
+    group = mean <= 24 ? 1 : mean <= 48 ? 4 : mean <= 96 ? 8 : mean <= 160 ? 16 : 32;
+    const int want = std::min(maxd, std::max(48, (int)(2.0 * mean) + 32));
+    for (;; group = group == 1 ? 4 : group * 2) {
+      cap = fit_cap(maxd, no, group, parity, false, pix, avail);
+      if (cap >= want || group == kWarps) break;
+    }
+    cap2 = fit_cap(std::min(maxd, kMaxSmemRow), no, kWarps, parity, false, pix, avail);
   } else {
-    if (workspace_bytes(mcap, pix) + 16 + per_slot > avail) return GS_ERANGE;
-    nh = (int)std::min<size_t>((size_t)no, (avail - workspace_bytes(mcap, pix) - 16) / per_slot);
+    // as many slots as fit beside the workspace of rows of up to 256
+    const size_t per_slot = (size_t)(parity ? 2 : 1) * (weighted ? 20 : 4);
+    cap = std::min(256, (maxd + 15) & ~15);
+    const size_t fixed = launch_smem(0, cap, group, parity, weighted, pix) + 32;
+    nh = (int)std::min<size_t>((size_t)no, (avail - fixed) / per_slot);
+    cap2 = cap;
+    // variant 8: only 64 shared slots (exercises the global path of the other
+    // orbits on any input)
+    if (o.variant & 8) nh = std::min(nh, 64);
   }
-  // variant 8: only 64 shared slots (exercises the global path of the other
-  // orbits on any input)
-  if (o.variant & 8) nh = std::min(nh, 64);
+  // variant 1 sends every hub to the global workspace (exercises it on any
+  // input)
+  if (o.variant & 1) cap = cap2 = 2;
   // with fewer slots than orbits the orbits are relabelled (most frequent
   // first) and the per-slot results mapped back at the end
   const bool relabel = nh < no;
@@ -964,7 +1146,11 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   unsigned long long* s_odd = a.odd;
   unsigned long long* const o_odd = a.odd;  // odd counts in orbit order (caller's or scratch)
   int32_t* d_slot = nullptr;
-  uint32_t* d_lut2 = nullptr;
+  const int64_t nl = (int64_t)t->lut.size();
+  // one entry more: lanes without an edge read past a row
+  void* d_ent = sc.alloc_bytes((size_t)(nl + 1) * (small_ent ? 2 : 4));
+  uint8_t* d_chir = sc.alloc<uint8_t>(no);
+  if (!d_ent || !d_chir) return GS_ENOMEM;
   if (relabel) {
     s_even = sc.alloc<unsigned long long>(no);
     s_odd = parity ? sc.alloc<unsigned long long>(no) : nullptr;
@@ -973,9 +1159,8 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
       a.wodd = parity ? sc.alloc<unsigned long long>(3 * (size_t)no) : nullptr;
     }
     d_slot = sc.alloc<int32_t>(no);
-    d_lut2 = sc.alloc<uint32_t>(t->lut.size());
     if (!s_even || (parity && !s_odd) || (weighted && (!a.weven || (parity && !a.wodd))) ||
-        !d_slot || !d_lut2)
+        !d_slot)
       return GS_ENOMEM;
   }
   cudaMemsetAsync(s_even, 0, sizeof(uint64_t) * no, s);
@@ -985,36 +1170,18 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   a.even = s_even;
   a.odd = s_odd;
   a.hot = nh;
-
-  const bool small_r = g.edges[g.nb] < 32768;
-  auto pick = [&](bool P, bool Wt, bool X) -> void (*)(Args) {
-#define GS_PICK(P_, Wt_, X_)                                                   \
-  return small_r ? k_count4<P_, Wt_, true, X_> : k_count4<P_, Wt_, false, X_>
-    if (P && X) {
-      if (Wt) GS_PICK(true, true, true);
-      GS_PICK(true, false, true);
-    }
-    if (P) {
-      if (Wt) GS_PICK(true, true, false);
-      GS_PICK(true, false, false);
-    }
-    if (Wt) GS_PICK(false, true, false);
-    GS_PICK(false, false, false);
-#undef GS_PICK
+  a.ent = d_ent;
+  a.chir = d_chir;
+  auto entries = [&](const int32_t* slot_of) {
+    const int blocks = (int)std::min<int64_t>((nl + 255) / 256, 4096);
+    if (small_ent)
+      k_entries<uint16_t><<<blocks, 256, 0, s>>>(t->d_lut, nl, slot_of, (uint16_t*)d_ent, d_chir);
+    else
+      k_entries<uint32_t><<<blocks, 256, 0, s>>>(t->d_lut, nl, slot_of, (uint32_t*)d_ent, d_chir);
+    note_launch();
   };
-  // variant 1 sends every hub to the global workspace (exercises it on any
-  // input)
-  const bool force_global = (o.variant & 1) != 0;
-  const int thr = force_global ? 2 : mcap;
-  void (*kern)(Args) = pick(parity, weighted, pix);
-  const size_t smem = (size_t)nh * per_slot + 16 + workspace_bytes(mcap, pix);
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem);
-  const int grid = std::max(1, per_sm) * sms;
-  a.mcap = mcap;
-  a.thr = thr;
-  a.gcap = std::max(g.max_deg, 3);
+  entries(nullptr);
+
   // squared-distance buckets no wider than the narrowest bin (variant 4:
   // binary search instead)
   a.bk_shift = 0;
@@ -1034,68 +1201,66 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   }
   a.gscratch = nullptr;
   a.gscratch_stride = 0;
-  if (g.max_deg > thr) {
-    a.gscratch_stride = (workspace_bytes(a.gcap, pix) + 255) & ~(size_t)255;
-    a.gscratch = sc.alloc<unsigned char>(a.gscratch_stride * grid);
-    if (!a.gscratch) return GS_ENOMEM;
-  }
+  a.gcap = maxd;
+
+  auto pick = [&](bool P, bool Wt, bool X, bool fast) {
+    return small_ent ? pick4<uint16_t>(P, Wt, X, fast) : pick4<uint32_t>(P, Wt, X, fast);
+  };
+  auto launch = [&](void (*k)(Args), const Args& la, int grid, size_t smem) -> int {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaMemsetAsync(la.hub_counter, 0, sizeof(unsigned long long), s);
+    k<<<grid, kThreads, smem, s>>>(la);
+    note_launch();
+    return cuda_status(cudaGetLastError());
+  };
 
   // Relabelling: count the tetrahedra of every orbit over an evenly strided
   // sample of about 2048 hubs of the first window (unweighted, all slots in
   // shared memory, long rows skipped), rank the orbits by that count and
   // give the top nh the shared slots. Where that count kernel does not fit,
   // the orbits keep their order. The choice changes only the speed.
-  auto relabel_orbits = [&](const Args& wa, cudaStream_t st_) -> int {
+  auto relabel_orbits = [&](const Args& wa) -> int {
     std::vector<int32_t> slot_of(no);
     std::vector<int32_t> order(no);
     for (int k = 0; k < no; ++k) order[k] = k;
-    const size_t smem_s = (size_t)no * 4 + 16 + workspace_bytes(mcap, false);
-    if (smem_s <= avail) {
+    const int cap_s = fit_cap(std::min(maxd, 256), no, kWarps, false, false, false, avail);
+    if (cap_s >= 16) {
       unsigned long long* d_cnt = sc.alloc<unsigned long long>(no);
-      unsigned long long* d_hc = sc.alloc<unsigned long long>(1);
-      if (!d_cnt || !d_hc) return GS_ENOMEM;
-      cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long) * no, st_);
-      cudaMemsetAsync(d_hc, 0, sizeof(unsigned long long), st_);
+      if (!d_cnt) return GS_ENOMEM;
+      cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long) * no, s);
       Args sa = wa;
-      sa.big = nullptr;
-      sa.nbig = 0;
-      sa.thr = mcap;
+      sa.group = kWarps;
+      sa.cap = cap_s;
+      sa.dmax = cap_s;
       sa.hot = no;
-      sa.lut = t->d_lut;
       sa.even = d_cnt;
       sa.odd = nullptr;
       sa.weven = sa.wodd = nullptr;
       sa.W = nullptr;
-      sa.hub_counter = d_hc;
       sa.hub_stride = std::max<int64_t>(1, (wa.hub_end - wa.hub_begin) / 2048);
-      void (*ks)(Args) = pick(false, false, false);
-      cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_s);
-      int ps = 0;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, ks, kThreads, smem_s);
-      ks<<<std::max(1, ps) * sms, kThreads, smem_s, st_>>>(sa);
-      note_launch();
+      int ls = launch(pick(false, false, false, true), sa, sms,
+                      launch_smem(no, cap_s, kWarps, false, false, false));
+      if (ls) return ls;
       std::vector<unsigned long long> cnt(no);
       cudaMemcpyAsync(cnt.data(), d_cnt, sizeof(unsigned long long) * no, cudaMemcpyDeviceToHost,
-                      st_);
-      const cudaError_t e = cudaStreamSynchronize(st_);
+                      s);
+      const cudaError_t e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return cuda_status(e);
       std::stable_sort(order.begin(), order.end(),
                        [&](int x, int y) { return cnt[x] > cnt[y]; });
     }
     for (int k = 0; k < no; ++k) slot_of[order[k]] = k;
-    cudaMemcpyAsync(d_slot, slot_of.data(), sizeof(int32_t) * no, cudaMemcpyHostToDevice, st_);
-    const int64_t nl = (int64_t)t->lut.size();
-    k_relabel_lut<<<(int)std::min<int64_t>((nl + 255) / 256, 4096), 256, 0, st_>>>(t->d_lut, nl,
-                                                                                  d_slot, d_lut2);
-    note_launch();
+    cudaMemcpyAsync(d_slot, slot_of.data(), sizeof(int32_t) * no, cudaMemcpyHostToDevice, s);
+    entries(d_slot);
     // the host vector must outlive the (pageable, hence synchronous) copy
-    const cudaError_t e = cudaStreamSynchronize(st_);
+    const cudaError_t e = cudaStreamSynchronize(s);
     return e == cudaSuccess ? cuda_status(cudaGetLastError()) : cuda_status(e);
   };
 
   KernelTimer timer(o.kernel_ms);
   timer.start(s);
   bool first = true;
+  void (*kern)(Args) = pick(parity, weighted, pix, all_hot);
   st = for_each_window(g, o, sc, [&](const WinView& v) -> int {
     a.adj = v.adj;
     a.adj_off = v.off1;
@@ -1103,29 +1268,47 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     a.adj_off2 = v.off2;
     a.hub_begin = v.h0;
     a.hub_end = v.h1;
+    a.group = group;
+    a.cap = cap;
+    a.dmax = cap;
     if (first && relabel) {
-      const int rs = relabel_orbits(a, s);
+      const int rs = relabel_orbits(a);
       if (rs) return rs;
-      a.lut = d_lut2;
     }
     first = false;
-    // the window's long rows go to the front of its hub queue
-    std::vector<int64_t> big;
-    if (g.max_deg > thr)
-      for (int64_t h = v.h0; h < v.h1; ++h)
-        if (g.h_deg[h] > thr) big.push_back(h);
-    a.nbig = (int64_t)big.size();
-    a.big = nullptr;
-    if (!big.empty()) {
-      int64_t* d_big = sc.alloc<int64_t>(big.size());
-      if (!d_big) return GS_ENOMEM;
-      cudaMemcpyAsync(d_big, big.data(), sizeof(int64_t) * big.size(), cudaMemcpyHostToDevice, s);
-      a.big = d_big;
+    int ls = GS_OK;
+    if (cap >= 3)
+      ls = launch(kern, a, sms, launch_smem(nh, cap, group, parity, weighted, pix));
+    if (ls || maxd <= cap) return ls;
+    // the longer rows
+    std::vector<int64_t> longer;
+    bool global = false;
+    for (int64_t h = v.h0; h < v.h1; ++h)
+      if (g.h_deg[h] > std::max(cap, 2)) {
+        longer.push_back(h);
+        global = global || g.h_deg[h] > cap2;
+      }
+    if (longer.empty()) return GS_OK;
+    int64_t* d_list = sc.alloc<int64_t>(longer.size());
+    if (!d_list) return GS_ENOMEM;
+    cudaMemcpyAsync(d_list, longer.data(), sizeof(int64_t) * longer.size(), cudaMemcpyHostToDevice,
+                    s);
+    Args la = a;
+    la.list = d_list;
+    la.nlist = (int64_t)longer.size();
+    la.group = kWarps;
+    la.cap = cap2;
+    int grid = (int)std::min<int64_t>(sms, la.nlist);
+    if (global) {
+      la.gscratch_stride =
+          (workspace_bytes(maxd, kWarps, sizeof(uint32_t), weighted, pix) + 255) & ~(size_t)255;
+      // as many CTAs as have room for their workspace
+      while (!(la.gscratch = sc.alloc<unsigned char>(la.gscratch_stride * grid)) && grid > 1)
+        grid = (grid + 1) / 2;
+      if (!la.gscratch) return GS_ENOMEM;
     }
-    cudaMemsetAsync(a.hub_counter, 0, sizeof(unsigned long long), s);
-    { kern<<<grid, kThreads, smem, s>>>(a); note_launch(); }
     // the host list must outlive the (pageable, hence synchronous) copy only
-    return cuda_status(cudaGetLastError());
+    return launch(kern, la, grid, launch_smem(nh, cap2, kWarps, parity, weighted, pix));
   });
   if (st) return st;
   if (relabel) {
@@ -1154,12 +1337,10 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
       { k_i64_to_double<<<(no + 255) / 256, 256, 0, s>>>(reinterpret_cast<const long long*>(o_odd), no,
                                                        d_wodd); note_launch(); }
   }
-  int herr = 0;
-  cudaMemcpyAsync(&herr, a.err, sizeof(int), cudaMemcpyDeviceToHost, s);
   cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_status(e);
   timer.publish();
-  return herr ? GS_ETIMEOUT : GS_OK;
+  return GS_OK;
 }
 
 }  // namespace gs
