@@ -1,12 +1,16 @@
 // Lattice quantisation and the device radius-search graph build (Sec. 2.1).
 //
-// Points are binned into a uniform cell grid whose cells are at least
-// E_nb wide, so every neighbour lies in the 27 surrounding cells. Points are
-// relabelled in cell order (cell-major, caller index within a cell), which
-// makes rows come out sorted when the stencil cells are visited in
-// increasing cell order, and keeps neighbour ids close to the hub id (good
-// L2 locality for the counting kernels). Only the oriented half
+// Points are binned into a uniform cell grid, kx x ky x kz cells per E_nb
+// cubed, so every neighbour lies in a stencil of (2 kx + 1)(2 ky + 1)(2 kz + 1)
+// cells. Points are relabelled in cell order (x-major, caller index within a
+// cell), which makes rows come out sorted when the stencil's cells are
+// visited in increasing cell order, and keeps neighbour ids close to the hub
+// id (good L2 locality for the counting kernels). Only the oriented half
 // N+(i) = {j > i} is stored: every tuple is counted at its smallest label.
+// Thin cells along x make N+(i) nearly the half ball ahead of i, so rows are
+// of nearly equal length: with cells as wide as E_nb they varied by 75% about
+// the mean with the hub's place in its cell, which cost the triangle kernel
+// pair tests and the tetrahedron kernel its longest rows.
 #include <algorithm>
 
 #include "gs_internal.cuh"
@@ -15,11 +19,15 @@ namespace gs {
 namespace {
 
 constexpr int kMaxCellsPerAxis = 256;
-constexpr int kCellThreads = 512;   // row pass: one CTA per cell
-constexpr int kCellCap = 4096;      // stencil points staged in shared memory (64 KB)
+constexpr int kRowThreads = 256;    // row pass: a warp per group of hubs
+constexpr int kRowWarps = kRowThreads / 32;
+constexpr int kRowHubs = 4;         // hubs of one cell that a warp takes together
+constexpr int kMaxRuns = 96;        // id ranges of a stencil (9 x 5 columns, split in z)
+constexpr int kBucketMax = 2048;    // squared-distance buckets of the bin lookup
 
 struct GridDesc {
   int nc[3];
+  int k[3];          // cells per E_nb along each axis
   int64_t lo[3];     // open box: grid origin
   int64_t width[3];  // open box: cell width
   int64_t box;       // periodic box side, 0 = open
@@ -28,14 +36,6 @@ struct GridDesc {
 __device__ inline int cell_axis(const GridDesc& G, int a, int x) {
   if (G.box) return (int)(((int64_t)x * G.nc[a]) / G.box);
   return (int)(((int64_t)x - G.lo[a]) / G.width[a]);
-}
-
-__device__ inline int64_t min_image(int64_t d, int64_t box) {
-  if (box) {
-    if (2 * d >= box) d -= box;
-    else if (2 * d < -box) d += box;
-  }
-  return d;
 }
 
 __global__ void k_quantize(const double* pos, int64_t n3, int64_t box_u, int periodic,
@@ -116,179 +116,231 @@ __global__ void k_scatter(const int32_t* key, int64_t n, int32_t* cursor, int32_
 // Orders each cell by caller index: slot s goes to cell_start + rank, rank =
 // number of points of the same cell with a smaller caller index.
 __global__ void k_rank_in_cell(const int32_t* key, const int32_t* tmp, int64_t n,
-                               const int32_t* cell_start, const int32_t* cell_count,
-                               const int32_t* xyz, int4* xyzp) {
+                               const int32_t* cell_start, const int32_t* xyz, int4* xyzp,
+                               int32_t* cell) {
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
        s += (int64_t)gridDim.x * blockDim.x) {
     const int32_t me = tmp[s];
     const int c = key[me];
-    const int b = cell_start[c], e = b + cell_count[c];
+    const int b = cell_start[c], e = cell_start[c + 1];
     int r = 0;
     for (int t = b; t < e; ++t) r += tmp[t] < me;
     xyzp[b + r] = make_int4(xyz[3 * (int64_t)me], xyz[3 * (int64_t)me + 1],
                             xyz[3 * (int64_t)me + 2], me);
+    cell[b + r] = c;
   }
 }
 
-// Warp-wide ascending sort of one int per lane (bitonic network).
-__device__ inline int warp_sort_asc(int v) {
+// Id ranges of the later neighbours' cells: points [beg, end) seen at the
+// periodic image code (two bits per axis: image + 1).
+struct Run {
+  int beg, end, code, pad;
+};
+constexpr int kNoShift = 1 | (1 << 2) | (1 << 4);
+
+// The runs of hubs i0.. of the cell (cx, cy, cz): per column of the stencil
+// the cells cz - kz .. cz + kz are consecutive ids (two runs where they wrap).
+// Ids up to i0 are cut off. Runs come out in ascending order; at the faces of
+// a periodic box they are ranked first. Returns their number.
+__device__ inline int stencil_runs(const GridDesc& G, const int32_t* __restrict__ start, int cx,
+                                   int cy, int cz, int i0, Run* run, Run* tmp) {
   const int lane = threadIdx.x & 31;
-  for (int k = 2; k <= 32; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      const int o = __shfl_xor_sync(0xffffffffu, v, j);
-      const bool up = ((lane & k) == 0);
-      const bool lower = ((lane & j) == 0);
-      const int mn = min(v, o), mx = max(v, o);
-      v = (lower == up) ? mn : mx;
+  const unsigned below = (1u << lane) - 1u;
+  const bool per = G.box != 0;
+  const bool faces = per && (cx < G.k[0] || cx >= G.nc[0] - G.k[0] || cy < G.k[1] ||
+                             cy >= G.nc[1] - G.k[1] || cz < G.k[2] || cz >= G.nc[2] - G.k[2]);
+  const int wy = 2 * G.k[1] + 1, ncol = (2 * G.k[0] + 1) * wy;
+  Run* out = faces ? tmp : run;
+  int n = 0;
+  for (int q0 = 0; q0 < ncol; q0 += 32) {
+    const int q = q0 + lane;
+    int x = cx + q / wy - G.k[0], y = cy + q % wy - G.k[1];
+    int code = kNoShift;
+    bool ok = q < ncol;
+    if (x < 0) {
+      ok = ok && per;
+      x += G.nc[0];
+      code -= 1;
+    } else if (x >= G.nc[0]) {
+      ok = ok && per;
+      x -= G.nc[0];
+      code += 1;
     }
-  return v;
-}
-
-// Squared minimum-image distance of a candidate pair, or a value >= E_nb^2
-// when the pair cannot be an edge. SMALL: E_nb <= 2^16 and every
-// coordinate difference fits 31 bits (box or extent below 2^30), so the
-// test runs in 32-bit arithmetic: a pair with any |component| >= 2^16 is no
-// edge, and otherwise each squared component is below 2^32.
-template <bool SMALL>
-__device__ inline int64_t cand_d2(const int4& P, const int4& Q, int64_t box, int64_t e2hi) {
-  if constexpr (SMALL) {
-    const int bx = (int)box;
-    auto mi32 = [bx](int d) {
-      if (bx) {
-        if (2 * d >= bx) d -= bx;
-        else if (2 * d < -bx) d += bx;
+    if (y < 0) {
+      ok = ok && per;
+      y += G.nc[1];
+      code -= 1 << 2;
+    } else if (y >= G.nc[1]) {
+      ok = ok && per;
+      y -= G.nc[1];
+      code += 1 << 2;
+    }
+    const int64_t col = ((int64_t)x * G.nc[1] + y) * G.nc[2];
+    auto add = [&](bool use, int z0, int z1, int cd) {
+      Run r{0, 0, cd, 0};
+      if (use) {
+        r.beg = max(start[col + z0], i0 + 1);
+        r.end = start[col + z1 + 1];
       }
-      return d;
+      const bool v = r.beg < r.end;
+      const unsigned m = __ballot_sync(0xffffffffu, v);
+      if (v) out[n + __popc(m & below)] = r;
+      n += __popc(m);
     };
-    const unsigned ax = (unsigned)abs(mi32(Q.x - P.x)), ay = (unsigned)abs(mi32(Q.y - P.y)),
-                   az = (unsigned)abs(mi32(Q.z - P.z));
-    return (max(ax, max(ay, az)) >= 65536u)
-               ? e2hi
-               : (int64_t)((unsigned long long)(ax * ax) + (ay * ay) + (az * az));
-  } else {
-    const int64_t dx = min_image((int64_t)Q.x - P.x, box);
-    const int64_t dy = min_image((int64_t)Q.y - P.y, box);
-    const int64_t dz = min_image((int64_t)Q.z - P.z, box);
-    return dx * dx + dy * dy + dz * dz;
+    const int z0 = cz - G.k[2], z1 = cz + G.k[2];
+    add(ok, max(z0, 0), min(z1, G.nc[2] - 1), code);
+    if (faces) {
+      add(ok && z0 < 0, z0 + G.nc[2], G.nc[2] - 1, code - (1 << 4));
+      add(ok && z1 >= G.nc[2], 0, z1 - G.nc[2], code + (1 << 4));
+    }
   }
+  __syncwarp();
+  if (faces) {
+    for (int q = lane; q < n; q += 32) {
+      const Run r = tmp[q];
+      int rank = 0;
+      for (int t = 0; t < n; ++t) rank += tmp[t].beg < r.beg ? 1 : 0;
+      run[rank] = r;
+    }
+    __syncwarp();
+  }
+  return n;
 }
 
-// Row pass, one CTA per cell (persistent over cells): every hub of a cell
-// has the same stencil, the cells with index >= its own (in increasing
-// order, so rows come out sorted). The CTA copies the points of those
-// cells into shared memory once (up to cap points; a cell whose stencil
-// holds more reads them from global memory), then each warp takes one hub
-// of the cell at a time and tests every candidate j > i.
-// FILL = false counts |N+(i)|; FILL = true writes the packed words. Only
-// hubs in [h0, h1) are processed (chunked out-of-core builds).
-template <bool FILL, bool SMALL>
-__global__ void __launch_bounds__(kCellThreads) k_rows_cells(
-    const int4* __restrict__ xyzp, GridDesc G, int64_t ncell, const int32_t* __restrict__ cell_start,
-    const int32_t* __restrict__ cell_count, const int64_t* __restrict__ e2g, int nb,
-    int32_t* deg, const int64_t* __restrict__ ptr, uint32_t* __restrict__ adj, int64_t h0,
-    int64_t h1, int64_t out_off, int cap) {
-  extern __shared__ int4 s_cand[];
+// Row pass: a warp takes up to kRowHubs consecutive hubs of one cell (they
+// share the stencil) and tests every candidate of its runs against all of
+// them, lanes over candidates (128-bit coalesced loads through L1/L2); a
+// ballot compacts the hits, so rows come out sorted without a sort. The
+// image of a run is fixed by its cell, so a candidate costs three
+// subtractions and three 64-bit multiply-adds per hub.
+// FILL = false counts |N+(i)| and takes the totals; FILL = true writes the
+// packed words (and sums |N+(j)| over the edges). Only hubs in [h0, h1) are
+// processed (chunked out-of-core builds).
+// Bound by instruction issue; the two passes over 3e6 uniform points (402
+// edges a row, E_nb = 40 h^-1Mpc) take 19.5 ms against 48 ms for a CTA per
+// cell of side E_nb with the stencil staged in shared memory (twice the
+// candidates, one hub per warp at a time, per-candidate minimum images).
+template <bool FILL>
+__global__ void __launch_bounds__(kRowThreads) k_rows(
+    const int4* __restrict__ xyzp, const int32_t* __restrict__ cell, GridDesc G,
+    const int32_t* __restrict__ start, const int64_t* __restrict__ e2g, int nb, int bk_shift,
+    int bk_n, int32_t* deg, const int64_t* __restrict__ ptr, uint32_t* __restrict__ adj,
+    int64_t h0, int64_t h1, int64_t out_off, unsigned long long* totals) {
+  __shared__ Run s_run[2][kRowWarps][kMaxRuns];
   __shared__ int64_t e2[kMaxBins + 1];
-  __shared__ int s_beg[27], s_cnt[27], s_off[28], s_cell[27];
-  __shared__ int s_ncell;
-  for (int b = threadIdx.x; b <= nb; b += blockDim.x) e2[b] = e2g[b];
+  __shared__ uint8_t s_bk[kBucketMax];
+  for (int b = threadIdx.x; b <= nb; b += kRowThreads) e2[b] = e2g[b];
+  if (FILL)
+    for (int k = threadIdx.x; k < bk_n; k += kRowThreads) {
+      const int64_t x = (int64_t)k << bk_shift;
+      int b = 0;
+      while (b + 1 < nb && e2g[b + 1] <= x) ++b;
+      s_bk[k] = (uint8_t)b;
+    }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int kW = kCellThreads / 32;
-  const int64_t e2lo = e2[0], e2hi = e2[nb];
-  for (int64_t own = blockIdx.x; own < ncell; own += gridDim.x) {
-    const int64_t cb = cell_start[own], ce = cb + cell_count[own];
-    const int64_t hb = cb > h0 ? cb : h0, he = ce < h1 ? ce : h1;
-    if (hb >= he) continue;  // the same decision in every thread
-    if (warp == 0) {
-      const int c2 = (int)(own % G.nc[2]), c1 = (int)((own / G.nc[2]) % G.nc[1]),
-                c0 = (int)(own / ((int64_t)G.nc[1] * G.nc[2]));
-      int cell = INT_MAX;
-      if (lane < 27) {
-        int q[3] = {c0 + lane / 9 - 1, c1 + (lane / 3) % 3 - 1, c2 + lane % 3 - 1};
-        bool ok = true;
-        for (int a = 0; a < 3; ++a) {
-          if (G.box) q[a] = (q[a] + G.nc[a]) % G.nc[a];
-          else if (q[a] < 0 || q[a] >= G.nc[a]) ok = false;
+  const unsigned below = (1u << lane) - 1u;
+  Run* run = s_run[0][warp];
+  const unsigned long long e2lo = (unsigned long long)e2[0],
+                           span = (unsigned long long)(e2[nb] - e2[0]);
+  unsigned long long edges = 0, probe = 0;
+  int longest = 0;
+  const int64_t nblk = (h1 + kRowHubs - 1) / kRowHubs;
+  for (int64_t q = h0 / kRowHubs + blockIdx.x * (int64_t)kRowWarps + warp; q < nblk;
+       q += (int64_t)gridDim.x * kRowWarps) {
+    int i = (int)max(q * kRowHubs, h0);
+    const int iend = (int)min((q + 1) * kRowHubs, h1);
+    while (i < iend) {
+      const int c = cell[i];
+      int H = 1;
+      while (i + H < iend && cell[i + H] == c) ++H;
+      const int cz = c % G.nc[2], cy = (c / G.nc[2]) % G.nc[1], cx = c / (G.nc[2] * G.nc[1]);
+      const int nr = stencil_runs(G, start, cx, cy, cz, i, run, s_run[1][warp]);
+      // hubs beyond H repeat the last one and keep nothing
+      int4 P[kRowHubs];
+      int px[kRowHubs], py[kRowHubs], pz[kRowHubs], cnt[kRowHubs];
+      uint32_t* out[kRowHubs];
+#pragma unroll
+      for (int h = 0; h < kRowHubs; ++h) {
+        P[h] = xyzp[min(i + h, i + H - 1)];
+        px[h] = P[h].x, py[h] = P[h].y, pz[h] = P[h].z;
+        cnt[h] = 0;
+        out[h] = FILL ? adj + (ptr[min(i + h, i + H - 1)] - out_off) : nullptr;
+      }
+      int code = kNoShift;
+      for (int r = 0; r < nr; ++r) {
+        const Run R = run[r];
+        if (R.code != code) {  // the hubs as seen from the run's image
+          code = R.code;
+          const unsigned sx = (unsigned)((code & 3) - 1) * (unsigned)G.box,
+                         sy = (unsigned)(((code >> 2) & 3) - 1) * (unsigned)G.box,
+                         sz = (unsigned)((code >> 4) - 1) * (unsigned)G.box;
+#pragma unroll
+          for (int h = 0; h < kRowHubs; ++h) {
+            px[h] = (int)((unsigned)P[h].x - sx);
+            py[h] = (int)((unsigned)P[h].y - sy);
+            pz[h] = (int)((unsigned)P[h].z - sz);
+          }
         }
-        if (ok) cell = (q[0] * G.nc[1] + q[1]) * G.nc[2] + q[2];
-        if (cell < own) cell = INT_MAX;
-      }
-      cell = warp_sort_asc(cell);
-      const int prev = __shfl_up_sync(0xffffffffu, cell, 1);
-      if (lane > 0 && prev == cell) cell = INT_MAX;  // duplicate stencil cell
-      cell = warp_sort_asc(cell);                    // valid cells first
-      const unsigned valid = __ballot_sync(0xffffffffu, cell != INT_MAX);
-      int c = 0;
-      if (cell != INT_MAX) {
-        s_cell[lane] = cell;
-        s_beg[lane] = cell_start[cell];
-        c = cell_count[cell];
-        s_cnt[lane] = c;
-      }
-      // exclusive offsets of the cells' points in the staged copy
-      int incl = c;
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      if (lane < 27) s_off[lane + 1] = incl;
-      if (lane == 0) {
-        s_off[0] = 0;
-        s_ncell = __popc(valid);
-      }
-    }
-    __syncthreads();
-    const int ncs = s_ncell;
-    const bool staged = s_off[ncs] <= cap;
-    if (staged) {
-      for (int k = 0; k < ncs; ++k)
-        for (int t = threadIdx.x; t < s_cnt[k]; t += kCellThreads)
-          s_cand[s_off[k] + t] = xyzp[(int64_t)s_beg[k] + t];
-    }
-    __syncthreads();
-    for (int64_t i = hb + warp; i < he; i += kW) {
-      const int4 P = xyzp[i];
-      int64_t count = 0;
-      int64_t out = FILL ? ptr[i] - out_off : 0;
-      for (int k = 0; k < ncs; ++k) {
-        const int64_t b = s_beg[k], e = b + s_cnt[k];
-        const int64_t st = (s_cell[k] == own) ? i + 1 : b;
-        const int sk = s_off[k];
-        for (int64_t t0 = st; t0 < e; t0 += 32) {
-          const int64_t t = t0 + lane;
-          bool hit = false;
-          uint32_t word = 0;
-          if (t < e) {
-            const int4 Q = staged ? s_cand[sk + (int)(t - b)] : xyzp[t];
-            const int64_t D2 = cand_d2<SMALL>(P, Q, G.box, e2hi);
-            if (D2 >= e2lo && D2 < e2hi) {
-              hit = true;
-              if (FILL) {
-                int lo = 0, hi = nb;
-                while (hi - lo > 1) {
-                  const int mid = (lo + hi) >> 1;
-                  if (e2[mid] <= D2) lo = mid;
+        for (int t0 = R.beg; t0 < R.end; t0 += 32) {
+          const int t = t0 + lane;
+          const bool in = t < R.end;
+          const int4 Q = in ? xyzp[t] : make_int4(0, 0, 0, 0);
+          const int dt = FILL && in ? deg[t] : 0;
+#pragma unroll
+          for (int h = 0; h < kRowHubs; ++h) {
+            if (h >= H) continue;  // uniform
+            // modulo 2^32 on purpose: the true difference is a few cells
+            const int x = (int)((unsigned)Q.x - (unsigned)px[h]),
+                      y = (int)((unsigned)Q.y - (unsigned)py[h]),
+                      z = (int)((unsigned)Q.z - (unsigned)pz[h]);
+            const unsigned long long D2 = (unsigned long long)((long long)x * x + (long long)y * y +
+                                                               (long long)z * z);
+            const bool hit = in && t > i + h && D2 - e2lo < span;
+            const unsigned m = __ballot_sync(0xffffffffu, hit);
+            if (FILL && hit) {
+              int b;
+              if (bk_n) {
+                b = s_bk[D2 >> bk_shift];
+                b += (long long)D2 >= e2[b + 1] ? 1 : 0;
+              } else {
+                b = 0;
+                int hi = nb;
+                while (hi - b > 1) {
+                  const int mid = (b + hi) >> 1;
+                  if (e2[mid] <= (long long)D2) b = mid;
                   else hi = mid;
                 }
-                word = ((uint32_t)t << 8) | (uint32_t)lo;
               }
+              out[h][cnt[h] + __popc(m & below)] = ((uint32_t)t << 8) | (uint32_t)b;
+              probe += (unsigned long long)dt;
             }
+            cnt[h] += __popc(m);
           }
-          const unsigned m = __ballot_sync(0xffffffffu, hit);
-          if (FILL && hit) adj[out + __popc(m & ((1u << lane) - 1u))] = word;
-          out += __popc(m);
-          count += __popc(m);
         }
       }
-      if (!FILL) {
-        if (lane == 0) deg[i] = (int32_t)count;
-      } else {
-        const int64_t end = ptr[i + 1] - out_off;
-        for (int64_t p = out + lane; p < end; p += 32) adj[p] = kSentinel;
+#pragma unroll
+      for (int h = 0; h < kRowHubs; ++h) {
+        if (h >= H) continue;
+        if (!FILL) {
+          if (lane == 0) deg[i + h] = cnt[h];
+          edges += (unsigned long long)cnt[h];
+          longest = max(longest, cnt[h]);
+        } else {
+          const int pad = (int)pad_row(cnt[h]);
+          if (cnt[h] + lane < pad) out[h][cnt[h] + lane] = kSentinel;
+        }
       }
+      __syncwarp();  // the runs are rewritten for the next group
+      i += H;
     }
-    __syncthreads();  // the staged copy is rewritten for the next cell
+  }
+  if (FILL) {
+    for (int o = 16; o; o >>= 1) probe += __shfl_xor_sync(0xffffffffu, probe, o);
+    if (lane == 0 && probe) atomicAdd(totals, probe);
+  } else if (lane == 0) {
+    if (edges) atomicAdd(totals + 1, edges);
+    atomicMax((int*)(totals + 2), longest);
   }
 }
 
@@ -296,37 +348,6 @@ __global__ void k_pad_lengths(const int32_t* deg, int64_t n, int64_t* len) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= n;
        i += (int64_t)gridDim.x * blockDim.x)
     len[i] = (i < n) ? pad_row(deg[i]) : 0;
-}
-
-// probe[i] = sum over j in N+(i) of |N+(j)|, and the largest degree.
-__global__ void k_graph_stats(const int32_t* __restrict__ deg, const int64_t* __restrict__ ptr,
-                              const uint32_t* __restrict__ adj, int64_t adj_off, int64_t h0,
-                              int64_t h1, unsigned long long* probe_total,
-                              unsigned long long* edge_total, int* max_deg) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  unsigned long long pw = 0, ew = 0;
-  int md = 0;
-  for (int64_t i = h0 + blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < h1;
-       i += warps) {
-    const int d = deg[i];
-    const int64_t p = ptr[i] - adj_off;
-    for (int k = lane; k < d; k += 32) pw += (unsigned long long)deg[edge_id(adj[p + k])];
-    if (lane == 0) {
-      ew += (unsigned long long)d;
-      md = max(md, d);
-    }
-  }
-  for (int o = 16; o; o >>= 1) {
-    pw += __shfl_xor_sync(0xffffffffu, pw, o);
-    ew += __shfl_xor_sync(0xffffffffu, ew, o);
-    md = max(md, __shfl_xor_sync(0xffffffffu, md, o));
-  }
-  if (lane == 0) {
-    atomicAdd(probe_total, pw);
-    atomicAdd(edge_total, ew);
-    atomicMax(max_deg, md);
-  }
 }
 
 int grid_blocks(int64_t work, int threads) {
@@ -397,60 +418,77 @@ int build_graph_device(const int32_t* d_xyz, int64_t n, int64_t box_u,
   if (ce != cudaSuccess) return cuda_status(ce);
   if (h[6]) return GS_ERANGE;
 
+  // Cells of side E_nb, split further where they hold enough points to fill a
+  // warp's candidate loads: (4, 2, 2) from 32 points a cell on, where the
+  // stencil's later half shrinks from 14 to 7.1 E_nb^3 and rows become even,
+  // (2, 1, 1) from 8 on.
   GridDesc G;
   G.box = box_u;
-  for (int a = 0; a < 3; ++a) {
-    if (box_u) {
-      G.nc[a] = (int)std::max<int64_t>(1, std::min<int64_t>(box_u / rmax, kMaxCellsPerAxis));
-      G.lo[a] = 0;
-      G.width[a] = 0;
-    } else {
-      const int64_t ext = (int64_t)h[3 + a] - h[a];
-      G.lo[a] = h[a];
-      G.width[a] = std::max<int64_t>(rmax, ext / kMaxCellsPerAxis + 1);
-      G.nc[a] = (int)(ext / G.width[a] + 1);
+  auto grid = [&](int kx, int ky, int kz) {
+    const int k[3] = {kx, ky, kz};
+    for (int a = 0; a < 3; ++a) {
+      G.k[a] = k[a];
+      if (box_u) {
+        G.nc[a] = (int)std::max<int64_t>(1, std::min<int64_t>(box_u * k[a] / rmax,
+                                                              (int64_t)kMaxCellsPerAxis * k[a]));
+        G.lo[a] = 0;
+        G.width[a] = 0;
+      } else {
+        const int64_t ext = (int64_t)h[3 + a] - h[a];
+        G.lo[a] = h[a];
+        G.width[a] = std::max<int64_t>((rmax + k[a] - 1) / k[a],
+                                       ext / ((int64_t)kMaxCellsPerAxis * k[a]) + 1);
+        G.nc[a] = (int)(ext / G.width[a] + 1);
+      }
+      g->cells[a] = G.nc[a];
     }
-    g->cells[a] = G.nc[a];
-  }
-  const int64_t ncell = (int64_t)G.nc[0] * G.nc[1] * G.nc[2];
+    return (int64_t)G.nc[0] * G.nc[1] * G.nc[2];
+  };
+  int64_t ncell = grid(1, 1, 1);
+  if (n >= 32 * ncell) ncell = grid(4, 2, 2);
+  else if (n >= 8 * ncell) ncell = grid(2, 1, 1);
 
   int32_t* key = sc.alloc<int32_t>(n);
   int32_t* tmp = sc.alloc<int32_t>(n);
-  int32_t* cnt = sc.alloc<int32_t>(ncell);
-  int32_t* start = sc.alloc<int32_t>(ncell);
+  int32_t* start = sc.alloc<int32_t>(ncell + 1);
   int32_t* cursor = sc.alloc<int32_t>(ncell);
+  int32_t* cell = sc.alloc<int32_t>(n);
   int64_t* len = sc.alloc<int64_t>(n + 1);
-  if (!key || !tmp || !cnt || !start || !cursor || !len) return GS_ENOMEM;
-  cudaMemsetAsync(cnt, 0, sizeof(int32_t) * ncell, s);
-  { k_cell_keys<<<grid_blocks(n, 256), 256, 0, s>>>(d_xyz, n, G, key, cnt); note_launch(); }
-  st = scan_exclusive_i32(cnt, start, ncell, nullptr, s, sc);
+  if (!key || !tmp || !start || !cursor || !cell || !len) return GS_ENOMEM;
+  cudaMemsetAsync(start, 0, sizeof(int32_t) * (ncell + 1), s);
+  { k_cell_keys<<<grid_blocks(n, 256), 256, 0, s>>>(d_xyz, n, G, key, start); note_launch(); }
+  st = scan_exclusive_i32(start, start, ncell + 1, nullptr, s, sc);
   if (st) return st;
   cudaMemcpyAsync(cursor, start, sizeof(int32_t) * ncell, cudaMemcpyDeviceToDevice, s);
   { k_scatter<<<grid_blocks(n, 256), 256, 0, s>>>(key, n, cursor, tmp); note_launch(); }
-  { k_rank_in_cell<<<grid_blocks(n, 256), 256, 0, s>>>(key, tmp, n, start, cnt, d_xyz, g->d_xyzp); note_launch(); }
+  { k_rank_in_cell<<<grid_blocks(n, 256), 256, 0, s>>>(key, tmp, n, start, d_xyz, g->d_xyzp, cell); note_launch(); }
 
-  // row passes: persistent CTAs over the cells
-  const size_t cell_smem = (size_t)kCellCap * sizeof(int4);
-  // 32-bit candidate tests when E_nb <= 2^16 and coordinate differences fit
-  // 31 bits
-  // (variant bit 1: the 64-bit test everywhere)
-  bool small = rmax <= 65536 && !(o.variant & 1);
-  for (int a = 0; a < 3 && small; ++a)
-    small = box_u ? box_u < (int64_t(1) << 30) : (int64_t)h[3 + a] - h[a] < (int64_t(1) << 30);
-  auto rows_count = small ? k_rows_cells<false, true> : k_rows_cells<false, false>;
-  auto rows_fill = small ? k_rows_cells<true, true> : k_rows_cells<true, false>;
-  int dev = 0, sms = 0, per_sm = 0;
+  // squared-distance buckets no wider than the narrowest bin
+  int bk_shift = 0, bk_n = 0;
+  {
+    int64_t gap = INT64_MAX;
+    for (int b = 0; b < nb; ++b) gap = std::min(gap, e2[b + 1] - e2[b]);
+    while (bk_shift < 62 && (int64_t(1) << (bk_shift + 1)) <= gap) ++bk_shift;
+    const int64_t nbk = ((e2[nb] - 1) >> bk_shift) + 1;
+    if (nbk <= kBucketMax) bk_n = (int)nbk;
+  }
+  int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  for (auto k : {rows_count, rows_fill})
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cell_smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rows_fill, kCellThreads, cell_smem);
-  const int row_blocks = (int)std::min<int64_t>(ncell, (int64_t)std::max(1, per_sm) * sms * 8);
+  unsigned long long* tot = sc.alloc<unsigned long long>(3);  // probe words, edges, longest row
+  if (!tot) return GS_ENOMEM;
+  cudaMemsetAsync(tot, 0, sizeof(unsigned long long) * 3, s);
+  auto rows = [&](bool fill, uint32_t* adj, int64_t h0, int64_t h1, int64_t off) {
+    const int64_t groups = (h1 - h0 + kRowHubs - 1) / kRowHubs + 1;
+    const int blocks = (int)std::min<int64_t>((groups + kRowWarps - 1) / kRowWarps, sms * 16);
+    auto kern = fill ? k_rows<true> : k_rows<false>;
+    kern<<<blocks, kRowThreads, 0, s>>>(g->d_xyzp, cell, G, start, g->d_edges2, nb, bk_shift, bk_n,
+                                        g->d_deg, fill ? g->d_ptr : nullptr, adj, h0, h1, off, tot);
+    note_launch();
+  };
   KernelTimer timer(o.kernel_ms);
   timer.start(s);
-  { rows_count<<<row_blocks, kCellThreads, cell_smem, s>>>(g->d_xyzp, G, ncell, start, cnt,
-                                                          g->d_edges2, nb, g->d_deg, nullptr,
-                                                          nullptr, 0, n, 0, kCellCap); note_launch(); }
+  rows(false, nullptr, 0, n, 0);
   timer.stop(s);
   { k_pad_lengths<<<grid_blocks(n + 1, 256), 256, 0, s>>>(g->d_deg, n, len); note_launch(); }
   st = scan_exclusive_i64(len, g->d_ptr, n + 1, s, sc);
@@ -460,21 +498,14 @@ int build_graph_device(const int32_t* d_xyz, int64_t n, int64_t box_u,
   ce = cudaStreamSynchronize(s);
   if (ce != cudaSuccess) return cuda_status(ce);
   g->slots = g->h_ptr[n];
-  unsigned long long* tot = sc.alloc<unsigned long long>(3);
-  if (!tot) return GS_ENOMEM;
-  cudaMemsetAsync(tot, 0, sizeof(unsigned long long) * 3, s);
   const uint64_t edge_bytes = sizeof(uint32_t) * (uint64_t)g->slots;
   const bool out_of_core = o.force_windows > 0 || (o.budget && edge_bytes > o.budget);
   if (!out_of_core) {
     st = dev_alloc((void**)&g->d_adj, edge_bytes);
     if (st) return st;
     timer.start(s);
-    { rows_fill<<<row_blocks, kCellThreads, cell_smem, s>>>(g->d_xyzp, G, ncell, start, cnt,
-                                                           g->d_edges2, nb, g->d_deg, g->d_ptr,
-                                                           g->d_adj, 0, n, 0, kCellCap); note_launch(); }
+    rows(true, g->d_adj, 0, n, 0);
     timer.stop(s);
-    { k_graph_stats<<<grid_blocks(n * 32, 256), 256, 0, s>>>(g->d_deg, g->d_ptr, g->d_adj, 0, 0, n, tot,
-                                                           tot + 1, (int*)(tot + 2)); note_launch(); }
   } else {
     // Out of core: the edges live in pinned host memory. Rows are filled a
     // chunk of hubs at a time into a device staging buffer and copied out.
@@ -502,12 +533,8 @@ int build_graph_device(const int32_t* d_xyz, int64_t n, int64_t box_u,
       const int64_t off = g->h_ptr[h0];
       const int64_t words = g->h_ptr[h1] - off;
       timer.start(s);
-      { rows_fill<<<row_blocks, kCellThreads, cell_smem, s>>>(g->d_xyzp, G, ncell, start, cnt,
-                                                             g->d_edges2, nb, g->d_deg, g->d_ptr,
-                                                             stage, h0, h1, off, kCellCap); note_launch(); }
+      rows(true, stage, h0, h1, off);
       timer.stop(s);
-      { k_graph_stats<<<grid_blocks((h1 - h0) * 32, 256), 256, 0, s>>>(g->d_deg, g->d_ptr, stage, off, h0, h1,
-                                                                     tot, tot + 1, (int*)(tot + 2)); note_launch(); }
       ce = cudaMemcpyAsync(g->h_adj + off, stage, sizeof(uint32_t) * words, cudaMemcpyDeviceToHost, s);
       if (ce != cudaSuccess) return cuda_status(ce);
       ce = cudaStreamSynchronize(s);  // the staging buffer is reused
@@ -516,11 +543,11 @@ int build_graph_device(const int32_t* d_xyz, int64_t n, int64_t box_u,
     }
     std::vector<int32_t> hdeg(n);
     cudaMemcpy(hdeg.data(), g->d_deg, sizeof(int32_t) * n, cudaMemcpyDeviceToHost);
-    // first id of the last x-slab (cells are x-major); open boxes: n
+    // first id of the last E_nb in x (cells are x-major); open boxes: n
     g->wrap_start = n;
     if (box_u) {
       int32_t ws = 0;
-      const int64_t c_last = (int64_t)(G.nc[0] - 1) * G.nc[1] * G.nc[2];
+      const int64_t c_last = (int64_t)(G.nc[0] - G.k[0]) * G.nc[1] * G.nc[2];
       cudaMemcpy(&ws, start + c_last, sizeof(int32_t), cudaMemcpyDeviceToHost);
       g->wrap_start = ws;
     }
