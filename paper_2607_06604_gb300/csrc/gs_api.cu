@@ -412,6 +412,7 @@ int prepare_weights(const Graph& g, const float* w, FixedW* out, Scratch& sc, cu
   if (h[0] > h[1]) h[0] = h[1] = 0;  // all weights zero
   out->scale = 24 - h[0];
   out->bits = 25 + (h[1] - h[0]) + 1;
+  out->mag = 24 + (h[1] - h[0]);  // mantissas below 1
   out->nonneg = h[3] == 0;
   if (out->bits > max_bits) return GS_EUNSUPPORTED;
   { k_weight_fixed<<<304, 256, 0, s>>>(dw, g.d_xyzp, g.n, out->scale, W); note_launch(); }
@@ -433,6 +434,7 @@ int count3_wide(const Graph& g, const FixedW& fw, uint64_t* d_counts, double* d_
   ft.d_W = Wt;
   ft.scale = fw.scale;
   ft.bits = 30;
+  ft.mag = 29;
   ft.nonneg = false;
   int st = GS_OK;
   for (int k = 0; k < npts && !st; ++k) {
@@ -458,6 +460,7 @@ int count4_wide(const Graph& g, const FixedW& fw, bool parity, bool pix, uint64_
   ft.d_W = Wt;
   ft.scale = fw.scale;
   ft.bits = 30;
+  ft.mag = 29;
   ft.nonneg = false;
   for (int k = 0; k < npts && !st; ++k) {
     st = split_weights_device(fw, g.n, wide_eval_point(k), Wt, o.stream);

@@ -29,6 +29,8 @@
 // sums of W_j W_k kept in 32-bit limbs, multiplied by W_i into the CTA's
 // 128-bit sums, flushed into 192-bit global accumulators.
 #include <algorithm>
+#include <cmath>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -1141,6 +1143,480 @@ __global__ void __launch_bounds__(kPThreads, 2) k_count3p(PArgs a) {
   flush();
 }
 
+// ----------------------------------------------------------------------------
+// Tiled pair kernel (the default for evenly spaced bins). As k_count3p it
+// tests every pair (j, k) of N+(i) geometrically, with the pair test taken to
+// single precision and the operands to registers:
+//  * The row is dealt into tiles of at most 32 neighbours (neighbour t to tile
+//    t mod ntile, so a tile's lanes are spread over the row and their
+//    histogram cells over the banks). A work item is one pair of tiles: the
+//    k's sit in the lanes' registers, the j's are broadcast from shared
+//    memory, four per 128-bit load. A pair then costs a quarter of four
+//    broadcasts instead of a 16-byte load per lane.
+//  * The displacements are integers below 2^20, exact in single precision, and
+//    so are their differences. u = sqrt(D2) c + m, one fused multiply-add,
+//    puts the position of the pair in units of the bin width, in fixed point
+//    with 16 fraction bits, into the low mantissa bits of u: the bin is a
+//    shift away. A pair within the error bound (amb, below) of a bin edge is
+//    decided by integer comparisons instead; there are about 1e-4 of them.
+//  * Unweighted counts go to cells of the raw triple (b_ij, b_ik, b_jk), whose
+//    index is a sum of one term of j, one of k and the bin: no table lookup.
+//    Weighted cells are those of ({b_ij, b_ik}, b_jk); see below. A pair that
+//    is no edge goes to the extra bin nb, so that updates need no predicate
+//    (a predicated shared atomic is compiled to a branch, four instructions).
+// Bound by instruction issue and shared-memory atomics together; figures at
+// the launch rule (tile_launch).
+//
+// Weighted (exact): per hub and cell the sum of x = W_j W_k, |x| < 2^60, and
+// the number of pairs, in three 32-bit words updated by two shared atomics: lo
+// takes the low words of x (its carry goes on), Z takes (high word + carry)
+// 2^cb + 1, so its low cb bits count the pairs; T takes, rarely, the carries
+// out of Z (upper half, signed) and of Z's count field (lower half). fold
+// adds the cells of one configuration, multiplies by W_i and adds to the
+// CTA's 128-bit sums.
+struct TArgs {
+  Cat one;
+  const Cat* cats;      // batched launches
+  const int64_t* base;
+  int ncats;
+  int nb, nconf;
+  int cap;              // neighbours staged in shared memory per group (multiple of 32)
+  int group;            // warps per hub (all of the CTA's when weighted or batched)
+  float c, m;           // u = sqrt(D2) c + m
+  uint32_t amb;         // ambiguous iff the low 16 bits of u are <= amb
+  int cb;               // weighted: bits of Z's count field
+  const int64_t* e2g;
+  unsigned char* gscratch;  // hubs above cap: per-CTA staging in global memory
+  size_t gstride;
+  unsigned long long* hub_counter;
+};
+
+constexpr int kTThreads = 512;
+constexpr int kTWarps = kTThreads / 32;
+// Rows above this are left to the walk and pair kernels: C(8192, 2) < 2^25
+// pairs per hub keep the shared counters below 2^32 between flushes.
+constexpr int kTMaxDeg = 8192;
+// Absent j's and k's stand at these x (in units): farther from every point,
+// and from one another, than twice the largest E_nb (2^19).
+constexpr float kFarJ = 4.0e6f, kFarK = -4.0e6f;
+
+__device__ inline unsigned long long t_pack(float x, float y) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ inline void t_unpack(unsigned long long v, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ inline unsigned long long t_add(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ inline unsigned long long t_mul(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ inline unsigned long long t_fma(unsigned long long a, unsigned long long b,
+                                           unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ inline float t_sqrt(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// u of a pair in bin b lies in [kTileM + b, kTileM + b + 1): 16 fraction bits.
+constexpr float kTileM = 192.0f;
+constexpr uint32_t kTileBits = 0x43400000u;  // bits of kTileM
+constexpr int kTileMaxBins = 62;             // kTileM + nb + 1 below 256
+
+// The bin that u says, nb when none, plus kBin0 (taken off in the cells' base
+// address). LOWER: u may lie below kTileM.
+template <bool LOWER>
+constexpr uint32_t kBin0 = LOWER ? 0u : kTileBits >> 16;
+template <bool LOWER>
+__device__ inline uint32_t t_bin(float u, int nb) {
+  const uint32_t bits = __float_as_uint(u);
+  return min((LOWER ? bits - kTileBits : bits) >> 16, kBin0<LOWER> + (uint32_t)nb);
+}
+
+__device__ inline void t_red(uint32_t addr, uint32_t v) {
+  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ inline uint32_t t_atom(uint32_t addr, uint32_t v) {
+  uint32_t old;
+  asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(v) : "memory");
+  return old;
+}
+
+// Records a pair with weights Wj, Wk in the weighted cell at `at` (words lo,
+// Z, T, zoff bytes apart; scale = 2^cb).
+template <int WM>
+__device__ inline void t_record(uint32_t at, uint32_t zoff, int Wj, int Wk, uint32_t scale) {
+  const long long x = (long long)Wj * Wk;
+  const uint32_t x0 = (uint32_t)x;
+  const uint32_t o0 = t_atom(at, x0);
+  uint32_t x1, n, c;  // the high word with the low word's carry
+  asm("{\n\t.reg .u32 s;\n\tadd.cc.u32 s, %1, %2;\n\taddc.u32 %0, %3, 0;\n\t}"
+      : "=r"(x1)
+      : "r"(o0), "r"(x0), "r"((uint32_t)((unsigned long long)x >> 32)));
+  const uint32_t a1 = x1 * scale + 1u;
+  const uint32_t o1 = t_atom(at + zoff, a1);
+  asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, 0, 0;" : "=&r"(n), "=r"(c) : "r"(o1), "r"(a1));
+  if (WM != kExactPos) c -= (uint32_t)((int)a1 < 0 ? 1 : 0);  // sign extension
+  const bool wrap = (n & (scale - 1u)) == 0u;  // the count field has come round
+  if (wrap || c) t_red(at + 2u * zoff, (c << 16) + (wrap ? 1u : 0u));
+}
+
+// Staged neighbours of one hub, one array per quantity: x, y, z (float);
+// unweighted: p = b nb rows, q = b rows of nb + 1 cells; weighted: p =
+// b (b + 1) / 2 rows, q = b rows, W. p and q as byte offsets of 32-bit cells.
+struct Stage {
+  float *x, *y, *z;
+  int *p, *q, *W;
+};
+__host__ __device__ inline size_t stage_bytes(int64_t cap, bool weighted) {
+  return (size_t)cap * (weighted ? 24 : 20);
+}
+__device__ inline Stage stage_at(unsigned char* b, int64_t cap) {
+  Stage s;
+  s.x = reinterpret_cast<float*>(b);
+  s.y = s.x + cap;
+  s.z = s.y + cap;
+  s.p = reinterpret_cast<int*>(s.z + cap);
+  s.q = s.p + cap;
+  s.W = s.q + cap;
+  return s;
+}
+
+template <int WM, bool BATCH, bool LOWER>
+__global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
+  constexpr bool WEIGHTED = WM != kNone;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int nb = a.nb, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int group = a.group, gthreads = group * 32, g = warp / group, gt = tid - g * gthreads,
+            wg = gt >> 5;
+  const int npair = WEIGHTED ? nb * (nb + 1) / 2 : nb * nb;
+  const int nr = nb + 1;  // a row of cells: the bins of (j, k) and one for no edge
+  const int ncell = npair * nr;
+  unsigned char* sp = smem;
+  unsigned long long* whist = reinterpret_cast<unsigned long long*>(sp);  // [nconf][2]
+  if (WEIGHTED) sp += (size_t)a.nconf * 16;
+  int64_t* s_e2 = reinterpret_cast<int64_t*>(sp);
+  sp += ((size_t)(nb + 1) * 8 + 15) & ~(size_t)15;
+  uint32_t* s_cfg = reinterpret_cast<uint32_t*>(sp);  // sorted triple of each configuration
+  sp += ((size_t)a.nconf * 4 + 15) & ~(size_t)15;
+  unsigned* hist = reinterpret_cast<unsigned*>(sp);  // weighted: [nconf] counts
+  if (WEIGHTED) sp += ((size_t)a.nconf * 4 + 15) & ~(size_t)15;
+  unsigned* cell = reinterpret_cast<unsigned*>(sp);  // unweighted counts; weighted lo, Z, T
+  sp += ((size_t)ncell * (WEIGHTED ? 12 : 4) + 15) & ~(size_t)15;
+  const Stage st_s = stage_at(sp + (size_t)g * stage_bytes(a.cap, WEIGHTED), a.cap);
+  __shared__ int64_t s_hub[kTWarps];
+  __shared__ int s_flush[kTWarps], s_cat, s_cur;
+  __shared__ Cat s_c;  // batched: the current catalogue
+  __shared__ unsigned long long s_pending;
+
+  for (int k = tid; k < ncell * (WEIGHTED ? 3 : 1); k += kTThreads) cell[k] = 0u;
+  for (int k = tid; k < nb * nb * nb; k += kTThreads) {
+    const int p = k / (nb * nb), q = (k / nb) % nb, r = k % nb;
+    if (p <= q && q <= r) s_cfg[conf3_rank(p, q, r, nb)] = p | (q << 8) | (r << 16);
+  }
+  if (WEIGHTED)
+    for (int k = tid; k < a.nconf; k += kTThreads) {
+      hist[k] = 0u;
+      whist[2 * k] = whist[2 * k + 1] = 0ull;
+    }
+  for (int b = tid; b <= nb; b += kTThreads) s_e2[b] = a.e2g[b];
+  if (tid == 0) {
+    s_pending = 0;
+    s_cur = BATCH ? -1 : 0;
+  }
+  __syncthreads();
+  const Cat& c = BATCH ? s_c : a.one;
+  int cur = BATCH ? -1 : 0;
+
+  auto sync = [&]() {
+    if (gthreads == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(gthreads) : "memory");
+  };
+  // Adds the shared counts (and sums) to the global ones and clears them;
+  // exchanges, so that one group can do it while the others count on.
+  auto flush = [&](int t, int threads) {
+    if (cur < 0) return;
+    for (int k = t; k < a.nconf; k += threads) {
+      if constexpr (WEIGHTED) {
+        const unsigned v = hist[k];
+        if (v) {
+          atomicAdd(c.counts + k, (unsigned long long)v);
+          hist[k] = 0u;
+        }
+        const unsigned long long lo = whist[2 * k], hi = whist[2 * k + 1];
+        if (lo | hi) {
+          atomic_add_i192(c.wacc + 3 * k, lo, hi);
+          whist[2 * k] = whist[2 * k + 1] = 0ull;
+        }
+      } else {
+        const uint32_t f = s_cfg[k];
+        const int p = f & 255, q = (f >> 8) & 255, r = f >> 16;
+        unsigned long long v = 0;
+        auto take = [&](int x, int y, int z) {
+          v += atomicExch(cell + (x * nb + y) * nr + z, 0u);
+        };
+        take(p, q, r);
+        if (q != r) take(p, r, q);
+        if (p != q) take(q, p, r);
+        if (p != q) take(q, r, p);
+        if (p != r && q != r) take(r, p, q);
+        if (p != q && p != r && q != r) take(r, q, p);
+        if (v) atomicAdd(c.counts + k, v);
+      }
+    }
+  };
+  // Weighted: the hub's cells, times W_i, into the CTA's sums.
+  auto fold = [&](int64_t Wi) {
+    if constexpr (WEIGHTED) {
+      const uint32_t cm = (1u << a.cb) - 1u;
+      for (int k = tid; k < a.nconf; k += kTThreads) {
+        const uint32_t f = s_cfg[k];
+        const int p = f & 255, q = (f >> 8) & 255, r = f >> 16;
+        unsigned long long slo = 0, n = 0;
+        long long shi = 0;
+        auto take = [&](int x, int y, int z) {  // x <= y the hub edges' bins
+          const int i = (y * (y + 1) / 2 + x) * nr + z;
+          const uint32_t lo = cell[i], Z = cell[ncell + i], T = cell[2 * ncell + i];
+          if (!(lo | Z | T)) return;
+          cell[i] = cell[ncell + i] = 0u;
+          if (T) cell[2 * ncell + i] = 0u;
+          const long long num = (long long)(((unsigned long long)(T & 0xFFFFu) << a.cb) + (Z & cm));
+          // Z with its carries: H 2^cb + num
+          const long long full = (long long)(((unsigned long long)(long long)((int)T >> 16) << 32) |
+                                             Z);
+          const long long H = (full - num) >> a.cb;
+          n += (unsigned long long)num;
+          const unsigned long long add = ((unsigned long long)H << 32) | lo;
+          slo += add;
+          shi += (H >> 32) + (slo < add ? 1 : 0);
+        };
+        take(p, q, r);
+        if (q != r) take(p, r, q);
+        if (p != q) take(q, r, p);
+        if (!n) continue;
+        hist[k] += (unsigned)n;
+        // (shi, slo) W_i modulo 2^128
+        const unsigned long long w = (unsigned long long)Wi;
+        const unsigned long long plo = slo * w;
+        const unsigned long long phi = __umul64hi(slo, w) - (Wi < 0 ? slo : 0ull) +
+                                       (unsigned long long)shi * w;
+        const unsigned long long old = whist[2 * k], now = old + plo;
+        whist[2 * k] = now;
+        whist[2 * k + 1] += phi + (now < old ? 1ull : 0ull);
+      }
+    }
+  };
+
+  const uint32_t s_cell = (uint32_t)__cvta_generic_to_shared(cell);
+  [[maybe_unused]] const uint32_t zoff = (uint32_t)ncell * 4u, scale = 1u << a.cb;
+  // Exact bin of a pair near a bin edge, nb when it is no edge.
+  auto exact_bin = [&](float dx, float dy, float dz) -> int {
+    const long long x = (long long)(int)dx, y = (long long)(int)dy, z = (long long)(int)dz;
+    const long long D2 = x * x + y * y + z * z;
+    if (D2 < s_e2[0] || D2 >= s_e2[nb]) return nb;
+    int b = 0, e = nb;
+    while (e - b > 1) {
+      const int mid = (b + e) >> 1;
+      if (s_e2[mid] <= D2) b = mid;
+      else e = mid;
+    }
+    return b;
+  };
+
+  // Pairs of one item: the lane's k (tile tk) with the nj j's of tile tj.
+  auto item = [&](const Stage& S, int tk, int tj, int nk, int nj, auto diag) {
+    constexpr bool DIAG = decltype(diag)::value;
+    const int k = tk * 32 + lane;
+    const float xk = lane < nk ? S.x[k] : kFarK, yk = S.y[k], zk = S.z[k];
+    const int qk = S.q[k];
+    [[maybe_unused]] const int pk = WEIGHTED ? S.p[k] : 0, Wk = WEIGHTED ? S.W[k] : 0;
+    const unsigned long long nx = t_pack(-xk, -xk), ny = t_pack(-yk, -yk), nz = t_pack(-zk, -zk);
+        const uint32_t base = s_cell - 4u * kBin0<LOWER> + (WEIGHTED ? 0u : (uint32_t)qk);
+    for (int j = tj * 32; j < tj * 32 + nj; j += 4) {
+      float u[4];
+      {
+        const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(S.x + j);
+        const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(S.y + j);
+        const ulonglong2 Z = *reinterpret_cast<const ulonglong2*>(S.z + j);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const unsigned long long dx = t_add(h ? X.y : X.x, nx), dy = t_add(h ? Y.y : Y.x, ny),
+                                   dz = t_add(h ? Z.y : Z.x, nz);
+          float e0, e1;
+          t_unpack(t_fma(dz, dz, t_fma(dy, dy, t_mul(dx, dx))), e0, e1);
+          u[2 * h] = fmaf(t_sqrt(e0), a.c, a.m);
+          u[2 * h + 1] = fmaf(t_sqrt(e1), a.c, a.m);
+        }
+      }
+      if (DIAG) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v)  // each pair once
+          if (j - tj * 32 + v >= lane) u[v] = __uint_as_float(0x7F7FFFFFu);
+      }
+      // the smallest low halves, two to a word
+      const uint32_t near2 = __vminu2(
+          __byte_perm(__float_as_uint(u[0]), __float_as_uint(u[1]), 0x5410),
+          __byte_perm(__float_as_uint(u[2]), __float_as_uint(u[3]), 0x5410));
+      const bool near = min(near2 & 0xFFFFu, near2 >> 16) <= a.amb;
+      const int4 pj = *reinterpret_cast<const int4*>(S.p + j);
+      const int pp[4] = {pj.x, pj.y, pj.z, pj.w};
+      if constexpr (!WEIGHTED) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+          t_red(base + (uint32_t)pp[v] + 4u * t_bin<LOWER>(u[v], nb), 1u);
+        if (near) {
+          // move the count of a pair whose exact bin is another
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            if ((__float_as_uint(u[v]) & 0xFFFFu) > a.amb) continue;
+            const int was = (int)(t_bin<LOWER>(u[v], nb) - kBin0<LOWER>);
+            const int b = exact_bin(S.x[j + v] - xk, S.y[j + v] - yk, S.z[j + v] - zk);
+            if (b == was) continue;
+            unsigned* row = cell + (pp[v] + qk) / 4;
+            atomicSub(row + was, 1u);
+            atomicAdd(row + b, 1u);
+          }
+        }
+      } else {
+        const int4 qj = *reinterpret_cast<const int4*>(S.q + j);
+        const int4 wj = *reinterpret_cast<const int4*>(S.W + j);
+        const int qq[4] = {qj.x, qj.y, qj.z, qj.w}, ww[4] = {wj.x, wj.y, wj.z, wj.w};
+        uint32_t b[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) b[v] = t_bin<LOWER>(u[v], nb);
+        if (near) {
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+            if ((__float_as_uint(u[v]) & 0xFFFFu) <= a.amb)
+              b[v] = kBin0<LOWER> +
+                     (uint32_t)exact_bin(S.x[j + v] - xk, S.y[j + v] - yk, S.z[j + v] - zk);
+        }
+        // misses branch off: returning atomics to one trash cell per row took
+        // 4.4 wavefronts each, those of the hits alone 2.6
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+          if (b[v] < kBin0<LOWER> + (uint32_t)nb)
+          t_record<WM>(base + (uint32_t)(max(pp[v], pk) + min(qq[v], qk)) + 4u * b[v], zoff, ww[v],
+                       Wk, scale);
+      }
+    }
+  };
+  // One hub: stage the row, then the items over the group's warps.
+  auto hub = [&](const Stage& S, int64_t i, int d) {
+    const uint32_t* row = row_at(c.adj, c.ptr, i, c.adj_off, c.split, c.adj_off2);
+    const int4 P = c.xyzp[i];
+    const int nt = (d + 31) >> 5;
+    for (int s = gt; s < nt * 32; s += gthreads) {
+      const int t = (s & 31) * nt + (s >> 5);
+      if (t < d) {
+        const uint32_t w = row[t];
+        const uint32_t id = edge_id(w);
+        const int b = (int)edge_bin(w);
+        const int4 Q = c.xyzp[id];
+        S.x[s] = (float)(int)min_image((int64_t)Q.x - P.x, c.box);
+        S.y[s] = (float)(int)min_image((int64_t)Q.y - P.y, c.box);
+        S.z[s] = (float)(int)min_image((int64_t)Q.z - P.z, c.box);
+        S.p[s] = 4 * nr * (WEIGHTED ? b * (b + 1) / 2 : b * nb);
+        S.q[s] = 4 * nr * b;
+        if (WEIGHTED) S.W[s] = (int)c.W[id];
+      } else {
+        S.x[s] = kFarJ;
+        S.y[s] = S.z[s] = 0.f;
+        S.p[s] = S.q[s] = 0;
+        if (WEIGHTED) S.W[s] = 0;
+      }
+    }
+    sync();
+    // tile t holds dq + (t < dr) neighbours; items (tk, tj), tj <= tk, go
+    // round the warps
+    const int dq = d / nt, dr = d - dq * nt;
+    for (int tk = 0, tj = wg;; tj += group) {
+      while (tk < nt && tj > tk) tj -= ++tk;
+      if (tk >= nt) break;
+      const int nk = dq + (tk < dr ? 1 : 0), nj = dq + (tj < dr ? 1 : 0);
+      if (tj == tk) item(S, tk, tj, nk, nk - 1, std::true_type{});
+      else item(S, tk, tj, nk, nj, std::false_type{});
+    }
+    sync();
+  };
+
+  for (;;) {
+    if (gt == 0) {
+      int64_t i = -1;
+      int k = 0;
+      const int64_t q = (int64_t)atomicAdd(a.hub_counter, 1ull);
+      if (BATCH) {
+        if (q < a.base[a.ncats]) {
+          int lo = 0, hi = a.ncats;  // largest k with base[k] <= q
+          while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (a.base[mid] <= q) lo = mid;
+            else hi = mid;
+          }
+          k = lo;
+          i = q - a.base[k];
+        }
+      } else {
+        i = a.one.hub_begin + q;
+        if (i >= a.one.hub_end) i = -1;
+      }
+      s_hub[g] = i;
+      if (BATCH) s_cat = k;
+      s_flush[g] = 0;
+      if (i >= 0) {
+        const unsigned long long d = (unsigned long long)(BATCH ? a.cats[k].deg : a.one.deg)[i];
+        const unsigned long long need = d * (d - (d > 0)) / 2;  // triangles at i <= C(d, 2)
+        // The shared counters stay below 2^32: between two flushes they take
+        // what was registered since the last reset (2^29 and one hub), what
+        // registers while a flush runs (the same) and the hubs under way at a
+        // reset (15 of at most 2^25).
+        if ((BATCH && k != s_cur) || atomicAdd(&s_pending, need) + need > (1ull << 29)) {
+          atomicExch(&s_pending, BATCH ? need : 0ull);
+          s_flush[g] = 1;
+          if (BATCH) s_cur = k;
+        }
+      }
+    }
+    sync();
+    const int64_t i = s_hub[g];
+    if (i < 0) break;
+    if (s_flush[g]) {
+      flush(gt, gthreads);
+      if (WEIGHTED || BATCH) sync();
+    }
+    if (BATCH && s_cat != cur) {
+      cur = s_cat;
+      if (tid == 0) s_c = a.cats[cur];
+      sync();
+    }
+    const int d = c.deg[i];
+    if (d < 2) {
+      sync();
+      continue;
+    }
+    if (d > a.cap)
+      hub(stage_at(a.gscratch + ((size_t)blockIdx.x * (kTWarps / group) + g) * a.gstride,
+                   a.gstride / (WEIGHTED ? 24 : 20)),
+          i, d);
+    else hub(st_s, i, d);
+    if (WEIGHTED) fold(c.W[i]);  // ordered by the barrier at the top
+  }
+  __syncthreads();
+  flush(tid, kTThreads);
+}
+
 // Equilateral configurations (b, b, b) by pair geometry: a triangle is
 // equilateral in this sense only when both hub edges share bin b, so the CTA
 // stages N+(i) grouped by the hub edge's bin (a counting sort in shared
@@ -1451,6 +1927,84 @@ PairLaunch pair_launch(int nb, int nconf, bool weighted, bool use_lut,
   return L;  // cap 0: the configuration tables leave no room (walk kernel instead)
 }
 
+// Launch plan of the tiled pair kernel; cap 0: another kernel takes the call.
+struct TileLaunch {
+  int cap = 0, group = kTWarps, blocks = 0;
+  size_t smem = 0;
+  TArgs a;  // the binning constants
+};
+
+// mean: mean row length. Conditions: bins evenly spaced to within 1/128 of
+// their width (edges rounded to the lattice are), two CTAs per SM, and
+// (weighted) rows long enough to pay for folding the cells at every hub.
+TileLaunch tile_launch(int nb, int nconf, const FixedW* fw, bool batch, double mean, int max_deg,
+                       const std::vector<int64_t>& edges) {
+  TileLaunch L;
+  if (max_deg > kTMaxDeg) return L;
+  const bool weighted = fw != nullptr;
+  const double w = (double)(edges[nb] - edges[0]) / nb;
+  if (nb > kTileMaxBins) return L;
+  double dev = 0.0;  // edges off the even spacing, in bin widths
+  for (int b = 0; b <= nb; ++b)
+    dev = std::max(dev, std::fabs((double)(edges[b] - edges[0]) / w - b));
+  // D = sqrt(D2): relative error below 0.75 2^-21 from the squared distance
+  // (three roundings, halved), the approximate square root (2^-23) and c
+  // (2^-24), at most E_nb / w bin widths; m's rounding; half a unit for u
+  const double off = (double)edges[0] / w, one = 65536.0;
+  const double err = (double)edges[nb] / w * std::ldexp(0.75, -21) + dev +
+                     std::max(kTileM + 1.0, off) * std::ldexp(1.0, -24);
+  if (err > 1.0 / 128) return L;
+  const int delta = (int)std::ceil(err * one + 0.75);
+  L.a.c = (float)(1.0 / w);
+  L.a.m = (float)(kTileM + delta / one - off);
+  L.a.amb = 2u * (uint32_t)delta;
+  L.a.cb = 0;
+  if (weighted) {
+    // |x| < 2^(2 mag): high words below 2^hb; the count field and the sum's
+    // carries are then equally rare
+    const int hb = std::max(2 * fw->mag - 32, 0);
+    L.a.cb = std::min((32 - hb) / 2, 12);
+    const double pairs = 0.5 * max_deg * (max_deg - 1.0);
+    if (pairs >= std::ldexp(1.0, 14 + L.a.cb)) return L;  // T's halves
+    if (0.5 * mean * (mean - 1.0) < 2.0 * nconf) return L;
+  }
+  L.a.nb = nb;
+  L.a.nconf = nconf;
+  int dev_id = 0, per_sm_bytes = 0, sms = 0;
+  cudaGetDevice(&dev_id);
+  cudaDeviceGetAttribute(&per_sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev_id);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id);
+  auto pad16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
+  const size_t ncell = (size_t)(weighted ? nb * (nb + 1) / 2 : nb * nb) * (nb + 1);
+  const size_t fixed = (weighted ? (size_t)nconf * 16 + pad16((size_t)nconf * 4) : 0) +
+                       pad16((size_t)(nb + 1) * 8) + pad16((size_t)nconf * 4) +
+                       pad16(ncell * (weighted ? 12 : 4));
+  const size_t budget = (size_t)per_sm_bytes / 2 - 1024 - 512;  // static shared memory and slack
+  if (fixed + 2 * stage_bytes(32, weighted) > budget) return L;
+  const int want = std::min(max_deg, std::max(64, (int)(2.5 * mean)));
+  // few warps per hub where rows are short
+  int group = (weighted || batch) ? kTWarps : mean <= 64 ? 1 : mean <= 160 ? 4 : mean <= 320 ? 8 : kTWarps;
+  for (;; group = group == 1 ? 4 : group * 2) {
+    const size_t room = (budget - fixed) / (kTWarps / group);
+    L.cap = (int)(room / (weighted ? 24 : 20)) & ~31;
+    if (L.cap >= want || group == kTWarps) break;
+  }
+  L.cap = std::min(L.cap, (max_deg + 31) & ~31);
+  if (L.cap < 32) L.cap = 0;
+  L.group = group;
+  L.smem = fixed + (size_t)(kTWarps / group) * stage_bytes(L.cap, weighted);
+  L.blocks = 2 * sms;
+  return L;
+}
+
+template <bool BATCH>
+void (*pick_count3t(int wm, bool nonneg, bool lower))(TArgs) {
+#define GS_T(W) (lower ? k_count3t<W, BATCH, true> : k_count3t<W, BATCH, false>)
+  if (wm == kNone) return GS_T(kNone);
+  return nonneg ? GS_T(kExactPos) : GS_T(kExact);
+#undef GS_T
+}
+
 }  // namespace
 
 // An exact 192-bit two's-complement sum times 2^-scale, rounded to the
@@ -1560,8 +2114,13 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
   // more than 65,535 neighbours (whose triangles could overflow the 32-bit
   // shared counters within one hub) take the merge-walk kernel.
   const bool pair_ok = !equi && (o.variant & ~4) == 0 && g.max_deg <= kMaxSmemHistDeg;
-  const PairLaunch PL = pair_ok ? pair_launch(g.nb, nconf, wm != kNone, use_lut, g.edges)
-                                : PairLaunch{};
+  // evenly spaced bins: the tiled pair kernel (variant bit 4 keeps the other)
+  TileLaunch TL;
+  if (pair_ok && !(o.variant & 4) && g.n > 0)
+    TL = tile_launch(g.nb, nconf, wm != kNone ? fw : nullptr, false,
+                     (double)g.edges_total / (double)g.n, g.max_deg, g.edges);
+  const PairLaunch PL = pair_ok && !TL.cap ? pair_launch(g.nb, nconf, wm != kNone, use_lut, g.edges)
+                                           : PairLaunch{};
   // equilateral configurations: pair geometry within hub-edge bin groups
   // (variant bit 512 keeps the walk's EQUI instantiation)
   const bool equi_pair = equi && !(o.variant & 512) && g.max_deg <= kMaxSmemHistDeg;
@@ -1606,6 +2165,41 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
       pa.one.hub_end = v.h1;
       cudaMemsetAsync(pa.hub_counter, 0, sizeof(unsigned long long), s);
       { kern<<<grid, kPThreads, smem, s>>>(pa); note_launch(); }
+      return cuda_status(cudaGetLastError());
+    });
+    timer.stop(s);
+  } else if (TL.cap > 0) {
+    TArgs ta = TL.a;
+    ta.one = a.one;
+    ta.cats = nullptr;
+    ta.base = nullptr;
+    ta.ncats = 0;
+    ta.cap = TL.cap;
+    ta.group = TL.group;
+    ta.e2g = g.d_edges2;
+    ta.hub_counter = a.hub_counter;
+    void (*kern)(TArgs) = pick_count3t<false>(wm, fw && fw->nonneg, g.edges[0] > 0);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TL.smem);
+    // no more CTAs than the hubs keep busy
+    const int groups = kTWarps / TL.group;
+    const int grid = (int)std::min<int64_t>(TL.blocks, (g.n + groups - 1) / groups);
+    ta.gscratch = nullptr;
+    ta.gstride = 0;
+    if (g.max_deg > TL.cap) {
+      ta.gstride = stage_bytes((g.max_deg + 31) & ~31, wm != kNone);
+      ta.gscratch = sc.alloc<unsigned char>(ta.gstride * grid * groups);
+      if (!ta.gscratch) return GS_ENOMEM;
+    }
+    timer.start(s);
+    st = for_each_window(g, o, sc, [&](const WinView& v) -> int {
+      ta.one.adj = v.adj;
+      ta.one.adj_off = v.off1;
+      ta.one.split = v.split;
+      ta.one.adj_off2 = v.off2;
+      ta.one.hub_begin = v.h0;
+      ta.one.hub_end = v.h1;
+      cudaMemsetAsync(ta.hub_counter, 0, sizeof(unsigned long long), s);
+      { kern<<<grid, kTThreads, TL.smem, s>>>(ta); note_launch(); }
       return cuda_status(cudaGetLastError());
     });
     timer.stop(s);
@@ -1765,10 +2359,43 @@ int count3_batch_device(const Graph* const* gr, int ng, const FixedW* fws, uint6
   bool same_edges = true;
   for (int k = 1; k < ng; ++k) same_edges = same_edges && gr[k]->edges == gr[0]->edges;
   const bool pair_ok = same_edges && (o.variant & ~4) == 0 && max_deg <= kMaxSmemHistDeg;
-  const PairLaunch PL = pair_ok ? pair_launch(nb, nconf, wm != kNone, !(o.variant & 4),
-                                              gr[0]->edges)
-                                : PairLaunch{};
-  if (PL.cap > 0) {
+  double mean = 0.0;
+  for (int k = 0; k < ng; ++k) mean += (double)gr[k]->edges_total;
+  if (base[ng] > 0) mean /= (double)base[ng];
+  // the weights' width over all catalogues
+  FixedW wide;
+  wide.nonneg = nonneg;
+  for (int k = 0; k < ng && fws; ++k) wide.mag = std::max(wide.mag, fws[k].mag);
+  TileLaunch TL;
+  if (pair_ok && !(o.variant & 4) && base[ng] > 0)
+    TL = tile_launch(nb, nconf, wm != kNone ? &wide : nullptr, true, mean, max_deg, gr[0]->edges);
+  const PairLaunch PL = pair_ok && !TL.cap
+                            ? pair_launch(nb, nconf, wm != kNone, !(o.variant & 4), gr[0]->edges)
+                            : PairLaunch{};
+  if (TL.cap > 0) {
+    TArgs ta = TL.a;
+    ta.one = cats[0];
+    ta.cats = d_cats;
+    ta.base = d_base;
+    ta.ncats = ng;
+    ta.cap = TL.cap;
+    ta.group = TL.group;
+    ta.e2g = gr[0]->d_edges2;
+    ta.hub_counter = a.hub_counter;
+    void (*kern)(TArgs) = pick_count3t<true>(wm, nonneg, gr[0]->edges[0] > 0);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TL.smem);
+    const int grid = (int)std::min<int64_t>(TL.blocks, base[ng]);
+    ta.gscratch = nullptr;
+    ta.gstride = 0;
+    if (max_deg > TL.cap) {
+      ta.gstride = stage_bytes((max_deg + 31) & ~31, wm != kNone);
+      ta.gscratch = sc.alloc<unsigned char>(ta.gstride * grid);
+      if (!ta.gscratch) return GS_ENOMEM;
+    }
+    timer.start(s);
+    { kern<<<grid, kTThreads, TL.smem, s>>>(ta); note_launch(); }
+    timer.stop(s);
+  } else if (PL.cap > 0) {
     PArgs pa;
     pa.one = cats[0];
     pa.cats = d_cats;

@@ -63,8 +63,8 @@ struct Graph {
   std::vector<int64_t> h_ptr;   // host copy of d_ptr (window planning)
   std::vector<int32_t> h_deg;   // host copy of d_deg
   // out-of-core planning. In a periodic box the ids are x-major, so hubs
-  // of the first x-slab have wrap-around neighbours in the last one:
-  // wrap_start is the first id of the last x-slab (n for an open box);
+  // of the first E_nb in x have wrap-around neighbours in the last one:
+  // wrap_start is the first id of the cells there (n for an open box);
   // h_reach[i] is the largest neighbour id of i below wrap_start (or i) and
   // h_far[i] says whether i has neighbours at or above wrap_start.
   std::vector<int32_t> h_reach;
@@ -151,7 +151,8 @@ int64_t num_conf3(int nb);
 struct FixedW {
   int64_t* d_W = nullptr;  // [n], internal order
   int scale = 0;
-  int bits = 0;  // max bit length of |W_i| plus one sign bit
+  int bits = 0;  // max bit length of |W_i| plus one sign bit (an upper bound)
+  int mag = 0;   // |W_i| < 2^mag
   bool nonneg = true;  // no weight is negative
 };
 // max_bits: the widest |W| (bits, sign included) the caller can sum exactly:
