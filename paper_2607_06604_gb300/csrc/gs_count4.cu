@@ -94,7 +94,7 @@ struct Args {
   const void* __restrict__ ent;      // orbit table (see Ent)
   const uint8_t* __restrict__ chir;  // chirality per slot (parity)
   int64_t box;
-  int nb, nb3;
+  int nb, tab3;  // bins; table entries per (b_01, b_02, b_12): nb^2 (nb + 1)
   int cap;   // shared-memory workspace capacity (neighbours) of a group
   int gcap;  // global workspace capacity
   int group; // warps per group
@@ -115,12 +115,22 @@ struct Args {
 // Table entries: twice the slot, plus 1 when the relabelling onto the
 // representative of a chiral orbit is odd; the top bit marks chiral orbits.
 // Two bytes when the slots fit 14 bits (nb <= 8): half the lines per gather.
+// The last digit (b_23) has one value more, no edge, whose entries say slot
+// n_orbits: the counters have a cell for it, so that updates need no predicate
+// (a predicated shared atomic is compiled to a branch, four instructions).
 template <class E>
 struct Ent {
   static constexpr int kTop = sizeof(E) * 8 - 1;
   static constexpr uint32_t kMask = (1u << kTop) - 1u;
-  using Signed = typename std::make_signed<E>::type;
 };
+
+// A table entry, sign-extended (the chirality bit fills the top).
+__device__ inline int load_entry(const uint16_t* p) {
+  int v;
+  asm("ld.global.nc.s16 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ inline int load_entry(const uint32_t* p) { return (int)__ldg(p); }
 
 __device__ inline int64_t mi(int64_t d, int64_t box) {
   if (box) {
@@ -371,22 +381,9 @@ struct Shared {
   unsigned long long pending;     // tetrahedra the shared counters may hold
 };
 
-// Adds 1 to a counter at a shared address when b < nb (no branch).
-__device__ inline void inc_shared_below(uint32_t addr, uint32_t b, uint32_t nb) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t"
-      "@p red.shared.add.u32 [%0], 1;\n\t}" ::"r"(addr),
-      "r"(b), "r"(nb)
-      : "memory");
-}
-
-// The same for a global 64-bit counter.
-__device__ inline void inc_global_below(unsigned long long* p, uint32_t b, uint32_t nb) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t"
-      "@p red.global.add.u64 [%0], 1;\n\t}" ::"l"(p),
-      "r"(b), "r"(nb)
-      : "memory");
+// Adds 1 to a counter at a shared address.
+__device__ inline void inc_shared(uint32_t addr) {
+  asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory");
 }
 
 // Pairs of floats in one 64-bit register (low half first); each half is
@@ -618,7 +615,7 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
         if (p < n) {
           const int b = (int)list[p];
           const int4 db = w.disp[b];
-          tri = (uint32_t)((b01 * nb + db.w) * nb + Ba[b]) * (uint32_t)a.nb3;
+          tri = (uint32_t)((b01 * nb + db.w) * nb + Ba[b]) * (uint32_t)a.tab3;
           brow = GW ? b : row_off<int>(b, m + 1);
           if (PARITY) {
             if constexpr (PIX) {
@@ -649,19 +646,21 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
         const bool in = p < n;
         const int c = in ? (int)list[p] : m;  // column m: no edges
         const int4 dc = w.disp[c];
-        const uint32_t lane_idx = (uint32_t)((dc.w * nb + (in ? (int)Ba[c] : 0)) * nb);
+        const uint32_t lane_idx = (uint32_t)((dc.w * nb + (in ? (int)Ba[c] : 0)) * (nb + 1));
         const int Wc = WEIGHTED && in ? w.wv[c] : 0;
         float ux = 0.f, uy = 0.f, uz = 0.f;
         if constexpr (PIX) {
           const float4 u3 = spoke(dc, in ? lpix[p] : 0);
           ux = u3.x, uy = u3.y, uz = u3.z;
         } else if (PARITY) {
-          ux = (float)dc.x, uy = (float)dc.y, uz = (float)dc.z;
+          // unused lanes: a volume far from zero
+          ux = in ? (float)dc.x : 1e20f, uy = (float)dc.y, uz = (float)dc.z;
         }
         const int ns = t0 > k0 ? 32 : min(31, n - 1 - k0);
         if constexpr (FAST) {
           const uint8_t* Bc = w.B + c;
-          const auto* ent_c = reinterpret_cast<const typename Ent<E>::Signed*>(ent) + lane_idx;
+          const E* ent_c = ent + lane_idx;
+          const uint32_t trash = (uint32_t)(PARITY ? 2 * a.hot : a.hot);
           const uint32_t cells = (uint32_t)__cvta_generic_to_shared(h.cnt);
           const unsigned long long ux2 = pack2(ux, ux), uy2 = pack2(uy, uy), uz2 = pack2(uz, uz);
           auto steps = [&](auto diag) {
@@ -676,11 +675,9 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
               const uint32_t tt[U] = {t.x, t.y, t.z, t.w};
 #pragma unroll
               for (int u = 0; u < U; ++u) {
-                // a lane without an edge here reads the next table entry
-                // (same lines) and adds nothing
                 b23[u] = (uint32_t)nb;
                 if (!decltype(diag)::value || s0 + u < lane) b23[u] = Bc[rr[u]];
-                en[u] = ent_c[tt[u] + b23[u]];
+                en[u] = load_entry(ent_c + (tt[u] + b23[u]));
               }
               if (PARITY) {
                 const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(ch->nx + s0);
@@ -693,24 +690,23 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
 #pragma unroll
               for (int u = 0; u < U; ++u) {
                 uint32_t cell;
-                uint32_t below = (uint32_t)nb;
                 if constexpr (PARITY) {
-                  // V < 0 on a chiral orbit (the entry is read sign-extended)
+                  // V < 0 on a chiral orbit
                   const uint32_t neg = (__float_as_uint(V[u]) & (uint32_t)en[u]) >> 31;
                   cell = ((uint32_t)en[u] ^ neg) & Ent<E>::kMask;
                   if constexpr (PIX) {
                     // degenerate pixel volumes are a few percent: even channel
                     if (fabsf(V[u]) < a.eps && en[u] < 0) {
-                      inc_global_below(a.even + (cell >> 1), b23[u], (uint32_t)nb);
-                      below = 0u;
+                      atomicAdd(a.even + (cell >> 1), 1ull);
+                      cell = trash;
                     }
-                  } else {
-                    if (b23[u] < (uint32_t)nb) vmin = fminf(vmin, fabsf(V[u]));
+                  } else if (!decltype(diag)::value || s0 + u < lane) {
+                    vmin = fminf(vmin, fabsf(V[u]));
                   }
                 } else {
                   cell = ((uint32_t)en[u] & Ent<E>::kMask) >> 1;
                 }
-                inc_shared_below(cells + 4u * cell, b23[u], below);
+                inc_shared(cells + 4u * cell);
               }
               if (PARITY && !PIX && vmin < a.eps) {
                 // a volume within its error bound of zero: move the count if
@@ -793,7 +789,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
   h.sum = reinterpret_cast<unsigned long long*>(sp);
   if (WEIGHTED) sp += (size_t)ncell * 16;
   h.cnt = reinterpret_cast<unsigned*>(sp);
-  sp += pad16((size_t)ncell * 4);
+  sp += pad16((size_t)ncell * 4 + 8);
   float4* pixu = reinterpret_cast<float4*>(sp);
   if (PIX) sp += 256 * sizeof(float4);
   Chunk* ch = reinterpret_cast<Chunk*>(sp) + warp;
@@ -804,7 +800,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
       sp + (size_t)g * workspace_bytes(a.cap, group, sizeof(uint16_t), WEIGHTED, PIX), a.cap,
       group, WEIGHTED, PIX);
 
-  for (int k = tid; k < ncell; k += kThreads) {
+  for (int k = tid; k < ncell; k += kThreads) {  // the cell of no edge is never read
     h.cnt[k] = 0u;
     if (WEIGHTED) h.sum[2 * k] = h.sum[2 * k + 1] = 0ull;
   }
@@ -971,11 +967,17 @@ const float4* pixel_centres(int* status) {
 // Table entries (see Ent) and chirality by slot from the orbit table: orbit o
 // takes slot slot_of[o] (its own index when slot_of is null).
 template <class E>
-__global__ void k_entries(const uint32_t* __restrict__ lut, int64_t n,
+__global__ void k_entries(const uint32_t* __restrict__ lut, int64_t n, int nb, int n_orbits,
                           const int32_t* __restrict__ slot_of, E* out, uint8_t* chir) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t e = lut[k], o = e & 0x3FFFFFFFu, chiral = e >> 31;
+    const int64_t row = k / (nb + 1);
+    const int b = (int)(k - row * (nb + 1));
+    if (b == nb) {
+      out[k] = (E)(n_orbits << 1);
+      continue;
+    }
+    const uint32_t e = lut[row * nb + b], o = e & 0x3FFFFFFFu, chiral = e >> 31;
     const uint32_t slot = slot_of ? (uint32_t)slot_of[o] : o;
     out[k] = (E)((slot << 1) | ((e >> 30) & chiral) | (chiral << Ent<E>::kTop));
     chir[slot] = (uint8_t)chiral;  // every raw tuple of an orbit agrees
@@ -1028,7 +1030,7 @@ void (*pick4(bool parity, bool weighted, bool pix, bool fast))(Args) {
 // the workspaces of 32 / group groups.
 size_t launch_smem(int64_t hot, int cap, int group, bool parity, bool weighted, bool pix) {
   const size_t ncell = (size_t)hot * (parity ? 2 : 1);
-  return (weighted ? ncell * 16 : 0) + pad16(ncell * 4) + (pix ? 256 * sizeof(float4) : 0) +
+  return (weighted ? ncell * 16 : 0) + pad16(ncell * 4 + 8) + (pix ? 256 * sizeof(float4) : 0) +
          (size_t)kWarps * sizeof(Chunk) + (weighted ? (size_t)kThreads * 8 : 0) +
          (size_t)(kWarps / group) * workspace_bytes(cap, group, sizeof(uint16_t), weighted, pix);
 }
@@ -1073,7 +1075,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   a.e2g = g.d_edges2;
   a.box = g.box_u;
   a.nb = g.nb;
-  a.nb3 = g.nb * g.nb * g.nb;
+  a.tab3 = g.nb * g.nb * (g.nb + 1);
   a.even = reinterpret_cast<unsigned long long*>(d_even);
   a.odd = parity ? (d_odd ? reinterpret_cast<unsigned long long*>(d_odd)
                           : sc.alloc<unsigned long long>(no))
@@ -1105,7 +1107,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const size_t avail = (size_t)optin - sizeof(Shared) - 64;
   // two-byte entries hold slots below 2^14 (nb <= 8)
-  const bool small_ent = no <= 16384;
+  const bool small_ent = no < 16384;
   // Launch 1: groups of `group` warps over every hub of at most `cap`
   // neighbours; launch 2 (when longer rows exist): whole CTAs over a list of
   // the longer ones, in shared memory up to cap2, else in global scratch.
@@ -1146,9 +1148,8 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   unsigned long long* s_odd = a.odd;
   unsigned long long* const o_odd = a.odd;  // odd counts in orbit order (caller's or scratch)
   int32_t* d_slot = nullptr;
-  const int64_t nl = (int64_t)t->lut.size();
-  // one entry more: lanes without an edge read past a row
-  void* d_ent = sc.alloc_bytes((size_t)(nl + 1) * (small_ent ? 2 : 4));
+  const int64_t nl = (int64_t)t->lut.size() / g.nb * (g.nb + 1);
+  void* d_ent = sc.alloc_bytes((size_t)nl * (small_ent ? 2 : 4));
   uint8_t* d_chir = sc.alloc<uint8_t>(no);
   if (!d_ent || !d_chir) return GS_ENOMEM;
   if (relabel) {
@@ -1175,9 +1176,11 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   auto entries = [&](const int32_t* slot_of) {
     const int blocks = (int)std::min<int64_t>((nl + 255) / 256, 4096);
     if (small_ent)
-      k_entries<uint16_t><<<blocks, 256, 0, s>>>(t->d_lut, nl, slot_of, (uint16_t*)d_ent, d_chir);
+      k_entries<uint16_t><<<blocks, 256, 0, s>>>(t->d_lut, nl, g.nb, no, slot_of, (uint16_t*)d_ent,
+                                               d_chir);
     else
-      k_entries<uint32_t><<<blocks, 256, 0, s>>>(t->d_lut, nl, slot_of, (uint32_t*)d_ent, d_chir);
+      k_entries<uint32_t><<<blocks, 256, 0, s>>>(t->d_lut, nl, g.nb, no, slot_of, (uint32_t*)d_ent,
+                                               d_chir);
     note_launch();
   };
   entries(nullptr);
