@@ -30,13 +30,13 @@
 // 128-bit sums, flushed into 192-bit global accumulators.
 #include <algorithm>
 #include <cmath>
-#include <cstring>
 #include <map>
 #include <mutex>
 #include <tuple>
 #include <type_traits>
 
 #include "gs_internal.cuh"
+#include "gs_tiles.cuh"
 
 namespace gs {
 namespace {
@@ -1164,16 +1164,27 @@ __global__ void __launch_bounds__(kPThreads, 2) k_count3p(PArgs a) {
 //    Weighted cells are those of ({b_ij, b_ik}, b_jk); see below. A pair that
 //    is no edge goes to the extra bin nb, so that updates need no predicate
 //    (a predicated shared atomic is compiled to a branch, four instructions).
-// Bound by instruction issue and shared-memory atomics together; figures at
-// the launch rule (tile_launch).
+// Bound by instruction issue and the shared-memory pipe together (81% and 82%;
+// 20 instructions and 5 wavefronts per 32 pairs, weighted 47 and 11). Kernel
+// times on one GB300, k_count3p -> this: 3e6 uniform points, 402 edges a row,
+// weighted 596 -> 409 ms; 1e6 of them unweighted 148 -> 59 ms; 1e6 clustered
+// points, 134 a row, weighted 42 -> 25 ms.
 //
-// Weighted (exact): per hub and cell the sum of x = W_j W_k, |x| < 2^60, and
-// the number of pairs, in three 32-bit words updated by two shared atomics: lo
-// takes the low words of x (its carry goes on), Z takes (high word + carry)
-// 2^cb + 1, so its low cb bits count the pairs; T takes, rarely, the carries
-// out of Z (upper half, signed) and of Z's count field (lower half). fold
-// adds the cells of one configuration, multiplies by W_i and adds to the
-// CTA's 128-bit sums.
+// Weighted (exact), two modes. Both keep per cell the sum of integer products
+// and the number of pairs in 32-bit words; the last word of the sum, Z, takes
+// (high word + carry) 2^cb + 1, so its low cb bits count the pairs, and T takes,
+// rarely, the carries out of Z (upper half, signed) and of Z's count field
+// (lower half).
+//  * FOLD, long rows: x = W_j W_k, |x| < 2^60, two shared atomics per pair; the
+//    CTA works on one hub, after which fold adds the cells of one
+//    configuration, times W_i, to the CTA's 128-bit sums.
+//  * else: x = W_i W_j W_k, |x| < 2^90, three atomics, but the cells outlive
+//    the hub, so a hub may be one warp's and nothing passes over every
+//    configuration at its end.
+// Pairs that are no edge update a word of their lane's own bank, so that four
+// pairs' atomics go out together (a branch around them left each pair waiting
+// for its own chain of returned values: 1e6 uniform points, 402 edges a row,
+// 144 ms against 138).
 struct TArgs {
   Cat one;
   const Cat* cats;      // batched launches
@@ -1181,9 +1192,10 @@ struct TArgs {
   int ncats;
   int nb, nconf;
   int cap;              // neighbours staged in shared memory per group (multiple of 32)
-  int group;            // warps per hub (all of the CTA's when weighted or batched)
-  float c, m;           // u = sqrt(D2) c + m
-  uint32_t amb;         // ambiguous iff the low 16 bits of u are <= amb
+  int group;            // warps per hub (all of the CTA's when FOLD or batched)
+  float c, m;           // see TileBins
+  uint32_t amb;
+  unsigned long long limit;  // pairs between two flushes
   int cb;               // weighted: bits of Z's count field
   const int64_t* e2g;
   unsigned char* gscratch;  // hubs above cap: per-CTA staging in global memory
@@ -1191,146 +1203,108 @@ struct TArgs {
   unsigned long long* hub_counter;
 };
 
-constexpr int kTThreads = 512;
-constexpr int kTWarps = kTThreads / 32;
-// Rows above this are left to the walk and pair kernels: C(8192, 2) < 2^25
-// pairs per hub keep the shared counters below 2^32 between flushes.
-constexpr int kTMaxDeg = 8192;
-// Absent j's and k's stand at these x (in units): farther from every point,
-// and from one another, than twice the largest E_nb (2^19).
-constexpr float kFarJ = 4.0e6f, kFarK = -4.0e6f;
-
-__device__ inline unsigned long long t_pack(float x, float y) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ inline void t_unpack(unsigned long long v, float& x, float& y) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-}
-__device__ inline unsigned long long t_add(unsigned long long a, unsigned long long b) {
-  unsigned long long r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ inline unsigned long long t_mul(unsigned long long a, unsigned long long b) {
-  unsigned long long r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ inline unsigned long long t_fma(unsigned long long a, unsigned long long b,
-                                           unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ inline float t_sqrt(float x) {
-  float r;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
-// u of a pair in bin b lies in [kTileM + b, kTileM + b + 1): 16 fraction bits.
-constexpr float kTileM = 192.0f;
-constexpr uint32_t kTileBits = 0x43400000u;  // bits of kTileM
-constexpr int kTileMaxBins = 62;             // kTileM + nb + 1 below 256
-
-// The bin that u says, nb when none, plus kBin0 (taken off in the cells' base
-// address). LOWER: u may lie below kTileM.
-template <bool LOWER>
-constexpr uint32_t kBin0 = LOWER ? 0u : kTileBits >> 16;
-template <bool LOWER>
-__device__ inline uint32_t t_bin(float u, int nb) {
-  const uint32_t bits = __float_as_uint(u);
-  return min((LOWER ? bits - kTileBits : bits) >> 16, kBin0<LOWER> + (uint32_t)nb);
-}
-
-__device__ inline void t_red(uint32_t addr, uint32_t v) {
-  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-__device__ inline uint32_t t_atom(uint32_t addr, uint32_t v) {
-  uint32_t old;
-  asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(v) : "memory");
-  return old;
-}
-
-// Records a pair with weights Wj, Wk in the weighted cell at `at` (words lo,
-// Z, T, zoff bytes apart; scale = 2^cb).
-template <int WM>
-__device__ inline void t_record(uint32_t at, uint32_t zoff, int Wj, int Wk, uint32_t scale) {
-  const long long x = (long long)Wj * Wk;
-  const uint32_t x0 = (uint32_t)x;
-  const uint32_t o0 = t_atom(at, x0);
-  uint32_t x1, n, c;  // the high word with the low word's carry
-  asm("{\n\t.reg .u32 s;\n\tadd.cc.u32 s, %1, %2;\n\taddc.u32 %0, %3, 0;\n\t}"
-      : "=r"(x1)
-      : "r"(o0), "r"(x0), "r"((uint32_t)((unsigned long long)x >> 32)));
-  const uint32_t a1 = x1 * scale + 1u;
-  const uint32_t o1 = t_atom(at + zoff, a1);
-  asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, 0, 0;" : "=&r"(n), "=r"(c) : "r"(o1), "r"(a1));
-  if (WM != kExactPos) c -= (uint32_t)((int)a1 < 0 ? 1 : 0);  // sign extension
-  const bool wrap = (n & (scale - 1u)) == 0u;  // the count field has come round
-  if (wrap || c) t_red(at + 2u * zoff, (c << 16) + (wrap ? 1u : 0u));
+// Records four pairs in the weighted cells at[] (their words zoff bytes apart;
+// scale = 2^cb). V = W_k (FOLD) or W_i W_k; the words are [w0,] w1, Z, T.
+template <int WM, bool FOLD>
+__device__ inline void t_record(const uint32_t (&at)[4], uint32_t zoff, const int (&Wj)[4],
+                                long long V, uint32_t scale) {
+  constexpr bool POS = WM == kExactPos;
+  uint32_t lo[4], hi[4], o[4];  // x = (hi, lo) or (hi, lo, w0), hi its last word
+  if constexpr (FOLD) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const long long x = (long long)Wj[v] * (int)V;
+      lo[v] = (uint32_t)x;
+      hi[v] = (uint32_t)((unsigned long long)x >> 32);
+      o[v] = t_atom(at[v], lo[v]);
+    }
+  } else {
+    const uint32_t vl = (uint32_t)V, vh = (uint32_t)((unsigned long long)V >> 32);
+    uint32_t w0[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      unsigned long long p0, p1;  // x = p1 2^32 + low word of p0
+      if constexpr (POS) {
+        p0 = (unsigned long long)(uint32_t)Wj[v] * vl;
+        p1 = (unsigned long long)(uint32_t)Wj[v] * vh + (p0 >> 32);
+      } else {
+        const long long q0 = (long long)Wj[v] * (long long)(unsigned long long)vl;
+        p0 = (unsigned long long)q0;
+        p1 = (unsigned long long)((long long)Wj[v] * (int)vh + (q0 >> 32));
+      }
+      w0[v] = (uint32_t)p0;
+      lo[v] = (uint32_t)p1;
+      hi[v] = (uint32_t)(p1 >> 32);
+      o[v] = t_atom(at[v], w0[v]);
+    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      asm("{\n\t.reg .u32 s;\n\tadd.cc.u32 s, %2, %3;\n\taddc.cc.u32 %0, %0, 0;\n\t"
+          "addc.u32 %1, %1, 0;\n\t}"
+          : "+r"(lo[v]), "+r"(hi[v])
+          : "r"(o[v]), "r"(w0[v]));
+      o[v] = t_atom(at[v] + zoff, lo[v]);
+    }
+  }
+  const uint32_t zo = FOLD ? zoff : 2u * zoff;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    asm("{\n\t.reg .u32 s;\n\tadd.cc.u32 s, %1, %2;\n\taddc.u32 %0, %0, 0;\n\t}"
+        : "+r"(hi[v])
+        : "r"(o[v]), "r"(lo[v]));
+    hi[v] = hi[v] * scale + 1u;
+    o[v] = t_atom(at[v] + zo, hi[v]);
+  }
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    uint32_t n, c;
+    asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, 0, 0;" : "=&r"(n), "=r"(c) : "r"(o[v]), "r"(hi[v]));
+    if (!POS) c -= (uint32_t)((int)hi[v] < 0 ? 1 : 0);  // sign extension
+    const bool wrap = (n & (scale - 1u)) == 0u;         // the count field has come round
+    if (wrap || c) t_red(at[v] + zo + zoff, (c << 16) + (wrap ? 1u : 0u));
+  }
 }
 
-// Staged neighbours of one hub, one array per quantity: x, y, z (float);
-// unweighted: p = b nb rows, q = b rows of nb + 1 cells; weighted: p =
-// b (b + 1) / 2 rows, q = b rows, W. p and q as byte offsets of 32-bit cells.
-struct Stage {
-  float *x, *y, *z;
-  int *p, *q, *W;
-};
-__host__ __device__ inline size_t stage_bytes(int64_t cap, bool weighted) {
-  return (size_t)cap * (weighted ? 24 : 20);
-}
-__device__ inline Stage stage_at(unsigned char* b, int64_t cap) {
-  Stage s;
-  s.x = reinterpret_cast<float*>(b);
-  s.y = s.x + cap;
-  s.z = s.y + cap;
-  s.p = reinterpret_cast<int*>(s.z + cap);
-  s.q = s.p + cap;
-  s.W = s.q + cap;
-  return s;
-}
-
-template <int WM, bool BATCH, bool LOWER>
+template <int WM, bool BATCH, bool LOWER, bool FOLD>
 __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
   constexpr bool WEIGHTED = WM != kNone;
+  constexpr int kWords = !WEIGHTED ? 1 : FOLD ? 3 : 4;
   extern __shared__ __align__(16) unsigned char smem[];
   const int nb = a.nb, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int group = a.group, gthreads = group * 32, g = warp / group, gt = tid - g * gthreads,
             wg = gt >> 5;
   const int npair = WEIGHTED ? nb * (nb + 1) / 2 : nb * nb;
-  const int nr = nb + 1;  // a row of cells: the bins of (j, k) and one for no edge
-  const int ncell = npair * nr;
+  // cells: rows of the bins of (j, k), unweighted one more for no edge;
+  // weighted, a word per lane for no edge after them
+  const int nr = WEIGHTED ? nb : nb + 1;
+  const int ncell = npair * nr, stride = ncell + (WEIGHTED ? 32 : 0);
   unsigned char* sp = smem;
-  unsigned long long* whist = reinterpret_cast<unsigned long long*>(sp);  // [nconf][2]
-  if (WEIGHTED) sp += (size_t)a.nconf * 16;
+  unsigned long long* whist = reinterpret_cast<unsigned long long*>(sp);  // FOLD: [nconf][2]
+  if (FOLD) sp += (size_t)a.nconf * 16;
   int64_t* s_e2 = reinterpret_cast<int64_t*>(sp);
   sp += ((size_t)(nb + 1) * 8 + 15) & ~(size_t)15;
   uint32_t* s_cfg = reinterpret_cast<uint32_t*>(sp);  // sorted triple of each configuration
   sp += ((size_t)a.nconf * 4 + 15) & ~(size_t)15;
-  unsigned* hist = reinterpret_cast<unsigned*>(sp);  // weighted: [nconf] counts
-  if (WEIGHTED) sp += ((size_t)a.nconf * 4 + 15) & ~(size_t)15;
-  unsigned* cell = reinterpret_cast<unsigned*>(sp);  // unweighted counts; weighted lo, Z, T
-  sp += ((size_t)ncell * (WEIGHTED ? 12 : 4) + 15) & ~(size_t)15;
+  unsigned* hist = reinterpret_cast<unsigned*>(sp);  // FOLD: [nconf] counts
+  if (FOLD) sp += ((size_t)a.nconf * 4 + 15) & ~(size_t)15;
+  unsigned* cell = reinterpret_cast<unsigned*>(sp);  // counts; weighted [w0,] w1, Z, T
+  sp += ((size_t)stride * kWords * 4 + 15) & ~(size_t)15;
   const Stage st_s = stage_at(sp + (size_t)g * stage_bytes(a.cap, WEIGHTED), a.cap);
   __shared__ int64_t s_hub[kTWarps];
   __shared__ int s_flush[kTWarps], s_cat, s_cur;
   __shared__ Cat s_c;  // batched: the current catalogue
   __shared__ unsigned long long s_pending;
 
-  for (int k = tid; k < ncell * (WEIGHTED ? 3 : 1); k += kTThreads) cell[k] = 0u;
-  for (int k = tid; k < nb * nb * nb; k += kTThreads) {
-    const int p = k / (nb * nb), q = (k / nb) % nb, r = k % nb;
-    if (p <= q && q <= r) s_cfg[conf3_rank(p, q, r, nb)] = p | (q << 8) | (r << 16);
-  }
-  if (WEIGHTED)
+  for (int k = tid; k < stride * kWords; k += kTThreads) cell[k] = 0u;
+  if (FOLD)
     for (int k = tid; k < a.nconf; k += kTThreads) {
       hist[k] = 0u;
       whist[2 * k] = whist[2 * k + 1] = 0ull;
     }
+  for (int k = tid; k < nb * nb * nb; k += kTThreads) {
+    const int p = k / (nb * nb), q = (k / nb) % nb, r = k % nb;
+    if (p <= q && q <= r) s_cfg[conf3_rank(p, q, r, nb)] = p | (q << 8) | (r << 16);
+  }
   for (int b = tid; b <= nb; b += kTThreads) s_e2[b] = a.e2g[b];
   if (tid == 0) {
     s_pending = 0;
@@ -1344,25 +1318,50 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
     if (gthreads == 32) __syncwarp();
     else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(gthreads) : "memory");
   };
-  // Adds the shared counts (and sums) to the global ones and clears them;
-  // exchanges, so that one group can do it while the others count on.
+  // Adds the cells to the global counts (and sums) and clears them; exchanges,
+  // so that one group can do it while the others count on. (Every word is its
+  // additions modulo 2^32 and every carry is added somewhere, so the global
+  // sums are right whichever flush takes a word or its carry.)
   auto flush = [&](int t, int threads) {
     if (cur < 0) return;
     for (int k = t; k < a.nconf; k += threads) {
-      if constexpr (WEIGHTED) {
+      const uint32_t f = s_cfg[k];
+      const int p = f & 255, q = (f >> 8) & 255, r = f >> 16;
+      if constexpr (FOLD) {  // one group: plain reads and writes
         const unsigned v = hist[k];
+        const unsigned long long lo = whist[2 * k], hi = whist[2 * k + 1];
         if (v) {
           atomicAdd(c.counts + k, (unsigned long long)v);
           hist[k] = 0u;
         }
-        const unsigned long long lo = whist[2 * k], hi = whist[2 * k + 1];
         if (lo | hi) {
           atomic_add_i192(c.wacc + 3 * k, lo, hi);
           whist[2 * k] = whist[2 * k + 1] = 0ull;
         }
+      } else if constexpr (WEIGHTED) {
+        const uint32_t cm = (1u << a.cb) - 1u;
+        unsigned long long slo = 0, num = 0;
+        long long shi = 0;
+        auto take = [&](int x, int y, int z) {  // x <= y the hub edges' bins
+          unsigned* w = cell + (y * (y + 1) / 2 + x) * nr + z;
+          const uint32_t w0 = atomicExch(w, 0u), w1 = atomicExch(w + stride, 0u),
+                         Z = atomicExch(w + 2 * stride, 0u), T = atomicExch(w + 3 * stride, 0u);
+          // Z with its carries is H 2^cb + the number of pairs
+          const long long n = (long long)(((unsigned long long)(T & 0xFFFFu) << a.cb) + (Z & cm));
+          const long long full =
+              (long long)(((unsigned long long)(long long)((int)T >> 16) << 32) | Z);
+          const unsigned long long add = ((unsigned long long)w1 << 32) | w0;
+          num += (unsigned long long)n;
+          slo += add;
+          shi += ((full - n) >> a.cb) + (slo < add ? 1 : 0);
+        };
+        take(p, q, r);
+        if (q != r) take(p, r, q);
+        if (p != q) take(q, r, p);
+        if (num) atomicAdd(c.counts + k, num);
+        if (slo | (unsigned long long)shi)
+          atomic_add_i192(c.wacc + 3 * k, slo, (unsigned long long)shi);
       } else {
-        const uint32_t f = s_cfg[k];
-        const int p = f & 255, q = (f >> 8) & 255, r = f >> 16;
         unsigned long long v = 0;
         auto take = [&](int x, int y, int z) {
           v += atomicExch(cell + (x * nb + y) * nr + z, 0u);
@@ -1377,63 +1376,52 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
       }
     }
   };
-  // Weighted: the hub's cells, times W_i, into the CTA's sums.
-  auto fold = [&](int64_t Wi) {
-    if constexpr (WEIGHTED) {
-      const uint32_t cm = (1u << a.cb) - 1u;
-      for (int k = tid; k < a.nconf; k += kTThreads) {
-        const uint32_t f = s_cfg[k];
-        const int p = f & 255, q = (f >> 8) & 255, r = f >> 16;
-        unsigned long long slo = 0, n = 0;
-        long long shi = 0;
-        auto take = [&](int x, int y, int z) {  // x <= y the hub edges' bins
-          const int i = (y * (y + 1) / 2 + x) * nr + z;
-          const uint32_t lo = cell[i], Z = cell[ncell + i], T = cell[2 * ncell + i];
-          if (!(lo | Z | T)) return;
-          cell[i] = cell[ncell + i] = 0u;
-          if (T) cell[2 * ncell + i] = 0u;
-          const long long num = (long long)(((unsigned long long)(T & 0xFFFFu) << a.cb) + (Z & cm));
-          // Z with its carries: H 2^cb + num
-          const long long full = (long long)(((unsigned long long)(long long)((int)T >> 16) << 32) |
-                                             Z);
-          const long long H = (full - num) >> a.cb;
-          n += (unsigned long long)num;
-          const unsigned long long add = ((unsigned long long)H << 32) | lo;
-          slo += add;
-          shi += (H >> 32) + (slo < add ? 1 : 0);
-        };
-        take(p, q, r);
-        if (q != r) take(p, r, q);
-        if (p != q) take(q, r, p);
-        if (!n) continue;
-        hist[k] += (unsigned)n;
-        // (shi, slo) W_i modulo 2^128
-        const unsigned long long w = (unsigned long long)Wi;
-        const unsigned long long plo = slo * w;
-        const unsigned long long phi = __umul64hi(slo, w) - (Wi < 0 ? slo : 0ull) +
-                                       (unsigned long long)shi * w;
-        const unsigned long long old = whist[2 * k], now = old + plo;
-        whist[2 * k] = now;
-        whist[2 * k + 1] += phi + (now < old ? 1ull : 0ull);
-      }
+
+  // FOLD: the hub's cells, times W_i, into the CTA's sums.
+  auto fold = [&](long long Wi) {
+    const uint32_t cm = (1u << a.cb) - 1u;
+    for (int k = tid; k < a.nconf; k += kTThreads) {
+      const uint32_t f = s_cfg[k];
+      const int p = f & 255, q = (f >> 8) & 255, r = f >> 16;
+      unsigned long long slo = 0, num = 0;
+      long long shi = 0;
+      auto take = [&](int x, int y, int z) {  // x <= y the hub edges' bins
+        unsigned* w = cell + (y * (y + 1) / 2 + x) * nr + z;
+        const uint32_t lo = w[0], Z = w[stride], T = w[2 * stride];
+        if (!(lo | Z | T)) return;
+        w[0] = w[stride] = 0u;
+        if (T) w[2 * stride] = 0u;
+        // Z with its carries is H 2^cb + the number of pairs
+        const long long n = (long long)(((unsigned long long)(T & 0xFFFFu) << a.cb) + (Z & cm));
+        const long long full =
+            (long long)(((unsigned long long)(long long)((int)T >> 16) << 32) | Z);
+        const long long H = (full - n) >> a.cb;
+        const unsigned long long add = ((unsigned long long)H << 32) | lo;
+        num += (unsigned long long)n;
+        slo += add;
+        shi += (H >> 32) + (slo < add ? 1 : 0);
+      };
+      take(p, q, r);
+      if (q != r) take(p, r, q);
+      if (p != q) take(q, r, p);
+      if (!num) continue;
+      hist[k] += (unsigned)num;
+      // (shi, slo) W_i modulo 2^128
+      const unsigned long long w = (unsigned long long)Wi;
+      const unsigned long long plo = slo * w;
+      const unsigned long long phi =
+          __umul64hi(slo, w) - (Wi < 0 ? slo : 0ull) + (unsigned long long)shi * w;
+      const unsigned long long old = whist[2 * k], now = old + plo;
+      whist[2 * k] = now;
+      whist[2 * k + 1] += phi + (now < old ? 1ull : 0ull);
     }
   };
 
   const uint32_t s_cell = (uint32_t)__cvta_generic_to_shared(cell);
-  [[maybe_unused]] const uint32_t zoff = (uint32_t)ncell * 4u, scale = 1u << a.cb;
-  // Exact bin of a pair near a bin edge, nb when it is no edge.
-  auto exact_bin = [&](float dx, float dy, float dz) -> int {
-    const long long x = (long long)(int)dx, y = (long long)(int)dy, z = (long long)(int)dz;
-    const long long D2 = x * x + y * y + z * z;
-    if (D2 < s_e2[0] || D2 >= s_e2[nb]) return nb;
-    int b = 0, e = nb;
-    while (e - b > 1) {
-      const int mid = (b + e) >> 1;
-      if (s_e2[mid] <= D2) b = mid;
-      else e = mid;
-    }
-    return b;
-  };
+  [[maybe_unused]] const uint32_t zoff = (uint32_t)stride * 4u, scale = 1u << a.cb,
+                                  none = s_cell + 4u * (uint32_t)(ncell + lane);
+  auto exact_bin = [&](float dx, float dy, float dz) { return t_exact_bin(s_e2, nb, dx, dy, dz); };
+  long long Wi = 0;
 
   // Pairs of one item: the lane's k (tile tk) with the nj j's of tile tj.
   auto item = [&](const Stage& S, int tk, int tj, int nk, int nj, auto diag) {
@@ -1441,7 +1429,8 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
     const int k = tk * 32 + lane;
     const float xk = lane < nk ? S.x[k] : kFarK, yk = S.y[k], zk = S.z[k];
     const int qk = S.q[k];
-    [[maybe_unused]] const int pk = WEIGHTED ? S.p[k] : 0, Wk = WEIGHTED ? S.W[k] : 0;
+    [[maybe_unused]] const int pk = WEIGHTED ? S.p[k] : 0;
+    [[maybe_unused]] const long long V = WEIGHTED ? (FOLD ? 1 : Wi) * S.W[k] : 0;
     const unsigned long long nx = t_pack(-xk, -xk), ny = t_pack(-yk, -yk), nz = t_pack(-zk, -zk);
         const uint32_t base = s_cell - 4u * kBin0<LOWER> + (WEIGHTED ? 0u : (uint32_t)qk);
     for (int j = tj * 32; j < tj * 32 + nj; j += 4) {
@@ -1503,13 +1492,13 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
               b[v] = kBin0<LOWER> +
                      (uint32_t)exact_bin(S.x[j + v] - xk, S.y[j + v] - yk, S.z[j + v] - zk);
         }
-        // misses branch off: returning atomics to one trash cell per row took
-        // 4.4 wavefronts each, those of the hits alone 2.6
+        uint32_t at[4];
 #pragma unroll
         for (int v = 0; v < 4; ++v)
-          if (b[v] < kBin0<LOWER> + (uint32_t)nb)
-          t_record<WM>(base + (uint32_t)(max(pp[v], pk) + min(qq[v], qk)) + 4u * b[v], zoff, ww[v],
-                       Wk, scale);
+          at[v] = b[v] < kBin0<LOWER> + (uint32_t)nb
+                      ? base + (uint32_t)(max(pp[v], pk) + min(qq[v], qk)) + 4u * b[v]
+                      : none;
+        t_record<WM, FOLD>(at, zoff, ww, V, scale);
       }
     }
   };
@@ -1517,6 +1506,7 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
   auto hub = [&](const Stage& S, int64_t i, int d) {
     const uint32_t* row = row_at(c.adj, c.ptr, i, c.adj_off, c.split, c.adj_off2);
     const int4 P = c.xyzp[i];
+    if (WEIGHTED) Wi = c.W[i];
     const int nt = (d + 31) >> 5;
     for (int s = gt; s < nt * 32; s += gthreads) {
       const int t = (s & 31) * nt + (s >> 5);
@@ -1578,11 +1568,10 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
       if (i >= 0) {
         const unsigned long long d = (unsigned long long)(BATCH ? a.cats[k].deg : a.one.deg)[i];
         const unsigned long long need = d * (d - (d > 0)) / 2;  // triangles at i <= C(d, 2)
-        // The shared counters stay below 2^32: between two flushes they take
-        // what was registered since the last reset (2^29 and one hub), what
-        // registers while a flush runs (the same) and the hubs under way at a
-        // reset (15 of at most 2^25).
-        if ((BATCH && k != s_cur) || atomicAdd(&s_pending, need) + need > (1ull << 29)) {
+        // Between two flushes the cells take what was registered since the
+        // last reset (limit and one hub), what registers while a flush runs
+        // (the same) and the hubs under way at a reset (tile_launch).
+        if ((BATCH && k != s_cur) || atomicAdd(&s_pending, need) + need > a.limit) {
           atomicExch(&s_pending, BATCH ? need : 0ull);
           s_flush[g] = 1;
           if (BATCH) s_cur = k;
@@ -1594,7 +1583,7 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
     if (i < 0) break;
     if (s_flush[g]) {
       flush(gt, gthreads);
-      if (WEIGHTED || BATCH) sync();
+      if (BATCH || FOLD) sync();
     }
     if (BATCH && s_cat != cur) {
       cur = s_cat;
@@ -1611,7 +1600,7 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
                    a.gstride / (WEIGHTED ? 24 : 20)),
           i, d);
     else hub(st_s, i, d);
-    if (WEIGHTED) fold(c.W[i]);  // ordered by the barrier at the top
+    if constexpr (FOLD) fold(Wi);  // ordered by the barrier at the top
   }
   __syncthreads();
   flush(tid, kTThreads);
@@ -1930,43 +1919,33 @@ PairLaunch pair_launch(int nb, int nconf, bool weighted, bool use_lut,
 // Launch plan of the tiled pair kernel; cap 0: another kernel takes the call.
 struct TileLaunch {
   int cap = 0, group = kTWarps, blocks = 0;
+  bool lower = false, fold = false;
   size_t smem = 0;
-  TArgs a;  // the binning constants
+  TArgs a;  // binning and flush constants
 };
 
-// mean: mean row length. Conditions: bins evenly spaced to within 1/128 of
-// their width (edges rounded to the lattice are), two CTAs per SM, and
-// (weighted) rows long enough to pay for folding the cells at every hub.
+// mean: mean row length. The kernel takes evenly spaced bins whose cells leave
+// room for two CTAs per SM.
 TileLaunch tile_launch(int nb, int nconf, const FixedW* fw, bool batch, double mean, int max_deg,
                        const std::vector<int64_t>& edges) {
   TileLaunch L;
-  if (max_deg > kTMaxDeg) return L;
+  const TileBins bins = tile_bins(edges);
+  if (!bins.ok || max_deg > kTMaxDeg) return L;
   const bool weighted = fw != nullptr;
-  const double w = (double)(edges[nb] - edges[0]) / nb;
-  if (nb > kTileMaxBins) return L;
-  double dev = 0.0;  // edges off the even spacing, in bin widths
-  for (int b = 0; b <= nb; ++b)
-    dev = std::max(dev, std::fabs((double)(edges[b] - edges[0]) / w - b));
-  // D = sqrt(D2): relative error below 0.75 2^-21 from the squared distance
-  // (three roundings, halved), the approximate square root (2^-23) and c
-  // (2^-24), at most E_nb / w bin widths; m's rounding; half a unit for u
-  const double off = (double)edges[0] / w, one = 65536.0;
-  const double err = (double)edges[nb] / w * std::ldexp(0.75, -21) + dev +
-                     std::max(kTileM + 1.0, off) * std::ldexp(1.0, -24);
-  if (err > 1.0 / 128) return L;
-  const int delta = (int)std::ceil(err * one + 0.75);
-  L.a.c = (float)(1.0 / w);
-  L.a.m = (float)(kTileM + delta / one - off);
-  L.a.amb = 2u * (uint32_t)delta;
+  L.a.c = bins.c;
+  L.a.m = bins.m;
+  L.a.amb = bins.amb;
+  L.lower = bins.lower;
   L.a.cb = 0;
+  // sums per hub (two atomics a pair) where the pairs of a row outweigh its
+  // pass over the configurations: 402 edges a row and 1540 configurations, 409
+  // ms against 539 with three atomics; 134 a row, 39 against 25
+  L.fold = weighted && 0.5 * mean * mean >= 16.0 * nconf;
   if (weighted) {
-    // |x| < 2^(2 mag): high words below 2^hb; the count field and the sum's
-    // carries are then equally rare
-    const int hb = std::max(2 * fw->mag - 32, 0);
+    // |x| < 2^(2 mag) or 2^(3 mag): high words below 2^hb; the count field and
+    // the sum's carries are then equally rare
+    const int hb = std::max(L.fold ? 2 * fw->mag - 32 : 3 * fw->mag - 64, 0);
     L.a.cb = std::min((32 - hb) / 2, 12);
-    const double pairs = 0.5 * max_deg * (max_deg - 1.0);
-    if (pairs >= std::ldexp(1.0, 14 + L.a.cb)) return L;  // T's halves
-    if (0.5 * mean * (mean - 1.0) < 2.0 * nconf) return L;
   }
   L.a.nb = nb;
   L.a.nconf = nconf;
@@ -1975,19 +1954,39 @@ TileLaunch tile_launch(int nb, int nconf, const FixedW* fw, bool batch, double m
   cudaDeviceGetAttribute(&per_sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev_id);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id);
   auto pad16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
-  const size_t ncell = (size_t)(weighted ? nb * (nb + 1) / 2 : nb * nb) * (nb + 1);
-  const size_t fixed = (weighted ? (size_t)nconf * 16 + pad16((size_t)nconf * 4) : 0) +
+  const size_t ncell = weighted ? (size_t)nb * (nb + 1) / 2 * nb + 32 : (size_t)nb * nb * (nb + 1);
+  const size_t fixed = (L.fold ? (size_t)nconf * 16 + pad16((size_t)nconf * 4) : 0) +
                        pad16((size_t)(nb + 1) * 8) + pad16((size_t)nconf * 4) +
-                       pad16(ncell * (weighted ? 12 : 4));
+                       pad16(ncell * 4 * (!weighted ? 1 : L.fold ? 3 : 4));
   const size_t budget = (size_t)per_sm_bytes / 2 - 1024 - 512;  // static shared memory and slack
-  if (fixed + 2 * stage_bytes(32, weighted) > budget) return L;
-  const int want = std::min(max_deg, std::max(64, (int)(2.5 * mean)));
-  // few warps per hub where rows are short
-  int group = (weighted || batch) ? kTWarps : mean <= 64 ? 1 : mean <= 160 ? 4 : mean <= 320 ? 8 : kTWarps;
+  if (fixed + 8 * stage_bytes(32, weighted) > budget) return L;
+  const int want = std::min(max_deg, std::max(64, (int)(1.8 * mean)));
+  // few warps per hub where rows are short (a hub's barriers cost the same
+  // however many warps wait for them); more where the staging would not fit
+  int group = batch || L.fold ? kTWarps : mean <= 64 ? 1 : mean <= 160 ? 4 : 8;
   for (;; group = group == 1 ? 4 : group * 2) {
     const size_t room = (budget - fixed) / (kTWarps / group);
     L.cap = (int)(room / (weighted ? 24 : 20)) & ~31;
     if (L.cap >= want || group == kTWarps) break;
+  }
+  // Pairs a cell may take between flushes: 2 limit + (groups + 1) hubs, see
+  // the kernel. Counts below 2^32; weighted, T's halves below 2^15, that is
+  // 2^(15 + cb) pairs.
+  // (FOLD: T's halves hold one hub, the counts below 2^32 many.)
+  const double hub = 0.5 * max_deg * (max_deg - 1.0);
+  const int room_bits = weighted && !L.fold ? 15 + L.a.cb : 32;
+  L.a.limit = 1ull << (room_bits - 2);
+  if (L.fold && hub >= std::ldexp(1.0, 14 + L.a.cb)) {
+    L.cap = 0;
+    return L;
+  }
+  if (hub * (kTWarps / group + 1) >= std::ldexp(1.0, room_bits - 1)) {
+    group = kTWarps;
+    if (hub * 2 >= std::ldexp(1.0, room_bits - 1)) {
+      L.cap = 0;
+      return L;
+    }
+    L.cap = (int)((budget - fixed) / (weighted ? 24 : 20)) & ~31;
   }
   L.cap = std::min(L.cap, (max_deg + 31) & ~31);
   if (L.cap < 32) L.cap = 0;
@@ -1998,11 +1997,12 @@ TileLaunch tile_launch(int nb, int nconf, const FixedW* fw, bool batch, double m
 }
 
 template <bool BATCH>
-void (*pick_count3t(int wm, bool nonneg, bool lower))(TArgs) {
-#define GS_T(W) (lower ? k_count3t<W, BATCH, true> : k_count3t<W, BATCH, false>)
-  if (wm == kNone) return GS_T(kNone);
-  return nonneg ? GS_T(kExactPos) : GS_T(kExact);
-#undef GS_T
+void (*pick_count3t(int wm, bool nonneg, const TileLaunch& L))(TArgs) {
+  if (wm == kNone)
+    return L.lower ? k_count3t<kNone, BATCH, true, false> : k_count3t<kNone, BATCH, false, false>;
+  if (nonneg)
+    return L.fold ? k_count3t<kExactPos, BATCH, true, true> : k_count3t<kExactPos, BATCH, true, false>;
+  return L.fold ? k_count3t<kExact, BATCH, true, true> : k_count3t<kExact, BATCH, true, false>;
 }
 
 }  // namespace
@@ -2178,7 +2178,7 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
     ta.group = TL.group;
     ta.e2g = g.d_edges2;
     ta.hub_counter = a.hub_counter;
-    void (*kern)(TArgs) = pick_count3t<false>(wm, fw && fw->nonneg, g.edges[0] > 0);
+    void (*kern)(TArgs) = pick_count3t<false>(wm, fw && fw->nonneg, TL);
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TL.smem);
     // no more CTAs than the hubs keep busy
     const int groups = kTWarps / TL.group;
@@ -2382,7 +2382,7 @@ int count3_batch_device(const Graph* const* gr, int ng, const FixedW* fws, uint6
     ta.group = TL.group;
     ta.e2g = gr[0]->d_edges2;
     ta.hub_counter = a.hub_counter;
-    void (*kern)(TArgs) = pick_count3t<true>(wm, nonneg, gr[0]->edges[0] > 0);
+    void (*kern)(TArgs) = pick_count3t<true>(wm, nonneg, TL);
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TL.smem);
     const int grid = (int)std::min<int64_t>(TL.blocks, base[ng]);
     ta.gscratch = nullptr;
