@@ -19,8 +19,10 @@
 // weighted sums of W_i W_j W_k go straight to 192-bit global sums.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "gs_internal.cuh"
+#include "gs_tiles.cuh"
 
 namespace gs {
 
@@ -254,6 +256,318 @@ __global__ void __launch_bounds__(kMThreads, 2) k_count3mu(MArgs a) {
   flush();
 }
 
+// ----------------------------------------------------------------------------
+// Tiled kernel (unweighted, evenly spaced bins, counters in shared memory): the
+// row in tiles and the pair test as in k_count3t, the normal in single
+// precision too. The cross product's components carry an error below 2^-22.2 L,
+// L = |D_j| |D_k|, so t = nmu |n_z| / |n| is within 2^-12 nmu / (2^3.5 s) + nmu
+// 2^-21 < 2^-12 of its value where |n| >= s L, s = nmu 2^-8.5; it is kept in
+// fixed point with 16 fraction bits, and pairs with t within 2^-12 of an
+// integer or a smaller |n| (about one in a thousand) go to the exact
+// comparisons, as do pairs near a bin edge. The configuration comes from a
+// shared table with an extra bin for pairs that are no edge.
+// 1e6 uniform points (402 edges a row, 20 bins, 10 mu bins): 158 ms against 330
+// for k_count3mu on the same graph.
+struct MTArgs {
+  const int64_t* __restrict__ ptr;
+  const int32_t* __restrict__ deg;
+  const uint32_t* __restrict__ adj;
+  int64_t adj_off, split, adj_off2;
+  int64_t hub_begin, hub_end;
+  const int4* __restrict__ xyzp;
+  int64_t box;
+  const int64_t* __restrict__ e2g;
+  int nb, nconf, nmu;
+  int cap, group;
+  float c, m;    // see TileBins
+  uint32_t amb;
+  float kappa;   // s^2
+  unsigned long long* counts;
+  unsigned long long* hub_counter;
+  unsigned char* gscratch;
+  size_t gstride;
+};
+constexpr uint32_t kMuAmb = 32;  // 2^-12 to both sides, in 2^-16
+constexpr float kMuM = kTileM + 16.0f / 65536.0f;
+
+template <bool LOWER>
+__global__ void __launch_bounds__(kTThreads, 2) k_mu_tiles(MTArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int nb = a.nb, nm1 = a.nmu + 1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int group = a.group, gthreads = group * 32, g = warp / group, gt = tid - g * gthreads,
+            wg = gt >> 5;
+  const int ncell = a.nconf * nm1;
+  unsigned char* sp = smem;
+  int64_t* s_e2 = reinterpret_cast<int64_t*>(sp);
+  sp += ((size_t)(nb + 1) * 8 + 15) & ~(size_t)15;
+  uint16_t* s_lut = reinterpret_cast<uint16_t*>(sp);  // [nb][nb][nb + 1]
+  sp += ((size_t)nb * nb * (nb + 1) * 2 + 15) & ~(size_t)15;
+  unsigned* hist = reinterpret_cast<unsigned*>(sp);  // [nconf + 1][nmu + 1]
+  sp += ((size_t)(ncell + nm1) * 4 + 15) & ~(size_t)15;
+  const size_t sbytes = stage_bytes(a.cap, false) + (size_t)a.cap * 4;
+  const Stage st_s = stage_at(sp + (size_t)g * sbytes, a.cap);
+  __shared__ int64_t s_hub[kTWarps];
+  __shared__ int s_flush[kTWarps];
+  __shared__ unsigned long long s_pending;
+  for (int k = tid; k < ncell; k += kTThreads) hist[k] = 0u;
+  for (int k = tid; k < nb * nb * (nb + 1); k += kTThreads) {
+    const int r = k % (nb + 1), q = (k / (nb + 1)) % nb, p = k / ((nb + 1) * nb);
+    s_lut[k] = (uint16_t)(r == nb ? a.nconf : conf3_rank(p, q, r, nb));
+  }
+  for (int b = tid; b <= nb; b += kTThreads) s_e2[b] = a.e2g[b];
+  if (tid == 0) s_pending = 0;
+  __syncthreads();
+
+  auto sync = [&]() {
+    if (gthreads == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(gthreads) : "memory");
+  };
+  auto flush = [&](int t, int threads) {
+    for (int k = t; k < ncell; k += threads) {
+      const unsigned v = atomicExch(hist + k, 0u);
+      if (v) atomicAdd(a.counts + k, (unsigned long long)v);
+    }
+  };
+  const uint32_t lut0 =
+      (uint32_t)__cvta_generic_to_shared(s_lut) - 2u * kBin0<LOWER>;
+  const uint32_t hist0 = (uint32_t)__cvta_generic_to_shared(hist);
+
+  // Pairs of the lane's k (tile tk) with the nj j's of tile tj. S.W holds
+  // s^2 |D_j|^2 as a float.
+  auto item = [&](const Stage& S, int tk, int tj, int nk, int nj, auto diag) {
+    constexpr bool DIAG = decltype(diag)::value;
+    const int k = tk * 32 + lane;
+    const float xk = lane < nk ? S.x[k] : kFarK, yk = S.y[k], zk = S.z[k];
+    const uint32_t lrow = lut0 + (uint32_t)S.q[k];
+    const unsigned long long nx = t_pack(-xk, -xk), ny = t_pack(-yk, -yk), nz = t_pack(-zk, -zk);
+    const unsigned long long px = t_pack(xk, xk), py = t_pack(yk, yk), pz = t_pack(zk, zk);
+    const float lk = fmaf(zk, zk, fmaf(yk, yk, xk * xk));
+    for (int j = tj * 32; j < tj * 32 + nj; j += 4) {
+      float u[4], t[4], q[4];
+      {
+        const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(S.x + j);
+        const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(S.y + j);
+        const ulonglong2 Z = *reinterpret_cast<const ulonglong2*>(S.z + j);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const unsigned long long xj = h ? X.y : X.x, yj = h ? Y.y : Y.x, zj = h ? Z.y : Z.x;
+          const unsigned long long dx = t_add(xj, nx), dy = t_add(yj, ny), dz = t_add(zj, nz);
+          float e0, e1;
+          t_unpack(t_fma(dz, dz, t_fma(dy, dy, t_mul(dx, dx))), e0, e1);
+          u[2 * h] = fmaf(t_sqrt(e0), a.c, a.m);
+          u[2 * h + 1] = fmaf(t_sqrt(e1), a.c, a.m);
+          const unsigned long long cx = t_fma(yj, pz, t_mul(zj, ny)),
+                                   cy = t_fma(zj, px, t_mul(xj, nz)),
+                                   cz = t_fma(xj, py, t_mul(yj, nx));
+          t_unpack(t_fma(cx, cx, t_fma(cy, cy, t_mul(cz, cz))), q[2 * h], q[2 * h + 1]);
+          t_unpack(cz, t[2 * h], t[2 * h + 1]);
+        }
+      }
+      if (DIAG) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v)  // each pair once
+          if (j - tj * 32 + v >= lane) {
+            u[v] = __uint_as_float(0x7F7FFFFFu);
+            q[v] = 3.0e38f;
+          }
+      }
+      const float4 sj = *reinterpret_cast<const float4*>(S.W + j);
+      const float ss[4] = {sj.x, sj.y, sj.z, sj.w};
+      const int4 pj = *reinterpret_cast<const int4*>(S.p + j);
+      const int pp[4] = {pj.x, pj.y, pj.z, pj.w};
+      float flat = 3.0e38f;  // the least |n|^2 - s^2 L^2
+      uint32_t b[4], mu[4];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        flat = fminf(flat, fmaf(-ss[v], lk, q[v]));
+        t[v] = fmaf(fabsf(t[v]) * rsqrtf(q[v]), (float)a.nmu, kMuM);
+        if (DIAG && j - tj * 32 + v >= lane) t[v] = __uint_as_float(0x7F7FFFFFu);
+        b[v] = t_bin<LOWER>(u[v], nb);
+        mu[v] = min((__float_as_uint(t[v]) >> 16) - (kTileBits >> 16), (uint32_t)a.nmu);
+      }
+      const uint32_t near2 = __vminu2(
+          __byte_perm(__float_as_uint(u[0]), __float_as_uint(u[1]), 0x5410),
+          __byte_perm(__float_as_uint(u[2]), __float_as_uint(u[3]), 0x5410));
+      const uint32_t nearm = __vminu2(
+          __byte_perm(__float_as_uint(t[0]), __float_as_uint(t[1]), 0x5410),
+          __byte_perm(__float_as_uint(t[2]), __float_as_uint(t[3]), 0x5410));
+      if (min(near2 & 0xFFFFu, near2 >> 16) <= a.amb || min(nearm & 0xFFFFu, nearm >> 16) <= kMuAmb ||
+          !(flat > 0.f)) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          if ((__float_as_uint(u[v]) & 0xFFFFu) <= a.amb)
+            b[v] = kBin0<LOWER> +
+                   (uint32_t)t_exact_bin(s_e2, nb, S.x[j + v] - xk, S.y[j + v] - yk, S.z[j + v] - zk);
+          if (b[v] < kBin0<LOWER> + (uint32_t)nb &&
+              ((__float_as_uint(t[v]) & 0xFFFFu) <= kMuAmb || !(fmaf(-ss[v], lk, q[v]) > 0.f))) {
+            const long long jx = (long long)(int)S.x[j + v], jy = (long long)(int)S.y[j + v],
+                            jz = (long long)(int)S.z[j + v], kx = (long long)(int)xk,
+                            ky = (long long)(int)yk, kz = (long long)(int)zk;
+            mu[v] = (uint32_t)mu_bin(jy * kz - jz * ky, jz * kx - jx * kz, jx * ky - jy * kx, a.nmu);
+          }
+        }
+      }
+      uint32_t cf[4];
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+        asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}"
+                     : "=r"(cf[v])
+                     : "r"(lrow + (uint32_t)pp[v] + 2u * b[v]));
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+        t_red(hist0 + cf[v] * (uint32_t)(4 * nm1) + 4u * mu[v], 1u);
+    }
+  };
+  auto hub = [&](const Stage& S, int64_t i, int d) {
+    const uint32_t* row = row_at(a.adj, a.ptr, i, a.adj_off, a.split, a.adj_off2);
+    const int4 P = a.xyzp[i];
+    const int nt = (d + 31) >> 5;
+    for (int s = gt; s < nt * 32; s += gthreads) {
+      const int t = (s & 31) * nt + (s >> 5);
+      float x = kFarJ, y = 0.f, z = 0.f;
+      int b = 0;
+      if (t < d) {
+        const uint32_t w = row[t];
+        const int4 Q = a.xyzp[edge_id(w)];
+        b = (int)edge_bin(w);
+        x = (float)t_min_image(Q.x, P.x, a.box);
+        y = (float)t_min_image(Q.y, P.y, a.box);
+        z = (float)t_min_image(Q.z, P.z, a.box);
+      }
+      S.x[s] = x;
+      S.y[s] = y;
+      S.z[s] = z;
+      S.p[s] = 2 * (nb + 1) * nb * b;
+      S.q[s] = 2 * (nb + 1) * b;
+      S.W[s] = __float_as_int(a.kappa * fmaf(z, z, fmaf(y, y, x * x)));
+    }
+    sync();
+    const int dq = d / nt, dr = d - dq * nt;
+    for (int tk = 0, tj = wg;; tj += group) {
+      while (tk < nt && tj > tk) tj -= ++tk;
+      if (tk >= nt) break;
+      const int nk = dq + (tk < dr ? 1 : 0), nj = dq + (tj < dr ? 1 : 0);
+      if (tj == tk) item(S, tk, tj, nk, nk - 1, std::true_type{});
+      else item(S, tk, tj, nk, nj, std::false_type{});
+    }
+    sync();
+  };
+
+  for (;;) {
+    if (gt == 0) {
+      int64_t i = a.hub_begin + (int64_t)atomicAdd(a.hub_counter, 1ull);
+      if (i >= a.hub_end) i = -1;
+      s_hub[g] = i;
+      s_flush[g] = 0;
+      if (i >= 0) {
+        const unsigned long long d = (unsigned long long)a.deg[i];
+        const unsigned long long need = d * (d - (d > 0)) / 2;
+        // counters below 2^32: twice the limit and the hubs under way (16 of
+        // at most 2^25 pairs)
+        if (atomicAdd(&s_pending, need) + need > (1ull << 30)) {
+          atomicExch(&s_pending, 0ull);
+          s_flush[g] = 1;
+        }
+      }
+    }
+    sync();
+    const int64_t i = s_hub[g];
+    if (i < 0) break;
+    if (s_flush[g]) flush(gt, gthreads);
+    const int d = a.deg[i];
+    if (d < 2) {
+      sync();
+      continue;
+    }
+    if (d > a.cap)
+      hub(stage_at(a.gscratch + ((size_t)blockIdx.x * (kTWarps / group) + g) * a.gstride,
+                   a.gstride / 24),
+          i, d);
+    else hub(st_s, i, d);
+  }
+  __syncthreads();
+  flush(tid, kTThreads);
+}
+
+// Launches k_mu_tiles; false when the call is another kernel's.
+bool mu_tiles(const Graph& g, int nmu, int nconf, uint64_t* d_counts, unsigned long long* counter,
+              const Opts& o, Scratch& sc, KernelTimer& timer, int* status) {
+  const TileBins bins = tile_bins(g.edges);
+  if (!bins.ok || g.max_deg > kTMaxDeg || g.n == 0 || nmu > kTileMaxBins || nconf > 65534)
+    return false;
+  int dev = 0, sms = 0, per_sm = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  auto pad16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
+  const size_t nb = (size_t)g.nb;
+  const size_t fixed = pad16((nb + 1) * 8) + pad16(nb * nb * (nb + 1) * 2) +
+                       pad16(((size_t)nconf + 1) * (nmu + 1) * 4);
+  // two CTAs per SM, or one where the counters need it
+  size_t budget = (size_t)per_sm / 2 - 1024 - 512;
+  int ctas = 2;
+  const int mean = (int)(g.edges_total / g.n);
+  const int want = std::min(g.max_deg, std::max(64, mean * 9 / 5));
+  if (fixed + 24 * 256 > budget) {
+    budget = (size_t)optin - 512;
+    ctas = 1;
+    if (fixed + 24 * 256 > budget) return false;
+  }
+  MTArgs a;
+  a.group = mean <= 64 ? 1 : mean <= 160 ? 4 : 8;
+  for (;; a.group = a.group == 1 ? 4 : a.group * 2) {
+    a.cap = (int)((budget - fixed) / (kTWarps / a.group) / 24) & ~31;
+    if (a.cap >= want || a.group == kTWarps) break;
+  }
+  a.cap = std::min(a.cap, (g.max_deg + 31) & ~31);
+  if (a.cap < 32) return false;
+  const int groups = kTWarps / a.group;
+  const size_t smem = fixed + (size_t)groups * a.cap * 24;
+  a.ptr = g.d_ptr;
+  a.deg = g.d_deg;
+  a.xyzp = g.d_xyzp;
+  a.box = g.box_u;
+  a.e2g = g.d_edges2;
+  a.nb = g.nb;
+  a.nconf = nconf;
+  a.nmu = nmu;
+  a.c = bins.c;
+  a.m = bins.m;
+  a.amb = bins.amb;
+  a.kappa = (float)(nmu * nmu * std::ldexp(1.0, -17));
+  a.counts = reinterpret_cast<unsigned long long*>(d_counts);
+  a.hub_counter = counter;
+  void (*kern)(MTArgs) = bins.lower ? k_mu_tiles<true> : k_mu_tiles<false>;
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int grid = (int)std::min<int64_t>((int64_t)ctas * sms, (g.n + groups - 1) / groups);
+  a.gscratch = nullptr;
+  a.gstride = 0;
+  *status = GS_OK;
+  if (g.max_deg > a.cap) {
+    a.gstride = (size_t)((g.max_deg + 31) & ~31) * 24;
+    a.gscratch = sc.alloc<unsigned char>(a.gstride * grid * groups);
+    if (!a.gscratch) {
+      *status = GS_ENOMEM;
+      return true;
+    }
+  }
+  timer.start(o.stream);
+  *status = for_each_window(g, o, sc, [&](const WinView& v) -> int {
+    a.adj = v.adj;
+    a.adj_off = v.off1;
+    a.split = v.split;
+    a.adj_off2 = v.off2;
+    a.hub_begin = v.h0;
+    a.hub_end = v.h1;
+    cudaMemsetAsync(a.hub_counter, 0, sizeof(unsigned long long), o.stream);
+    { kern<<<grid, kTThreads, smem, o.stream>>>(a); note_launch(); }
+    return cuda_status(cudaGetLastError());
+  });
+  timer.stop(o.stream);
+  return true;
+}
+
 }  // namespace
 
 int count3mu_device(const Graph& g, const FixedW* fw, int nmu, uint64_t* d_counts,
@@ -287,6 +601,20 @@ int count3mu_device(const Graph& g, const FixedW* fw, int nmu, uint64_t* d_count
   cudaMemsetAsync(d_counts, 0, sizeof(uint64_t) * ncell, s);
   if (weighted) cudaMemsetAsync(a.wacc, 0, sizeof(unsigned long long) * 3 * ncell, s);
 
+  KernelTimer timer(o.kernel_ms);
+  int st = GS_OK;
+  if (!weighted && mu_tiles(g, nmu, nconf, d_counts, a.hub_counter, o, sc, timer, &st)) {
+    if (st) return st;
+    if (d_wsum) {
+      const int blocks = (int)std::min<int64_t>((ncell + 255) / 256, 4096);
+      k_u64_to_double<<<blocks, 256, 0, s>>>(a.counts, ncell, d_wsum);
+      note_launch();
+    }
+    const cudaError_t e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cuda_status(e);
+    timer.publish();
+    return cuda_status(cudaGetLastError());
+  }
   int dev = 0, sms = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -336,9 +664,7 @@ int count3mu_device(const Graph& g, const FixedW* fw, int nmu, uint64_t* d_count
     a.gscratch = sc.alloc<unsigned char>(a.gstride * grid);
     if (!a.gscratch) return GS_ENOMEM;
   }
-  KernelTimer timer(o.kernel_ms);
   timer.start(s);
-  int st = GS_OK;
   if (g.n > 0)
     st = for_each_window(g, o, sc, [&](const WinView& v) -> int {
       a.adj = v.adj;

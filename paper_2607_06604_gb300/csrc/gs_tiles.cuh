@@ -94,6 +94,16 @@ __device__ inline Stage stage_at(unsigned char* b, int64_t cap) {
   return s;
 }
 
+// Minimum-image difference q - p of coordinates.
+__device__ inline int t_min_image(int q, int p, int64_t box) {
+  int64_t d = (int64_t)q - p;
+  if (box) {
+    if (2 * d >= box) d -= box;
+    else if (2 * d < -box) d += box;
+  }
+  return (int)d;
+}
+
 // Exact bin of a pair from its displacement (integers held in floats), nb
 // when it is no edge.
 __device__ inline int t_exact_bin(const int64_t* e2, int nb, float dx, float dy, float dz) {

@@ -115,3 +115,23 @@ def test_batch_of_unequal_catalogues_and_windows(gs):
     assert np.array_equal(c, refs[2][0]) and np.array_equal(s, refs[2][1])
     parts = [gs.gs_count_3pcf(graphs[2], shard=k, shards=3) for k in range(3)]
     assert np.array_equal(sum(parts), refs[2][0])
+
+
+@pytest.mark.parametrize("n", [33, 64, 130])
+@pytest.mark.parametrize("nmu", [1, 5, 62, 64])
+@pytest.mark.parametrize("flat", [False, True])
+def test_mu_rows_and_degenerate_normals(gs, n, nmu, flat):
+    """Rows around multiples of 32; a coarse lattice (normals exactly on mu
+    edges, collinear and coincident points) or a plate two units thick."""
+    rng = np.random.default_rng(n + nmu)
+    d = rng.integers(-2, 3, size=(n, 3)) * 800
+    if flat:
+        d = rng.integers(-2500, 2501, size=(n, 3))
+        d[:, 1] = rng.integers(0, 3, size=n)
+    X = (50_000 + d).astype(np.int32)
+    for edges in (1600 * np.arange(6), np.array([500, 1901, 3300, 4700, 6100])):
+        edges = edges.astype(np.int64)
+        ref = oracle.Graph(X, 200_000, edges).count_3pcf_mu(nmu)
+        ref = ref[0] if isinstance(ref, tuple) else ref
+        got = gs.gs_count_3pcf_mu(gs.gs_build_graph(X, 200_000, edges), nmu)
+        assert np.array_equal(got, np.asarray(ref).reshape(got.shape))
