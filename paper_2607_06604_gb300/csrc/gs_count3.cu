@@ -1607,174 +1607,261 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
 }
 
 // Equilateral configurations (b, b, b) by pair geometry: a triangle is
-// equilateral in this sense only when both hub edges share bin b, so the CTA
-// stages N+(i) grouped by the hub edge's bin (a counting sort in shared
-// memory) and tests only the pairs within a group, against the one range
-// [E_b, E_b+1). Counts go to per-CTA 32-bit histograms [nb]; weighted, W_j W_k
-// to the hub's 96-bit sums [nb] folded by W_i into the CTA's 128-bit sums,
-// as in the other triangle kernels.
-template <int WM>
-__global__ void __launch_bounds__(kPThreads, 2) k_equi3p(PArgs a) {
-  constexpr bool WEIGHTED = WM != kNone;
+// equilateral in this sense only when both hub edges share bin b, so a hub's
+// neighbours are staged by hub-edge bin (a counting sort in shared memory) and
+// only pairs within a bin are tested, against the one range [E_b, E_b+1).
+// Within a bin the pairs go tile by tile as in k_count3t: k in the lanes, four
+// j's per broadcast. v = |D2 s_b - o_b| - 1 in single precision is negative
+// inside the range; pairs with |v| within the bound of zero are decided in
+// integers. A lane counts its hits and sums their W_j in registers; one warp
+// sum per tile pair, times W_k and W_i, goes to the CTA's counts and 128-bit
+// sums [nb]. Groups of a few warps take a hub each.
+// Bound by instruction issue in the staging and the tiles' ragged ends. 1e6
+// uniform points (402 edges a row, 20 bins), weighted: 20.4 ms against 45.5
+// for a CTA per hub that spread the pairs of four rows over the lanes as one
+// list (two random 16-byte loads a pair).
+struct EArgs {
+  Cat one;
+  int nb, cap, group;
+  const int64_t* e2g;
+  unsigned char* gscratch;  // hubs above cap: per-group staging in global memory
+  size_t gstride;
+  unsigned long long* hub_counter;
+};
+
+// Staging entries of a hub of d neighbours: bins start at multiples of four.
+__host__ __device__ inline int64_t equi_entries(int64_t d, int nb) {
+  return (d + 3 * (int64_t)(nb < d ? nb : d) + 7) & ~(int64_t)3;
+}
+
+template <bool WEIGHTED>
+__global__ void __launch_bounds__(kTThreads, 2) k_equi_tiles(EArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  int4* s_stage = reinterpret_cast<int4*>(smem);
-  __shared__ int64_t s_e2[kMaxBins + 1];
-  __shared__ int s_cnt[kMaxBins + 1], s_cur[kMaxBins + 1];
-  __shared__ unsigned s_hist[kMaxBins];
-  __shared__ unsigned s_hacc[WEIGHTED ? 3 * kMaxBins : 1];
-  __shared__ unsigned long long s_whist[WEIGHTED ? 2 * kMaxBins : 1];
-  __shared__ int64_t s_hub;
+  const int nb = a.nb, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int group = a.group, gthreads = group * 32, g = warp / group, gt = tid - g * gthreads,
+            wg = gt >> 5;
+  const int ngroups = kTWarps / group;
+  unsigned char* sp = smem;
+  unsigned long long* s_sum = reinterpret_cast<unsigned long long*>(sp);  // [nb][2]
+  if (WEIGHTED) sp += (size_t)nb * 16;
+  int64_t* s_e2 = reinterpret_cast<int64_t*>(sp);
+  sp += ((size_t)(nb + 1) * 8 + 15) & ~(size_t)15;
+  float4* s_rng = reinterpret_cast<float4*>(sp);  // s_b, o_b, bound
+  sp += (size_t)nb * 16;
+  unsigned* s_cnt = reinterpret_cast<unsigned*>(sp);
+  sp += ((size_t)nb * 4 + 15) & ~(size_t)15;
+  int* s_off = reinterpret_cast<int*>(sp) + g * 2 * (nb + 1);  // starts, then ends, by bin
+  int* s_end = s_off + nb + 1;
+  sp += ((size_t)ngroups * 2 * (nb + 1) * 4 + 15) & ~(size_t)15;
+  const int words = WEIGHTED ? 4 : 3;
+  float* st_s = reinterpret_cast<float*>(sp) + (size_t)g * a.cap * words;
+  __shared__ int64_t s_hub[kTWarps];
+  __shared__ int s_flush[kTWarps];
   __shared__ unsigned long long s_pending;
-  __shared__ int s_flush, s_next;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int nb = a.nb;
-  for (int b = tid; b <= nb; b += kPThreads) s_e2[b] = a.e2g[b];
-  for (int b = tid; b < nb; b += kPThreads) {
-    s_hist[b] = 0u;
-    if (WEIGHTED) {
-      s_hacc[3 * b] = s_hacc[3 * b + 1] = s_hacc[3 * b + 2] = 0u;
-      s_whist[2 * b] = s_whist[2 * b + 1] = 0ull;
-    }
+  for (int b = tid; b <= nb; b += kTThreads) s_e2[b] = a.e2g[b];
+  for (int b = tid; b < nb; b += kTThreads) {
+    // half the range's width in D2 is 1 / s_b; the squared distance's three
+    // roundings and those of the product and the constants stay below
+    // 6 2^-24 of o_b + 2
+    const double lo = (double)a.e2g[b], hi = (double)a.e2g[b + 1];
+    const double o = (hi + lo) / (hi - lo);
+    s_rng[b] = make_float4((float)(2.0 / (hi - lo)), (float)o, (float)((o + 2.0) * 3.6e-7), 0.f);
+    s_cnt[b] = 0u;
+    if (WEIGHTED) s_sum[2 * b] = s_sum[2 * b + 1] = 0ull;
   }
   if (tid == 0) s_pending = 0;
+  for (int k = gt; k <= nb; k += gthreads) s_end[k] = 0;
   __syncthreads();
-  const Cat c = a.one;
-
-  auto flush = [&]() {
-    for (int b = tid; b < nb; b += kPThreads) {
-      const unsigned v = s_hist[b];
-      if (v) {
-        atomicAdd(c.counts + b, (unsigned long long)v);
-        s_hist[b] = 0u;
-      }
+  const Cat& c = a.one;
+  auto sync = [&]() {
+    if (gthreads == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(gthreads) : "memory");
+  };
+  auto flush = [&](int t, int threads) {
+    for (int b = t; b < nb; b += threads) {
+      const unsigned v = atomicExch(s_cnt + b, 0u);
+      if (v) atomicAdd(c.counts + b, (unsigned long long)v);
       if (WEIGHTED) {
-        const unsigned long long lo = s_whist[2 * b], hi = s_whist[2 * b + 1];
-        if (lo | hi) {
-          atomic_add_i192(c.wacc + 3 * b, lo, hi);
-          s_whist[2 * b] = s_whist[2 * b + 1] = 0ull;
-        }
+        const unsigned long long lo = atomicExch(s_sum + 2 * b, 0ull),
+                                 hi = atomicExch(s_sum + 2 * b + 1, 0ull);
+        if (lo | hi) atomic_add_i192(c.wacc + 3 * b, lo, hi);
       }
     }
   };
 
-  for (;;) {
-    if (tid == 0) {
-      const int64_t i = c.hub_begin + (int64_t)atomicAdd(a.hub_counter, 1ull);
-      s_hub = i < c.hub_end ? i : -1;
-      s_flush = 0;
-      s_next = 0;
-      if (i < c.hub_end) {
-        const unsigned long long d = (unsigned long long)c.deg[i];
-        const unsigned long long need = d * (d - (d > 0)) / 2;
-        if (s_pending + need > 0xFFFFFFFFull) {
-          s_flush = 1;
-          s_pending = need;
-        } else {
-          s_pending += need;
+  // The pairs of the lane's k in [k0, k0 + nk) with the j's [j0, j0 + nj).
+  auto item = [&](const float* X, const float* Y, const float* Z, const int* W, int b, int k0,
+                  int nk, int j0, int nj, long long Wi, auto diag) {
+    constexpr bool DIAG = decltype(diag)::value;
+    const float4 rng = s_rng[b];
+    const int k = k0 + min(lane, nk - 1);
+    const float xk = lane < nk ? X[k] : kFarK, yk = Y[k], zk = Z[k];
+    const unsigned long long nx = t_pack(-xk, -xk), ny = t_pack(-yk, -yk), nz = t_pack(-zk, -zk);
+    unsigned hits = 0;
+    long long sum = 0;  // of W_j over the lane's hits
+    for (int j = j0; j < j0 + nj; j += 4) {
+      float v[4];
+      {
+        const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(X + j);
+        const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(Y + j);
+        const ulonglong2 z = *reinterpret_cast<const ulonglong2*>(Z + j);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const unsigned long long dx = t_add(h ? x.y : x.x, nx), dy = t_add(h ? y.y : y.x, ny),
+                                   dz = t_add(h ? z.y : z.x, nz);
+          t_unpack(t_fma(dz, dz, t_fma(dy, dy, t_mul(dx, dx))), v[2 * h], v[2 * h + 1]);
         }
       }
+      int4 w4 = make_int4(0, 0, 0, 0);
+      if (WEIGHTED) w4 = *reinterpret_cast<const int4*>(W + j);
+      const int ww[4] = {w4.x, w4.y, w4.z, w4.w};
+      float near = 3.0e38f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        v[q] = fabsf(fmaf(v[q], rng.x, -rng.y)) - 1.0f;
+        if (DIAG && j - j0 + q >= lane) v[q] = 3.0e38f;  // each pair once
+        near = fminf(near, fabsf(v[q]));
+      }
+      if (near <= rng.z) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (!(fabsf(v[q]) <= rng.z)) continue;
+          const long long x = (long long)(int)(X[j + q] - xk), y = (long long)(int)(Y[j + q] - yk),
+                          z = (long long)(int)(Z[j + q] - zk);
+          const long long D2 = x * x + y * y + z * z;
+          v[q] = D2 >= s_e2[b] && D2 < s_e2[b + 1] ? -1.0f : 1.0f;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        hits += __float_as_uint(v[q]) >> 31;
+        if (WEIGHTED) sum += v[q] < 0.f ? ww[q] : 0;
+      }
     }
-    for (int b = tid; b <= nb; b += kPThreads) s_cnt[b] = 0;
-    __syncthreads();
-    const int64_t i = s_hub;
-    if (i < 0) break;
-    if (s_flush) {
-      flush();
-      __syncthreads();
+    const unsigned total = __reduce_add_sync(0xffffffffu, hits);
+    if (!total) return;
+    if (lane == 0) atomicAdd(s_cnt + b, total);
+    if constexpr (WEIGHTED) {
+      // |sum| < 2^35, |W_i W_k| < 2^60: the lanes' 128-bit products are added
+      // 24 bits at a time (modulo 2^128)
+      long long lo = 0, hi = 0;
+      mul_i128(sum, Wi * W[k], &lo, &hi);
+      const unsigned long long l = (unsigned long long)lo, h = (unsigned long long)hi;
+      unsigned part[6] = {(unsigned)(l & 0xFFFFFFu),
+                          (unsigned)((l >> 24) & 0xFFFFFFu),
+                          (unsigned)(((l >> 48) | (h << 16)) & 0xFFFFFFu),
+                          (unsigned)((h >> 8) & 0xFFFFFFu),
+                          (unsigned)((h >> 32) & 0xFFFFFFu),
+                          (unsigned)(h >> 56)};
+#pragma unroll
+      for (int q = 0; q < 6; ++q) part[q] = __reduce_add_sync(0xffffffffu, part[q]);
+      if (lane == 0) {
+        unsigned long long tl = 0, th = 0;
+        auto add = [&](unsigned long long p, int s) {  // p 2^s, s a multiple of 24
+          const unsigned long long al = s < 64 ? p << s : 0ull;
+          const unsigned long long ah = s == 0 ? 0ull : s < 64 ? p >> (64 - s) : p << (s - 64);
+          tl += al;
+          th += ah + (tl < al ? 1ull : 0ull);
+        };
+#pragma unroll
+        for (int q = 0; q < 6; ++q) add(part[q], 24 * q);
+        atomic_add_i128(s_sum + 2 * b, (long long)tl, (long long)th);
+      }
     }
-    const int d = c.deg[i];
-    if (d < 2) {
-      __syncthreads();
-      continue;
-    }
+  };
+  auto hub = [&](float* st, int64_t cap, int64_t i, int d) {
+    float *X = st, *Y = st + cap, *Z = st + 2 * cap;
+    int* W = reinterpret_cast<int*>(st + 3 * cap);
     const uint32_t* row = row_at(c.adj, c.ptr, i, c.adj_off, c.split, c.adj_off2);
     const int4 P = c.xyzp[i];
-    int4* S = d > a.cap ? reinterpret_cast<int4*>(a.gscratch + (size_t)blockIdx.x * a.gstride)
-                        : s_stage;
-    uint8_t* G = reinterpret_cast<uint8_t*>(S + (d > a.cap ? d : a.cap));  // group of each entry
-    // counting sort of the row by hub-edge bin
-    for (int t = tid; t < d; t += kPThreads) atomicAdd(&s_cnt[edge_bin(row[t]) + 1], 1);
-    __syncthreads();
-    if (tid == 0) {
-      for (int b = 1; b <= nb; ++b) s_cnt[b] += s_cnt[b - 1];
-      for (int b = 0; b < nb; ++b) s_cur[b] = s_cnt[b];
-    }
-    __syncthreads();
-    for (int t = tid; t < d; t += kPThreads) {
-      const uint32_t w = row[t];
-      const uint32_t k = edge_id(w);
-      const int4 Q = c.xyzp[k];
-      const int pos = atomicAdd(&s_cur[edge_bin(w)], 1);
-      G[pos] = (uint8_t)edge_bin(w);
-      S[pos] = make_int4((int)min_image((int64_t)Q.x - P.x, c.box),
-                         (int)min_image((int64_t)Q.y - P.y, c.box),
-                         (int)min_image((int64_t)Q.z - P.z, c.box),
-                         WEIGHTED ? (int)c.W[k] : (int)edge_bin(w));
-    }
-    __syncthreads();
-    // warps take four rows ra0..ra0+3 at a time; the pairs (ra, rb) with rb
-    // later in ra's group are spread over the lanes as one list
-    for (;;) {
-      int ra0 = 0;
-      if (lane == 0) ra0 = atomicAdd(&s_next, 4);
-      ra0 = __shfl_sync(0xffffffffu, ra0, 0);
-      if (ra0 >= d - 1) break;
-      int nk = 0;  // partners of row ra0 + lane (lanes 0..3)
-      if (lane < 4 && ra0 + lane < d - 1) nk = s_cnt[G[ra0 + lane] + 1] - (ra0 + lane) - 1;
-      int pre = nk;
-      for (int o = 1; o < 4; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, pre, o);
-        if (lane >= o) pre += v;
+    for (int t = gt; t < d; t += gthreads) atomicAdd(s_end + edge_bin(row[t]), 1);
+    sync();
+    if (wg == 0) {  // starts, rounded up to four; the tails are filled with absent j's
+      int base = 0;
+      for (int b0 = 0; b0 < nb; b0 += 32) {
+        const int b = b0 + lane, n = b < nb ? s_end[b] : 0, n4 = (n + 3) & ~3;
+        int incl = n4;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += t;
+        }
+        const int start = base + incl - n4;
+        if (b < nb) s_off[b] = s_end[b] = start;
+        for (int t = n; t < n4; ++t) {
+          X[start + t] = kFarJ;
+          Y[start + t] = Z[start + t] = 0.f;
+          if (WEIGHTED) W[start + t] = 0;
+        }
+        base += __shfl_sync(0xffffffffu, incl, 31);
       }
-      const int p0 = __shfl_sync(0xffffffffu, pre, 0), p1 = __shfl_sync(0xffffffffu, pre, 1),
-                p2 = __shfl_sync(0xffffffffu, pre, 2), T = __shfl_sync(0xffffffffu, pre, 3);
-      for (int t = lane; t < T; t += 32) {
-        const int k = (t >= p0 ? 1 : 0) + (t >= p1 ? 1 : 0) + (t >= p2 ? 1 : 0);
-        const int base = k == 0 ? 0 : (k == 1 ? p0 : (k == 2 ? p1 : p2));
-        const int ra = ra0 + k, rb = ra + 1 + (t - base);
-        const int b = G[ra];
-        const int4 Da = S[ra], Db = S[rb];
-        const int64_t x = (int64_t)Db.x - Da.x, y = (int64_t)Db.y - Da.y,
-                      z = (int64_t)Db.z - Da.z;
-        const int64_t D2 = x * x + y * y + z * z;
-        if (D2 < s_e2[b] || D2 >= s_e2[b + 1]) continue;
-        atomicAdd(&s_hist[b], 1u);
-        if constexpr (WEIGHTED) {
-          const long long xw = (long long)Da.w * Db.w;  // |.| < 2^60
-          const uint32_t x0 = (uint32_t)xw, x1 = (uint32_t)((unsigned long long)xw >> 32);
-          const uint32_t o0 = atomicAdd(&s_hacc[3 * b], x0);
-          const uint32_t a1 = x1 + ((o0 + x0 < o0) ? 1u : 0u);
-          uint32_t a2 = (xw < 0 ? 0xFFFFFFFFu : 0u) + ((a1 < x1) ? 1u : 0u);
-          if (a1) {
-            const uint32_t o1 = atomicAdd(&s_hacc[3 * b + 1], a1);
-            a2 += (o1 + a1 < o1) ? 1u : 0u;
-          }
-          if (a2) atomicAdd(&s_hacc[3 * b + 2], a2);
+    }
+    sync();
+    for (int t = gt; t < d; t += gthreads) {
+      const uint32_t w = row[t];
+      const uint32_t id = edge_id(w);
+      const int4 Q = c.xyzp[id];
+      const int pos = atomicAdd(s_end + edge_bin(w), 1);
+      X[pos] = (float)t_min_image(Q.x, P.x, c.box);
+      Y[pos] = (float)t_min_image(Q.y, P.y, c.box);
+      Z[pos] = (float)t_min_image(Q.z, P.z, c.box);
+      if (WEIGHTED) W[pos] = (int)c.W[id];
+    }
+    sync();
+    const long long Wi = WEIGHTED ? c.W[i] : 0;
+    int turn = 0;
+    for (int b = 0; b < nb; ++b) {
+      const int o = s_off[b], n = s_end[b] - o;
+      if (n < 2) continue;
+      // tiles of equal size, a multiple of four
+      const int nt = (n + 31) >> 5, size = ((n + nt - 1) / nt + 3) & ~3;
+      for (int tk = 0; tk * size < n; ++tk)
+        for (int tj = 0; tj <= tk; ++tj) {
+          if (turn++ % group != wg) continue;
+          const int nk = min(size, n - tk * size);
+          if (tj == tk)
+            item(X, Y, Z, W, b, o + tk * size, nk, o + tj * size, nk - 1, Wi, std::true_type{});
+          else
+            item(X, Y, Z, W, b, o + tk * size, nk, o + tj * size, size, Wi, std::false_type{});
+        }
+    }
+    sync();
+    for (int k = gt; k < nb; k += gthreads) s_end[k] = 0;  // for the next hub
+  };
+
+  for (;;) {
+    if (gt == 0) {
+      int64_t i = c.hub_begin + (int64_t)atomicAdd(a.hub_counter, 1ull);
+      if (i >= c.hub_end) i = -1;
+      s_hub[g] = i;
+      s_flush[g] = 0;
+      if (i >= 0) {
+        const unsigned long long d = (unsigned long long)c.deg[i];
+        const unsigned long long need = d * (d - (d > 0)) / 2;
+        // counts below 2^32: twice the limit and the hubs under way (16 of at
+        // most 2^25 pairs, or one of fewer than 2^31)
+        if (atomicAdd(&s_pending, need) + need > (1ull << 29)) {
+          atomicExch(&s_pending, 0ull);
+          s_flush[g] = 1;
         }
       }
     }
-    __syncthreads();
-    if constexpr (WEIGHTED) {
-      // the hub's 96-bit sums times W_i into the CTA's 128-bit sums
-      const int64_t Wi = c.W[i];
-      for (int b = tid; b < nb; b += kPThreads) {
-        const uint32_t l = s_hacc[3 * b], m = s_hacc[3 * b + 1], h = s_hacc[3 * b + 2];
-        if (!(l | m | h)) continue;
-        s_hacc[3 * b] = s_hacc[3 * b + 1] = s_hacc[3 * b + 2] = 0u;
-        const unsigned long long ml = ((unsigned long long)m << 32) | l;
-        const unsigned long long uw = (unsigned long long)Wi;
-        const unsigned long long plo = ml * uw;
-        unsigned long long phi = __umul64hi(ml, uw) - (Wi < 0 ? ml : 0ull);
-        phi += (unsigned long long)((long long)(int32_t)h * Wi);
-        const unsigned long long olo = s_whist[2 * b];
-        const unsigned long long nlo = olo + plo;
-        s_whist[2 * b] = nlo;
-        s_whist[2 * b + 1] += phi + ((nlo < olo) ? 1ull : 0ull);
-      }
+    sync();
+    const int64_t i = s_hub[g];
+    if (i < 0) break;
+    if (s_flush[g]) flush(gt, gthreads);
+    const int d = c.deg[i];
+    if (d < 2) {
+      sync();
+      continue;
     }
+    const int64_t need = equi_entries(d, nb);
+    if (need > a.cap)
+      hub(reinterpret_cast<float*>(a.gscratch + ((size_t)blockIdx.x * ngroups + g) * a.gstride),
+          need, i, d);
+    else hub(st_s, a.cap, i, d);
   }
   __syncthreads();
-  flush();
+  flush(tid, kTThreads);
 }
 
 template <bool BATCH>
@@ -2125,46 +2212,53 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
   // (variant bit 512 keeps the walk's EQUI instantiation)
   const bool equi_pair = equi && !(o.variant & 512) && g.max_deg <= kMaxSmemHistDeg;
   if (equi_pair) {
-    PArgs pa;
-    pa.one = a.one;
-    pa.cats = nullptr;
-    pa.base = nullptr;
-    pa.ncats = 0;
-    pa.nb = g.nb;
-    pa.nconf = nconf;
-    pa.use_lut = 0;
-    pa.bk_shift = pa.bk_n = 0;
-    pa.lin_c = 0.0f;
-    pa.e2g = g.d_edges2;
-    pa.hub_counter = a.hub_counter;
+    EArgs ea;
+    ea.one = a.one;
+    ea.nb = g.nb;
+    ea.e2g = g.d_edges2;
+    ea.hub_counter = a.hub_counter;
     int per_sm_bytes = 0;
     cudaDeviceGetAttribute(&per_sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    // two CTAs per SM: the staging buffer takes what the static arrays leave
-    const size_t budget = (size_t)per_sm_bytes / 2 - 1024 - 16 * 1024;
-    pa.cap = (int)std::min<size_t>(4096, budget / 17) & ~31;
-    const size_t smem = (size_t)pa.cap * 17;
-    void (*kern)(PArgs) = wm == kNone ? k_equi3p<kNone> : k_equi3p<kExact>;
+    const bool weighted_e = wm != kNone;
+    const size_t words = weighted_e ? 4 : 3;
+    const int mean = g.n ? (int)(g.edges_total / g.n) : 0;
+    const int64_t want = equi_entries(std::min(g.max_deg, std::max(64, 2 * mean)), g.nb);
+    const int64_t most = equi_entries(g.max_deg, g.nb);
+    const size_t budget = (size_t)per_sm_bytes / 2 - 1024 - 512;  // two CTAs per SM
+    auto pad16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
+    // the fewest warps per hub whose staging fits (all of the CTA's when a
+    // hub's pairs alone could fill the counters)
+    size_t fixed = 0;
+    for (ea.group = g.max_deg > kTMaxDeg ? kTWarps : 1;; ea.group *= 2) {
+      fixed = (weighted_e ? (size_t)g.nb * 16 : 0) + pad16((size_t)(g.nb + 1) * 8) +
+              (size_t)g.nb * 16 + pad16((size_t)g.nb * 4) +
+              pad16((size_t)(kTWarps / ea.group) * 2 * (g.nb + 1) * 4);
+      const size_t room = budget > fixed ? (budget - fixed) / (kTWarps / ea.group) : 0;
+      ea.cap = (int)std::min<int64_t>(most, (int64_t)(room / (4 * words)) & ~(int64_t)3);
+      if (ea.cap >= want || ea.group == kTWarps) break;
+    }
+    const int groups = kTWarps / ea.group;
+    const size_t smem = fixed + (size_t)groups * ea.cap * 4 * words;
+    void (*kern)(EArgs) = weighted_e ? k_equi_tiles<true> : k_equi_tiles<false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPThreads, smem);
-    const int grid = std::max(1, per_sm) * sms;
-    pa.gscratch = nullptr;
-    pa.gstride = 0;
-    if (g.max_deg > pa.cap) {
-      pa.gstride = ((size_t)g.max_deg * 17 + 255) & ~(size_t)255;
-      pa.gscratch = sc.alloc<unsigned char>(pa.gstride * grid);
-      if (!pa.gscratch) return GS_ENOMEM;
+    const int grid = (int)std::min<int64_t>((int64_t)2 * sms, (g.n + groups - 1) / groups);
+    ea.gscratch = nullptr;
+    ea.gstride = 0;
+    if (most > ea.cap) {
+      ea.gstride = ((size_t)most * 4 * words + 255) & ~(size_t)255;
+      ea.gscratch = sc.alloc<unsigned char>(ea.gstride * grid * groups);
+      if (!ea.gscratch) return GS_ENOMEM;
     }
     timer.start(s);
     st = for_each_window(g, o, sc, [&](const WinView& v) -> int {
-      pa.one.adj = v.adj;
-      pa.one.adj_off = v.off1;
-      pa.one.split = v.split;
-      pa.one.adj_off2 = v.off2;
-      pa.one.hub_begin = v.h0;
-      pa.one.hub_end = v.h1;
-      cudaMemsetAsync(pa.hub_counter, 0, sizeof(unsigned long long), s);
-      { kern<<<grid, kPThreads, smem, s>>>(pa); note_launch(); }
+      ea.one.adj = v.adj;
+      ea.one.adj_off = v.off1;
+      ea.one.split = v.split;
+      ea.one.adj_off2 = v.off2;
+      ea.one.hub_begin = v.h0;
+      ea.one.hub_end = v.h1;
+      cudaMemsetAsync(ea.hub_counter, 0, sizeof(unsigned long long), s);
+      { kern<<<grid, kTThreads, smem, s>>>(ea); note_launch(); }
       return cuda_status(cudaGetLastError());
     });
     timer.stop(s);
