@@ -40,46 +40,99 @@ __global__ void __launch_bounds__(kThreads) k_pairs_count(const uint4* __restric
 }
 
 // Weighted pair sums sum_{i<j} W_i W_j per bin (192-bit), and the weight
-// moments sum W_i and sum W_i^2 (for the analytic random pair count).
+// moments sum W_i and sum W_i^2 (for the analytic random pair count). A warp
+// per hub sums the W_j of each bin in its own shared counters, the low and high
+// halves apart (both below 2^31 for kPairChunk edges), which needs no carries;
+// per hub each bin's sum, times W_i, goes to a 128-bit sum that only this warp's
+// lane adds to. Bound by the gathers of W_j from L2: 4e8 edges (1e6 points, 20
+// bins) 0.97 ms against 4.8 with 64-bit shared atomics per edge (24 cycles
+// per warp) and global atomics per hub for the moments.
+constexpr int kPairChunk = 32768;
+__host__ __device__ inline int pair_copies(int nb) { return nb <= 32 ? 4 : 1; }
+__host__ __device__ inline size_t pair_warp_bytes(int nb) {
+  return (size_t)nb * 16 + (((size_t)nb * pair_copies(nb) * 12 + 15) & ~(size_t)15);
+}
 __global__ void __launch_bounds__(kThreads) k_pairs_weighted(
     const int64_t* __restrict__ ptr, const int32_t* __restrict__ deg,
     const uint32_t* __restrict__ adj, int64_t adj_off, int64_t split, int64_t adj_off2,
     const int64_t* __restrict__ W, int64_t h0, int64_t h1, int nb, unsigned long long* pairs,
     unsigned long long* wpairs, unsigned long long* moments) {
-  __shared__ unsigned long long acc[2 * (kMaxBins + 1)];
-  __shared__ unsigned cnt[kMaxBins + 1];
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-    acc[2 * b] = acc[2 * b + 1] = 0;
-    cnt[b] = 0;
-  }
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ unsigned total[kMaxBins + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, copies = pair_copies(nb);
+  unsigned char* mine = smem + (size_t)warp * pair_warp_bytes(nb);
+  unsigned long long* acc = reinterpret_cast<unsigned long long*>(mine);  // [nb][2]
+  // per bin and copy (lanes use copy lane mod copies): count, low and high sums
+  unsigned* cnt = reinterpret_cast<unsigned*>(mine + (size_t)nb * 16);
+  unsigned* low = cnt + nb * copies;
+  unsigned* high = low + nb * copies;
+  for (int b = lane; b < 2 * nb; b += 32) acc[b] = 0ull;
+  for (int b = lane; b < 3 * nb * copies; b += 32) cnt[b] = 0u;
+  for (int b = threadIdx.x; b < nb; b += blockDim.x) total[b] = 0u;
   __syncthreads();
-  const int lane = threadIdx.x & 31;
+  const int copy = lane & (copies - 1);
+  long long m1 = 0;                        // lane 0: sum of W_i (below 2^54)
+  unsigned long long m2lo = 0, m2hi = 0;   // and of W_i^2
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t i = h0 + blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < h1;
-       i += warps) {
-    const int64_t Wi = W[i];
+  for (int64_t i = h0 + blockIdx.x * (int64_t)(blockDim.x >> 5) + warp; i < h1; i += warps) {
+    const long long Wi = W[i];
     const int d = deg[i];
     const uint32_t* r = row_at(adj, ptr, i, adj_off, split, adj_off2);
-    for (int k = lane; k < d; k += 32) {
-      const uint32_t w = r[k];
-      const int b = (int)edge_bin(w);
-      long long lo, hi;
-      mul_i128(Wi, W[edge_id(w)], &lo, &hi);
-      atomic_add_i128(acc + 2 * b, lo, hi);
-      atomicAdd(cnt + b, 1u);
+    for (int c0 = 0; c0 < d; c0 += kPairChunk) {
+      const int c1 = min(d, c0 + kPairChunk);
+      for (int k0 = c0; k0 < c1; k0 += 128) {
+        uint32_t w[4];
+        int x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int k = k0 + 32 * q + lane;
+          w[q] = k < c1 ? r[k] : kSentinel;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = w[q] != kSentinel ? (int)W[edge_id(w[q])] : 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (w[q] != kSentinel) {
+            const int at = (int)edge_bin(w[q]) * copies + copy;
+            atomicAdd(cnt + at, 1u);
+            atomicAdd(low + at, (unsigned)x[q] & 0xFFFFu);
+            atomicAdd(high + at, (unsigned)(x[q] >> 16));
+          }
+      }
+      __syncwarp();
+      for (int b = lane; b < nb; b += 32) {
+        long long s = 0;
+        unsigned n = 0;
+        for (int q = 0; q < copies; ++q) {
+          const int at = b * copies + q;
+          n += cnt[at];
+          s += (long long)low[at] + ((long long)(int)high[at] << 16);
+          cnt[at] = low[at] = high[at] = 0u;
+        }
+        if (!n) continue;
+        atomicAdd(total + b, n);
+        long long lo, hi;
+        mul_i128(Wi, s, &lo, &hi);  // below 2^30 2^45
+        const unsigned long long old = acc[2 * b], now = old + (unsigned long long)lo;
+        acc[2 * b] = now;
+        acc[2 * b + 1] += (unsigned long long)hi + (now < old ? 1ull : 0ull);
+      }
+      __syncwarp();
     }
-    if (lane == 0) {
-      long long lo, hi;
-      mul_i128(Wi, Wi, &lo, &hi);
-      atomic_add_i192(moments + 3, (unsigned long long)lo, (unsigned long long)hi);
-      atomic_add_i192(moments, (unsigned long long)Wi, (unsigned long long)(Wi < 0 ? -1ll : 0ll));
-    }
+    m1 += Wi;
+    const unsigned long long sq = (unsigned long long)(Wi * Wi);  // below 2^60
+    m2lo += sq;
+    m2hi += m2lo < sq ? 1ull : 0ull;
   }
-  __syncthreads();
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+  if (lane == 0) {
+    if (m1) atomic_add_i192(moments, (unsigned long long)m1, (unsigned long long)(m1 < 0 ? -1ll : 0ll));
+    if (m2lo | m2hi) atomic_add_i192(moments + 3, m2lo, m2hi);
+  }
+  for (int b = lane; b < nb; b += 32)
     if (acc[2 * b] | acc[2 * b + 1]) atomic_add_i192(wpairs + 3 * b, acc[2 * b], acc[2 * b + 1]);
-    if (cnt[b]) atomicAdd(pairs + b, (unsigned long long)cnt[b]);
-  }
+  __syncthreads();
+  for (int b = threadIdx.x; b < nb; b += blockDim.x)
+    if (total[b]) atomicAdd(pairs + b, (unsigned long long)total[b]);
 }
 
 __global__ void k_xi_disc(const unsigned long long* pairs, const double* wpairs_d,
@@ -142,9 +195,13 @@ int pairs_weighted_device(const Graph& g, const FixedW& fw, unsigned long long* 
   cudaMemsetAsync(wacc, 0, sizeof(unsigned long long) * (3 * nb + 6), s);
   timer.start(s);
   int st = GS_OK;
+  const size_t smem = (kThreads / 32) * pair_warp_bytes(nb);
+  cudaFuncSetAttribute(k_pairs_weighted, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // a CTA's counts stay below 2^32: at most 2^31 edges each
+  const int grid = (int)std::max<int64_t>(sms * 8, (g.edges_total >> 24) + 1);
   if (g.n)
     st = for_each_window(g, o, sc, [&](const WinView& v) -> int {
-      { k_pairs_weighted<<<sms * 8, kThreads, 0, s>>>(g.d_ptr, g.d_deg, v.adj, v.off1, v.split, v.off2,
+      { k_pairs_weighted<<<grid, kThreads, smem, s>>>(g.d_ptr, g.d_deg, v.adj, v.off1, v.split, v.off2,
                                                     fw.d_W, v.h0, v.h1, nb, pairs, wacc,
                                                     wacc + 3 * nb); note_launch(); }
       return cuda_status(cudaGetLastError());

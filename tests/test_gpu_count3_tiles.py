@@ -135,3 +135,27 @@ def test_mu_rows_and_degenerate_normals(gs, n, nmu, flat):
         ref = ref[0] if isinstance(ref, tuple) else ref
         got = gs.gs_count_3pcf_mu(gs.gs_build_graph(X, 200_000, edges), nmu)
         assert np.array_equal(got, np.asarray(ref).reshape(got.shape))
+
+
+@pytest.mark.parametrize("n", [2, 33, 64, 130, 700])
+@pytest.mark.parametrize("kind", ["uniform", "signed", "span"])
+def test_equilateral_and_weighted_pairs(gs, n, kind):
+    """One, few and many neighbours per bin, pairs exactly on bin edges, uneven
+    bins, more bins than lanes."""
+    rng = np.random.default_rng(n)
+    X = (50_000 + np.concatenate([rng.integers(-3, 4, size=(n // 2, 3)) * 1000,
+                                  rng.integers(-2500, 2501, size=(n - n // 2, 3))])).astype(np.int32)
+    w = weights(kind, len(X), 9)
+    for edges in (np.array([0, 20_000]), 1000 * np.arange(12), np.array([0, 700, 1000, 5000, 5001, 9000]),
+                  np.linspace(0, 11_000, 41)):
+        edges = edges.astype(np.int64)
+        og = oracle.Graph(X, 200_000, edges)
+        g = gs.gs_build_graph(X, 200_000, edges)
+        rc, rw = oracle.equilateral_3pcf(og, w)
+        assert np.array_equal(gs.gs_count_3pcf_equilateral(g), rc)
+        gc, gw = gs.gs_count_3pcf_equilateral(g, w)
+        assert np.array_equal(gc, rc) and np.array_equal(gw, rw)
+        rr = np.ones(len(edges) - 1)
+        rp, rsum = og.pairs(w)
+        gp, gxi, _ = gs.gs_disconnected_4pcf(g, w, rr=rr, zeta=False)
+        assert np.array_equal(gp, rp) and np.array_equal(gxi, rsum - 1.0)
