@@ -46,11 +46,14 @@
 // so that the orbits met most often in a sample of hubs come first, and a
 // tetrahedron of any other orbit goes to the global counters directly.
 //
-// Weighted sums (exact, fixed-point W): the hub's sums of W_a W_b W_c are
-// kept per cell in shared 128-bit words (32-bit limbs) and multiplied by W_i
-// into the global 192-bit sums when the hub ends. Shared memory holds these
-// words (and the counts) only for the `hot` orbits, as above; a tetrahedron
-// of any other orbit goes straight to the global sums with its full product.
+// Weighted sums (exact, fixed-point W): the hub's sums of x = W_a W_b W_c are
+// kept per cell in three 32-bit words, one array per word (cells of 16 bytes in
+// a row left an atomic eight of the 32 banks: 4.3 wavefronts each), and
+// multiplied by W_i into the global 192-bit sums when the hub ends; the rare
+// carry out of the top word goes there at once. Shared memory holds the words
+// (and the counts) only for the `hot` orbits, as above; a tetrahedron of any
+// other orbit goes straight to the global sums with its full product. Pairs that
+// are no edge update words of the lane's own bank.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -58,6 +61,7 @@
 #include <type_traits>
 
 #include "gs_internal.cuh"
+#include "gs_tiles.cuh"
 
 namespace gs {
 namespace {
@@ -239,35 +243,6 @@ __host__ __device__ inline int dir_pixel(int64_t x, int64_t y, int64_t z) {
   return 16 * band + sector;
 }
 
-// A 128-bit two's complement value (lo, hi) into a shared 128-bit sum kept
-// as four 32-bit limbs, least significant first (sums modulo 2^128; the
-// caller keeps the true sum in range). 32-bit shared atomics are native;
-// the carries ripple through the returned old values, and a limb whose
-// addend (with the carry in) is zero is skipped. (64-bit shared atomic adds
-// measured 2.3 times slower in the triangle kernel's record.)
-__device__ inline void shared_add_i128(unsigned long long* p64, unsigned long long lo,
-                                       unsigned long long hi) {
-  unsigned* p = reinterpret_cast<unsigned*>(p64);
-  const uint32_t x0 = (uint32_t)lo, x1 = (uint32_t)(lo >> 32), x2 = (uint32_t)hi,
-                 x3 = (uint32_t)(hi >> 32);
-  uint32_t o = atomicAdd(p, x0);
-  uint32_t c = (o + x0 < o) ? 1u : 0u;
-  const uint32_t s1 = x1 + c;
-  c = (s1 < x1) ? 1u : 0u;  // x1 = 2^32 - 1 and a carry: s1 = 0
-  if (s1) {
-    o = atomicAdd(p + 1, s1);
-    c |= (o + s1 < o) ? 1u : 0u;
-  }
-  const uint32_t s2 = x2 + c;
-  c = (s2 < x2) ? 1u : 0u;
-  if (s2) {
-    o = atomicAdd(p + 2, s2);
-    c |= (o + s2 < o) ? 1u : 0u;
-  }
-  const uint32_t s3 = x3 + c;
-  if (s3) atomicAdd(p + 3, s3);
-}
-
 // A 192-bit two's complement value into three global 64-bit words.
 __device__ inline void atomic_add_w192(unsigned long long* g, unsigned long long w0,
                                        unsigned long long w1, unsigned long long w2) {
@@ -417,28 +392,27 @@ struct Chunk {
   uint32_t tab[32];
 };
 
-// The counters and sums of one CTA (cells of the slots below a.hot).
+// The counters of one CTA: cells of the slots below a.hot (parity: two per
+// slot), then a word per lane for no edge. Weighted: three more arrays, `stride`
+// words apart, the low to high words of the hub's sums.
 struct Hist {
-  unsigned* cnt;             // [cells]
-  unsigned long long* sum;   // weighted: [cells][2]
+  unsigned* cnt;
+  uint32_t stride;
 };
+// The top word starts at half its range, so that sums of either sign stay clear
+// of its carry (from zero, every change of a sum's sign carried: 2.5 ms of
+// global atomics per 1e9 tetrahedra).
+constexpr uint32_t kTopZero = 0x80000000u;
+__host__ __device__ inline size_t hist_words(int64_t hot, bool parity) {
+  return (size_t)hot * (parity ? 2 : 1) + 32;
+}
 
-// One tetrahedron in cell `cell` (parity: twice the slot plus the sign; else
-// the slot). deg: V = 0 on a chiral orbit, even channel only. Wab = W_a W_b.
+// One tetrahedron straight to the global counts and sums. cell: twice the slot
+// plus the sign (parity) or the slot; deg: V = 0 on a chiral orbit, even
+// channel only. Wab = W_a W_b.
 template <bool PARITY, bool WEIGHTED>
-__device__ inline void record4(const Args& a, const Hist& h, bool hist_ok, uint32_t cell, bool deg,
-                               int64_t Wi, int64_t Wab, int Wc) {
-  const uint32_t hotc = (uint32_t)(PARITY ? 2 * a.hot : a.hot);
-  const bool hot = hist_ok && !deg && cell < hotc;
-  if (hot) {
-    atomicAdd(h.cnt + cell, 1u);
-    if constexpr (WEIGHTED) {
-      long long lo, hi;
-      mul_i128(Wab, (long long)Wc, &lo, &hi);  // below 2^90
-      shared_add_i128(h.sum + 2 * (size_t)cell, (unsigned long long)lo, (unsigned long long)hi);
-    }
-    return;
-  }
+__device__ inline void record_global(const Args& a, uint32_t cell, bool deg, int64_t Wi,
+                                     int64_t Wab, int Wc) {
   const uint32_t slot = PARITY ? cell >> 1 : cell;
   const bool neg = PARITY && (cell & 1u);
   const bool odd = PARITY && !deg && a.chir[slot];
@@ -455,6 +429,61 @@ __device__ inline void record4(const Args& a, const Hist& h, bool hist_ok, uint3
         hi = ~hi + (lo == 0ull ? 1ull : 0ull);
       }
       atomic_add_i192(a.wodd + 3 * (size_t)slot, lo, hi);
+    }
+  }
+}
+
+// Two weighted tetrahedra with products Wc V[] in the cells at[] (shared
+// addresses of their counts, `none` for the lane's unused words); cell[] for the
+// carries out of the top word (about one in 2^21 for weights within a factor of
+// two).
+template <bool PARITY>
+__device__ inline void record_weighted(const Args& a, const uint32_t (&at)[2],
+                                       const uint32_t (&cell)[2], uint32_t none, uint32_t stride,
+                                       int64_t Wi, int Wc, const long long (&V)[2]) {
+  uint32_t w0[2], w1[2], w2[2], o[2];
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    inc_shared(at[v]);
+    // x = p1 2^32 + low word of p0
+    const long long p0 = (long long)Wc * (long long)(V[v] & 0xFFFFFFFFll);
+    const long long p1 = (long long)Wc * (int)(V[v] >> 32) + (p0 >> 32);
+    w0[v] = (uint32_t)p0;
+    w1[v] = (uint32_t)p1;
+    w2[v] = (uint32_t)((unsigned long long)p1 >> 32);
+    o[v] = t_atom(at[v] + stride, w0[v]);
+  }
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    asm("{\n\t.reg .u32 s;\n\tadd.cc.u32 s, %2, %3;\n\taddc.cc.u32 %0, %0, 0;\n\t"
+        "addc.u32 %1, %1, 0;\n\t}"
+        : "+r"(w1[v]), "+r"(w2[v])
+        : "r"(o[v]), "r"(w0[v]));
+    o[v] = t_atom(at[v] + 2u * stride, w1[v]);
+  }
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    asm("{\n\t.reg .u32 s;\n\tadd.cc.u32 s, %1, %2;\n\taddc.u32 %0, %0, 0;\n\t}"
+        : "+r"(w2[v])
+        : "r"(o[v]), "r"(w1[v]));
+    o[v] = t_atom(at[v] + 3u * stride, w2[v]);
+  }
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    uint32_t n, c;
+    asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, 0, 0;" : "=&r"(n), "=r"(c) : "r"(o[v]), "r"(w2[v]));
+    c -= w2[v] >> 31;  // sign extension
+    if (c != 0u && at[v] != none) {
+      // c 2^96 W_i
+      const long long t = (long long)(int)c * Wi;
+      const uint32_t slot = PARITY ? cell[v] >> 1 : cell[v];
+      atomic_add_w192(a.weven + 3 * (size_t)slot, 0ull, (unsigned long long)t << 32,
+                      (unsigned long long)(t >> 32));
+      if (PARITY && a.chir[slot]) {
+        const long long u = (cell[v] & 1u) ? -t : t;
+        atomic_add_w192(a.wodd + 3 * (size_t)slot, 0ull, (unsigned long long)u << 32,
+                        (unsigned long long)(u >> 32));
+      }
     }
   }
 }
@@ -730,9 +759,77 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
           };
           if (t0 > k0) steps(std::false_type{});
           else steps(std::true_type{});
+        } else if constexpr (WEIGHTED) {
+          const uint8_t* Bc = w.B + c;
+          const E* ent_c = ent + lane_idx;
+          const uint32_t hotc = hist_ok ? (uint32_t)(PARITY ? 2 * a.hot : a.hot) : 0u;
+          const uint32_t cells = (uint32_t)__cvta_generic_to_shared(h.cnt),
+                         none = cells + 4u * ((uint32_t)(PARITY ? 2 * a.hot : a.hot) + lane);
+          auto steps = [&](auto diag) {
+            for (int s0 = 0; s0 < ns; s0 += 2) {
+              uint32_t b23[2], cell[2], at[2];
+              int en[2];
+              float V[2] = {1.f, 1.f};
+              long long wab[2];
+              const int2 r = *reinterpret_cast<const int2*>(ch->row + s0);
+              const uint2 t = *reinterpret_cast<const uint2*>(ch->tab + s0);
+              const longlong2 w2 = *reinterpret_cast<const longlong2*>(wchunk + s0);
+              wab[0] = w2.x, wab[1] = w2.y;
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                const int ru = u ? r.y : r.x;
+                b23[u] = (uint32_t)nb;
+                if (!decltype(diag)::value || s0 + u < lane)
+                  b23[u] = Bc[GW ? row_off<I>((I)ru, m + 1) : (I)ru];
+                en[u] = load_entry(ent_c + ((u ? t.y : t.x) + b23[u]));
+              }
+              bool rare = false;
+              if constexpr (PARITY) {
+                const float2 x = *reinterpret_cast<const float2*>(ch->nx + s0),
+                             y = *reinterpret_cast<const float2*>(ch->ny + s0),
+                             z = *reinterpret_cast<const float2*>(ch->nz + s0);
+                V[0] = fmaf(z.x, uz, fmaf(y.x, uy, x.x * ux));
+                V[1] = fmaf(z.y, uz, fmaf(y.y, uy, x.y * ux));
+              }
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                if constexpr (PARITY) {
+                  const uint32_t neg = (__float_as_uint(V[u]) & (uint32_t)en[u]) >> 31;
+                  cell[u] = ((uint32_t)en[u] ^ neg) & Ent<E>::kMask;
+                  rare |= fabsf(V[u]) < a.eps;
+                } else {
+                  cell[u] = ((uint32_t)en[u] & Ent<E>::kMask) >> 1;
+                }
+                const bool hot = cell[u] < hotc;
+                rare |= !hot && b23[u] < (uint32_t)nb;
+                at[u] = hot ? cells + 4u * cell[u] : none;
+              }
+              if (rare) {
+                // a volume near zero is decided in integers; V = 0 and orbits
+                // without shared cells go to the global sums
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                  if (b23[u] >= (uint32_t)nb) continue;
+                  bool deg = false;
+                  if (PARITY && fabsf(V[u]) < a.eps && en[u] < 0) {
+                    const long long Vx = PIX ? 0 : det3(da, w.disp[list[k0 + s0 + u]], dc);
+                    deg = Vx == 0;
+                    cell[u] = ((uint32_t)en[u] ^ (Vx < 0 ? 1u : 0u)) & Ent<E>::kMask;
+                    at[u] = cell[u] < hotc && !deg ? cells + 4u * cell[u] : none;
+                  }
+                  if (deg || cell[u] >= hotc)
+                    record_global<PARITY, true>(a, cell[u], deg, Wi, wab[u], Wc);
+                }
+              }
+              record_weighted<PARITY>(a, at, cell, none, 4u * h.stride, Wi, Wc, wab);
+            }
+          };
+          if (t0 > k0) steps(std::false_type{});
+          else steps(std::true_type{});
         } else {
           // entries [0, lim) of the chunk come before c
           const int lim = min(ns, in ? (t0 > k0 ? 32 : lane) : 0);
+          const uint32_t hotc = hist_ok ? (uint32_t)(PARITY ? 2 * a.hot : a.hot) : 0u;
           constexpr int U = 2;  // two steps' loads before their updates
           for (int s0 = 0; s0 < lim; s0 += U) {
             uint32_t b23[U], e[U];
@@ -766,8 +863,8 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
               } else {
                 cell >>= 1;
               }
-              record4<PARITY, WEIGHTED>(a, h, hist_ok, cell, deg, Wi,
-                                        WEIGHTED ? wchunk[s0 + u] : 0, Wc);
+              if (!deg && cell < hotc) atomicAdd(h.cnt + cell, 1u);
+              else record_global<PARITY, false>(a, cell, deg, 0, 0, 0);
             }
           }
         }
@@ -783,13 +880,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
   __shared__ Shared s;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int group = a.group, gthreads = group * 32, g = warp / group, gt = tid - g * gthreads;
-  const int ncell = PARITY ? 2 * a.hot : a.hot;
   unsigned char* sp = smem;
   Hist h;
-  h.sum = reinterpret_cast<unsigned long long*>(sp);
-  if (WEIGHTED) sp += (size_t)ncell * 16;
+  h.stride = (uint32_t)hist_words(a.hot, PARITY);
   h.cnt = reinterpret_cast<unsigned*>(sp);
-  sp += pad16((size_t)ncell * 4 + 8);
+  sp += pad16((size_t)h.stride * (WEIGHTED ? 16 : 4));
   float4* pixu = reinterpret_cast<float4*>(sp);
   if (PIX) sp += 256 * sizeof(float4);
   Chunk* ch = reinterpret_cast<Chunk*>(sp) + warp;
@@ -800,10 +895,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
       sp + (size_t)g * workspace_bytes(a.cap, group, sizeof(uint16_t), WEIGHTED, PIX), a.cap,
       group, WEIGHTED, PIX);
 
-  for (int k = tid; k < ncell; k += kThreads) {  // the cell of no edge is never read
-    h.cnt[k] = 0u;
-    if (WEIGHTED) h.sum[2 * k] = h.sum[2 * k + 1] = 0ull;
-  }
+  for (uint32_t k = tid; k < h.stride * (WEIGHTED ? 4 : 1); k += kThreads)
+    h.cnt[k] = k < 3 * h.stride ? 0u : kTopZero;
   for (int k = tid; k < kWarps * kMaxBins4; k += kThreads) s.cur[k] = 0;
   for (int b = tid; b <= a.nb; b += kThreads) s.e2[b] = a.e2g[b];
   for (int k = tid; k < a.bk_n; k += kThreads) {
@@ -894,20 +987,29 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
       // the clearing before the next hub's additions)
       const long long Wi = a.W[i];
       for (int k = gt; k < a.hot; k += gthreads) {
-        unsigned long long* c = h.sum + (PARITY ? 4 : 2) * (size_t)k;
-        unsigned long long elo = c[0], ehi = c[1];
+        // the words as a signed 96-bit number (carries out of it are in the
+        // global sums already); cleared
+        auto take = [&](int cell, unsigned long long& lo, unsigned long long& hi) {
+          unsigned* c = h.cnt + h.stride + cell;
+          const uint32_t w0 = c[0], w1 = c[h.stride], w2 = c[2 * h.stride];
+          lo = ((unsigned long long)w1 << 32) | w0;
+          hi = (unsigned long long)(long long)(int)(w2 ^ kTopZero);
+          if (lo | hi) {
+            c[0] = c[h.stride] = 0u;
+            c[2 * h.stride] = kTopZero;
+          }
+        };
+        unsigned long long elo, ehi;
+        take(PARITY ? 2 * k : k, elo, ehi);
         if (PARITY) {
-          // even = S+ + S-, odd = S+ - S- (each below 2^115 in magnitude, so
-          // no 128-bit overflow)
-          const unsigned long long nlo = c[2], nhi = c[3];
+          // even = S+ + S-, odd = S+ - S-
+          unsigned long long nlo, nhi;
+          take(2 * k + 1, nlo, nhi);
           if (!(elo | ehi | nlo | nhi)) continue;
           const unsigned long long olo = elo - nlo, ohi = ehi - nhi - (elo < nlo ? 1ull : 0ull);
           elo += nlo;
           ehi += nhi + (elo < nlo ? 1ull : 0ull);
-          c[0] = c[1] = c[2] = c[3] = 0ull;
           if ((olo | ohi) && a.chir[k]) fold_i128(a.wodd + 3 * k, olo, ohi, Wi);
-        } else {
-          c[0] = c[1] = 0ull;
         }
         if (elo | ehi) fold_i128(a.weven + 3 * k, elo, ehi, Wi);
       }
@@ -1029,8 +1131,7 @@ void (*pick4(bool parity, bool weighted, bool pix, bool fast))(Args) {
 // Shared memory of a launch: cells of `hot` slots, chunks, pixel centres and
 // the workspaces of 32 / group groups.
 size_t launch_smem(int64_t hot, int cap, int group, bool parity, bool weighted, bool pix) {
-  const size_t ncell = (size_t)hot * (parity ? 2 : 1);
-  return (weighted ? ncell * 16 : 0) + pad16(ncell * 4 + 8) + (pix ? 256 * sizeof(float4) : 0) +
+  return pad16(hist_words(hot, parity) * (weighted ? 16 : 4)) + (pix ? 256 * sizeof(float4) : 0) +
          (size_t)kWarps * sizeof(Chunk) + (weighted ? (size_t)kThreads * 8 : 0) +
          (size_t)(kWarps / group) * workspace_bytes(cap, group, sizeof(uint16_t), weighted, pix);
 }
@@ -1128,9 +1229,11 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     }
     cap2 = fit_cap(std::min(maxd, kMaxSmemRow), no, kWarps, parity, false, pix, avail);
   } else {
-    // as many slots as fit beside the workspace of rows of up to 256
-    const size_t per_slot = (size_t)(parity ? 2 : 1) * (weighted ? 20 : 4);
-    cap = std::min(256, (maxd + 15) & ~15);
+    // as many slots as fit beside the workspace: of rows of up to 352 when
+    // weighted (1e5 clustered points, nb = 8: rows beyond 256 took 114 of 400 ms
+    // in global scratch; the 3,300 slots left hold all but 0.3% of tetrahedra)
+    const size_t per_slot = (size_t)(parity ? 2 : 1) * (weighted ? 16 : 4);
+    cap = std::min(weighted ? 352 : 256, (maxd + 15) & ~15);
     const size_t fixed = launch_smem(0, cap, group, parity, weighted, pix) + 32;
     nh = (int)std::min<size_t>((size_t)no, (avail - fixed) / per_slot);
     cap2 = cap;
