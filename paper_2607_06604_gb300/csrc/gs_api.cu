@@ -71,10 +71,38 @@ Scratch::~Scratch() {
   for (void* p : ptrs_) cudaFreeAsync(p, s_);
 }
 
+cudaMemPool_t memory_pool() {
+  static std::mutex mu;
+  static cudaMemPool_t pools[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64) return nullptr;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!pools[dev]) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    uint64_t keep = kPoolKeep;
+    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess)
+      cudaGetLastError();
+    pools[dev] = p;
+  }
+  return pools[dev];
+}
+
 void* Scratch::alloc_bytes(size_t bytes) {
   if (bytes == 0) bytes = 16;
   void* p = nullptr;
-  if (cudaMallocAsync(&p, bytes, s_) != cudaSuccess) {
+  cudaMemPool_t pool = memory_pool();
+  if ((pool ? cudaMallocFromPoolAsync(&p, bytes, pool, s_) : cudaMallocAsync(&p, bytes, s_)) !=
+      cudaSuccess) {
     cudaGetLastError();
     failed_ = true;
     return nullptr;
@@ -600,6 +628,13 @@ int gs_build_graph(const int32_t* xyz, int64_t n, int64_t box_u, const int64_t* 
 void gs_free_graph(gs_graph* G) {
   if (!G) return;
   Graph& g = G->g;
+  // work in flight on the device (a recorded launch being replayed) finishes
+  // first: freeing pool memory does not wait for it as cudaFree otherwise does
+  int cur = 0;
+  cudaGetDevice(&cur);
+  if (cur != g.device) cudaSetDevice(g.device);
+  cudaDeviceSynchronize();
+  if (cur != g.device) cudaSetDevice(cur);
   cudaFree(g.d_edges2);
   cudaFree(g.d_xyzp);
   cudaFree(g.d_deg);

@@ -1389,10 +1389,11 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     // the longer rows
     std::vector<int64_t> longer;
     bool global = false;
+    const std::vector<int32_t>& deg = host_deg(g);
     for (int64_t h = v.h0; h < v.h1; ++h)
-      if (g.h_deg[h] > std::max(cap, 2)) {
+      if (deg[h] > std::max(cap, 2)) {
         longer.push_back(h);
-        global = global || g.h_deg[h] > cap2;
+        global = global || deg[h] > cap2;
       }
     if (longer.empty()) return GS_OK;
     int64_t* d_list = sc.alloc<int64_t>(longer.size());

@@ -12,6 +12,7 @@
 // the mean with the hub's place in its cell, which cost the triangle kernel
 // pair tests and the tetrahedron kernel its longest rows.
 #include <algorithm>
+#include <mutex>
 
 #include "gs_internal.cuh"
 
@@ -386,10 +387,23 @@ int build_graph_device(const int32_t* d_xyz, int64_t n, int64_t box_u,
   for (int b = 0; b <= nb; ++b) e2[b] = edges[b] * edges[b];
   auto dev_alloc = [&](void** p, size_t bytes) -> int {
     if (bytes == 0) bytes = 16;
-    cudaError_t e = cudaMalloc(p, bytes);
+    // small arrays from the library's pool (ready in the order of the build's
+    // stream, which the build synchronises), large ones of their own
+    cudaMemPool_t pool = memory_pool();
+    cudaError_t e = pool && bytes <= kPoolKeep / 8 ? cudaMallocFromPoolAsync(p, bytes, pool, s)
+                                                   : cudaMalloc(p, bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
-      return GS_ENOMEM;
+      // give back what the pool keeps, and try again
+      if (pool) {
+        cudaDeviceSynchronize();
+        cudaMemPoolTrimTo(pool, 0);
+      }
+      if (cudaMalloc(p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        *p = nullptr;
+        return GS_ENOMEM;
+      }
     }
     g->device_bytes += (int64_t)bytes;
     return GS_OK;
@@ -493,11 +507,9 @@ int build_graph_device(const int32_t* d_xyz, int64_t n, int64_t box_u,
   { k_pad_lengths<<<grid_blocks(n + 1, 256), 256, 0, s>>>(g->d_deg, n, len); note_launch(); }
   st = scan_exclusive_i64(len, g->d_ptr, n + 1, s, sc);
   if (st) return st;
-  g->h_ptr.resize(n + 1);
-  cudaMemcpyAsync(g->h_ptr.data(), g->d_ptr, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, s);
+  cudaMemcpyAsync(&g->slots, g->d_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
   ce = cudaStreamSynchronize(s);
   if (ce != cudaSuccess) return cuda_status(ce);
-  g->slots = g->h_ptr[n];
   const uint64_t edge_bytes = sizeof(uint32_t) * (uint64_t)g->slots;
   const bool out_of_core = o.force_windows > 0 || (o.budget && edge_bytes > o.budget);
   if (!out_of_core) {
@@ -507,6 +519,11 @@ int build_graph_device(const int32_t* d_xyz, int64_t n, int64_t box_u,
     rows(true, g->d_adj, 0, n, 0);
     timer.stop(s);
   } else {
+    g->h_ptr.resize(n + 1);
+    ce = cudaMemcpyAsync(g->h_ptr.data(), g->d_ptr, sizeof(int64_t) * (n + 1),
+                         cudaMemcpyDeviceToHost, s);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+    if (ce != cudaSuccess) return cuda_status(ce);
     // Out of core: the edges live in pinned host memory. Rows are filled a
     // chunk of hubs at a time into a device staging buffer and copied out.
     ce = cudaHostAlloc((void**)&g->h_adj, std::max<uint64_t>(edge_bytes, 16), cudaHostAllocDefault);
@@ -576,9 +593,6 @@ int build_graph_device(const int32_t* d_xyz, int64_t n, int64_t box_u,
   g->probe_words = (int64_t)ht[0];
   g->edges_total = (int64_t)ht[1];
   g->max_deg = (int)(ht[2] & 0xffffffffu);
-  g->h_deg.resize(n);
-  ce = cudaMemcpy(g->h_deg.data(), g->d_deg, sizeof(int32_t) * n, cudaMemcpyDeviceToHost);
-  if (ce != cudaSuccess) return cuda_status(ce);
   timer.publish();
   return cuda_status(cudaGetLastError());
 }
@@ -709,17 +723,41 @@ int walk_words_device(Graph* g) {
   return GS_OK;
 }
 
+namespace {
+std::mutex g_host_mu;
+}
+const std::vector<int64_t>& host_ptr(const Graph& g) {
+  std::lock_guard<std::mutex> lock(g_host_mu);
+  if (g.h_ptr.empty()) {
+    std::vector<int64_t> p((size_t)g.n + 1, 0);
+    // an error stays for the calling query to report
+    (void)cudaMemcpy(p.data(), g.d_ptr, sizeof(int64_t) * p.size(), cudaMemcpyDeviceToHost);
+    g.h_ptr.swap(p);
+  }
+  return g.h_ptr;
+}
+const std::vector<int32_t>& host_deg(const Graph& g) {
+  std::lock_guard<std::mutex> lock(g_host_mu);
+  if (g.h_deg.empty() && g.n) {
+    std::vector<int32_t> d((size_t)g.n, 0);
+    (void)cudaMemcpy(d.data(), g.d_deg, sizeof(int32_t) * d.size(), cudaMemcpyDeviceToHost);
+    g.h_deg.swap(d);
+  }
+  return g.h_deg;
+}
+
 void shard_range(const Graph& g, const Opts& o, int64_t* lo, int64_t* hi) {
   *lo = 0;
   *hi = g.n;
   if (o.shards <= 1 || g.n == 0) return;
-  // boundaries at equal shares of the edge words (h_ptr is nondecreasing)
-  const int64_t total = g.h_ptr[g.n];
+  // boundaries at equal shares of the edge words (row starts do not decrease)
+  const std::vector<int64_t>& P = host_ptr(g);
+  const int64_t total = P[g.n];
   auto bound = [&](int k) -> int64_t {
     if (k <= 0) return 0;
     if (k >= o.shards) return g.n;
     const int64_t target = (int64_t)((__int128)total * k / o.shards);
-    return std::lower_bound(g.h_ptr.begin(), g.h_ptr.begin() + g.n, target) - g.h_ptr.begin();
+    return std::lower_bound(P.begin(), P.begin() + g.n, target) - P.begin();
   };
   *lo = bound(o.shard);
   *hi = bound(o.shard + 1);

@@ -60,8 +60,10 @@ struct Graph {
   int64_t* d_ptr = nullptr;     // [n+1] row starts (words)
   uint32_t* d_adj = nullptr;    // [slots] packed edge words (resident graphs)
   uint32_t* h_adj = nullptr;    // [slots] pinned host copy (out-of-core graphs)
-  std::vector<int64_t> h_ptr;   // host copy of d_ptr (window planning)
-  std::vector<int32_t> h_deg;   // host copy of d_deg
+  // host copies of d_ptr and d_deg, made when a query first needs them (see
+  // host_ptr, host_deg); out-of-core graphs have h_ptr from the start
+  mutable std::vector<int64_t> h_ptr;
+  mutable std::vector<int32_t> h_deg;
   // out-of-core planning. In a periodic box the ids are x-major, so hubs
   // of the first E_nb in x have wrap-around neighbours in the last one:
   // wrap_start is the first id of the cells there (n for an open box);
@@ -93,12 +95,24 @@ struct Opts {
   int shard = 0, shards = 0;
 };
 
+// Host copies of the row starts [n+1] and lengths [n].
+const std::vector<int64_t>& host_ptr(const Graph& g);
+const std::vector<int32_t>& host_deg(const Graph& g);
+
 // Hub range [lo, hi) of the query's shard (the whole graph when unsharded).
 void shard_range(const Graph& g, const Opts& o, int64_t* lo, int64_t* hi);
 Opts read_opts(const gs_options* o);
 
 // Whether p is device-accessible memory of the current device.
 bool is_device_ptr(const void* p);
+
+// The library's memory pool on the current device (nullptr: the device's own).
+// It keeps up to kPoolKeep bytes over synchronisations, so that a call's scratch
+// and a small graph's arrays are not mapped and unmapped by every call (a
+// 2e4-point chain of calls: 0.88 -> 0.33 ms); more than that goes back to the driver at the
+// next synchronisation. Pools are safe between threads and streams.
+constexpr uint64_t kPoolKeep = 64ull << 20;
+cudaMemPool_t memory_pool();
 
 // Stream-ordered scratch allocations released at scope exit.
 class Scratch {
