@@ -49,6 +49,13 @@ __device__ inline float t_sqrt(float x) {
   return r;
 }
 
+// Relative error below 2^-22; |x| below 2^-126 counts as zero.
+__device__ inline float t_rsqrt(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // u of a pair in bin b lies in [kTileM + b, kTileM + b + 1): 16 fraction bits.
 constexpr float kTileM = 192.0f;
 constexpr uint32_t kTileBits = 0x43400000u;  // bits of kTileM
