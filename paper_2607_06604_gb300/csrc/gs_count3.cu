@@ -1174,7 +1174,8 @@ __global__ void __launch_bounds__(kPThreads, 2) k_count3p(PArgs a) {
 // and the number of pairs in 32-bit words; the last word of the sum, Z, takes
 // (high word + carry) 2^cb + 1, so its low cb bits count the pairs, and T takes,
 // rarely, the carries out of Z (upper half, signed) and of Z's count field
-// (lower half).
+// (lower half). For weights of both signs Z starts at half its range: from zero,
+// every change of a sum's sign would carry.
 //  * FOLD, long rows: x = W_j W_k, |x| < 2^60, two shared atomics per pair; the
 //    CTA works on one hub, after which fold adds the cells of one
 //    configuration, times W_i, to the CTA's 128-bit sums.
@@ -1269,6 +1270,7 @@ template <int WM, bool BATCH, bool LOWER, bool FOLD>
 __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
   constexpr bool WEIGHTED = WM != kNone;
   constexpr int kWords = !WEIGHTED ? 1 : FOLD ? 3 : 4;
+  constexpr uint32_t kZ0 = WM == kExact ? 0x80000000u : 0u;  // Z of no pairs
   extern __shared__ __align__(16) unsigned char smem[];
   const int nb = a.nb, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int group = a.group, gthreads = group * 32, g = warp / group, gt = tid - g * gthreads,
@@ -1295,7 +1297,8 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
   __shared__ Cat s_c;  // batched: the current catalogue
   __shared__ unsigned long long s_pending;
 
-  for (int k = tid; k < stride * kWords; k += kTThreads) cell[k] = 0u;
+  for (int k = tid; k < stride * kWords; k += kTThreads)
+    cell[k] = WEIGHTED && k / stride == kWords - 2 ? kZ0 : 0u;
   if (FOLD)
     for (int k = tid; k < a.nconf; k += kTThreads) {
       hist[k] = 0u;
@@ -1345,11 +1348,11 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
         auto take = [&](int x, int y, int z) {  // x <= y the hub edges' bins
           unsigned* w = cell + (y * (y + 1) / 2 + x) * nr + z;
           const uint32_t w0 = atomicExch(w, 0u), w1 = atomicExch(w + stride, 0u),
-                         Z = atomicExch(w + 2 * stride, 0u), T = atomicExch(w + 3 * stride, 0u);
+                         Z = atomicExch(w + 2 * stride, kZ0), T = atomicExch(w + 3 * stride, 0u);
           // Z with its carries is H 2^cb + the number of pairs
           const long long n = (long long)(((unsigned long long)(T & 0xFFFFu) << a.cb) + (Z & cm));
           const long long full =
-              (long long)(((unsigned long long)(long long)((int)T >> 16) << 32) | Z);
+              (long long)(((unsigned long long)(long long)((int)T >> 16) << 32) | Z) - (long long)kZ0;
           const unsigned long long add = ((unsigned long long)w1 << 32) | w0;
           num += (unsigned long long)n;
           slo += add;
@@ -1388,13 +1391,14 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
       auto take = [&](int x, int y, int z) {  // x <= y the hub edges' bins
         unsigned* w = cell + (y * (y + 1) / 2 + x) * nr + z;
         const uint32_t lo = w[0], Z = w[stride], T = w[2 * stride];
-        if (!(lo | Z | T)) return;
-        w[0] = w[stride] = 0u;
+        if (!(lo | (Z ^ kZ0) | T)) return;
+        w[0] = 0u;
+        w[stride] = kZ0;
         if (T) w[2 * stride] = 0u;
         // Z with its carries is H 2^cb + the number of pairs
         const long long n = (long long)(((unsigned long long)(T & 0xFFFFu) << a.cb) + (Z & cm));
         const long long full =
-            (long long)(((unsigned long long)(long long)((int)T >> 16) << 32) | Z);
+            (long long)(((unsigned long long)(long long)((int)T >> 16) << 32) | Z) - (long long)kZ0;
         const long long H = (full - n) >> a.cb;
         const unsigned long long add = ((unsigned long long)H << 32) | lo;
         num += (unsigned long long)n;
