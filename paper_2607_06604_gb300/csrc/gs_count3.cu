@@ -1,7 +1,11 @@
-// Binned triangle counts (Sec. 2.2), GB300 layout. Two kernels give the same
+// Binned triangle counts (Sec. 2.2), GB300 layout. Three kernels give the same
 // counts and exact weighted sums:
 //
-// k_count3p (the default): every triangle i < j < k is found at its smallest
+// k_count3t (the default for evenly spaced bins, described where it stands):
+// the pair test of k_count3p in register tiles and single precision, with exact
+// decisions near bin edges.
+//
+// k_count3p (other bins): every triangle i < j < k is found at its smallest
 // vertex i from the pair (j, k) of N+(i). The CTA stages the hub-relative
 // displacement of every neighbour and tests each pair of N+(i) directly: it
 // is an edge exactly when its lattice distance lies in [E_0, E_nb), and the
@@ -23,8 +27,8 @@
 // (wrap-around neighbours of a periodic box, very sparse catalogues) use a
 // shared hash of N+(i) in the same memory, staged in segments.
 //
-// Both: the configuration index comes from a shared table over (b_ij, b_ik,
-// b_jk); counts go to per-CTA shared-memory histograms flushed with one
+// The last two: the configuration index comes from a shared table over (b_ij,
+// b_ik, b_jk); counts go to per-CTA shared-memory histograms flushed with one
 // 64-bit atomic per bin. Weighted sums use exact fixed point: per hub, 96-bit
 // sums of W_j W_k kept in 32-bit limbs, multiplied by W_i into the CTA's
 // 128-bit sums, flushed into 192-bit global accumulators.
@@ -788,7 +792,7 @@ void (*pick_equi3(int wm, bool nonneg, bool smem_hist))(Args) {
 }
 
 // ----------------------------------------------------------------------------
-// Pair-geometry triangle counting (the default launch).
+// Pair-geometry triangle counting (bins that are not evenly spaced).
 //
 // Every triangle i < j < k has j and k in N+(i). The walk above finds the
 // pairs (j, k) of N+(i) that are edges by intersecting sorted rows; this
@@ -2200,7 +2204,7 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   KernelTimer timer(o.kernel_ms);
   int st = GS_OK;
-  // The pair kernel is the default. Launch bits of the walk's own paths
+  // The pair kernels are the default. Launch bits of the walk's own paths
   // (1, 2, 8, 16, 32, 64, 512), the equilateral configurations and rows of
   // more than 65,535 neighbours (whose triangles could overflow the 32-bit
   // shared counters within one hub) take the merge-walk kernel.
@@ -2245,12 +2249,12 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
     const size_t smem = fixed + (size_t)groups * ea.cap * 4 * words;
     void (*kern)(EArgs) = weighted_e ? k_equi_tiles<true> : k_equi_tiles<false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int grid = (int)std::min<int64_t>((int64_t)2 * sms, (g.n + groups - 1) / groups);
+    int grid = (int)std::min<int64_t>((int64_t)2 * sms, (g.n + groups - 1) / groups);
     ea.gscratch = nullptr;
     ea.gstride = 0;
     if (most > ea.cap) {
       ea.gstride = ((size_t)most * 4 * words + 255) & ~(size_t)255;
-      ea.gscratch = sc.alloc<unsigned char>(ea.gstride * grid * groups);
+      ea.gscratch = staging(sc, ea.gstride * groups, &grid);
       if (!ea.gscratch) return GS_ENOMEM;
     }
     timer.start(s);
@@ -2280,12 +2284,12 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TL.smem);
     // no more CTAs than the hubs keep busy
     const int groups = kTWarps / TL.group;
-    const int grid = (int)std::min<int64_t>(TL.blocks, (g.n + groups - 1) / groups);
+    int grid = (int)std::min<int64_t>(TL.blocks, (g.n + groups - 1) / groups);
     ta.gscratch = nullptr;
     ta.gstride = 0;
     if (g.max_deg > TL.cap) {
       ta.gstride = stage_bytes((g.max_deg + 31) & ~31, wm != kNone);
-      ta.gscratch = sc.alloc<unsigned char>(ta.gstride * grid * groups);
+      ta.gscratch = staging(sc, ta.gstride * groups, &grid);
       if (!ta.gscratch) return GS_ENOMEM;
     }
     timer.start(s);
@@ -2482,12 +2486,12 @@ int count3_batch_device(const Graph* const* gr, int ng, const FixedW* fws, uint6
     ta.hub_counter = a.hub_counter;
     void (*kern)(TArgs) = pick_count3t<true>(wm, nonneg, TL);
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TL.smem);
-    const int grid = (int)std::min<int64_t>(TL.blocks, base[ng]);
+    int grid = (int)std::min<int64_t>(TL.blocks, base[ng]);
     ta.gscratch = nullptr;
     ta.gstride = 0;
     if (max_deg > TL.cap) {
       ta.gstride = stage_bytes((max_deg + 31) & ~31, wm != kNone);
-      ta.gscratch = sc.alloc<unsigned char>(ta.gstride * grid);
+      ta.gscratch = staging(sc, ta.gstride, &grid);
       if (!ta.gscratch) return GS_ENOMEM;
     }
     timer.start(s);

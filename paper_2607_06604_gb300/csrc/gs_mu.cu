@@ -7,7 +7,8 @@
 // vertices changes it), its bin the largest m < nmu with m / nmu <= mu, and
 // collinear triangles (n = 0) go to the extra bin nmu.
 //
-// Kernel: the pair geometry of the triangle kernel. A persistent CTA takes
+// Kernels: k_mu_tiles (unweighted counts over evenly spaced bins, below) and
+// k_count3mu, the pair geometry of the triangle kernel. A persistent CTA takes
 // one hub i at a time, stages the hub-relative displacement of every
 // neighbour (and its hub-edge bin), and tests every pair (j, k) of N+(i):
 // an edge exactly when E_0^2 <= |D_k - D_j|^2 < E_nb^2. For each triangle
@@ -542,13 +543,13 @@ bool mu_tiles(const Graph& g, int nmu, int nconf, uint64_t* d_counts, unsigned l
   a.hub_counter = counter;
   void (*kern)(MTArgs) = bins.lower ? k_mu_tiles<true> : k_mu_tiles<false>;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  const int grid = (int)std::min<int64_t>((int64_t)ctas * sms, (g.n + groups - 1) / groups);
+  int grid = (int)std::min<int64_t>((int64_t)ctas * sms, (g.n + groups - 1) / groups);
   a.gscratch = nullptr;
   a.gstride = 0;
   *status = GS_OK;
   if (g.max_deg > a.cap) {
     a.gstride = (size_t)((g.max_deg + 31) & ~31) * 24;
-    a.gscratch = sc.alloc<unsigned char>(a.gstride * grid * groups);
+    a.gscratch = staging(sc, a.gstride * groups, &grid);
     if (!a.gscratch) {
       *status = GS_ENOMEM;
       return true;

@@ -111,6 +111,15 @@ __device__ inline int t_min_image(int q, int p, int64_t box) {
   return (int)d;
 }
 
+// Global staging of `each` bytes per CTA for rows beyond the shared one, with
+// as many CTAs of *grid as there is memory for (nullptr: not even one).
+inline unsigned char* staging(Scratch& sc, size_t each, int* grid) {
+  for (;; *grid = (*grid + 1) / 2) {
+    unsigned char* p = sc.alloc<unsigned char>(each * *grid);
+    if (p || *grid <= 1) return p;
+  }
+}
+
 // Exact bin of a pair from its displacement (integers held in floats), nb
 // when it is no edge.
 __device__ inline int t_exact_bin(const int64_t* e2, int nb, float dx, float dy, float dz) {
