@@ -83,10 +83,10 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-KERNEL_VERSION = "k_count3p.v1"  # bump when k_count3 changes; stale captures then report null
+KERNEL_VERSION = "k_count3t.v1"  # bump when k_count3 changes; stale captures then report null
 
 
-KERNEL4_VERSION = "k_count4.v5"  # likewise for k_count4
+KERNEL4_VERSION = "k_count4.v6"  # likewise for k_count4
 
 
 def _profile_values(name):
@@ -407,8 +407,8 @@ def run_ours(args):
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
             "per_unit": "5 B per edge of the hub row and of every spoke row N+(j)",
-            "limiter": "shared-memory pipe (pair tests on staged neighbours, histogram atomics)",
-            "kernel": "k_count3p (RRR)", "kernel_ms": k_ms, "alg_bytes_per_launch": alg_bytes,
+            "limiter": "instruction issue and the shared-memory pipe (pair tests on staged tiles, atomics)",
+            "kernel": "k_count3t (RRR)", "kernel_ms": k_ms, "alg_bytes_per_launch": alg_bytes,
             "strict_bytes_per_launch": strict_bytes,
             "strict_frac": strict_bytes / (k_ms / 1e3) / 1e9 / peak,
             "triangles_per_launch": float(counts[1].sum().item())}
@@ -504,7 +504,7 @@ def measure_4pcf(gs, torch, runs=2):
                          "kernel": "k_count4 (parity)", "alg_bytes_per_launch": b4,
                          "per_unit": "5 B per edge: hub rows, spoke rows, and the row of each "
                                      "triangle's third vertex",
-                         "limiter": "instruction issue on shared-memory bit rows (the rows of "
+                         "limiter": "shared-memory pipe: broadcasts, bin-matrix rows and counters (the rows of "
                                     "a hub's neighbourhood are staged once per hub)"}}
 
 
