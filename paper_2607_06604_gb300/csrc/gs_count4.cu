@@ -105,6 +105,7 @@ struct Args {
   int bk_shift, bk_n;  // squared-distance buckets (bk_n = 0: binary search)
   int hot;             // orbits (slots) below this are accumulated in shared memory
   float eps;           // volumes within eps of zero are decided in integers
+  unsigned long long limit;  // tetrahedra between two flushes of the shared counters
   unsigned long long* even;
   unsigned long long* odd;
   unsigned long long* weven;  // [n_orbits][3] 192-bit
@@ -715,7 +716,28 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
                 unpack2(fma2(z.x, uz2, fma2(y.x, uy2, mul2(x.x, ux2))), V[0], V[1]);
                 unpack2(fma2(z.y, uz2, fma2(y.y, uy2, mul2(x.y, ux2))), V[2], V[3]);
               }
-              float vmin = 3.0e38f;
+              // Signs are settled before any counter is touched: counters only
+              // grow, so another group's flush may take them at any moment.
+              if constexpr (PARITY && !PIX) {
+                float vmin = 3.0e38f;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                  if (!decltype(diag)::value || s0 + u < lane) vmin = fminf(vmin, fabsf(V[u]));
+                if (vmin < a.eps) {
+                  // a volume within its error bound of zero: the exact sign, or
+                  // the even channel alone if V = 0
+#pragma unroll
+                  for (int u = 0; u < U; ++u) {
+                    if (b23[u] >= (uint32_t)nb || !(fabsf(V[u]) < a.eps) || en[u] >= 0) continue;
+                    const long long Vx = det3(da, w.disp[list[k0 + s0 + u]], dc);
+                    V[u] = Vx < 0 ? -1.0f : 1.0f;
+                    if (Vx == 0) {
+                      atomicAdd(a.even + (((uint32_t)en[u] & Ent<E>::kMask) >> 1), 1ull);
+                      en[u] = (int)trash;
+                    }
+                  }
+                }
+              }
 #pragma unroll
               for (int u = 0; u < U; ++u) {
                 uint32_t cell;
@@ -723,37 +745,15 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
                   // V < 0 on a chiral orbit
                   const uint32_t neg = (__float_as_uint(V[u]) & (uint32_t)en[u]) >> 31;
                   cell = ((uint32_t)en[u] ^ neg) & Ent<E>::kMask;
-                  if constexpr (PIX) {
-                    // degenerate pixel volumes are a few percent: even channel
-                    if (fabsf(V[u]) < a.eps && en[u] < 0) {
-                      atomicAdd(a.even + (cell >> 1), 1ull);
-                      cell = trash;
-                    }
-                  } else if (!decltype(diag)::value || s0 + u < lane) {
-                    vmin = fminf(vmin, fabsf(V[u]));
+                  // degenerate pixel volumes are a few percent: even channel
+                  if (PIX && fabsf(V[u]) < a.eps && en[u] < 0) {
+                    atomicAdd(a.even + (cell >> 1), 1ull);
+                    cell = trash;
                   }
                 } else {
                   cell = ((uint32_t)en[u] & Ent<E>::kMask) >> 1;
                 }
                 inc_shared(cells + 4u * cell);
-              }
-              if (PARITY && !PIX && vmin < a.eps) {
-                // a volume within its error bound of zero: move the count if
-                // the exact sign is another, or to the even channel if V = 0
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                  if (b23[u] >= (uint32_t)nb || !(fabsf(V[u]) < a.eps) || en[u] >= 0) continue;
-                  const uint32_t neg = __float_as_uint(V[u]) >> 31;
-                  const uint32_t cell = ((uint32_t)en[u] ^ neg) & Ent<E>::kMask;
-                  const long long Vx = det3(da, w.disp[list[k0 + s0 + u]], dc);
-                  if (Vx == 0) {
-                    atomicSub(h.cnt + cell, 1u);
-                    atomicAdd(a.even + (cell >> 1), 1ull);
-                  } else if ((Vx < 0 ? 1u : 0u) != neg) {
-                    atomicSub(h.cnt + cell, 1u);
-                    atomicAdd(h.cnt + (cell ^ 1u), 1u);
-                  }
-                }
               }
             }
           };
@@ -961,7 +961,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
         // hub), those registered while a flush runs (the same) and those
         // under way at a reset (31 hubs of at most 2^26).
         if (need <= kMaxHubNeed &&
-            atomicAdd(&s.pending, need) + need > (1ull << 29)) {
+            atomicAdd(&s.pending, need) + need > a.limit) {
           atomicExch(&s.pending, 0ull);
           s.flush[g] = 1;
         }
@@ -1190,6 +1190,9 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     const double r = (double)g.edges[g.nb];
     a.eps = pix ? kPixZero : (float)std::ldexp(r * r * r, -21);
   }
+  // variant 1024: a flush before every hub (exercises flushes while other
+  // groups count)
+  a.limit = (o.variant & 1024) ? 0 : 1ull << 29;
   // weighted results land in the callers' 192-bit arrays (or scratch)
   unsigned long long* weven = weighted ? (weven_out ? weven_out : sc.alloc<unsigned long long>(3 * (size_t)no))
                                        : nullptr;

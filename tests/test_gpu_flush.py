@@ -1,0 +1,48 @@
+"""Shared counters emptied by one group of warps while the others count on:
+variant 1024 flushes before every hub, on catalogues whose counts the kernels
+decide in integers (points on a mesh or in planes: volumes of zero), with one
+warp to half a CTA per hub. Against the oracle bit for bit."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gs():
+    import torch
+    assert torch.cuda.is_available()
+    import paper_2607_06604_gb300 as m
+    return m
+
+
+def mesh(m):
+    at = np.stack(np.meshgrid(*[np.arange(m)] * 3, indexing="ij"), -1).reshape(-1, 3) * 1000
+    return at.astype(np.int32), m * 1000
+
+
+def planes(n, box_u):
+    """Uniform points on planes 2,500 apart."""
+    X = np.random.default_rng(n).integers(0, box_u, size=(n, 3))
+    X[:, 2] = X[:, 2] // 2500 * 2500
+    return X.astype(np.int32), box_u
+
+
+# rows of about 15, 27, 60 and 100: 1, 4, 8 and 16 warps per hub
+CATALOGUES = [(mesh, (20,), 2100), (mesh, (18,), 2300), (mesh, (14,), 3100), (mesh, (15,), 3700),
+              (planes, (7000, 40_000), 4000), (planes, (13_000, 40_000), 4000),
+              (planes, (12_000, 30_000), 4000), (planes, (3700, 17_000), 4000)]
+
+
+@pytest.mark.parametrize("kind,args,rmax", CATALOGUES)
+def test_parity_flush_between_groups(gs, kind, args, rmax):
+    X, box_u = kind(*args)
+    edges = np.linspace(0, rmax, 6).astype(np.int64)
+    re, ro = oracle.Graph(X, box_u, edges).count_4pcf()
+    g = gs.gs_build_graph(X, box_u, edges)
+    for _ in range(3):
+        ge, go = gs.gs_count_4pcf_parity(g, variant=1024)
+        assert np.array_equal(ge, re) and np.array_equal(go, ro)
+    assert np.array_equal(gs.gs_count_4pcf(g, variant=1024), re)
