@@ -84,8 +84,8 @@ typedef struct {
    * let their copies land (tests of the failure path). 32 = weighted
    * gs_count_3pcf compacts each warp's hits before recording them. 64 =
    * gs_count_3pcf streams spoke rows through a per-warp ring of
-   * asynchronous copies (deeper prefetch). 1024 = gs_count_4pcf* empties
-   * its shared counters before every hub. Other results are identical;
+   * asynchronous copies (deeper prefetch). 1024 = gs_count_4pcf* and
+   * gs_count_3pcf's tiled kernel empty their shared counters before every hub. Other results are identical;
    * the bits exist for testing and tuning. */
   int32_t variant;
   /* cudaStream_t for all device work; NULL = legacy default stream. */

@@ -1326,9 +1326,10 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
     else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(gthreads) : "memory");
   };
   // Adds the cells to the global counts (and sums) and clears them; exchanges,
-  // so that one group can do it while the others count on. (Every word is its
-  // additions modulo 2^32 and every carry is added somewhere, so the global
-  // sums are right whichever flush takes a word or its carry.)
+  // so that one group can do it while the others count on. (Unweighted counters
+  // only grow. Weighted, every word is its additions modulo 2^32 and every carry
+  // is added somewhere, so the global sums are right whichever flush takes a
+  // word or its carry.)
   auto flush = [&](int t, int threads) {
     if (cur < 0) return;
     for (int k = t; k < a.nconf; k += threads) {
@@ -1440,7 +1441,7 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
     [[maybe_unused]] const int pk = WEIGHTED ? S.p[k] : 0;
     [[maybe_unused]] const long long V = WEIGHTED ? (FOLD ? 1 : Wi) * S.W[k] : 0;
     const unsigned long long nx = t_pack(-xk, -xk), ny = t_pack(-yk, -yk), nz = t_pack(-zk, -zk);
-        const uint32_t base = s_cell - 4u * kBin0<LOWER> + (WEIGHTED ? 0u : (uint32_t)qk);
+    const uint32_t base = s_cell - 4u * kBin0<LOWER> + (WEIGHTED ? 0u : (uint32_t)qk);
     for (int j = tj * 32; j < tj * 32 + nj; j += 4) {
       float u[4];
       {
@@ -1470,22 +1471,18 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
       const int4 pj = *reinterpret_cast<const int4*>(S.p + j);
       const int pp[4] = {pj.x, pj.y, pj.z, pj.w};
       if constexpr (!WEIGHTED) {
+        // near an edge the exact bin, before the counter is touched: counters
+        // only grow, so another group's flush may take them at any moment
+        if (near) {
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+            if ((__float_as_uint(u[v]) & 0xFFFFu) <= a.amb)
+              u[v] = kTileM + 0.5f +
+                     (float)exact_bin(S.x[j + v] - xk, S.y[j + v] - yk, S.z[j + v] - zk);
+        }
 #pragma unroll
         for (int v = 0; v < 4; ++v)
           t_red(base + (uint32_t)pp[v] + 4u * t_bin<LOWER>(u[v], nb), 1u);
-        if (near) {
-          // move the count of a pair whose exact bin is another
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            if ((__float_as_uint(u[v]) & 0xFFFFu) > a.amb) continue;
-            const int was = (int)(t_bin<LOWER>(u[v], nb) - kBin0<LOWER>);
-            const int b = exact_bin(S.x[j + v] - xk, S.y[j + v] - yk, S.z[j + v] - zk);
-            if (b == was) continue;
-            unsigned* row = cell + (pp[v] + qk) / 4;
-            atomicSub(row + was, 1u);
-            atomicAdd(row + b, 1u);
-          }
-        }
       } else {
         const int4 qj = *reinterpret_cast<const int4*>(S.q + j);
         const int4 wj = *reinterpret_cast<const int4*>(S.W + j);
@@ -2208,7 +2205,7 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
   // (1, 2, 8, 16, 32, 64, 512), the equilateral configurations and rows of
   // more than 65,535 neighbours (whose triangles could overflow the 32-bit
   // shared counters within one hub) take the merge-walk kernel.
-  const bool pair_ok = !equi && (o.variant & ~4) == 0 && g.max_deg <= kMaxSmemHistDeg;
+  const bool pair_ok = !equi && (o.variant & ~(4 | 1024)) == 0 && g.max_deg <= kMaxSmemHistDeg;
   // evenly spaced bins: the tiled pair kernel (variant bit 4 keeps the other)
   TileLaunch TL;
   if (pair_ok && !(o.variant & 4) && g.n > 0)
@@ -2272,6 +2269,9 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
     timer.stop(s);
   } else if (TL.cap > 0) {
     TArgs ta = TL.a;
+    // variant 1024: a flush before every hub (exercises flushes while other
+    // groups count)
+    if (o.variant & 1024) ta.limit = 0;
     ta.one = a.one;
     ta.cats = nullptr;
     ta.base = nullptr;

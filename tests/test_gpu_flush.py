@@ -1,7 +1,8 @@
 """Shared counters emptied by one group of warps while the others count on:
 variant 1024 flushes before every hub, on catalogues whose counts the kernels
-decide in integers (points on a mesh or in planes: volumes of zero), with one
-warp to half a CTA per hub. Against the oracle bit for bit."""
+decide in integers (points on a mesh or in planes: volumes of zero, pairs on
+bin edges), with one warp to half a CTA per hub. Against the oracle bit for
+bit."""
 import numpy as np
 import pytest
 
@@ -46,3 +47,24 @@ def test_parity_flush_between_groups(gs, kind, args, rmax):
         ge, go = gs.gs_count_4pcf_parity(g, variant=1024)
         assert np.array_equal(ge, re) and np.array_equal(go, ro)
     assert np.array_equal(gs.gs_count_4pcf(g, variant=1024), re)
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("kind,args,rmax", CATALOGUES)
+@pytest.mark.parametrize("rmin", [0, 1000])
+def test_3pcf_flush_between_groups(gs, kind, args, rmax, rmin, weighted):
+    """Bins of 200 units: on the mesh many pairs lie on an edge."""
+    X, box_u = kind(*args)
+    edges = np.arange(rmin, rmax + 1, 200, dtype=np.int64)
+    og, g = oracle.Graph(X, box_u, edges), gs.gs_build_graph(X, box_u, edges)
+    if weighted:
+        rng = np.random.default_rng(3)
+        w = (rng.uniform(0.5, 1.5, len(X)) * np.where(rng.random(len(X)) < 0.4, -1, 1)).astype(np.float32)
+        rc, rw = og.count_3pcf(w)
+        for _ in range(3):
+            c, s = gs.gs_count_3pcf(g, w, variant=1024)
+            assert np.array_equal(c, rc) and np.array_equal(s, rw)
+    else:
+        ref = og.count_3pcf()
+        for _ in range(3):
+            assert np.array_equal(gs.gs_count_3pcf(g, variant=1024), ref)
