@@ -1392,7 +1392,9 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     // the longer rows
     std::vector<int64_t> longer;
     bool global = false;
-    const std::vector<int32_t>& deg = host_deg(g);
+    const int32_t* deg = nullptr;
+    ls = host_deg(g, s, &deg);
+    if (ls) return ls;
     for (int64_t h = v.h0; h < v.h1; ++h)
       if (deg[h] > std::max(cap, 2)) {
         longer.push_back(h);

@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "gs_host_copy.h"
 #include "gs_internal.cuh"
 
 namespace gs {
@@ -725,42 +726,44 @@ int walk_words_device(Graph* g) {
 
 namespace {
 std::mutex g_host_mu;
+
+template <class T>
+int host_copy_of(std::vector<T>& kept, const T* src, size_t count, cudaStream_t s, const T** out) {
+  return host_copy(g_host_mu, kept, count, [&](T* dst) {
+    const cudaError_t e =
+        cudaMemcpyAsync(dst, src, sizeof(T) * count, cudaMemcpyDeviceToHost, s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);  // nothing may write to dst later
+    if (e != cudaSuccess || e2 != cudaSuccess) cudaGetLastError();
+    return cuda_status(e != cudaSuccess ? e : e2);
+  }, out);
 }
-const std::vector<int64_t>& host_ptr(const Graph& g) {
-  std::lock_guard<std::mutex> lock(g_host_mu);
-  if (g.h_ptr.empty()) {
-    std::vector<int64_t> p((size_t)g.n + 1, 0);
-    // an error stays for the calling query to report
-    (void)cudaMemcpy(p.data(), g.d_ptr, sizeof(int64_t) * p.size(), cudaMemcpyDeviceToHost);
-    g.h_ptr.swap(p);
-  }
-  return g.h_ptr;
+}  // namespace
+
+int host_ptr(const Graph& g, cudaStream_t s, const int64_t** out) {
+  return host_copy_of(g.h_ptr, g.d_ptr, (size_t)g.n + 1, s, out);
 }
-const std::vector<int32_t>& host_deg(const Graph& g) {
-  std::lock_guard<std::mutex> lock(g_host_mu);
-  if (g.h_deg.empty() && g.n) {
-    std::vector<int32_t> d((size_t)g.n, 0);
-    (void)cudaMemcpy(d.data(), g.d_deg, sizeof(int32_t) * d.size(), cudaMemcpyDeviceToHost);
-    g.h_deg.swap(d);
-  }
-  return g.h_deg;
+int host_deg(const Graph& g, cudaStream_t s, const int32_t** out) {
+  return host_copy_of(g.h_deg, g.d_deg, (size_t)g.n, s, out);
 }
 
-void shard_range(const Graph& g, const Opts& o, int64_t* lo, int64_t* hi) {
+int shard_range(const Graph& g, const Opts& o, int64_t* lo, int64_t* hi) {
   *lo = 0;
   *hi = g.n;
-  if (o.shards <= 1 || g.n == 0) return;
+  if (o.shards <= 1 || g.n == 0) return GS_OK;
   // boundaries at equal shares of the edge words (row starts do not decrease)
-  const std::vector<int64_t>& P = host_ptr(g);
+  const int64_t* P = nullptr;
+  const int st = host_ptr(g, o.stream, &P);
+  if (st) return st;
   const int64_t total = P[g.n];
   auto bound = [&](int k) -> int64_t {
     if (k <= 0) return 0;
     if (k >= o.shards) return g.n;
     const int64_t target = (int64_t)((__int128)total * k / o.shards);
-    return std::lower_bound(P.begin(), P.begin() + g.n, target) - P.begin();
+    return std::lower_bound(P, P + g.n, target) - P;
   };
   *lo = bound(o.shard);
   *hi = bound(o.shard + 1);
+  return GS_OK;
 }
 
 int plan_windows(const Graph& g, const Opts& o, WindowPlan* plan, int64_t lo, int64_t hi) {

@@ -95,12 +95,14 @@ struct Opts {
   int shard = 0, shards = 0;
 };
 
-// Host copies of the row starts [n+1] and lengths [n].
-const std::vector<int64_t>& host_ptr(const Graph& g);
-const std::vector<int32_t>& host_deg(const Graph& g);
+// Host copies of the row starts [n+1] and lengths [n] (valid as long as the
+// graph), made over the stream on first need. A copy that failed is not kept:
+// the call gets the status, the next one tries again.
+int host_ptr(const Graph& g, cudaStream_t s, const int64_t** out);
+int host_deg(const Graph& g, cudaStream_t s, const int32_t** out);
 
 // Hub range [lo, hi) of the query's shard (the whole graph when unsharded).
-void shard_range(const Graph& g, const Opts& o, int64_t* lo, int64_t* hi);
+int shard_range(const Graph& g, const Opts& o, int64_t* lo, int64_t* hi);
 Opts read_opts(const gs_options* o);
 
 // Whether p is device-accessible memory of the current device.
@@ -253,14 +255,14 @@ __host__ __device__ inline const uint32_t* row_at(const uint32_t* adj, const int
 template <class F>
 int for_each_window(const Graph& g, const Opts& o, Scratch& sc, F&& fn) {
   int64_t lo = 0, hi = 0;
-  shard_range(g, o, &lo, &hi);
-  if (lo >= hi) return GS_OK;
+  int st = shard_range(g, o, &lo, &hi);
+  if (st || lo >= hi) return st;
   if (g.d_adj) {
     const WinView v{g.d_adj, 0, g.n, 0, lo, hi};
     return fn(v);
   }
   WindowPlan plan;
-  int st = plan_windows(g, o, &plan, lo, hi);
+  st = plan_windows(g, o, &plan, lo, hi);
   if (st) return st;
   const size_t nw = plan.h0.size();
   uint32_t* buf[2] = {sc.alloc<uint32_t>(plan.max_words),

@@ -246,8 +246,11 @@ int pairs_disc_device(const Graph& g, const FixedW* fw, const double* d_rr, uint
     st = for_each_window(g, o, sc, [&](const WinView& v) -> int {
       // the window's own rows are contiguous from row h0 (below any split)
       const bool all = v.h0 == 0 && v.h1 == g.n;
-      const int64_t w0 = all ? 0 : host_ptr(g)[v.h0];
-      const int64_t words = (all ? g.slots : host_ptr(g)[v.h1]) - w0;
+      const int64_t* P = nullptr;
+      const int ps = all ? GS_OK : host_ptr(g, s, &P);
+      if (ps) return ps;
+      const int64_t w0 = all ? 0 : P[v.h0];
+      const int64_t words = (all ? g.slots : P[v.h1]) - w0;
       const uint32_t* own = v.adj + (w0 - v.off1);
       if (words)
         { k_pairs_count<<<sms * 8, kThreads, 0, s>>>(reinterpret_cast<const uint4*>(own), words / 4, nb,
