@@ -1258,7 +1258,9 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   void* d_ent = sc.alloc_bytes((size_t)nl * (small_ent ? 2 : 4));
   uint8_t* d_chir = sc.alloc<uint8_t>(no);
   if (!d_ent || !d_chir) return GS_ENOMEM;
+  unsigned long long* d_sample = nullptr;  // counts of the sample that ranks the orbits
   if (relabel) {
+    d_sample = sc.alloc<unsigned long long>(no);
     s_even = sc.alloc<unsigned long long>(no);
     s_odd = parity ? sc.alloc<unsigned long long>(no) : nullptr;
     if (weighted) {
@@ -1267,7 +1269,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     }
     d_slot = sc.alloc<int32_t>(no);
     if (!s_even || (parity && !s_odd) || (weighted && (!a.weven || (parity && !a.wodd))) ||
-        !d_slot)
+        !d_slot || !d_sample)
       return GS_ENOMEM;
   }
   cudaMemsetAsync(s_even, 0, sizeof(uint64_t) * no, s);
@@ -1334,15 +1336,13 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     for (int k = 0; k < no; ++k) order[k] = k;
     const int cap_s = fit_cap(std::min(maxd, 256), no, kWarps, false, false, false, avail);
     if (cap_s >= 16) {
-      unsigned long long* d_cnt = sc.alloc<unsigned long long>(no);
-      if (!d_cnt) return GS_ENOMEM;
-      cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long) * no, s);
+      cudaMemsetAsync(d_sample, 0, sizeof(unsigned long long) * no, s);
       Args sa = wa;
       sa.group = kWarps;
       sa.cap = cap_s;
       sa.dmax = cap_s;
       sa.hot = no;
-      sa.even = d_cnt;
+      sa.even = d_sample;
       sa.odd = nullptr;
       sa.weven = sa.wodd = nullptr;
       sa.W = nullptr;
@@ -1351,8 +1351,8 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
                       launch_smem(no, cap_s, kWarps, false, false, false));
       if (ls) return ls;
       std::vector<unsigned long long> cnt(no);
-      cudaMemcpyAsync(cnt.data(), d_cnt, sizeof(unsigned long long) * no, cudaMemcpyDeviceToHost,
-                      s);
+      cudaMemcpyAsync(cnt.data(), d_sample, sizeof(unsigned long long) * no,
+                      cudaMemcpyDeviceToHost, s);
       const cudaError_t e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return cuda_status(e);
       std::stable_sort(order.begin(), order.end(),
@@ -1369,6 +1369,9 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   KernelTimer timer(o.kernel_ms);
   timer.start(s);
   bool first = true;
+  std::vector<int64_t> longer;  // hubs of rows beyond cap, their device copy and their CTAs
+  int64_t* d_list = nullptr;
+  int grid2 = 0;
   void (*kern)(Args) = pick(parity, weighted, pix, all_hot);
   st = for_each_window(g, o, sc, [&](const WinView& v) -> int {
     a.adj = v.adj;
@@ -1390,37 +1393,44 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
       ls = launch(kern, a, sms, launch_smem(nh, cap, group, parity, weighted, pix));
     if (ls || maxd <= cap) return ls;
     // the longer rows
-    std::vector<int64_t> longer;
-    bool global = false;
+    const int64_t l0 = std::lower_bound(longer.begin(), longer.end(), v.h0) - longer.begin(),
+                  l1 = std::lower_bound(longer.begin(), longer.end(), v.h1) - longer.begin();
+    if (l0 == l1) return GS_OK;
+    Args la = a;
+    la.list = d_list + l0;
+    la.nlist = l1 - l0;
+    la.group = kWarps;
+    la.cap = cap2;
+    return launch(kern, la, (int)std::min<int64_t>(grid2, la.nlist),
+                  launch_smem(nh, cap2, kWarps, parity, weighted, pix));
+  }, [&]() -> int {
+    // the hubs of longer rows, in ascending order, and the workspace of those
+    // beyond the shared one: of as many CTAs as there is memory for
+    if (maxd <= cap) return GS_OK;
+    int64_t lo = 0, hi = 0;
+    int ls = shard_range(g, o, &lo, &hi);
     const int32_t* deg = nullptr;
-    ls = host_deg(g, s, &deg);
+    if (!ls) ls = host_deg(g, s, &deg);
     if (ls) return ls;
-    for (int64_t h = v.h0; h < v.h1; ++h)
+    bool global = false;
+    for (int64_t h = lo; h < hi; ++h)
       if (deg[h] > std::max(cap, 2)) {
         longer.push_back(h);
         global = global || deg[h] > cap2;
       }
     if (longer.empty()) return GS_OK;
-    int64_t* d_list = sc.alloc<int64_t>(longer.size());
+    d_list = sc.alloc<int64_t>(longer.size());
     if (!d_list) return GS_ENOMEM;
-    cudaMemcpyAsync(d_list, longer.data(), sizeof(int64_t) * longer.size(), cudaMemcpyHostToDevice,
-                    s);
-    Args la = a;
-    la.list = d_list;
-    la.nlist = (int64_t)longer.size();
-    la.group = kWarps;
-    la.cap = cap2;
-    int grid = (int)std::min<int64_t>(sms, la.nlist);
-    if (global) {
-      la.gscratch_stride =
-          (workspace_bytes(maxd, kWarps, sizeof(uint32_t), weighted, pix) + 255) & ~(size_t)255;
-      // as many CTAs as have room for their workspace
-      while (!(la.gscratch = sc.alloc<unsigned char>(la.gscratch_stride * grid)) && grid > 1)
-        grid = (grid + 1) / 2;
-      if (!la.gscratch) return GS_ENOMEM;
-    }
-    // the host list must outlive the (pageable, hence synchronous) copy only
-    return launch(kern, la, grid, launch_smem(nh, cap2, kWarps, parity, weighted, pix));
+    // (pageable memory: copied out of `longer` when the call returns)
+    const cudaError_t e = cudaMemcpyAsync(d_list, longer.data(), sizeof(int64_t) * longer.size(),
+                                          cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return cuda_status(e);
+    grid2 = (int)std::min<int64_t>(sms, (int64_t)longer.size());
+    if (!global) return GS_OK;
+    a.gscratch_stride =
+        (workspace_bytes(maxd, kWarps, sizeof(uint32_t), weighted, pix) + 255) & ~(size_t)255;
+    a.gscratch = staging(sc, a.gscratch_stride, &grid2);
+    return a.gscratch ? GS_OK : GS_ENOMEM;
   });
   if (st) return st;
   if (relabel) {

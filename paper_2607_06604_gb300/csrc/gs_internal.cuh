@@ -251,15 +251,17 @@ __host__ __device__ inline const uint32_t* row_at(const uint32_t* adj, const int
 // the copy of window k+1 (pinned host -> device, on a side stream) overlaps
 // the counting of window k on o.stream. fn(const WinView&) launches the
 // counting of the window's hubs. A resident graph makes one call with its
-// own edge array.
-template <class F>
-int for_each_window(const Graph& g, const Opts& o, Scratch& sc, F&& fn) {
+// own edge array. setup() allocates, once for all windows, what may take as
+// much memory as there is: the window buffers come first.
+template <class F, class S>
+int for_each_window(const Graph& g, const Opts& o, Scratch& sc, F&& fn, S&& setup) {
   int64_t lo = 0, hi = 0;
   int st = shard_range(g, o, &lo, &hi);
   if (st || lo >= hi) return st;
   if (g.d_adj) {
     const WinView v{g.d_adj, 0, g.n, 0, lo, hi};
-    return fn(v);
+    st = setup();
+    return st ? st : fn(v);
   }
   WindowPlan plan;
   st = plan_windows(g, o, &plan, lo, hi);
@@ -268,6 +270,8 @@ int for_each_window(const Graph& g, const Opts& o, Scratch& sc, F&& fn) {
   uint32_t* buf[2] = {sc.alloc<uint32_t>(plan.max_words),
                       nw > 1 ? sc.alloc<uint32_t>(plan.max_words) : nullptr};
   if (!buf[0] || (nw > 1 && !buf[1])) return GS_ENOMEM;
+  st = setup();
+  if (st) return st;
   cudaStream_t cs = nullptr;
   cudaEvent_t ready = nullptr, copied[2] = {nullptr, nullptr}, done[2] = {nullptr, nullptr};
   cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
@@ -312,6 +316,11 @@ int for_each_window(const Graph& g, const Opts& o, Scratch& sc, F&& fn) {
   if (ready) cudaEventDestroy(ready);
   if (cs) cudaStreamDestroy(cs);
   return st;
+}
+
+template <class F>
+int for_each_window(const Graph& g, const Opts& o, Scratch& sc, F&& fn) {
+  return for_each_window(g, o, sc, fn, [] { return (int)GS_OK; });
 }
 
 // Device helpers shared by the counting kernels --------------------------------

@@ -1,0 +1,77 @@
+"""Device memory of calls on graphs streamed in windows: what a call allocates
+for long rows does not grow with the number of windows."""
+import threading
+
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_mod():
+    import torch
+    assert torch.cuda.is_available()
+    return torch
+
+
+@pytest.fixture(scope="module")
+def gs():
+    import paper_2607_06604_gb300 as m
+    return m
+
+
+def stars(n_stars, rays):
+    """Background points and, per star, a hub with `rays` neighbours on the half
+    sphere ahead of it in x."""
+    rng = np.random.default_rng(5)
+    box_u, r = 200_000, 9500
+    out = [rng.integers(0, box_u, size=(20_000, 3))]
+    for k in range(n_stars):
+        at = np.array([(2 * k + 1) * box_u // (2 * n_stars), 100_000, 100_000])
+        d = rng.normal(size=(rays, 3))
+        d *= r / np.linalg.norm(d, axis=1)[:, None]
+        d[:, 0] = np.abs(d[:, 0])
+        out += [at[None], at + np.rint(d).astype(np.int64)]
+    return np.mod(np.concatenate(out), box_u).astype(np.int32), box_u
+
+
+def peak(torch, call):
+    """Most device memory taken during call(), sampled beside it."""
+    torch.cuda.synchronize()
+    base = low = torch.cuda.mem_get_info()[0]
+    done = threading.Event()
+
+    def sample():
+        nonlocal low
+        while not done.is_set():
+            low = min(low, torch.cuda.mem_get_info()[0])
+
+    t = threading.Thread(target=sample)
+    t.start()
+    out = call()
+    low = min(low, torch.cuda.mem_get_info()[0])
+    done.set()
+    t.join()
+    torch.cuda.synchronize()
+    return out, base - low
+
+
+def test_4pcf_workspace_is_one_for_all_windows(gs, torch_mod):
+    """Variant 1: every hub's workspace is in global memory, 152 CTAs of
+    more than 1,000^2 / 2 bytes."""
+    X, box_u = stars(8, 1500)
+    edges = np.array([9000, 9400, 10_000], dtype=np.int64)
+    ref = oracle.Graph(X, box_u, edges).count_4pcf()
+    used = {}
+    for windows in (2, 2, 10):
+        g = gs.gs_build_graph(X, box_u, edges, force_windows=windows)
+        info = gs.gs_graph_info(g)
+        assert info["windows"] >= windows and info["max_degree"] > 1000
+        for variant in (0, 1):
+            got, used[windows] = peak(torch_mod, lambda: gs.gs_count_4pcf_parity(g, variant=variant))
+            assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+    assert used[2] > 80 << 20
+    assert used[10] < 1.25 * used[2] + (32 << 20), used
