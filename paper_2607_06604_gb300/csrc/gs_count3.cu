@@ -2249,11 +2249,6 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
     int grid = (int)std::min<int64_t>((int64_t)2 * sms, (g.n + groups - 1) / groups);
     ea.gscratch = nullptr;
     ea.gstride = 0;
-    if (most > ea.cap) {
-      ea.gstride = ((size_t)most * 4 * words + 255) & ~(size_t)255;
-      ea.gscratch = staging(sc, ea.gstride * groups, &grid);
-      if (!ea.gscratch) return GS_ENOMEM;
-    }
     timer.start(s);
     st = for_each_window(g, o, sc, [&](const WinView& v) -> int {
       ea.one.adj = v.adj;
@@ -2265,6 +2260,11 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
       cudaMemsetAsync(ea.hub_counter, 0, sizeof(unsigned long long), s);
       { kern<<<grid, kTThreads, smem, s>>>(ea); note_launch(); }
       return cuda_status(cudaGetLastError());
+    }, [&]() -> int {
+      if (most <= ea.cap) return GS_OK;
+      ea.gstride = ((size_t)most * 4 * words + 255) & ~(size_t)255;
+      ea.gscratch = staging(sc, ea.gstride * groups, &grid);
+      return ea.gscratch ? GS_OK : GS_ENOMEM;
     });
     timer.stop(s);
   } else if (TL.cap > 0) {
@@ -2287,11 +2287,6 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
     int grid = (int)std::min<int64_t>(TL.blocks, (g.n + groups - 1) / groups);
     ta.gscratch = nullptr;
     ta.gstride = 0;
-    if (g.max_deg > TL.cap) {
-      ta.gstride = stage_bytes((g.max_deg + 31) & ~31, wm != kNone);
-      ta.gscratch = staging(sc, ta.gstride * groups, &grid);
-      if (!ta.gscratch) return GS_ENOMEM;
-    }
     timer.start(s);
     st = for_each_window(g, o, sc, [&](const WinView& v) -> int {
       ta.one.adj = v.adj;
@@ -2303,6 +2298,11 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
       cudaMemsetAsync(ta.hub_counter, 0, sizeof(unsigned long long), s);
       { kern<<<grid, kTThreads, TL.smem, s>>>(ta); note_launch(); }
       return cuda_status(cudaGetLastError());
+    }, [&]() -> int {
+      if (g.max_deg <= TL.cap) return GS_OK;
+      ta.gstride = stage_bytes((g.max_deg + 31) & ~31, wm != kNone);
+      ta.gscratch = staging(sc, ta.gstride * groups, &grid);
+      return ta.gscratch ? GS_OK : GS_ENOMEM;
     });
     timer.stop(s);
   } else if (PL.cap > 0) {

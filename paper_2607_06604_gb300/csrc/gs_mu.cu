@@ -546,15 +546,6 @@ bool mu_tiles(const Graph& g, int nmu, int nconf, uint64_t* d_counts, unsigned l
   int grid = (int)std::min<int64_t>((int64_t)ctas * sms, (g.n + groups - 1) / groups);
   a.gscratch = nullptr;
   a.gstride = 0;
-  *status = GS_OK;
-  if (g.max_deg > a.cap) {
-    a.gstride = (size_t)((g.max_deg + 31) & ~31) * 24;
-    a.gscratch = staging(sc, a.gstride * groups, &grid);
-    if (!a.gscratch) {
-      *status = GS_ENOMEM;
-      return true;
-    }
-  }
   timer.start(o.stream);
   *status = for_each_window(g, o, sc, [&](const WinView& v) -> int {
     a.adj = v.adj;
@@ -566,6 +557,11 @@ bool mu_tiles(const Graph& g, int nmu, int nconf, uint64_t* d_counts, unsigned l
     cudaMemsetAsync(a.hub_counter, 0, sizeof(unsigned long long), o.stream);
     { kern<<<grid, kTThreads, smem, o.stream>>>(a); note_launch(); }
     return cuda_status(cudaGetLastError());
+  }, [&]() -> int {
+    if (g.max_deg <= a.cap) return GS_OK;
+    a.gstride = (size_t)((g.max_deg + 31) & ~31) * 24;
+    a.gscratch = staging(sc, a.gstride * groups, &grid);
+    return a.gscratch ? GS_OK : GS_ENOMEM;
   });
   timer.stop(o.stream);
   return true;

@@ -112,7 +112,8 @@ __device__ inline int t_min_image(int q, int p, int64_t box) {
 }
 
 // Global staging of `each` bytes per CTA for rows beyond the shared one, with
-// as many CTAs of *grid as there is memory for (nullptr: not even one).
+// as many CTAs of *grid as there is memory for (nullptr: not even one). Last of
+// a call's allocations: it may leave nothing for others.
 inline unsigned char* staging(Scratch& sc, size_t each, int* grid) {
   for (;; *grid = (*grid + 1) / 2) {
     unsigned char* p = sc.alloc<unsigned char>(each * *grid);

@@ -75,3 +75,31 @@ def test_4pcf_workspace_is_one_for_all_windows(gs, torch_mod):
             assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
     assert used[2] > 80 << 20
     assert used[10] < 1.25 * used[2] + (32 << 20), used
+
+
+def test_streamed_calls_fit_beside_little_memory(gs, torch_mod):
+    """Rows of thousands beside short ones: the staging for long rows of every
+    group of warps would take 0.6 GB and makes do with less, but only after the
+    window buffers (2 of 60 MB) are there."""
+    torch = torch_mod
+    rng = np.random.default_rng(6)
+    box_u = 1_000_000
+    X = np.concatenate([rng.integers(0, box_u, size=(400_000, 3)),
+                        500_000 + rng.integers(-1500, 1501, size=(6500, 3))]).astype(np.int32)
+    edges = np.array([0, 2500, 5000], dtype=np.int64)
+    g = gs.gs_build_graph(X, box_u, edges, force_windows=2)
+    info = gs.gs_graph_info(g)
+    assert info["max_degree"] > 6000 and info["edges"] / len(X) < 64
+    w = rng.uniform(0.5, 1.5, len(X)).astype(np.float32)
+    calls = [lambda: gs.gs_count_3pcf(g), lambda: gs.gs_count_3pcf_mu(g, 2),
+             lambda: gs.gs_count_3pcf_equilateral(g), lambda: gs.gs_count_3pcf_equilateral(g, w)[1]]
+    refs = [c() for c in calls]
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    for spare in (240, 300, 360, 480):  # MB
+        free = torch.cuda.mem_get_info()[0]
+        held = torch.empty(free - (spare << 20), dtype=torch.uint8, device="cuda")
+        for call, ref in zip(calls, refs):
+            assert np.array_equal(call(), ref), spare
+        del held
+        torch.cuda.empty_cache()
