@@ -67,6 +67,24 @@ int cuda_status(cudaError_t e) {
   return GS_ECUDA;
 }
 
+cudaError_t allow_shared_bytes(const void* kern, size_t bytes) {
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, size_t> allowed;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  try {
+    size_t& have = allowed[{dev, kern}];
+    if (bytes <= have) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) have = bytes;
+  } catch (const std::bad_alloc&) {
+    e = cudaErrorMemoryAllocation;
+  }
+  return e;
+}
+
 Scratch::~Scratch() {
   for (void* p : ptrs_) cudaFreeAsync(p, s_);
 }

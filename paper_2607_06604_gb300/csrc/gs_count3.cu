@@ -2245,7 +2245,7 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
     const int groups = kTWarps / ea.group;
     const size_t smem = fixed + (size_t)groups * ea.cap * 4 * words;
     void (*kern)(EArgs) = weighted_e ? k_equi_tiles<true> : k_equi_tiles<false>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared(kern, smem);
     int grid = (int)std::min<int64_t>((int64_t)2 * sms, (g.n + groups - 1) / groups);
     ea.gscratch = nullptr;
     ea.gstride = 0;
@@ -2281,7 +2281,7 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
     ta.e2g = g.d_edges2;
     ta.hub_counter = a.hub_counter;
     void (*kern)(TArgs) = pick_count3t<false>(wm, fw && fw->nonneg, TL);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TL.smem);
+    allow_shared(kern, TL.smem);
     // no more CTAs than the hubs keep busy
     const int groups = kTWarps / TL.group;
     int grid = (int)std::min<int64_t>(TL.blocks, (g.n + groups - 1) / groups);
@@ -2322,7 +2322,7 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
     pa.lin_c = PL.lin_c;
     void (*kern)(PArgs) =
         pick_count3p<false>(wm, fw && fw->nonneg, PL.lut, PL.bin);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL.smem);
+    allow_shared(kern, PL.smem);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPThreads, PL.smem);
     const int grid = std::max(1, per_sm) * sms;
@@ -2362,7 +2362,7 @@ int count3_device(const Graph& g, const FixedW* fw, uint64_t* d_counts, double* 
   void (*kern)(Args);
   kern = equi ? pick_equi3(wm, fw && fw->nonneg, smem_hist)
               : pick_count3<false>(wm, fw && fw->nonneg, smem_hist, L.lut);
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_shared(kern, smem);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem);
   const int grid = std::max(1, per_sm) * sms;
@@ -2485,7 +2485,7 @@ int count3_batch_device(const Graph* const* gr, int ng, const FixedW* fws, uint6
     ta.e2g = gr[0]->d_edges2;
     ta.hub_counter = a.hub_counter;
     void (*kern)(TArgs) = pick_count3t<true>(wm, nonneg, TL);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TL.smem);
+    allow_shared(kern, TL.smem);
     int grid = (int)std::min<int64_t>(TL.blocks, base[ng]);
     ta.gscratch = nullptr;
     ta.gstride = 0;
@@ -2514,7 +2514,7 @@ int count3_batch_device(const Graph* const* gr, int ng, const FixedW* fws, uint6
     pa.lin_c = PL.lin_c;
     void (*kern)(PArgs) =
         pick_count3p<true>(wm, nonneg, PL.lut, PL.bin);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL.smem);
+    allow_shared(kern, PL.smem);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPThreads, PL.smem);
     const int grid = std::max(1, per_sm) * sms;
@@ -2543,7 +2543,7 @@ int count3_batch_device(const Graph* const* gr, int ng, const FixedW* fws, uint6
   const size_t smem = L.smem;
   void (*kern)(Args);
   kern = pick_count3<true>(wm, nonneg, smem_hist, L.lut);
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_shared(kern, smem);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem);
   timer.start(s);
@@ -2695,7 +2695,7 @@ extern "C" int gs_count_3pcf_noalloc(const gs_graph* G, uint64_t* counts,
     a.first_wait_limit = (o.variant & 16) ? 0u : kWaitLimit;
     a.stage_cap = std::min(a.stage_cap, L.stage_words);
     void (*kern)(Args) = pick_count3<false>(kNone, true, L.smem_hist, L.lut);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
+    allow_shared(kern, L.smem);
     int per_sm = 0, sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -2798,7 +2798,7 @@ extern "C" int gs_plan_3pcf_batch(const gs_graph* const* graphs, int32_t n_graph
   a.stage_cap = std::min(a.stage_cap, L.stage_words);
   void (*kern)(Args) = pick_count3<true>(kNone, true, L.smem_hist, L.lut);
   int per_sm = 0, sms = 0, dev = 0;
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
+  if (e == cudaSuccess) e = allow_shared(kern, L.smem);
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, L.smem);

@@ -1318,7 +1318,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     return small_ent ? pick4<uint16_t>(P, Wt, X, fast) : pick4<uint32_t>(P, Wt, X, fast);
   };
   auto launch = [&](void (*k)(Args), const Args& la, int grid, size_t smem) -> int {
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared(k, smem);
     cudaMemsetAsync(la.hub_counter, 0, sizeof(unsigned long long), s);
     k<<<grid, kThreads, smem, s>>>(la);
     note_launch();

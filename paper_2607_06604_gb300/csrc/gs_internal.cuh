@@ -141,6 +141,15 @@ const void* to_device(Scratch& sc, const void* p, size_t bytes, cudaStream_t s);
 // Status from a CUDA error.
 int cuda_status(cudaError_t e);
 
+// Lets launches of the kernel on the current device use up to `bytes` of dynamic
+// shared memory. The limit only ever grows: a call in another thread that needs
+// less must not take it away between here and the launch.
+cudaError_t allow_shared_bytes(const void* kern, size_t bytes);
+template <class... A>
+cudaError_t allow_shared(void (*kern)(A...), size_t bytes) {
+  return allow_shared_bytes(reinterpret_cast<const void*>(kern), bytes);
+}
+
 // Exclusive scans (device, stream ordered). out may alias in.
 int scan_exclusive_i32(const int32_t* in, int32_t* out, int64_t n, int32_t* total_dev,
                        cudaStream_t s, Scratch& sc);

@@ -542,7 +542,7 @@ bool mu_tiles(const Graph& g, int nmu, int nconf, uint64_t* d_counts, unsigned l
   a.counts = reinterpret_cast<unsigned long long*>(d_counts);
   a.hub_counter = counter;
   void (*kern)(MTArgs) = bins.lower ? k_mu_tiles<true> : k_mu_tiles<false>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_shared(kern, smem);
   int grid = (int)std::min<int64_t>((int64_t)ctas * sms, (g.n + groups - 1) / groups);
   a.gscratch = nullptr;
   a.gstride = 0;
@@ -652,7 +652,7 @@ int count3mu_device(const Graph& g, const FixedW* fw, int nmu, uint64_t* d_count
   const bool small = g.edges[g.nb] <= 65536;
   void (*kern)(MArgs) = weighted ? (small ? k_count3mu<true, true> : k_count3mu<true, false>)
                                  : (small ? k_count3mu<false, true> : k_count3mu<false, false>);
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_shared(kern, smem);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMThreads, smem);
   const int grid = std::max(1, per_sm) * sms;

@@ -196,7 +196,7 @@ int pairs_weighted_device(const Graph& g, const FixedW& fw, unsigned long long* 
   timer.start(s);
   int st = GS_OK;
   const size_t smem = (kThreads / 32) * pair_warp_bytes(nb);
-  cudaFuncSetAttribute(k_pairs_weighted, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_shared(k_pairs_weighted, smem);
   // a CTA's counts stay below 2^32: at most 2^31 edges each
   const int grid = (int)std::max<int64_t>(sms * 8, (g.edges_total >> 24) + 1);
   if (g.n)
