@@ -386,18 +386,19 @@ int build_graph_device(const int32_t* d_xyz, int64_t n, int64_t box_u,
   const int64_t rmax = edges[nb];
   std::vector<int64_t> e2(nb + 1);
   for (int b = 0; b <= nb; ++b) e2[b] = edges[b] * edges[b];
-  auto dev_alloc = [&](void** p, size_t bytes) -> int {
+  auto dev_alloc = [&](void** p, size_t bytes, bool pooled = true) -> int {
     if (bytes == 0) bytes = 16;
     // small arrays from the library's pool (ready in the order of the build's
     // stream, which the build synchronises), large ones of their own
     cudaMemPool_t pool = memory_pool();
-    cudaError_t e = pool && bytes <= kPoolKeep / 8 ? cudaMallocFromPoolAsync(p, bytes, pool, s)
-                                                   : cudaMalloc(p, bytes);
+    cudaError_t e = pool && pooled && bytes <= kPoolKeep / 8
+                        ? cudaMallocFromPoolAsync(p, bytes, pool, s)
+                        : cudaMalloc(p, bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
       // give back what the pool keeps, and try again
       if (pool) {
-        cudaDeviceSynchronize();
+        cudaStreamSynchronize(s);
         cudaMemPoolTrimTo(pool, 0);
       }
       if (cudaMalloc(p, bytes) != cudaSuccess) {
@@ -409,7 +410,8 @@ int build_graph_device(const int32_t* d_xyz, int64_t n, int64_t box_u,
     g->device_bytes += (int64_t)bytes;
     return GS_OK;
   };
-  int st = dev_alloc((void**)&g->d_edges2, sizeof(int64_t) * (nb + 1));
+  // not from the pool: freeing it is how gs_free_graph waits for the device
+  int st = dev_alloc((void**)&g->d_edges2, sizeof(int64_t) * (nb + 1), false);
   if (!st) st = dev_alloc((void**)&g->d_xyzp, sizeof(int4) * std::max<int64_t>(n, 1));
   if (!st) st = dev_alloc((void**)&g->d_deg, sizeof(int32_t) * std::max<int64_t>(n, 1));
   if (!st) st = dev_alloc((void**)&g->d_ptr, sizeof(int64_t) * (n + 1));
