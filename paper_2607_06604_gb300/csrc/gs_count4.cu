@@ -28,9 +28,9 @@
 // error bound of zero, exactly in integers. Counts use per-CTA
 // shared-memory histograms flushed with 64-bit atomics, one cell per orbit
 // and sign of V: even = V > 0 plus V < 0, odd = their difference (chiral
-// orbits), so a tetrahedron updates one cell; those with V = 0 go to the
-// global even count. Hubs with more neighbours than the shared workspace
-// holds run with their workspace in global scratch.
+// orbits), so a tetrahedron updates one cell; those with V = 0 go to the two
+// cells in turn (see take_turn). Hubs with more neighbours than the shared
+// workspace holds run with their workspace in global scratch.
 //
 // What bounds it: instruction issue (80% of slots, 32 instructions per step of
 // 14 tetrahedra) and the shared-memory/L1 pipe (73%) together. Measured on one
@@ -408,6 +408,19 @@ __host__ __device__ inline size_t hist_words(int64_t hot, bool parity) {
   return (size_t)hot * (parity ? 2 : 1) + 32;
 }
 
+// The cell that the next V = 0 of a chiral orbit goes to, unweighted: the two
+// cells of the orbit in turn, which leaves their difference alone, but for one
+// when the number of them is odd. The top bit of the first cell says whose turn
+// it is, and that much is taken off when the cells are emptied: every +1 there
+// stands for one more such tetrahedron in the first cell than in the second,
+// whichever flush takes which. (Global atomics for V = 0 cost planar catalogues
+// more than all else: 2e4 points in a plane, 1.5e10 tetrahedra, 214 ms against
+// 92.)
+constexpr uint32_t kTurn = 0x80000000u;
+__device__ inline uint32_t take_turn(const Hist& h, uint32_t slot) {
+  return 2u * slot + (atomicXor(h.cnt + 2u * slot, kTurn) >> 31);
+}
+
 // One tetrahedron straight to the global counts and sums. cell: twice the slot
 // plus the sign (parity) or the slot; deg: V = 0 on a chiral orbit, even
 // channel only. Wab = W_a W_b.
@@ -725,16 +738,14 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
                   if (!decltype(diag)::value || s0 + u < lane) vmin = fminf(vmin, fabsf(V[u]));
                 if (vmin < a.eps) {
                   // a volume within its error bound of zero: the exact sign, or
-                  // the even channel alone if V = 0
+                  // the two cells in turn if V = 0
 #pragma unroll
                   for (int u = 0; u < U; ++u) {
                     if (b23[u] >= (uint32_t)nb || !(fabsf(V[u]) < a.eps) || en[u] >= 0) continue;
                     const long long Vx = det3(da, w.disp[list[k0 + s0 + u]], dc);
                     V[u] = Vx < 0 ? -1.0f : 1.0f;
-                    if (Vx == 0) {
-                      atomicAdd(a.even + (((uint32_t)en[u] & Ent<E>::kMask) >> 1), 1ull);
-                      en[u] = (int)trash;
-                    }
+                    if (Vx == 0)
+                      en[u] = (int)take_turn(h, ((uint32_t)en[u] & Ent<E>::kMask) >> 1);
                   }
                 }
               }
@@ -863,7 +874,8 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
               } else {
                 cell >>= 1;
               }
-              if (!deg && cell < hotc) atomicAdd(h.cnt + cell, 1u);
+              if (PARITY && deg && cell < hotc) cell = take_turn(h, cell >> 1);
+              if (cell < hotc) atomicAdd(h.cnt + cell, 1u);
               else record_global<PARITY, false>(a, cell, deg, 0, 0, 0);
             }
           }
@@ -915,11 +927,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
   auto flush = [&](int t, int threads) {
     for (int k = t; k < a.hot; k += threads) {
       if (PARITY) {
-        const unsigned p = atomicExch(h.cnt + 2 * k, 0u), n = atomicExch(h.cnt + 2 * k + 1, 0u);
-        if (p | n) {
-          atomicAdd(a.even + k, (unsigned long long)p + n);
-          if (p != n && a.chir[k])
-            atomicAdd(a.odd + k, (unsigned long long)((long long)p - (long long)n));
+        const unsigned c = atomicExch(h.cnt + 2 * k, 0u), n = atomicExch(h.cnt + 2 * k + 1, 0u);
+        if (c | n) {
+          const unsigned p = c & ~kTurn;
+          const long long d = (long long)p - (long long)n - (long long)(c >> 31);
+          if (p | n) atomicAdd(a.even + k, (unsigned long long)p + n);
+          if (d && a.chir[k]) atomicAdd(a.odd + k, (unsigned long long)d);
         }
       } else {
         const unsigned p = atomicExch(h.cnt + k, 0u);
@@ -956,10 +969,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
       if (i >= 0) {
         const unsigned long long m = (unsigned long long)a.deg[i];
         const unsigned long long need = m * (m - 1) * (m - 2) / 6;
-        // The shared counters stay below 2^32: between two flushes they take
-        // the hubs registered since the last reset (at most 2^29 and one
+        // The shared counters stay below 2^31: between two flushes they take
+        // the hubs registered since the last reset (at most 2^28 and one
         // hub), those registered while a flush runs (the same) and those
-        // under way at a reset (31 hubs of at most 2^26).
+        // under way at a reset (31 hubs). A hub is at most 2^26, and below 2^25
+        // where a CTA has several groups (their rows are in shared memory).
         if (need <= kMaxHubNeed &&
             atomicAdd(&s.pending, need) + need > a.limit) {
           atomicExch(&s.pending, 0ull);
@@ -1192,7 +1206,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   }
   // variant 1024: a flush before every hub (exercises flushes while other
   // groups count)
-  a.limit = (o.variant & 1024) ? 0 : 1ull << 29;
+  a.limit = (o.variant & 1024) ? 0 : 1ull << 28;
   // weighted results land in the callers' 192-bit arrays (or scratch)
   unsigned long long* weven = weighted ? (weven_out ? weven_out : sc.alloc<unsigned long long>(3 * (size_t)no))
                                        : nullptr;

@@ -68,3 +68,25 @@ def test_3pcf_flush_between_groups(gs, kind, args, rmax, rmin, weighted):
         ref = og.count_3pcf()
         for _ in range(3):
             assert np.array_equal(gs.gs_count_3pcf(g, variant=1024), ref)
+
+
+@pytest.mark.parametrize("nb", [3, 5, 9])
+@pytest.mark.parametrize("kind,args,rmax", [CATALOGUES[k] for k in (0, 2, 4, 6)] + [
+    (planes, (3, 17_000), 4000), (planes, (12, 17_000), 4000), (planes, (150, 17_000), 4000)])
+def test_volumes_of_zero(gs, kind, args, rmax, nb):
+    """V = 0 tetrahedra in even and odd numbers per orbit, unweighted (all orbits
+    or 64 in shared memory, rows in global memory) and with weights of both
+    signs."""
+    X, box_u = kind(*args)
+    edges = np.linspace(0, rmax, nb + 1).astype(np.int64)
+    og, g = oracle.Graph(X, box_u, edges), gs.gs_build_graph(X, box_u, edges)
+    rng = np.random.default_rng(8)
+    w = (rng.uniform(0.5, 1.5, len(X)) * np.where(rng.random(len(X)) < 0.5, -1, 1)).astype(np.float32)
+    for pix in (False, True):
+        ref = og.count_4pcf(w, pixel=pix)
+        for variant in (0, 1, 8):
+            got = gs.gs_count_4pcf_parity(g, w, pix=pix, variant=variant)
+            for a, b in zip(got, ref):
+                assert np.array_equal(a, b), (pix, variant)
+            got = gs.gs_count_4pcf_parity(g, pix=pix, variant=variant)
+            assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1]), (pix, variant)
