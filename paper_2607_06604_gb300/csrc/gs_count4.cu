@@ -104,6 +104,7 @@ struct Args {
   int group; // warps per group
   int bk_shift, bk_n;  // squared-distance buckets (bk_n = 0: binary search)
   int hot;             // orbits (slots) below this are accumulated in shared memory
+  int even_hot;        // weighted parity, ZERO: slots below this have an even-only cell too
   float eps;           // volumes within eps of zero are decided in integers
   unsigned long long limit;  // tetrahedra between two flushes of the shared counters
   unsigned long long* even;
@@ -394,7 +395,9 @@ struct Chunk {
 };
 
 // The counters of one CTA: cells of the slots below a.hot (parity: two per
-// slot), then a word per lane for no edge. Weighted: three more arrays, `stride`
+// slot; ZERO: then one per slot below a.even_hot for what counts in the even
+// channel only, V = 0 and achiral orbits), then a word per lane for no edge.
+// Weighted: three more arrays, `stride`
 // words apart, the low to high words of the hub's sums.
 struct Hist {
   unsigned* cnt;
@@ -404,9 +407,7 @@ struct Hist {
 // of its carry (from zero, every change of a sum's sign carried: 2.5 ms of
 // global atomics per 1e9 tetrahedra).
 constexpr uint32_t kTopZero = 0x80000000u;
-__host__ __device__ inline size_t hist_words(int64_t hot, bool parity) {
-  return (size_t)hot * (parity ? 2 : 1) + 32;
-}
+__host__ __device__ inline size_t hist_words(int64_t cells) { return (size_t)cells + 32; }
 
 // The cell that the next V = 0 of a chiral orbit goes to, unweighted: the two
 // cells of the orbit in turn, which leaves their difference alone, but for one
@@ -451,7 +452,7 @@ __device__ inline void record_global(const Args& a, uint32_t cell, bool deg, int
 // addresses of their counts, `none` for the lane's unused words); cell[] for the
 // carries out of the top word (about one in 2^21 for weights within a factor of
 // two).
-template <bool PARITY>
+template <bool PARITY, bool ZERO>
 __device__ inline void record_weighted(const Args& a, const uint32_t (&at)[2],
                                        const uint32_t (&cell)[2], uint32_t none, uint32_t stride,
                                        int64_t Wi, int Wc, const long long (&V)[2]) {
@@ -490,10 +491,12 @@ __device__ inline void record_weighted(const Args& a, const uint32_t (&at)[2],
     if (c != 0u && at[v] != none) {
       // c 2^96 W_i
       const long long t = (long long)(int)c * Wi;
-      const uint32_t slot = PARITY ? cell[v] >> 1 : cell[v];
+      const uint32_t cells2 = 2u * (uint32_t)a.hot;  // from here on the even-only ones
+      const bool even = ZERO && cell[v] >= cells2;
+      const uint32_t slot = even ? cell[v] - cells2 : PARITY ? cell[v] >> 1 : cell[v];
       atomic_add_w192(a.weven + 3 * (size_t)slot, 0ull, (unsigned long long)t << 32,
                       (unsigned long long)(t >> 32));
-      if (PARITY && a.chir[slot]) {
+      if (PARITY && !even && a.chir[slot]) {
         const long long u = (cell[v] & 1u) ? -t : t;
         atomic_add_w192(a.wodd + 3 * (size_t)slot, 0ull, (unsigned long long)u << 32,
                         (unsigned long long)(u >> 32));
@@ -505,8 +508,9 @@ __device__ inline void record_weighted(const Args& a, const uint32_t (&at)[2],
 // One hub by one group of warps. GW: the workspace is in global memory.
 // gt: thread within the group; chunk (and wchunk): the warp's 32 entries.
 // FAST: unweighted, every slot's cells in shared memory, workspace in shared
-// memory; the inner loop is then free of branches.
-template <bool PARITY, bool WEIGHTED, bool PIX, bool GW, bool FAST, class E, class L>
+// memory; the inner loop is then free of branches. ZERO: weighted, with even-only
+// cells (their few instructions in every loop cost 10% where V = 0 is rare).
+template <bool PARITY, bool WEIGHTED, bool PIX, bool GW, bool FAST, bool ZERO, class E, class L>
 __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, const Hist& h,
                             const float4* pixu, Chunk* ch, long long* wchunk, int64_t i, int m,
                             int g, int gt) {
@@ -535,6 +539,13 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
       const uint32_t word = row[k], id = edge_id(word);
       place(pos, word, id, a.xyzp[id]);
     }
+  } else if constexpr (ZERO) {
+    // as they are: on a mesh or in a plane lanes with neighbouring c's of one bin
+    // would all add to one orbit's cells
+    for (int k = gt; k < m; k += gthreads) {
+      const uint32_t word = row[k], id = edge_id(word);
+      place(k, word, id, a.xyzp[id]);
+    }
   } else {
     // by the hub edge's bin (counting sort): lanes with neighbouring c's then
     // share b_03, so their table entries lie in few lines
@@ -556,7 +567,7 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
     }
   }
   group_sync(g, gthreads);
-  if (!PIX && gt < kMaxBins4) cur[gt] = 0;  // for the next hub (barriers below)
+  if (!PIX && !ZERO && gt < kMaxBins4) cur[gt] = 0;  // for the next hub (barriers below)
   using I = typename std::conditional<GW, int64_t, int>::type;
   // B: (a, c) is an edge iff E_0^2 <= |D_c - D_a|^2 < E_nb^2 on the staged
   // hub-relative displacements (4 E_nb < L makes their difference the pair's
@@ -775,7 +786,10 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
           const E* ent_c = ent + lane_idx;
           const uint32_t hotc = hist_ok ? (uint32_t)(PARITY ? 2 * a.hot : a.hot) : 0u;
           const uint32_t cells = (uint32_t)__cvta_generic_to_shared(h.cnt),
-                         none = cells + 4u * ((uint32_t)(PARITY ? 2 * a.hot : a.hot) + lane);
+                         cells2 = (uint32_t)(PARITY ? 2 * a.hot : a.hot),
+                         evenc = cells2 + (ZERO ? (uint32_t)a.even_hot : 0u),
+                         hotce = hist_ok ? evenc : 0u,
+                         none = cells + 4u * (evenc + lane);
           auto steps = [&](auto diag) {
             for (int s0 = 0; s0 < ns; s0 += 2) {
               uint32_t b23[2], cell[2], at[2];
@@ -811,13 +825,15 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
                 } else {
                   cell[u] = ((uint32_t)en[u] & Ent<E>::kMask) >> 1;
                 }
-                const bool hot = cell[u] < hotc;
+                const bool even = ZERO && en[u] >= 0;
+                if (ZERO) cell[u] = even ? cells2 + (cell[u] >> 1) : cell[u];
+                const bool hot = cell[u] < (even ? hotce : hotc);
                 rare |= !hot && b23[u] < (uint32_t)nb;
                 at[u] = hot ? cells + 4u * cell[u] : none;
               }
               if (rare) {
-                // a volume near zero is decided in integers; V = 0 and orbits
-                // without shared cells go to the global sums
+                // a volume near zero is decided in integers; what has no shared
+                // cell goes to the global sums
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                   if (b23[u] >= (uint32_t)nb) continue;
@@ -828,11 +844,21 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
                     cell[u] = ((uint32_t)en[u] ^ (Vx < 0 ? 1u : 0u)) & Ent<E>::kMask;
                     at[u] = cell[u] < hotc && !deg ? cells + 4u * cell[u] : none;
                   }
-                  if (deg || cell[u] >= hotc)
+                  if constexpr (ZERO) {
+                    if (deg) {
+                      cell[u] = cells2 + (cell[u] >> 1);
+                      at[u] = cell[u] < hotce ? cells + 4u * cell[u] : none;
+                    }
+                    if (at[u] == none)
+                      record_global<PARITY, true>(
+                          a, en[u] >= 0 || deg ? 2u * (cell[u] - cells2) : cell[u], deg, Wi, wab[u],
+                          Wc);
+                  } else if (deg || cell[u] >= hotc) {
                     record_global<PARITY, true>(a, cell[u], deg, Wi, wab[u], Wc);
+                  }
                 }
               }
-              record_weighted<PARITY>(a, at, cell, none, 4u * h.stride, Wi, Wc, wab);
+              record_weighted<PARITY, ZERO>(a, at, cell, none, 4u * h.stride, Wi, Wc, wab);
             }
           };
           if (t0 > k0) steps(std::false_type{});
@@ -886,15 +912,17 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
   }
 }
 
-template <bool PARITY, bool WEIGHTED, bool PIX, bool FAST, class E>
+// VARIANT: FAST of an unweighted launch, ZERO of a weighted one.
+template <bool PARITY, bool WEIGHTED, bool PIX, bool VARIANT, class E>
 __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
+  constexpr bool FAST = !WEIGHTED && VARIANT, ZERO = WEIGHTED && VARIANT;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Shared s;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int group = a.group, gthreads = group * 32, g = warp / group, gt = tid - g * gthreads;
   unsigned char* sp = smem;
   Hist h;
-  h.stride = (uint32_t)hist_words(a.hot, PARITY);
+  h.stride = (uint32_t)hist_words((PARITY ? 2 : 1) * a.hot + (ZERO ? a.even_hot : 0));
   h.cnt = reinterpret_cast<unsigned*>(sp);
   sp += pad16((size_t)h.stride * (WEIGHTED ? 16 : 4));
   float4* pixu = reinterpret_cast<float4*>(sp);
@@ -939,6 +967,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
         if (p) atomicAdd(a.even + k, (unsigned long long)p);
       }
     }
+    if (ZERO)
+      for (int k = t; k < a.even_hot; k += threads) {
+        const unsigned z = atomicExch(h.cnt + 2 * a.hot + k, 0u);
+        if (z) atomicAdd(a.even + k, (unsigned long long)z);
+      }
   };
 
   unsigned long long next = 0;  // the group's first thread: the next ticket, taken ahead
@@ -990,9 +1023,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
       const Workspace<uint32_t> ws_g =
           carve<uint32_t>(a.gscratch + (size_t)blockIdx.x * a.gscratch_stride, a.gcap, group,
                           WEIGHTED, PIX);
-      hub4<PARITY, WEIGHTED, PIX, true, false, E>(a, ws_g, s, h, pixu, ch, wchunk, i, m, g, gt);
+      hub4<PARITY, WEIGHTED, PIX, true, false, ZERO, E>(a, ws_g, s, h, pixu, ch, wchunk, i, m, g, gt);
     } else {
-      hub4<PARITY, WEIGHTED, PIX, false, FAST, E>(a, ws_s, s, h, pixu, ch, wchunk, i, m, g, gt);
+      hub4<PARITY, WEIGHTED, PIX, false, FAST, ZERO, E>(a, ws_s, s, h, pixu, ch, wchunk, i, m, g, gt);
     }
     group_sync(g, gthreads);
     if (WEIGHTED) {
@@ -1000,19 +1033,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
       // launches have one group; the barrier at the top of the loop orders
       // the clearing before the next hub's additions)
       const long long Wi = a.W[i];
+      // the words as a signed 96-bit number (carries out of it are in the
+      // global sums already); cleared
+      auto take = [&](int cell, unsigned long long& lo, unsigned long long& hi) {
+        unsigned* c = h.cnt + h.stride + cell;
+        const uint32_t w0 = c[0], w1 = c[h.stride], w2 = c[2 * h.stride];
+        lo = ((unsigned long long)w1 << 32) | w0;
+        hi = (unsigned long long)(long long)(int)(w2 ^ kTopZero);
+        if (lo | hi) {
+          c[0] = c[h.stride] = 0u;
+          c[2 * h.stride] = kTopZero;
+        }
+      };
       for (int k = gt; k < a.hot; k += gthreads) {
-        // the words as a signed 96-bit number (carries out of it are in the
-        // global sums already); cleared
-        auto take = [&](int cell, unsigned long long& lo, unsigned long long& hi) {
-          unsigned* c = h.cnt + h.stride + cell;
-          const uint32_t w0 = c[0], w1 = c[h.stride], w2 = c[2 * h.stride];
-          lo = ((unsigned long long)w1 << 32) | w0;
-          hi = (unsigned long long)(long long)(int)(w2 ^ kTopZero);
-          if (lo | hi) {
-            c[0] = c[h.stride] = 0u;
-            c[2 * h.stride] = kTopZero;
-          }
-        };
         unsigned long long elo, ehi;
         take(PARITY ? 2 * k : k, elo, ehi);
         if (PARITY) {
@@ -1027,6 +1060,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
         }
         if (elo | ehi) fold_i128(a.weven + 3 * k, elo, ehi, Wi);
       }
+      if (ZERO)
+        for (int k = gt; k < a.even_hot; k += gthreads) {
+          unsigned long long lo, hi;
+          take(2 * a.hot + k, lo, hi);
+          if (lo | hi) fold_i128(a.weven + 3 * k, lo, hi, Wi);
+        }
     }
   }
   __syncthreads();
@@ -1112,6 +1151,43 @@ __global__ void k_slots_to_orbits(const unsigned long long* __restrict__ src,
   }
 }
 
+// Fraction of volumes of zero, estimated: triples of neighbours of random hubs,
+// out[0] those with V = 0 (pixelised: of the pixels seen from the hub), out[1]
+// all. Any sequence of numbers will do; the answer only decides a layout.
+__global__ void k_zero_volumes(Args a, int pix, unsigned* out) {
+  uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) * kHashMul + 12345u;
+  auto next = [&](int n) {
+    r = r * 1664525u + 1013904223u;
+    return (int)__umulhi(r, (uint32_t)n);
+  };
+  const int64_t i = a.hub_begin + next((int)(a.hub_end - a.hub_begin));
+  const int m = a.deg[i];
+  if (m < 3) return;
+  const uint32_t* row = row_at(a.adj, a.ptr, i, a.adj_off, a.split, a.adj_off2);
+  const int4 P = a.xyzp[i];
+  const int at[3] = {next(m), next(m), next(m)};
+  if (at[0] == at[1] || at[0] == at[2] || at[1] == at[2]) return;
+  int4 d[3];
+  float4 u[3];
+  for (int v = 0; v < 3; ++v) {
+    const int4 Q = a.xyzp[edge_id(row[at[v]])];
+    d[v] = make_int4((int)mi((int64_t)Q.x - P.x, a.box), (int)mi((int64_t)Q.y - P.y, a.box),
+                     (int)mi((int64_t)Q.z - P.z, a.box), 0);
+    if (pix) u[v] = a.pixu[dir_pixel(d[v].x, d[v].y, d[v].z)];
+  }
+  bool zero;
+  if (pix) {
+    const float V = (u[0].y * u[1].z - u[0].z * u[1].y) * u[2].x +
+                    (u[0].z * u[1].x - u[0].x * u[1].z) * u[2].y +
+                    (u[0].x * u[1].y - u[0].y * u[1].x) * u[2].z;
+    zero = fabsf(V) < a.eps;
+  } else {
+    zero = det3(d[0], d[1], d[2]) == 0;
+  }
+  if (zero) atomicAdd(out, 1u);
+  atomicAdd(out + 1, 1u);
+}
+
 __global__ void k_dir_pixels(const int32_t* d, int64_t n, uint8_t* out) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x)
@@ -1129,32 +1205,33 @@ int direction_pixels_device(const int32_t* d_dirs, int64_t n, uint8_t* d_out, cu
 }
 
 namespace {
-// fast: unweighted with every slot in shared memory
+// variant: unweighted with every slot in shared memory; weighted parity with
+// cells for V = 0
 template <class E>
-void (*pick4(bool parity, bool weighted, bool pix, bool fast))(Args) {
-#define GS_K4(P, X)                                    \
-  (weighted ? k_count4<P, true, X, false, E>           \
-   : fast   ? k_count4<P, false, X, true, E>           \
-            : k_count4<P, false, X, false, E>)
+void (*pick4(bool parity, bool weighted, bool pix, bool variant))(Args) {
+#define GS_K4(P, X)                                                             \
+  (weighted ? (P && variant ? k_count4<P, true, X, P, E> : k_count4<P, true, X, false, E>) \
+   : variant ? k_count4<P, false, X, true, E>                                   \
+             : k_count4<P, false, X, false, E>)
   if (parity && pix) return GS_K4(true, true);
   if (parity) return GS_K4(true, false);
   return GS_K4(false, false);
 #undef GS_K4
 }
 
-// Shared memory of a launch: cells of `hot` slots, chunks, pixel centres and
-// the workspaces of 32 / group groups.
-size_t launch_smem(int64_t hot, int cap, int group, bool parity, bool weighted, bool pix) {
-  return pad16(hist_words(hot, parity) * (weighted ? 16 : 4)) + (pix ? 256 * sizeof(float4) : 0) +
+// Shared memory of a launch: `cells` counters, chunks, pixel centres and the
+// workspaces of 32 / group groups.
+size_t launch_smem(int64_t cells, int cap, int group, bool weighted, bool pix) {
+  return pad16(hist_words(cells) * (weighted ? 16 : 4)) + (pix ? 256 * sizeof(float4) : 0) +
          (size_t)kWarps * sizeof(Chunk) + (weighted ? (size_t)kThreads * 8 : 0) +
          (size_t)(kWarps / group) * workspace_bytes(cap, group, sizeof(uint16_t), weighted, pix);
 }
 
 // Largest row capacity (a multiple of 16, at most want) of a launch, 0 if
 // not even 16 fit.
-int fit_cap(int want, int64_t hot, int group, bool parity, bool weighted, bool pix, size_t avail) {
+int fit_cap(int want, int64_t cells, int group, bool weighted, bool pix, size_t avail) {
   int cap = (want + 15) & ~15;
-  while (cap >= 16 && launch_smem(hot, cap, group, parity, weighted, pix) > avail) cap -= 16;
+  while (cap >= 16 && launch_smem(cells, cap, group, weighted, pix) > avail) cap -= 16;
   return std::max(cap, 0);
 }
 }  // namespace
@@ -1232,8 +1309,12 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   const int maxd = std::max(g.max_deg, 3);
   const double mean = g.n ? (double)g.edges_total / (double)g.n : 0.0;
   int group = kWarps, cap = 0, cap2 = 0, nh = no;
+  const int64_t per = parity ? 2 : 1;  // cells per slot
+  int64_t room = 0;                   // cells that fit
+  bool even_cells = false, probe = false;  // ZERO, and whether a sample of volumes decides on it
+  a.even_hot = 0;
   const bool all_hot = !weighted && !(o.variant & 8) &&
-                       fit_cap(std::min(256, maxd), no, kWarps, parity, false, pix, avail) >=
+                       fit_cap(std::min(256, maxd), per * no, kWarps, false, pix, avail) >=
                            std::min(256, (maxd + 15) & ~15);
   if (all_hot) {
     // few warps per hub where rows are short: a hub's barriers and its rows'
@@ -1241,29 +1322,34 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     group = mean <= 24 ? 1 : mean <= 48 ? 4 : mean <= 96 ? 8 : mean <= 160 ? 16 : 32;
     const int want = std::min(maxd, std::max(48, (int)(2.0 * mean) + 32));
     for (;; group = group == 1 ? 4 : group * 2) {
-      cap = fit_cap(maxd, no, group, parity, false, pix, avail);
+      cap = fit_cap(maxd, per * no, group, false, pix, avail);
       if (cap >= want || group == kWarps) break;
     }
-    cap2 = fit_cap(std::min(maxd, kMaxSmemRow), no, kWarps, parity, false, pix, avail);
+    cap2 = fit_cap(std::min(maxd, kMaxSmemRow), per * no, kWarps, false, pix, avail);
   } else {
     // as many slots as fit beside the workspace: of rows of up to 352 when
     // weighted (1e5 clustered points, nb = 8: rows beyond 256 took 114 of 400 ms
     // in global scratch; the 3,300 slots left hold all but 0.3% of tetrahedra)
-    const size_t per_slot = (size_t)(parity ? 2 : 1) * (weighted ? 16 : 4);
     cap = std::min(weighted ? 352 : 256, (maxd + 15) & ~15);
-    const size_t fixed = launch_smem(0, cap, group, parity, weighted, pix) + 32;
-    nh = (int)std::min<size_t>((size_t)no, (avail - fixed) / per_slot);
+    room = (int64_t)((avail - launch_smem(0, cap, group, weighted, pix) - 32) / (weighted ? 16 : 4));
     cap2 = cap;
     // variant 8: only 64 shared slots (exercises the global path of the other
     // orbits on any input)
+    if (o.variant & 8) room = std::min<int64_t>(room, 64 * 3);
+    nh = (int)std::min<int64_t>(no, room / per);
     if (o.variant & 8) nh = std::min(nh, 64);
+    if (weighted && parity) {
+      probe = !(o.variant & 8);
+      even_cells = !probe;
+      if (even_cells) a.even_hot = nh;
+    }
   }
   // variant 1 sends every hub to the global workspace (exercises it on any
   // input)
   if (o.variant & 1) cap = cap2 = 2;
   // with fewer slots than orbits the orbits are relabelled (most frequent
   // first) and the per-slot results mapped back at the end
-  const bool relabel = nh < no;
+  const bool relabel = nh < no || (probe && room < 3 * (int64_t)no);
   unsigned long long* s_even = a.even;
   unsigned long long* s_odd = a.odd;
   unsigned long long* const o_odd = a.odd;  // odd counts in orbit order (caller's or scratch)
@@ -1271,7 +1357,8 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   const int64_t nl = (int64_t)t->lut.size() / g.nb * (g.nb + 1);
   void* d_ent = sc.alloc_bytes((size_t)nl * (small_ent ? 2 : 4));
   uint8_t* d_chir = sc.alloc<uint8_t>(no);
-  if (!d_ent || !d_chir) return GS_ENOMEM;
+  unsigned* d_probe = probe ? sc.alloc<unsigned>(2) : nullptr;
+  if (!d_ent || !d_chir || (probe && !d_probe)) return GS_ENOMEM;
   unsigned long long* d_sample = nullptr;  // counts of the sample that ranks the orbits
   if (relabel) {
     d_sample = sc.alloc<unsigned long long>(no);
@@ -1328,14 +1415,35 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   a.gscratch_stride = 0;
   a.gcap = maxd;
 
-  auto pick = [&](bool P, bool Wt, bool X, bool fast) {
-    return small_ent ? pick4<uint16_t>(P, Wt, X, fast) : pick4<uint32_t>(P, Wt, X, fast);
+  auto pick = [&](bool P, bool Wt, bool X, bool variant) {
+    return small_ent ? pick4<uint16_t>(P, Wt, X, variant) : pick4<uint32_t>(P, Wt, X, variant);
   };
   auto launch = [&](void (*k)(Args), const Args& la, int grid, size_t smem) -> int {
     allow_shared(k, smem);
     cudaMemsetAsync(la.hub_counter, 0, sizeof(unsigned long long), s);
     k<<<grid, kThreads, smem, s>>>(la);
     note_launch();
+    return cuda_status(cudaGetLastError());
+  };
+
+  // Weighted parity: even-only cells take instructions and room from the others,
+  // worth it when more than one volume in 64 is zero (planes, meshes, pixels);
+  // such a tetrahedron costs a global 192-bit sum otherwise. A third of the room,
+  // or three quarters where most volumes are zero. 2e4 points in a plane, nb = 8:
+  // 166 ms against 691 without.
+  auto probe_zero = [&](const Args& wa) -> int {
+    unsigned h[2] = {0, 0};
+    cudaMemsetAsync(d_probe, 0, sizeof(h), s);
+    k_zero_volumes<<<64, 256, 0, s>>>(wa, pix ? 1 : 0, d_probe);
+    note_launch();
+    cudaMemcpyAsync(h, d_probe, sizeof(h), cudaMemcpyDeviceToHost, s);
+    const cudaError_t e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cuda_status(e);
+    if (64ull * h[0] > h[1]) {
+      even_cells = true;
+      a.even_hot = (int)std::min<int64_t>(no, 2ull * h[0] > h[1] ? room * 3 / 4 : room / 3);
+      nh = (int)std::min<int64_t>(no, (room - a.even_hot) / 2);
+    }
     return cuda_status(cudaGetLastError());
   };
 
@@ -1348,21 +1456,22 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     std::vector<int32_t> slot_of(no);
     std::vector<int32_t> order(no);
     for (int k = 0; k < no; ++k) order[k] = k;
-    const int cap_s = fit_cap(std::min(maxd, 256), no, kWarps, false, false, false, avail);
-    if (cap_s >= 16) {
+    const int cap_s = fit_cap(std::min(maxd, 256), no, kWarps, false, false, avail);
+    if (nh < no && cap_s >= 16) {
       cudaMemsetAsync(d_sample, 0, sizeof(unsigned long long) * no, s);
       Args sa = wa;
       sa.group = kWarps;
       sa.cap = cap_s;
       sa.dmax = cap_s;
       sa.hot = no;
+      sa.even_hot = 0;
       sa.even = d_sample;
       sa.odd = nullptr;
       sa.weven = sa.wodd = nullptr;
       sa.W = nullptr;
       sa.hub_stride = std::max<int64_t>(1, (wa.hub_end - wa.hub_begin) / 2048);
       int ls = launch(pick(false, false, false, true), sa, sms,
-                      launch_smem(no, cap_s, kWarps, false, false, false));
+                      launch_smem(no, cap_s, kWarps, false, false));
       if (ls) return ls;
       std::vector<unsigned long long> cnt(no);
       cudaMemcpyAsync(cnt.data(), d_sample, sizeof(unsigned long long) * no,
@@ -1386,7 +1495,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   std::vector<int64_t> longer;  // hubs of rows beyond cap, their device copy and their CTAs
   int64_t* d_list = nullptr;
   int grid2 = 0;
-  void (*kern)(Args) = pick(parity, weighted, pix, all_hot);
+  void (*kern)(Args) = pick(parity, weighted, pix, weighted ? even_cells : all_hot);
   st = for_each_window(g, o, sc, [&](const WinView& v) -> int {
     a.adj = v.adj;
     a.adj_off = v.off1;
@@ -1397,6 +1506,12 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     a.group = group;
     a.cap = cap;
     a.dmax = cap;
+    if (first && probe) {
+      const int ps = probe_zero(a);
+      if (ps) return ps;
+      a.hot = nh;
+      kern = pick(parity, weighted, pix, even_cells);
+    }
     if (first && relabel) {
       const int rs = relabel_orbits(a);
       if (rs) return rs;
@@ -1404,7 +1519,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     first = false;
     int ls = GS_OK;
     if (cap >= 3)
-      ls = launch(kern, a, sms, launch_smem(nh, cap, group, parity, weighted, pix));
+      ls = launch(kern, a, sms, launch_smem(per * nh + a.even_hot, cap, group, weighted, pix));
     if (ls || maxd <= cap) return ls;
     // the longer rows
     const int64_t l0 = std::lower_bound(longer.begin(), longer.end(), v.h0) - longer.begin(),
@@ -1416,7 +1531,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     la.group = kWarps;
     la.cap = cap2;
     return launch(kern, la, (int)std::min<int64_t>(grid2, la.nlist),
-                  launch_smem(nh, cap2, kWarps, parity, weighted, pix));
+                  launch_smem(per * nh + a.even_hot, cap2, kWarps, weighted, pix));
   }, [&]() -> int {
     // the hubs of longer rows, in ascending order, and the workspace of those
     // beyond the shared one: of as many CTAs as there is memory for

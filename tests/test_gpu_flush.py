@@ -31,6 +31,13 @@ def planes(n, box_u):
     return X.astype(np.int32), box_u
 
 
+def patch(n, box_u):
+    """Uniform points, one in 20 on a plane."""
+    X = np.random.default_rng(n).integers(0, box_u, size=(n, 3))
+    X[::20, 2] = 5000
+    return X.astype(np.int32), box_u
+
+
 # rows of about 15, 27, 60 and 100: 1, 4, 8 and 16 warps per hub
 CATALOGUES = [(mesh, (20,), 2100), (mesh, (18,), 2300), (mesh, (14,), 3100), (mesh, (15,), 3700),
               (planes, (7000, 40_000), 4000), (planes, (13_000, 40_000), 4000),
@@ -72,11 +79,13 @@ def test_3pcf_flush_between_groups(gs, kind, args, rmax, rmin, weighted):
 
 @pytest.mark.parametrize("nb", [3, 5, 9])
 @pytest.mark.parametrize("kind,args,rmax", [CATALOGUES[k] for k in (0, 2, 4, 6)] + [
-    (planes, (3, 17_000), 4000), (planes, (12, 17_000), 4000), (planes, (150, 17_000), 4000)])
+    (planes, (3, 17_000), 4000), (planes, (12, 17_000), 4000), (planes, (150, 17_000), 4000),
+    (patch, (1000, 17_000), 4000)])
 def test_volumes_of_zero(gs, kind, args, rmax, nb):
     """V = 0 tetrahedra in even and odd numbers per orbit, unweighted (all orbits
     or 64 in shared memory, rows in global memory) and with weights of both
-    signs."""
+    signs (cells for V = 0 on planes and meshes, none for a few coplanar points
+    among others)."""
     X, box_u = kind(*args)
     edges = np.linspace(0, rmax, nb + 1).astype(np.int64)
     og, g = oracle.Graph(X, box_u, edges), gs.gs_build_graph(X, box_u, edges)
