@@ -111,6 +111,8 @@ struct Args {
   unsigned long long* odd;
   unsigned long long* weven;  // [n_orbits][3] 192-bit
   unsigned long long* wodd;
+  unsigned long long* limbs;  // weighted: see record_limbs
+  uint32_t even_limbs;        // its first cell of the even channel alone
   const int64_t* __restrict__ W;
   const float4* __restrict__ pixu;  // pixelised parity: unit vectors of the pixel centres
   unsigned long long* hub_counter;
@@ -422,29 +424,43 @@ __device__ inline uint32_t take_turn(const Hist& h, uint32_t slot) {
   return 2u * slot + (atomicXor(h.cnt + 2u * slot, kTurn) >> 31);
 }
 
-// One tetrahedron straight to the global counts and sums. cell: twice the slot
-// plus the sign (parity) or the slot; deg: V = 0 on a chiral orbit, even
-// channel only. Wab = W_a W_b.
-template <bool PARITY, bool WEIGHTED>
-__device__ inline void record_global(const Args& a, uint32_t cell, bool deg, int64_t Wi,
-                                     int64_t Wab, int Wc) {
+// One tetrahedron straight to the global counts. cell: twice the slot plus the
+// sign (parity) or the slot; odd: of the odd channel too.
+template <bool PARITY>
+__device__ inline void record_global(const Args& a, uint32_t cell, bool odd) {
   const uint32_t slot = PARITY ? cell >> 1 : cell;
-  const bool neg = PARITY && (cell & 1u);
-  const bool odd = PARITY && !deg && a.chir[slot];
   atomicAdd(a.even + slot, 1ull);
-  if (odd) atomicAdd(a.odd + slot, neg ? ~0ull : 1ull);
-  if constexpr (WEIGHTED) {
-    long long plo, phi;
-    mul_i128(Wab, Wi * (int64_t)Wc, &plo, &phi);  // (W_a W_b)(W_i W_c), below 2^120
-    unsigned long long lo = (unsigned long long)plo, hi = (unsigned long long)phi;
-    atomic_add_i192(a.weven + 3 * (size_t)slot, lo, hi);
-    if (odd) {
-      if (neg) {  // negate the 128-bit product
-        lo = ~lo + 1ull;
-        hi = ~hi + (lo == 0ull ? 1ull : 0ull);
-      }
-      atomic_add_i192(a.wodd + 3 * (size_t)slot, lo, hi);
-    }
+  if (PARITY && odd) atomicAdd(a.odd + slot, (cell & 1u) ? ~0ull : 1ull);
+}
+
+// A weighted one, by cell (parity: 2 n_orbits + slot for the even channel alone):
+// the count and the product (W_a W_b)(W_i W_c), below 2^120, in limbs of 25 bits
+// (the top one is zero for weights within a factor of two), each to a word of its
+// own. Nothing waits for a returned value, as carries
+// between words would, and the two channels are told apart at the end (k_limbs):
+// with few lanes of a warp at it, the round trips of 192-bit sums in both channels
+// were the whole time (rows of 30, nb = 12, where few orbits have shared cells:
+// 42 -> 15.7 ms).
+constexpr int kLimbs = 5, kLimbBits = 25, kLimbWords = 1 + kLimbs;
+// Additions that a word may take between two passes of k_limbs (it holds twice as
+// many): launches are split to stay below.
+constexpr double kLimbAdds = 274877906944.0;  // 2^38
+__device__ inline void record_limbs(unsigned long long* limbs, uint32_t cell, int64_t Wi,
+                                    int64_t Wab, int Wc) {
+  unsigned long long* L = limbs + (size_t)cell * kLimbWords;
+  long long lo, hi;
+  mul_i128(Wab, Wi * (int64_t)Wc, &lo, &hi);
+  atomicAdd(L, 1ull);
+#pragma unroll
+  for (int k = 0; k < kLimbs; ++k) {
+    // the lowest limb left; the top one keeps the sign
+    const unsigned long long x = k + 1 < kLimbs
+                                     ? (unsigned long long)lo & ((1ull << kLimbBits) - 1ull)
+                                     : (unsigned long long)lo;
+    if (x) atomicAdd(L + 1 + k, x);
+    lo = (long long)(((unsigned long long)lo >> kLimbBits) |
+                     ((unsigned long long)hi << (64 - kLimbBits)));
+    hi >>= kLimbBits;
   }
 }
 
@@ -850,11 +866,12 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
                       at[u] = cell[u] < hotce ? cells + 4u * cell[u] : none;
                     }
                     if (at[u] == none)
-                      record_global<PARITY, true>(
-                          a, en[u] >= 0 || deg ? 2u * (cell[u] - cells2) : cell[u], deg, Wi, wab[u],
-                          Wc);
+                      record_limbs(a.limbs,
+                                   en[u] >= 0 || deg ? a.even_limbs + (cell[u] - cells2) : cell[u],
+                                   Wi, wab[u], Wc);
                   } else if (deg || cell[u] >= hotc) {
-                    record_global<PARITY, true>(a, cell[u], deg, Wi, wab[u], Wc);
+                    record_limbs(a.limbs, deg ? a.even_limbs + (cell[u] >> 1) : cell[u], Wi, wab[u],
+                                 Wc);
                   }
                 }
               }
@@ -902,7 +919,7 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
               }
               if (PARITY && deg && cell < hotc) cell = take_turn(h, cell >> 1);
               if (cell < hotc) atomicAdd(h.cnt + cell, 1u);
-              else record_global<PARITY, false>(a, cell, deg, 0, 0, 0);
+              else record_global<PARITY>(a, cell, !deg && (e[u] >> Ent<E>::kTop));
             }
           }
         }
@@ -1073,6 +1090,62 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
 }
 
 }  // namespace
+
+// 192-bit sums: x += y or x -= y.
+__device__ inline void add_w192(unsigned long long (&x)[3], const unsigned long long (&y)[3],
+                                bool minus) {
+  unsigned long long c = minus ? 1ull : 0ull;
+  for (int k = 0; k < 3; ++k) {
+    const unsigned long long v = minus ? ~y[k] : y[k], s = x[k] + v;
+    const unsigned long long t = s + c;
+    c = (s < v ? 1ull : 0ull) + (t < s ? 1ull : 0ull);
+    x[k] = t;
+  }
+}
+
+// Adds the limbs (see record_limbs) of every slot to its counts and 192-bit sums
+// and clears them. odd, wodd: nullptr without parity.
+__global__ void k_limbs(unsigned long long* limbs, int64_t n, const uint8_t* chir,
+                        unsigned long long* even, unsigned long long* odd,
+                        unsigned long long* weven, unsigned long long* wodd) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    unsigned long long cnt[3] = {0, 0, 0}, sum[3][3] = {};
+    const int cells = odd ? 3 : 1;
+    bool any = false;
+    for (int c = 0; c < cells; ++c) {
+      unsigned long long* L =
+          limbs + (size_t)(odd ? (c < 2 ? 2 * k + c : 2 * n + k) : k) * kLimbWords;
+      cnt[c] = L[0];
+      if (!cnt[c]) continue;
+      any = true;
+      L[0] = 0ull;
+      for (int q = 0; q < kLimbs; ++q) {
+        const unsigned long long v = L[1 + q];
+        L[1 + q] = 0ull;
+        const unsigned long long ext = q + 1 == kLimbs && (long long)v < 0 ? ~0ull : 0ull;
+        const int sh = q * kLimbBits, w = sh >> 6, r = sh & 63;
+        unsigned long long y[3] = {0, 0, 0};
+        const unsigned long long part[2] = {v << r, r ? (v >> (64 - r)) | (ext << r) : ext};
+        for (int p = w; p < 3; ++p) y[p] = p - w < 2 ? part[p - w] : ext;
+        add_w192(sum[c], y, false);
+      }
+    }
+    if (!any) continue;
+    even[k] += cnt[0] + cnt[1] + cnt[2];
+    unsigned long long* E = weven + 3 * k;
+    unsigned long long x[3] = {E[0], E[1], E[2]};
+    for (int c = 0; c < cells; ++c) add_w192(x, sum[c], false);
+    for (int q = 0; q < 3; ++q) E[q] = x[q];
+    if (!odd || !chir[k]) continue;
+    odd[k] += cnt[0] - cnt[1];
+    unsigned long long* O = wodd + 3 * k;
+    unsigned long long z[3] = {O[0], O[1], O[2]};
+    add_w192(z, sum[0], false);
+    add_w192(z, sum[1], true);
+    for (int q = 0; q < 3; ++q) O[q] = z[q];
+  }
+}
 
 __global__ void k_i192_to_double(const unsigned long long* acc, int64_t n, int scale, double* out);
 __global__ void k_u64_to_double(const unsigned long long* c, int64_t n, double* out);
@@ -1291,8 +1364,11 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
                                                   : nullptr;
   a.weven = weven;
   a.wodd = wodd;
+  const size_t limb_words = weighted ? (size_t)(parity ? 3 : 1) * no * kLimbWords : 0;
+  a.limbs = weighted ? sc.alloc<unsigned long long>(limb_words) : nullptr;
+  a.even_limbs = 2u * (uint32_t)no;
   a.hub_counter = sc.alloc<unsigned long long>(1);
-  if (!a.hub_counter || (parity && !a.odd) || (weighted && !a.weven) ||
+  if (!a.hub_counter || (parity && !a.odd) || (weighted && (!a.weven || !a.limbs)) ||
       (weighted && parity && !a.wodd))
     return GS_ENOMEM;
 
@@ -1377,6 +1453,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   if (parity) cudaMemsetAsync(s_odd, 0, sizeof(uint64_t) * no, s);
   if (a.weven) cudaMemsetAsync(a.weven, 0, sizeof(unsigned long long) * 3 * no, s);
   if (a.wodd) cudaMemsetAsync(a.wodd, 0, sizeof(unsigned long long) * 3 * no, s);
+  if (a.limbs) cudaMemsetAsync(a.limbs, 0, sizeof(unsigned long long) * limb_words, s);
   a.even = s_even;
   a.odd = s_odd;
   a.hot = nh;
@@ -1424,6 +1501,41 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     k<<<grid, kThreads, smem, s>>>(la);
     note_launch();
     return cuda_status(cudaGetLastError());
+  };
+
+  // The same over the hubs of la, rows of at most `rows`, in as many launches as
+  // the limbs of weighted sums allow.
+  double added = 0.0;
+  auto fold_limbs = [&]() -> int {
+    if (!weighted) return GS_OK;
+    k_limbs<<<(int)std::min<int64_t>((no + 255) / 256, 4096), 256, 0, s>>>(
+        a.limbs, no, a.chir, a.even, parity ? a.odd : nullptr, a.weven, parity ? a.wodd : nullptr);
+    note_launch();
+    added = 0.0;
+    return cuda_status(cudaGetLastError());
+  };
+  auto launch_hubs = [&](void (*k)(Args), const Args& la, int grid, size_t smem, int rows) -> int {
+    if (!weighted) return launch(k, la, grid, smem);
+    const double hub = std::max(1.0, (double)rows * (rows - 1.0) * (rows - 2.0) / 6.0);
+    const int64_t n = la.list ? la.nlist : la.hub_end - la.hub_begin,
+                  step = (o.variant & 1024) ? 256  // exercises the split
+                                            : std::max<int64_t>(1, (int64_t)(kLimbAdds / hub));
+    int ls = GS_OK;
+    for (int64_t h = 0; h < n && !ls; h += step) {
+      const int64_t m = std::min(step, n - h);
+      if (added > 0.0 && (added + (double)m * hub > kLimbAdds || (o.variant & 1024))) ls = fold_limbs();
+      Args part = la;
+      if (la.list) {
+        part.list = la.list + h;
+        part.nlist = m;
+      } else {
+        part.hub_begin = la.hub_begin + h;
+        part.hub_end = part.hub_begin + m;
+      }
+      added += (double)m * hub;
+      if (!ls) ls = launch(k, part, grid, smem);
+    }
+    return ls;
   };
 
   // Weighted parity: even-only cells take instructions and room from the others,
@@ -1519,7 +1631,8 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     first = false;
     int ls = GS_OK;
     if (cap >= 3)
-      ls = launch(kern, a, sms, launch_smem(per * nh + a.even_hot, cap, group, weighted, pix));
+      ls = launch_hubs(kern, a, sms, launch_smem(per * nh + a.even_hot, cap, group, weighted, pix),
+                       cap);
     if (ls || maxd <= cap) return ls;
     // the longer rows
     const int64_t l0 = std::lower_bound(longer.begin(), longer.end(), v.h0) - longer.begin(),
@@ -1530,8 +1643,8 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     la.nlist = l1 - l0;
     la.group = kWarps;
     la.cap = cap2;
-    return launch(kern, la, (int)std::min<int64_t>(grid2, la.nlist),
-                  launch_smem(per * nh + a.even_hot, cap2, kWarps, weighted, pix));
+    return launch_hubs(kern, la, (int)std::min<int64_t>(grid2, la.nlist),
+                       launch_smem(per * nh + a.even_hot, cap2, kWarps, weighted, pix), maxd);
   }, [&]() -> int {
     // the hubs of longer rows, in ascending order, and the workspace of those
     // beyond the shared one: of as many CTAs as there is memory for
@@ -1561,6 +1674,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     a.gscratch = staging(sc, a.gscratch_stride, &grid2);
     return a.gscratch ? GS_OK : GS_ENOMEM;
   });
+  if (!st) st = fold_limbs();
   if (st) return st;
   if (relabel) {
     auto back = [&](const unsigned long long* src, int words, unsigned long long* dst) {

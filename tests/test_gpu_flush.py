@@ -93,9 +93,28 @@ def test_volumes_of_zero(gs, kind, args, rmax, nb):
     w = (rng.uniform(0.5, 1.5, len(X)) * np.where(rng.random(len(X)) < 0.5, -1, 1)).astype(np.float32)
     for pix in (False, True):
         ref = og.count_4pcf(w, pixel=pix)
-        for variant in (0, 1, 8):
+        for variant in (0, 1, 8, 1024, 1024 + 8):
             got = gs.gs_count_4pcf_parity(g, w, pix=pix, variant=variant)
             for a, b in zip(got, ref):
                 assert np.array_equal(a, b), (pix, variant)
             got = gs.gs_count_4pcf_parity(g, pix=pix, variant=variant)
             assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1]), (pix, variant)
+
+
+@pytest.mark.parametrize("signed", [False, True])
+@pytest.mark.parametrize("nb", [5, 10, 12])
+def test_orbits_without_shared_cells(gs, nb, signed):
+    """Weighted sums of orbits that have no cells in shared memory: 64 orbits in
+    it (variant 8), launches of 256 hubs (1024), weights of the full 30 bits."""
+    X, box_u = planes(3000, 17_000) if nb == 5 else patch(2500, 17_000)
+    edges = np.linspace(0, 4000, nb + 1).astype(np.int64)
+    og, g = oracle.Graph(X, box_u, edges), gs.gs_build_graph(X, box_u, edges)
+    rng = np.random.default_rng(nb)
+    w = 2.0 ** rng.uniform(-4.9, 0.0, len(X)) * np.where(rng.random(len(X)) < 0.5 * signed, -1.0, 1.0)
+    w = w.astype(np.float32)
+    ref = og.count_4pcf(w)
+    for variant in (0, 8, 1024, 1024 + 8):
+        for a, b in zip(gs.gs_count_4pcf_parity(g, w, variant=variant), ref):
+            assert np.array_equal(a, b), variant
+        even, weven = gs.gs_count_4pcf(g, w, variant=variant)
+        assert np.array_equal(even, ref[0]) and np.array_equal(weven, ref[2]), variant
