@@ -1405,8 +1405,12 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   } else {
     // as many slots as fit beside the workspace: of rows of up to 352 when
     // weighted (1e5 clustered points, nb = 8: rows beyond 256 took 114 of 400 ms
-    // in global scratch; the 3,300 slots left hold all but 0.3% of tetrahedra)
+    // in global scratch; the 3,300 slots left hold all but 0.3% of tetrahedra),
+    // longer ones where every slot fits all the same (a clump of 400, nb = 5: 38 ->
+    // 25 ms)
     cap = std::min(weighted ? 352 : 256, (maxd + 15) & ~15);
+    if (weighted)
+      cap = std::max(cap, fit_cap(std::min(maxd, kMaxSmemRow), per * no, kWarps, true, pix, avail));
     room = (int64_t)((avail - launch_smem(0, cap, group, weighted, pix) - 32) / (weighted ? 16 : 4));
     cap2 = cap;
     // variant 8: only 64 shared slots (exercises the global path of the other

@@ -118,3 +118,15 @@ def test_orbits_without_shared_cells(gs, nb, signed):
             assert np.array_equal(a, b), variant
         even, weven = gs.gs_count_4pcf(g, w, variant=variant)
         assert np.array_equal(even, ref[0]) and np.array_equal(weven, ref[2]), variant
+
+
+def test_weighted_rows_beyond_352(gs):
+    """Few bins: all orbits have shared cells beside the workspace of rows of
+    more than 352."""
+    X = (50_000 + np.random.default_rng(2).integers(-2500, 2501, size=(368, 3))).astype(np.int32)
+    edges = np.array([0, 4000, 9000], dtype=np.int64)
+    w = np.random.default_rng(3).uniform(0.5, 1.5, len(X)).astype(np.float32)
+    g = gs.gs_build_graph(X, 200_000, edges)
+    assert gs.gs_graph_info(g)["max_degree"] > 352
+    for a, b in zip(gs.gs_count_4pcf_parity(g, w), oracle.Graph(X, 200_000, edges).count_4pcf(w)):
+        assert np.array_equal(a, b)
