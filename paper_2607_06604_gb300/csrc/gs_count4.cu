@@ -1392,10 +1392,13 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   const bool all_hot = !weighted && !(o.variant & 8) &&
                        fit_cap(std::min(256, maxd), per * no, kWarps, false, pix, avail) >=
                            std::min(256, (maxd + 15) & ~15);
+  // few warps per hub where rows are short: a hub's barriers and its rows' ragged
+  // ends cost the same however many warps wait for them
+  auto warps_per_hub = [](double m) {
+    return m <= 24 ? 1 : m <= 48 ? 4 : m <= 96 ? 8 : m <= 160 ? 16 : kWarps;
+  };
   if (all_hot) {
-    // few warps per hub where rows are short: a hub's barriers and its rows'
-    // ragged ends cost the same however many warps wait for them
-    group = mean <= 24 ? 1 : mean <= 48 ? 4 : mean <= 96 ? 8 : mean <= 160 ? 16 : 32;
+    group = warps_per_hub(mean);
     const int want = std::min(maxd, std::max(48, (int)(2.0 * mean) + 32));
     for (;; group = group == 1 ? 4 : group * 2) {
       cap = fit_cap(maxd, per * no, group, false, pix, avail);
@@ -1411,6 +1414,13 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     cap = std::min(weighted ? 352 : 256, (maxd + 15) & ~15);
     if (weighted)
       cap = std::max(cap, fit_cap(std::min(maxd, kMaxSmemRow), per * no, kWarps, true, pix, avail));
+    // unweighted, groups as above while their workspaces take a quarter at most
+    if (!weighted) {
+      group = warps_per_hub(mean);
+      while (group < kWarps &&
+             (kWarps / group) * workspace_bytes(cap, group, sizeof(uint16_t), false, pix) > avail / 4)
+        group = group == 1 ? 4 : group * 2;
+    }
     room = (int64_t)((avail - launch_smem(0, cap, group, weighted, pix) - 32) / (weighted ? 16 : 4));
     cap2 = cap;
     // variant 8: only 64 shared slots (exercises the global path of the other
@@ -1564,8 +1574,8 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   };
 
   // Relabelling: count the tetrahedra of every orbit over an evenly strided
-  // sample of about 2048 hubs of the first window (unweighted, all slots in
-  // shared memory, long rows skipped), rank the orbits by that count and
+  // sample of about 2048 hubs of the first window (at most a quarter of them;
+  // unweighted, all slots in shared memory, long rows skipped), rank the orbits by that count and
   // give the top nh the shared slots. Where that count kernel does not fit,
   // the orbits keep their order. The choice changes only the speed.
   auto relabel_orbits = [&](const Args& wa) -> int {
@@ -1585,7 +1595,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
       sa.odd = nullptr;
       sa.weven = sa.wodd = nullptr;
       sa.W = nullptr;
-      sa.hub_stride = std::max<int64_t>(1, (wa.hub_end - wa.hub_begin) / 2048);
+      sa.hub_stride = std::max<int64_t>(4, (wa.hub_end - wa.hub_begin) / 2048);
       int ls = launch(pick(false, false, false, true), sa, sms,
                       launch_smem(no, cap_s, kWarps, false, false));
       if (ls) return ls;
