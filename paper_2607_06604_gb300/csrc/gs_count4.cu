@@ -113,6 +113,7 @@ struct Args {
   unsigned long long* wodd;
   unsigned long long* limbs;  // weighted: see record_limbs
   uint32_t even_limbs;        // its first cell of the even channel alone
+  unsigned long long limb_need;  // tetrahedra of a hub whose sums times W_i fit the limbs
   const int64_t* __restrict__ W;
   const float4* __restrict__ pixu;  // pixelised parity: unit vectors of the pixel centres
   unsigned long long* hub_counter;
@@ -445,12 +446,7 @@ constexpr int kLimbs = 5, kLimbBits = 25, kLimbWords = 1 + kLimbs;
 // Additions that a word may take between two passes of k_limbs (it holds twice as
 // many): launches are split to stay below.
 constexpr double kLimbAdds = 274877906944.0;  // 2^38
-__device__ inline void record_limbs(unsigned long long* limbs, uint32_t cell, int64_t Wi,
-                                    int64_t Wab, int Wc) {
-  unsigned long long* L = limbs + (size_t)cell * kLimbWords;
-  long long lo, hi;
-  mul_i128(Wab, Wi * (int64_t)Wc, &lo, &hi);
-  atomicAdd(L, 1ull);
+__device__ inline void add_limbs(unsigned long long* L, long long lo, long long hi) {
 #pragma unroll
   for (int k = 0; k < kLimbs; ++k) {
     // the lowest limb left; the top one keeps the sign
@@ -462,6 +458,14 @@ __device__ inline void record_limbs(unsigned long long* limbs, uint32_t cell, in
                      ((unsigned long long)hi << (64 - kLimbBits)));
     hi >>= kLimbBits;
   }
+}
+__device__ inline void record_limbs(unsigned long long* limbs, uint32_t cell, int64_t Wi,
+                                    int64_t Wab, int Wc) {
+  unsigned long long* L = limbs + (size_t)cell * kLimbWords;
+  long long lo, hi;
+  mul_i128(Wab, Wi * (int64_t)Wc, &lo, &hi);
+  atomicAdd(L, 1ull);
+  add_limbs(L, lo, hi);
 }
 
 // Two weighted tetrahedra with products Wc V[] in the cells at[] (shared
@@ -1062,6 +1066,24 @@ __global__ void __launch_bounds__(kThreads, 1) k_count4(Args a) {
           c[2 * h.stride] = kTopZero;
         }
       };
+      // a hub of few tetrahedra: every cell's sum times W_i is below 2^124 and
+      // goes to the limbs of its cell, which waits for nothing (1e5 points, rows
+      // of 8, nb = 8: 5.9 -> 4.9 ms)
+      const unsigned long long mm = (unsigned long long)m;
+      if (mm * (mm - 1) * (mm - 2) / 6 <= a.limb_need) {
+        const int n2 = (PARITY ? 2 : 1) * a.hot, all = n2 + (ZERO ? a.even_hot : 0);
+        for (int k = gt; k < all; k += gthreads) {
+          unsigned long long lo, hi;
+          take(k, lo, hi);
+          if (!(lo | hi)) continue;
+          const unsigned long long v = (unsigned long long)Wi;
+          add_limbs(a.limbs + (size_t)(k < n2 ? (uint32_t)k : a.even_limbs + (uint32_t)(k - n2)) *
+                                  kLimbWords,
+                    (long long)(lo * v),
+                    (long long)(__umul64hi(lo, v) - (Wi < 0 ? lo : 0ull) + hi * v));
+        }
+        continue;
+      }
       for (int k = gt; k < a.hot; k += gthreads) {
         unsigned long long elo, ehi;
         take(PARITY ? 2 * k : k, elo, ehi);
@@ -1116,13 +1138,13 @@ __global__ void k_limbs(unsigned long long* limbs, int64_t n, const uint8_t* chi
     for (int c = 0; c < cells; ++c) {
       unsigned long long* L =
           limbs + (size_t)(odd ? (c < 2 ? 2 * k + c : 2 * n + k) : k) * kLimbWords;
-      cnt[c] = L[0];
-      if (!cnt[c]) continue;
+      unsigned long long l[kLimbs], some = cnt[c] = L[0];
+      for (int q = 0; q < kLimbs; ++q) some |= l[q] = L[1 + q];
+      if (!some) continue;
       any = true;
-      L[0] = 0ull;
+      for (int q = 0; q < kLimbWords; ++q) L[q] = 0ull;
       for (int q = 0; q < kLimbs; ++q) {
-        const unsigned long long v = L[1 + q];
-        L[1 + q] = 0ull;
+        const unsigned long long v = l[q];
         const unsigned long long ext = q + 1 == kLimbs && (long long)v < 0 ? ~0ull : 0ull;
         const int sh = q * kLimbBits, w = sh >> 6, r = sh & 63;
         unsigned long long y[3] = {0, 0, 0};
@@ -1367,6 +1389,8 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   const size_t limb_words = weighted ? (size_t)(parity ? 3 : 1) * no * kLimbWords : 0;
   a.limbs = weighted ? sc.alloc<unsigned long long>(limb_words) : nullptr;
   a.even_limbs = 2u * (uint32_t)no;
+  // (need) 2^(4 mag) < 2^124
+  a.limb_need = weighted && fw->mag < 31 ? (1ull << std::min(40, 123 - 4 * fw->mag)) : 0;
   a.hub_counter = sc.alloc<unsigned long long>(1);
   if (!a.hub_counter || (parity && !a.odd) || (weighted && (!a.weven || !a.limbs)) ||
       (weighted && parity && !a.wodd))
