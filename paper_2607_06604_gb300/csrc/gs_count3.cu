@@ -1327,9 +1327,10 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
   };
   // Adds the cells to the global counts (and sums) and clears them; exchanges,
   // so that one group can do it while the others count on. (Unweighted counters
-  // only grow. Weighted, every word is its additions modulo 2^32 and every carry
-  // is added somewhere, so the global sums are right whichever flush takes a
-  // word or its carry.)
+  // are signed and below 2^31: a count being moved may leave -1 for a while.
+  // Weighted, every word is its additions modulo 2^32 and every carry is added
+  // somewhere, so the global sums are right whichever flush takes a word or its
+  // carry.)
   auto flush = [&](int t, int threads) {
     if (cur < 0) return;
     for (int k = t; k < a.nconf; k += threads) {
@@ -1370,9 +1371,9 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
         if (slo | (unsigned long long)shi)
           atomic_add_i192(c.wacc + 3 * k, slo, (unsigned long long)shi);
       } else {
-        unsigned long long v = 0;
+        long long v = 0;
         auto take = [&](int x, int y, int z) {
-          v += atomicExch(cell + (x * nb + y) * nr + z, 0u);
+          v += (int)atomicExch(cell + (x * nb + y) * nr + z, 0u);
         };
         take(p, q, r);
         if (q != r) take(p, r, q);
@@ -1380,7 +1381,7 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
         if (p != q) take(q, r, p);
         if (p != r && q != r) take(r, p, q);
         if (p != q && p != r && q != r) take(r, q, p);
-        if (v) atomicAdd(c.counts + k, v);
+        if (v) atomicAdd(c.counts + k, (unsigned long long)v);
       }
     }
   };
@@ -1471,18 +1472,25 @@ __global__ void __launch_bounds__(kTThreads, 2) k_count3t(TArgs a) {
       const int4 pj = *reinterpret_cast<const int4*>(S.p + j);
       const int pp[4] = {pj.x, pj.y, pj.z, pj.w};
       if constexpr (!WEIGHTED) {
-        // near an edge the exact bin, before the counter is touched: counters
-        // only grow, so another group's flush may take them at any moment
-        if (near) {
-#pragma unroll
-          for (int v = 0; v < 4; ++v)
-            if ((__float_as_uint(u[v]) & 0xFFFFu) <= a.amb)
-              u[v] = kTileM + 0.5f +
-                     (float)exact_bin(S.x[j + v] - xk, S.y[j + v] - yk, S.z[j + v] - zk);
-        }
 #pragma unroll
         for (int v = 0; v < 4; ++v)
           t_red(base + (uint32_t)pp[v] + 4u * t_bin<LOWER>(u[v], nb), 1u);
+        if (near) {
+          // Move the count of a pair whose exact bin is another. A flush by
+          // another group may come in between and leave -1: flush reads the
+          // counters as signed numbers. (Bins settled before the count cost 1%
+          // of 13.4 ms on three mocks, 4% of 56 ms with rows of 1,000 and more.)
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            if ((__float_as_uint(u[v]) & 0xFFFFu) > a.amb) continue;
+            const int was = (int)(t_bin<LOWER>(u[v], nb) - kBin0<LOWER>);
+            const int b = exact_bin(S.x[j + v] - xk, S.y[j + v] - yk, S.z[j + v] - zk);
+            if (b == was) continue;
+            unsigned* row = cell + (pp[v] + qk) / 4;
+            atomicSub(row + was, 1u);
+            atomicAdd(row + b, 1u);
+          }
+        }
       } else {
         const int4 qj = *reinterpret_cast<const int4*>(S.q + j);
         const int4 wj = *reinterpret_cast<const int4*>(S.W + j);
@@ -2062,12 +2070,13 @@ TileLaunch tile_launch(int nb, int nconf, const FixedW* fw, bool batch, double m
     if (L.cap >= want || group == kTWarps) break;
   }
   // Pairs a cell may take between flushes: 2 limit + (groups + 1) hubs, see
-  // the kernel. Counts below 2^32; weighted, T's halves below 2^15, that is
+  // the kernel. Counts below 2^31; weighted, T's halves below 2^15, that is
   // 2^(15 + cb) pairs.
   // (FOLD: T's halves hold one hub, the counts below 2^32 many.)
   const double hub = 0.5 * max_deg * (max_deg - 1.0);
-  const int room_bits = weighted && !L.fold ? 15 + L.a.cb : 32;
-  L.a.limit = 1ull << (room_bits - 2);
+  const int room_bits = !weighted ? 31 : L.fold ? 32 : 15 + L.a.cb;
+  // (one group: a flush is over before it counts on, and 1 limit + 1 hub)
+  auto limit = [&] { return 1ull << (room_bits - (!weighted && group == kTWarps ? 1 : 2)); };
   if (L.fold && hub >= std::ldexp(1.0, 14 + L.a.cb)) {
     L.cap = 0;
     return L;
@@ -2082,6 +2091,7 @@ TileLaunch tile_launch(int nb, int nconf, const FixedW* fw, bool batch, double m
   }
   L.cap = std::min(L.cap, (max_deg + 31) & ~31);
   if (L.cap < 32) L.cap = 0;
+  L.a.limit = limit();
   L.group = group;
   L.smem = fixed + (size_t)(kTWarps / group) * stage_bytes(L.cap, weighted);
   L.blocks = 2 * sms;
