@@ -1486,6 +1486,8 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
     if (!s_even || (parity && !s_odd) || (weighted && (!a.weven || (parity && !a.wodd))) ||
         !d_slot || !d_sample)
       return GS_ENOMEM;
+    // a call without hubs maps its zeros back by this (in range)
+    cudaMemsetAsync(d_slot, 0, sizeof(int32_t) * no, s);
   }
   cudaMemsetAsync(s_even, 0, sizeof(uint64_t) * no, s);
   if (parity) cudaMemsetAsync(s_odd, 0, sizeof(uint64_t) * no, s);
