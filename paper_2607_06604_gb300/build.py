@@ -28,9 +28,9 @@ def nvcc() -> str:
 
 
 def common_flags() -> list[str]:
-    # host code: no fused multiply-add contraction (the FP64 pixel-volume
-    # table is defined as separately rounded operations; Arm compilers
-    # contract by default)
+    # host code: no fused multiply-add contraction, so that the constants formed
+    # in FP64 on the host (pixel centres, error bounds of the binning) are the
+    # same on both machines (Arm compilers contract by default)
     return ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
                    "-Xcompiler", "-ffp-contract=off",
                    "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]

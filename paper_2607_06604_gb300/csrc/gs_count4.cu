@@ -32,13 +32,13 @@
 // cells in turn (see take_turn). Hubs with more neighbours than the shared
 // workspace holds run with their workspace in global scratch.
 //
-// What bounds it: instruction issue (80% of slots, 32 instructions per step of
-// 14 tetrahedra) and the shared-memory/L1 pipe (73%) together. Measured on one
-// GB300 against a kernel that queued (b, c) pairs per warp and gave every lane
-// one of them (7.5 instructions and two random 16-byte loads per tetrahedron):
-// parity on 2e5 clustered points (8.4e10 tetrahedra) 648 -> 231 ms, pixelised
-// parity on 1e5 (4.2e10) 810 -> 194 ms, connected 4pCF of 5e4 + 5e4 points
-// 520 -> 424 ms, 1e5 points with rows of 26 (mock, build included) 8.5 -> 2.7 ms.
+// What bounds it: the shared-memory pipe (87% of its wavefronts; 73% of issue
+// slots, 24 instructions per step of 14 tetrahedra). Measured on one GB300
+// against a kernel that queued (b, c) pairs per warp and gave every lane one of
+// them (7.5 instructions and two random 16-byte loads per tetrahedron): parity
+// on 2e5 clustered points (8.4e10 tetrahedra) 648 -> 171 ms, pixelised parity on
+// 1e5 (4.2e10) 810 -> 140 ms, connected 4pCF of 5e4 + 5e4 points 520 -> 254 ms,
+// 1e5 points with rows of 26 (mock, build included) 8.5 -> 1.83 ms.
 //
 // When the per-orbit counters of every orbit do not fit in shared memory
 // beside the hub workspace (unweighted: many bins; weighted: see below),
@@ -49,11 +49,13 @@
 // Weighted sums (exact, fixed-point W): the hub's sums of x = W_a W_b W_c are
 // kept per cell in three 32-bit words, one array per word (cells of 16 bytes in
 // a row left an atomic eight of the 32 banks: 4.3 wavefronts each), and
-// multiplied by W_i into the global 192-bit sums when the hub ends; the rare
+// multiplied by W_i into the global sums when the hub ends (into limbs, see
+// record_limbs, where the hub is small enough, else 192-bit sums); the rare
 // carry out of the top word goes there at once. Shared memory holds the words
 // (and the counts) only for the `hot` orbits, as above; a tetrahedron of any
-// other orbit goes straight to the global sums with its full product. Pairs that
-// are no edge update words of the lane's own bank.
+// other orbit goes to the limbs with its full product. Volumes of zero have
+// cells of their own where a sample finds many of them (ZERO). Pairs that are no
+// edge update words of the lane's own bank.
 #include <algorithm>
 #include <cmath>
 #include <mutex>

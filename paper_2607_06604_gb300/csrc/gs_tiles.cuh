@@ -13,7 +13,7 @@ namespace gs {
 constexpr int kTThreads = 512;  // two CTAs per SM
 constexpr int kTWarps = kTThreads / 32;
 // Rows above this are left to the walk and pair kernels: C(8192, 2) < 2^25
-// pairs per hub keep the shared counters below 2^32 between flushes.
+// pairs per hub keep the shared counters below 2^31 between flushes.
 constexpr int kTMaxDeg = 8192;
 // Absent j's and k's stand at these x (in units): farther from every point,
 // and from one another, than twice the largest E_nb (2^19).
