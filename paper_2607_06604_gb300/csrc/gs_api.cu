@@ -516,7 +516,7 @@ int count4_wide(const Graph& g, const FixedW& fw, bool parity, bool pix, uint64_
   for (int k = 0; k < npts && !st; ++k) {
     st = split_weights_device(fw, g.n, wide_eval_point(k), Wt, o.stream);
     if (!st)
-      st = count4_device(g, &ft, parity, d_even, d_odd, nullptr, nullptr, o, sc, pix,
+      st = count4_device(g, &ft, parity, d_even, d_odd, nullptr, nullptr, o, pix,
                          Pe + 3 * (size_t)no * k, parity ? Po + 3 * (size_t)no * k : nullptr);
   }
   if (!st && d_weven) st = combine_wide_device(Pe, no, 4, 4 * fw.scale, d_weven, o.stream);
@@ -863,7 +863,7 @@ static int count4_common(const gs_graph* G, const float* w, bool parity, uint64_
     if (w && fw.bits > kNarrowWeightBits)
       st = count4_wide(g, fw, parity, pix, de, dod, dwe, dwo, o, sc);
     else
-      st = count4_device(g, w ? &fw : nullptr, parity, de, dod, dwe, dwo, o, sc, pix);
+      st = count4_device(g, w ? &fw : nullptr, parity, de, dod, dwe, dwo, o, pix);
     OutBuf outs[4] = {{even, de, sizeof(uint64_t) * nc},
                       {odd, dod, sizeof(int64_t) * nc},
                       {weven, dwe, sizeof(double) * nc},

@@ -1334,9 +1334,10 @@ int fit_cap(int want, int64_t cells, int group, bool weighted, bool pix, size_t 
 }  // namespace
 
 int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_even,
-                  int64_t* d_odd, double* d_weven, double* d_wodd, const Opts& o, Scratch& sc,
-                  bool pix, unsigned long long* weven_out, unsigned long long* wodd_out) {
+                  int64_t* d_odd, double* d_weven, double* d_wodd, const Opts& o, bool pix,
+                  unsigned long long* weven_out, unsigned long long* wodd_out) {
   cudaStream_t s = o.stream;
+  Scratch sc(s);  // given back on return: wide weights make five of these calls
   int st = GS_OK;
   pix = pix && parity;
   const float4* pixu = nullptr;

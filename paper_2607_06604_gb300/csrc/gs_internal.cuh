@@ -214,7 +214,7 @@ int count3_batch_device(const Graph* const* gr, int ng, const FixedW* fws, uint6
                         double* const* d_wsum, const Opts& o, Scratch& sc);
 // pix: the odd channel from pixelised spoke directions (parity only)
 int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_even,
-                  int64_t* d_odd, double* d_weven, double* d_wodd, const Opts& o, Scratch& sc,
+                  int64_t* d_odd, double* d_weven, double* d_wodd, const Opts& o,
                   bool pix = false, unsigned long long* weven_out = nullptr,
                   unsigned long long* wodd_out = nullptr);
 int direction_pixels_device(const int32_t* d_dirs, int64_t n, uint8_t* d_out, cudaStream_t s);

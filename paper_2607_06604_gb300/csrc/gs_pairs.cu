@@ -333,10 +333,10 @@ int connected_device(const Graph& gdr, const FixedW& fdr, const Graph& gr, const
     timer.publish();
   }
   sub.kernel_ms = o.kernel_ms ? ms + 1 : nullptr;
-  st = count4_device(gdr, &fdr, true, cnt, odd, ne, nodd, sub, sc);
+  st = count4_device(gdr, &fdr, true, cnt, odd, ne, nodd, sub);
   if (st) return st;
   sub.kernel_ms = o.kernel_ms ? ms + 2 : nullptr;
-  st = count4_device(gr, &fr, false, cnt, nullptr, re, nullptr, sub, sc);
+  st = count4_device(gr, &fr, false, cnt, nullptr, re, nullptr, sub);
   if (st) return st;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);

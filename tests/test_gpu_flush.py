@@ -130,3 +130,20 @@ def test_weighted_rows_beyond_352(gs):
     assert gs.gs_graph_info(g)["max_degree"] > 352
     for a, b in zip(gs.gs_count_4pcf_parity(g, w), oracle.Graph(X, 200_000, edges).count_4pcf(w)):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [500, 511, 520, 2040, 2060])
+@pytest.mark.parametrize("kind", ["span", "uniform"])
+def test_3pcf_rows_at_the_count_fields_limit(gs, n, kind):
+    """Complete rows on both sides of the lengths up to which the weighted tiles
+    can count pairs beside the sums (512 for weights of 30 bits, 2,048 for weights
+    within a factor of two)."""
+    rng = np.random.default_rng(n)
+    X = (50_000 + rng.integers(-2500, 2501, size=(n, 3))).astype(np.int32)
+    edges = 2560 * np.arange(5, dtype=np.int64)
+    w = 2.0 ** rng.uniform(-4.9, 0.0, n) * np.where(rng.random(n) < 0.5, -1, 1) if kind == "span" \
+        else rng.uniform(0.5, 1.5, n)
+    w = w.astype(np.float32)
+    rc, rw = oracle.Graph(X, 200_000, edges).count_3pcf(w)
+    c, s = gs.gs_count_3pcf(gs.gs_build_graph(X, 200_000, edges), w)
+    assert np.array_equal(c, rc) and np.array_equal(s, rw)

@@ -103,3 +103,22 @@ def test_streamed_calls_fit_beside_little_memory(gs, torch_mod):
             assert np.array_equal(call(), ref), spare
         del held
         torch.cuda.empty_cache()
+
+
+def test_wide_weights_hold_one_evaluations_scratch(gs, torch_mod):
+    """Wide weights make five weighted 4pCF evaluations; their scratch (hundreds of
+    MB at 14 bins) is that of one."""
+    rng = np.random.default_rng(8)
+    X = rng.integers(0, 60_000, size=(3000, 3)).astype(np.int32)
+    edges = np.linspace(0, 9000, 15).astype(np.int64)
+    g = gs.gs_build_graph(X, 60_000, edges)
+    narrow = rng.uniform(0.5, 1.5, len(X)).astype(np.float32)
+    wide = (2.0 ** rng.uniform(-9, 1, len(X))).astype(np.float32)
+    gs.gs_count_4pcf_parity(g, narrow)
+    one = peak(torch_mod, lambda: gs.gs_count_4pcf_parity(g, narrow))[1]
+    got, five = peak(torch_mod, lambda: gs.gs_count_4pcf_parity(g, wide))
+    for a, b in zip(got, oracle.Graph(X, 60_000, edges).count_4pcf(wide)):
+        assert np.array_equal(a, b)
+    # beside it the evaluations' own sums, 10 x 24 bytes an orbit
+    orbits = gs.gs_num_configs(4, 14)
+    assert five < 1.3 * one + 240 * orbits + (64 << 20), (one, five)
