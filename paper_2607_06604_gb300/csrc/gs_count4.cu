@@ -32,7 +32,7 @@
 // cells in turn (see take_turn). Hubs with more neighbours than the shared
 // workspace holds run with their workspace in global scratch.
 //
-// What bounds it: the shared-memory pipe (87% of its wavefronts; 73% of issue
+// What bounds it: the shared-memory pipe (90% of its wavefronts; 71% of issue
 // slots, 24 instructions per step of 14 tetrahedra). Measured on one GB300
 // against a kernel that queued (b, c) pairs per warp and gave every lane one of
 // them (7.5 instructions and two random 16-byte loads per tetrahedron): parity
