@@ -115,6 +115,7 @@ struct Args {
   unsigned long long* wodd;
   unsigned long long* limbs;  // weighted: see record_limbs
   uint32_t even_limbs;        // its first cell of the even channel alone
+  int long_rows;              // see record_sum
   unsigned long long limb_need;  // tetrahedra of a hub whose sums times W_i fit the limbs
   const int64_t* __restrict__ W;
   const float4* __restrict__ pixu;  // pixelised parity: unit vectors of the pixel centres
@@ -468,6 +469,17 @@ __device__ inline void record_limbs(unsigned long long* limbs, uint32_t cell, in
   mul_i128(Wab, Wi * (int64_t)Wc, &lo, &hi);
   atomicAdd(L, 1ull);
   add_limbs(L, lo, hi);
+}
+
+// The same straight to the count and the 192-bit sum of a slot, without parity:
+// half the atomics, but each waits for the carry of the one before. Better where
+// rows are long and more lanes have one (3e4 points, rows of 200, nb = 12: 339 ms
+// against 373 to 411; rows of 30: 22 against 12.8).
+__device__ inline void record_sum(const Args& a, uint32_t slot, int64_t Wi, int64_t Wab, int Wc) {
+  long long lo, hi;
+  atomicAdd(a.even + slot, 1ull);
+  mul_i128(Wab, Wi * (int64_t)Wc, &lo, &hi);
+  atomic_add_i192(a.weven + 3 * (size_t)slot, (unsigned long long)lo, (unsigned long long)hi);
 }
 
 // Two weighted tetrahedra with products Wc V[] in the cells at[] (shared
@@ -876,8 +888,11 @@ __device__ inline void hub4(const Args& a, const Workspace<L>& w, Shared& s, con
                                    en[u] >= 0 || deg ? a.even_limbs + (cell[u] - cells2) : cell[u],
                                    Wi, wab[u], Wc);
                   } else if (deg || cell[u] >= hotc) {
-                    record_limbs(a.limbs, deg ? a.even_limbs + (cell[u] >> 1) : cell[u], Wi, wab[u],
-                                 Wc);
+                    if (!PARITY && a.long_rows)
+                      record_sum(a, cell[u], Wi, wab[u], Wc);
+                    else
+                      record_limbs(a.limbs, deg ? a.even_limbs + (cell[u] >> 1) : cell[u], Wi,
+                                   wab[u], Wc);
                   }
                 }
               }
@@ -1411,6 +1426,7 @@ int count4_device(const Graph& g, const FixedW* fw, bool parity, uint64_t* d_eve
   // the longer ones, in shared memory up to cap2, else in global scratch.
   const int maxd = std::max(g.max_deg, 3);
   const double mean = g.n ? (double)g.edges_total / (double)g.n : 0.0;
+  a.long_rows = mean > 100.0;
   int group = kWarps, cap = 0, cap2 = 0, nh = no;
   const int64_t per = parity ? 2 : 1;  // cells per slot
   int64_t room = 0;                   // cells that fit
